@@ -195,23 +195,30 @@ def _buffers(w, rows):
                    "perm": z(B, N, dtype=i32), "points_out": z(B, N, C), "feat_out": z(B, N, w.feat_c)}}
 
 
+def _inputs(case, w, seed):
+    """The call's inputs on the GPU: some of points [B, N, C], proj [B, K, 3, 4] and feat."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    B, K, call = w.B, w.K, case["call"]
+    maps = (B, K, w.feat_c, w.feat_h, w.feat_w) if call == "maps" else (B, K, w.feat_h, w.feat_w, w.feat_c)
+    s = {}
+    if call != "lidar":
+        s["feat"] = torch.randn(maps, generator=g, device="cuda")
+    if call != "maps":
+        s["points"] = _points(case, w, g, "cuda")
+    if call not in ("lidar", "maps"):
+        s["proj"] = torch.from_numpy(gen.make_projection(w)).cuda()[None].expand(B, -1, -1, -1).contiguous()
+    return s
+
+
 def prepare(case, seed):
     w = _workload(case)
-    g = torch.Generator(device="cuda").manual_seed(seed)
     B, K = w.B, w.K
-    s = {"case": case, "w": w, "bridge": pkg.Bridge(pkg.config_from_workload(w))}
-    maps = (B, K, w.feat_c, w.feat_h, w.feat_w) if case["call"] == "maps" else (B, K, w.feat_h, w.feat_w, w.feat_c)
-    if case["call"] == "lidar":
-        s["points"] = _points(case, w, g, "cuda")
-    else:
-        s["feat"] = torch.randn(maps, generator=g, device="cuda")
-        if case["call"] == "maps":
-            p = case["pool"]
-            s["last"] = torch.zeros((B, K, w.feat_h, w.feat_w, w.feat_c), device="cuda")
-            s["pooled"] = torch.zeros((B, K, -(-w.feat_h // p), -(-w.feat_w // p), w.feat_c), device="cuda")
-            return s
-        s["points"] = _points(case, w, g, "cuda")
-        s["proj"] = torch.from_numpy(gen.make_projection(w)).cuda()[None].expand(B, -1, -1, -1).contiguous()
+    s = {"case": case, "w": w, "bridge": pkg.Bridge(pkg.config_from_workload(w)), **_inputs(case, w, seed)}
+    if case["call"] == "maps":
+        p = case["pool"]
+        s["last"] = torch.zeros((B, K, w.feat_h, w.feat_w, w.feat_c), device="cuda")
+        s["pooled"] = torch.zeros((B, K, -(-w.feat_h // p), -(-w.feat_w // p), w.feat_c), device="cuda")
+        return s
     s["bufs"] = _buffers(w, case["rows"] or case["call"] != "bridge")
     M = B * w.N
     if case["call"] == "staged":
@@ -259,6 +266,162 @@ def run(s):
         return {"vox": vox, "rules": [br.rulebook(vox, k, out=s["rules"][k]) for k in range(2)]}
     vox, pg = bufs["vox"], bufs["pg"]
     return [br.voxel_image_sampled(vox, k, pg["uvd"], pg["cam"], s["feat"], out=s["images"][k]) for k in range(2)]
+
+
+# ------------------------------------------------------------------------------------------------ the values in 64 bits
+# Which cell, camera and expert a point belongs to is decided in 32 bits by definition (one rounding per
+# operation), and feature rows are sampled at the 32-bit pixel that the call returns; those are taken in 32 bits here
+# too, and every value is then computed in 64 bits.
+def _fma(a, b, c):
+    """a * b + c of 32-bit numbers with one rounding (the product is exact in 64 bits)."""
+    return (a.double() * b.double() + c.double()).float()
+
+
+def _voxels64(pts, gr):
+    """Per scale: row of every point's voxel (-1: outside, or past the cap), points kept per row, means, cell ids."""
+    B, N, C = pts.shape
+    flat = pts.reshape(-1, C)
+    # a vector divisor: a plain number would be turned into a multiplication by its reciprocal
+    lo, size = (torch.tensor(v, device=pts.device).expand(len(flat), 3) for v in (gr.min, gr.voxel))
+    f = torch.floor((flat[:, :3] - lo) / size)
+    dims = torch.tensor(gr.dims, device=pts.device)
+    ok = ((f >= 0) & (f < dims)).all(1)
+    c = torch.where(ok[:, None], f, torch.zeros_like(f)).long()
+    frame = torch.arange(B, device=pts.device).repeat_interleave(N)
+    cell = ((frame * gr.dims[2] + c[:, 2]) * gr.dims[1] + c[:, 1]) * gr.dims[0] + c[:, 0]
+    at = ok.nonzero()[:, 0]
+    ids, row = torch.unique(cell[at], return_inverse=True)
+    if gr.max_points:                                                # the first points of every voxel, by index
+        order = torch.argsort(row, stable=True)
+        start = torch.searchsorted(row[order], torch.arange(len(ids), device=pts.device))
+        keep = torch.arange(len(order), device=pts.device) - start[row[order]] < gr.max_points
+        at, row = at[order[keep]], row[order[keep]]
+    n = torch.bincount(row, minlength=len(ids))
+    total = torch.zeros((len(ids), C), dtype=torch.float64, device=pts.device).index_add_(0, row, flat[at].double())
+    point_row = torch.full((B * N,), -1, device=pts.device).index_put_((at,), row)
+    return point_row, n, total / n[:, None], ids
+
+
+def _vox64(pts, w):
+    means, rows = [], []
+    B, N, C = pts.shape
+    gx, gy = w.grids[1].dims[:2]
+    for gr in w.grids:
+        point_row, _, mean, ids = _voxels64(pts, gr)
+        rows.append(point_row)
+        means.append(torch.zeros((B * N, C), dtype=torch.float64, device=pts.device))
+        means[-1][:len(ids)] = mean
+    bev = torch.zeros((B, gy * gx, C), dtype=torch.float64, device=pts.device)
+    bev.view(-1, C)[ids] = mean                                      # pillars: one cell high
+    bev = bev.transpose(1, 2).reshape(B, C, gy, gx)
+    return {"coords": [None] * 2, "counts": [None] * 2, "mean": means, "point_voxel": [None] * 2,
+            "num_voxels": None, "bev": bev}, rows
+
+
+def _project64(pts, proj, w):
+    """Per frame: uvd in 64 bits, the pixel in 32 bits, the lowest camera that sees each point (-1: none), and per
+    camera its mask, pixel and depth."""
+    x, y, z = pts[:, 0], pts[:, 1], pts[:, 2]
+    N = len(pts)
+    best = torch.full((N,), -1, device=pts.device)
+    uvd = torch.full((N, 3), -1.0, dtype=torch.float64, device=pts.device)
+    pixel = torch.zeros((N, 2), device=pts.device)
+    views = []
+    for k in range(w.K):
+        P = proj[k]
+        t = [_fma(P[r, 0], x, _fma(P[r, 1], y, _fma(P[r, 2], z, P[r, 3]))) for r in range(3)]
+        u, v = t[0] / t[2], t[1] / t[2]
+        vis = (t[2] > w.min_depth) & (u >= 0) & (u < w.img_w) & (v >= 0) & (v < w.img_h)
+        q = pts[:, :3].double() @ P[:, :3].double().T + P[:, 3].double()
+        if k == 0:
+            uvd[:, 2] = q[:, 2]
+        first = vis & (best < 0)
+        uvd[first] = torch.stack([q[:, 0] / q[:, 2], q[:, 1] / q[:, 2], q[:, 2]], dim=1)[first]
+        pixel[first] = torch.stack([u, v], dim=1)[first]
+        best[first] = k
+        views.append((vis, u, v, q[:, 2], t[2]))
+    return uvd, pixel, best, views
+
+
+def _rows64(pixel, best, feat, w):
+    """Feature rows of one frame, blended in 64 bits; zeros for points that no camera sees."""
+    rows = torch.zeros((len(best), w.feat_c), dtype=torch.float64, device=feat.device)
+    seen = (best >= 0).nonzero()[:, 0]
+    for at in seen.split(1 << 18):
+        fx, fy = ((pixel[at, d].double() - w.feat_offset) / w.feat_stride for d in (0, 1))
+        x0, y0 = torch.floor(fx), torch.floor(fy)
+        wx, wy = (fx - x0)[:, None], (fy - y0)[:, None]
+
+        def tap(dy, dx):
+            return feat[best[at], (y0.long() + dy).clamp(0, w.feat_h - 1), (x0.long() + dx).clamp(0, w.feat_w - 1)].double()
+
+        rows[at] = (1 - wy) * ((1 - wx) * tap(0, 0) + wx * tap(0, 1)) + wy * ((1 - wx) * tap(1, 0) + wx * tap(1, 1))
+    return rows
+
+
+def _experts(pts, visible, w):
+    r2 = _fma(pts[:, 0], pts[:, 0], pts[:, 1] * pts[:, 1])
+    bucket = torch.zeros(len(pts), dtype=torch.long, device=pts.device)
+    for t in w.thresholds:
+        t = torch.tensor(t, device=pts.device)                       # 32 bits, and so is its square
+        bucket += (r2 >= t * t).long()
+    return torch.tensor(w.lut, device=pts.device)[visible.long(), bucket]
+
+
+def exact(case, seed):
+    """What `run` returns, its numbers computed in 64 bits by plain torch; None for whole numbers."""
+    w, call = _workload(case), case["call"]
+    s = _inputs(case, w, seed)
+    if call == "maps":
+        last = s["feat"].permute(0, 1, 3, 4, 2).double()
+        p = case["pool"]
+        pooled = torch.nn.functional.avg_pool2d(s["feat"].double().flatten(0, 1), p, ceil_mode=True,
+                                                count_include_pad=False)
+        pooled = pooled.permute(0, 2, 3, 1).unflatten(0, last.shape[:2])
+        return {"last": last.contiguous(), "pooled": pooled.contiguous()}
+    pts = s["points"]
+    vox, point_rows = _vox64(pts, w)
+    if call == "lidar":
+        return {"vox": vox, "rules": [None, None]}
+    B, N, C = pts.shape
+    f64 = {"dtype": torch.float64, "device": pts.device}
+    uvd, rows = torch.zeros((B, N, 3), **f64), torch.zeros((B, N, w.feat_c), **f64)
+    best = torch.zeros((B, N), dtype=torch.long, device=pts.device)
+    views = []
+    for b in range(B):
+        uvd[b], pixel, best[b], v = _project64(pts[b], s["proj"][b], w)
+        views.append(v if call == "staged" else None)
+        rows[b] = _rows64(pixel, best[b], s["feat"][b], w)
+    if call == "fusion":
+        images, seen = [], (best >= 0).flatten()
+        for point_row in point_rows:
+            at = ((point_row >= 0) & seen).nonzero()[:, 0]
+            total = torch.zeros((B * N, w.feat_c), **f64).index_add_(0, point_row[at], rows.view(B * N, -1)[at])
+            n = torch.bincount(point_row[at], minlength=B * N).clamp(min=1)
+            images.append({"vox_img": total / n[:, None], "vox_img_count": None})
+        return images
+    visible, occ = best >= 0, None
+    if call == "staged":
+        hz, wz = -(-w.img_h // OCCLUSION_CELL), -(-w.img_w // OCCLUSION_CELL)
+        zbuf = torch.full((B, w.K, hz * wz), float("inf"), **f64)
+        for b in range(B):
+            visible[b] = False
+            for k, (vis, u, v, depth, depth32) in enumerate(views[b]):
+                cell = (v[vis] / OCCLUSION_CELL).long() * wz + (u[vis] / OCCLUSION_CELL).long()
+                zbuf[b, k].scatter_reduce_(0, cell, depth[vis], "amin")
+                near = torch.full((hz * wz,), float("inf"), device=pts.device).scatter_reduce_(0, cell, depth32[vis], "amin")
+                visible[b, vis.nonzero()[:, 0][~(depth32[vis] > near[cell] + OCCLUSION_MARGIN)]] = True
+        occ = {"zbuf": zbuf.view(B, w.K, hz, wz), "occ_mask": None, "clear_mask": None}
+    points_out, feat_out = torch.zeros((B, N, C), **f64), torch.zeros((B, N, w.feat_c), **f64)
+    for b in range(B):
+        order = torch.argsort(_experts(pts[b], visible[b], w), stable=True)
+        points_out[b], feat_out[b] = pts[b, order].double(), rows[b, order]
+    pg = {"uvd": uvd, "vis_mask": None, "cam": None, "gathered": rows if case["rows"] or call != "bridge" else None}
+    rd = {"expert": None, "offsets": None, "perm": None, "points_out": points_out, "feat_out": feat_out}
+    out = {"vox": vox, "pg": pg, "rd": rd}
+    if call == "staged":
+        return {**out, "occ": occ}
+    return {"bufs": out, "offsets": None, "num_voxels": None} if call == "host" else out
 
 
 # ------------------------------------------------------------------------------------------------ what a pass is
