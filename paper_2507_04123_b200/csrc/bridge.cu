@@ -8,7 +8,7 @@
 namespace emc2 {
 
 static const char* const kKernelNames[K_KINDS] = {
-    "vox_mark", "vox_count", "vox_prefix", "vox_rank", "vox_accum", "vox_over_find", "vox_over_fill", "vox_finalize", "arm_keys", "arm_sort", "arm_hash", "arm_rank",
+    "vox_mark", "vox_count", "vox_rank", "vox_accum", "vox_over_find", "vox_over_fill", "vox_finalize", "arm_keys", "arm_sort", "arm_hash", "arm_rank",
     "project_gather", "project_route", "gather_scatter", "route_hist", "route_scan", "dispatch_scatter", "scene_route", "pool_features",
     "vif_scan", "vif_fill", "vif_mean", "vif_sample", "occl_fill", "occl_splat", "occl_test",
     "channels_last", "rb_mark", "rb_count", "rb_scan", "rb_fill", "rb_clear"};
@@ -143,7 +143,7 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out) {
 
     // Plan the slab: everything the stage calls need, allocated once.
     SlabPlan plan;
-    size_t o_store[2], o_flag[2], o_acc[2], o_cl[2], o_ovf[2][5], o_tot[2];
+    size_t o_store[2], o_acc[2], o_cl[2], o_ovf[2][5], o_tot[2];
     for (int s = 0; s < 2; ++s) {
         ScaleDev& d = h->scale[s];
         const emc2_grid_t& g = c.grid[s];
@@ -157,12 +157,13 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out) {
         d.cells = (uint32_t)((uint64_t)g.dims[0] * g.dims[1] * g.dims[2]);
         const uint64_t total_cells = (uint64_t)d.cells * c.max_batch;
         d.mode = total_cells <= (uint64_t)kMaxTableCells ? MODE_TABLE : MODE_BITMAP;
-        const uint64_t per_group = d.mode == MODE_BITMAP ? kBitmapGroupCells : kTableGroupCells;
-        d.ngroups = (uint32_t)((total_cells + per_group - 1) / per_group);
+        const uint64_t per_tile = d.mode == MODE_BITMAP ? kBitmapTileCells : kTableTileCells;
+        d.tiles = (uint32_t)((total_cells + per_tile - 1) / per_tile + kCountTiles - 1) / kCountTiles * kCountTiles;
+        // A table store knows the cells' point counts without accumulating them: four channels need one float4.
+        d.acc_f4 = d.mode == MODE_TABLE && c.point_floats == 4 ? 1 : 2;
         d.max_ovf = d.cap > 0 ? (uint32_t)(maxpts / ((size_t)d.cap + 1) + 1) : 0;
         d.max_list = (uint32_t)maxpts;
-        o_store[s] = plan.take((size_t)d.ngroups * 1024);
-        o_flag[s] = plan.take((size_t)d.ngroups * sizeof(int4));
+        o_store[s] = plan.take((size_t)d.tiles * kScanTileBytes);
         o_acc[s] = plan.take(maxpts * 2 * sizeof(float4));
         o_cl[s] = plan.take(maxpts * sizeof(uint32_t));
         for (int k = 0; k < 3; ++k) o_ovf[s][k] = d.cap > 0 ? plan.take((size_t)d.max_ovf * sizeof(int)) : 0;
@@ -170,11 +171,12 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out) {
         o_ovf[s][4] = d.cap > 0 ? plan.take((size_t)d.max_ovf * kCursorStride * sizeof(int)) : 0;
         o_tot[s] = plan.take(4 * sizeof(int));
     }
-    // The rank scan gives a CTA 32 groups of one scale.
-    const size_t scan_ctas = (size_t)(h->scale[0].ngroups + 31) / 32 + (size_t)(h->scale[1].ngroups + 31) / 32;
-    const size_t o_part = plan.take(scan_ctas * 3 * sizeof(int));
-    const size_t o_pbase = plan.take(scan_ctas * 3 * sizeof(int));
-    const size_t o_units = plan.take(scan_ctas * sizeof(int));
+    const size_t tiles[2] = {h->scale[0].tiles, h->scale[1].tiles};
+    const size_t groups[2] = {(tiles[0] + kTilesPerGroup - 1) / kTilesPerGroup, (tiles[1] + kTilesPerGroup - 1) / kTilesPerGroup};
+    const size_t o_tiles = plan.take((tiles[0] + tiles[1]) * sizeof(uint32_t));
+    const size_t o_list = plan.take((tiles[0] + tiles[1]) * sizeof(uint32_t));
+    h->scan_reset_words = (int)(groups[0] + groups[1] + 1);
+    const size_t o_groups = plan.take((size_t)h->scan_reset_words * sizeof(uint32_t));
     const size_t o_vif_start = plan.take(maxpts * sizeof(int));
     const size_t o_vif_cursor = plan.take(maxpts * sizeof(int));
     const size_t o_vif_list = plan.take(maxpts * sizeof(int));
@@ -200,7 +202,6 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out) {
     for (int s = 0; s < 2; ++s) {
         ScaleDev& d = h->scale[s];
         d.store = reinterpret_cast<uint32_t*>(base + o_store[s]);
-        d.group_info = reinterpret_cast<int4*>(base + o_flag[s]);
         d.acc = reinterpret_cast<float4*>(base + o_acc[s]);
         d.cell_list = reinterpret_cast<uint32_t*>(base + o_cl[s]);
         d.ovf_off = d.cap > 0 ? reinterpret_cast<int*>(base + o_ovf[s][0]) : nullptr;
@@ -210,9 +211,12 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out) {
         d.ovf_cursor = d.cap > 0 ? reinterpret_cast<int*>(base + o_ovf[s][4]) : nullptr;
         d.totals = reinterpret_cast<int*>(base + o_tot[s]);
     }
-    h->d_scan_tot = reinterpret_cast<int*>(base + o_part);
-    h->d_scan_base = reinterpret_cast<int*>(base + o_pbase);
-    h->d_scan_units = reinterpret_cast<int*>(base + o_units);
+    h->scan.tile_voxels[0] = reinterpret_cast<uint32_t*>(base + o_tiles);
+    h->scan.tile_voxels[1] = h->scan.tile_voxels[0] + tiles[0];
+    h->scan.list = reinterpret_cast<uint32_t*>(base + o_list);
+    h->scan.group_voxels[0] = reinterpret_cast<uint32_t*>(base + o_groups);
+    h->scan.group_voxels[1] = h->scan.group_voxels[0] + groups[0];
+    h->scan.listed = h->scan.group_voxels[1] + groups[1];
     h->d_vif_start = reinterpret_cast<int*>(base + o_vif_start);
     h->d_vif_cursor = reinterpret_cast<int*>(base + o_vif_cursor);
     h->d_vif_list = reinterpret_cast<int*>(base + o_vif_list);
@@ -552,6 +556,8 @@ int emc2_bridge_set_tuning(emc2_bridge_t* h, int32_t knob, int32_t value) {
             if (rc != EMC2_OK) return rc;
         }
         h->scale[s].design = value;
+        // The other designs keep no counts per cell: the accumulators do.
+        h->scale[s].acc_f4 = value == 0 && h->scale[s].mode == MODE_TABLE && h->cfg.point_floats == 4 ? 1 : 2;
         h->scale[s].point_rank = value ? h->arm.point_rank[s] : nullptr;
     }
     h->tune[knob] = value;

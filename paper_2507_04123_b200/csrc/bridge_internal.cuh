@@ -12,16 +12,22 @@ namespace emc2 {
 
 constexpr int kTile = 256;           // points per CTA tile in the per-point kernels
 constexpr int kThreads = 256;
-constexpr int kBitmapGroupCells = 32 * 4 * 32;  // a 1 KB bitmap group: 32 sectors of four {bits, rank} pairs
-constexpr int kTableGroupCells = 32 * 2;         // a 1 KB table group: 32 sectors of two cell records
-constexpr int kMaxTableCells = 1 << 24;  // per-cell records up to 16 Mi cells per batch (256 MB)
+// The cell stores.  Large grids: 16-byte units of 96 cell bits and the rank of the unit's first voxel, so that
+// one 128-bit load answers a look-up and the scan streams 1.33 bits per cell (a {32 bits, rank} pair per 32
+// cells streams 2: 75 instead of 50 MB for four frames of the nuScenes-shaped grid, and the scan is paid by
+// the grid's volume).  Small grids: one word per cell.
+constexpr uint32_t kUnitCells = 96;
+constexpr size_t kScanTileBytes = 8192;   // of the store, per CTA of the ranking pass
+constexpr uint32_t kBitmapTileCells = (uint32_t)(kScanTileBytes / 16) * kUnitCells;
+constexpr uint32_t kTableTileCells = (uint32_t)(kScanTileBytes / 4);
+constexpr int kMaxTableCells = 1 << 24;  // a word per cell up to 16 Mi cells per batch (64 MB)
+constexpr uint32_t kOverCap = 0x80000000u;  // table word / list entry of a cell over the cap
 constexpr int kCursorStride = 8;         // ints between list cursors: one 32-byte sector each
 
 // Kernel kinds, for the launch counters and the optional event timing.
 enum KernelKind {
     K_VOX_MARK = 0,
     K_VOX_COUNT,
-    K_VOX_PREFIX,
     K_VOX_RANK,
     K_VOX_ACCUM,
     K_VOX_OVER_FIND,
@@ -91,14 +97,14 @@ struct ScaleDev {
     int cap;                // 0 = none
     int mode;               // ScaleMode
     uint32_t cells;         // cells per frame
-    uint32_t ngroups;       // 1 KB groups of `store` for the largest batch
+    uint32_t tiles;         // 8 KB tiles of `store` for the largest batch, a multiple of kCountTiles
     uint32_t max_ovf;       // most cells that can exceed the cap
     uint32_t max_list;      // entries of acc / cell_list / ovf_list: the most points of a call
-    uint32_t* store;        // bitmap: {bits, rank} per 32 cells; table: {count, rank, over-cap rank, -} per cell;
-                            // bits / counts are zero between calls
-    int4* group_info;       // [ngroups] {voxels, cells over the cap, their points} of the group (rewritten by
-                            // every call)
-    float4* acc;            // [max voxels][2] per-voxel accumulators
+    uint32_t* store;        // bitmap: 16-byte units {96 cell bits, rank}; table: one word per cell, its point
+                            // count while marking, then its rank or kOverCap | index among the cells over the
+                            // cap.  All zero between calls
+    int acc_f4;             // float4 per accumulator: 1 or 2
+    float4* acc;            // [max voxels][acc_f4] per-voxel accumulators
     uint32_t* cell_list;    // [max voxels] cell id of each unique voxel (table stores: bit 31 = over the cap)
     int* ovf_off;           // per cell over the cap j: start of its points in ovf_list
     int* ovf_cursor;        // per cell over the cap j: points appended so far, at [j * kCursorStride]
@@ -108,7 +114,8 @@ struct ScaleDev {
     int design;             // dedup design of this scale: 0 = this direct-addressed store, 1 = hash, 2 = sort
                             // (dedup_arms.cu); with 1 or 2 the store is not used and rows come from point_rank
     const int* point_rank;  // design != 0: [points of the call] row of every point's voxel, -1 if outside
-    int* totals;            // [0] voxels, [1] cells over the cap, [2] points in cells over the cap, [3] CTAs of the rank scan that found voxels
+    int* totals;            // [0] voxels, [2] points in cells over the cap, [3] cells over the cap ([2] and [3] are
+                            // one 64-bit ticket counter)
 };
 
 // Routing tables as the kernels take them (Sec. 3.2 distance rule, per point with visibility).
@@ -116,6 +123,23 @@ struct RouteParams {
     int T, E;
     float thr2[EMC2_MAX_THRESHOLDS];    // squared thresholds
     uint8_t lut[16];                    // [visible ? 8 : 0] + number of thresholds reached -> expert
+};
+
+// State of the rank scan.
+constexpr int kTilesPerGroup = 128;
+constexpr int kCountTiles = 4;  // tiles per CTA of the counting pass
+struct ScanState {
+    uint32_t* tile_voxels[2];   // [tiles] voxels per tile
+    uint32_t* group_voxels[2];  // [ceil(tiles / 128)] per group of tiles; zero when the scan begins
+    uint32_t* listed;           // tiles in `list`; zero when the scan begins
+    uint32_t* list;             // [tiles of both scales] tiles that hold voxels, in any order; bit 31: scale 1
+};
+
+// What of it is zeroed when a call begins, by whichever kernel marks the cells.
+struct ScanReset {
+    uint32_t* words;            // group_voxels of both scales and `listed`, side by side
+    int n;
+    int* totals[2];             // null: nothing to reset (second half of a split batch)
 };
 
 // Scratch of the alternative dedup designs (allocated when one is first selected).
@@ -150,9 +174,8 @@ struct emc2_bridge {
     int* d_status = nullptr;       // sticky device status word
     int* d_tile_counts = nullptr;  // [B, tiles per frame, E]
     int* d_tile_base = nullptr;    // same shape, exclusive bases
-    int* d_scan_tot = nullptr;     // [CTAs of the voxel rank scan, both scales][3] per-CTA totals
-    int* d_scan_base = nullptr;    // same shape: their exclusive prefix sums inside each scale
-    int* d_scan_units = nullptr;   // per scale the CTAs that found voxels
+    emc2::ScanState scan = {};
+    int scan_reset_words = 0;
     int* d_vif_start = nullptr;    // emc2_voxel_image: [max points] list starts, cursors, lists
     int* d_vif_cursor = nullptr;
     int* d_vif_list = nullptr;
@@ -206,6 +229,14 @@ int launch_project_gather(emc2_bridge* h, int B, int N, const float* d_points, c
 int launch_route_dispatch(emc2_bridge* h, int B, int N, const float* d_points, const uint8_t* d_vis_mask,
                           const float* d_gathered, uint8_t* d_expert, int32_t* d_offsets, int32_t* d_perm,
                           float* d_points_out, float* d_feat_out, cudaStream_t st);
+
+inline ScanReset scan_reset(const emc2_bridge* h) {
+    ScanReset r;
+    r.words = h->scan.group_voxels[0];
+    r.n = h->scan_reset_words;
+    for (int s = 0; s < 2; ++s) r.totals[s] = h->scale[s].totals;
+    return r;
+}
 
 inline RouteParams route_params(const emc2_bridge* h) {
     RouteParams rp;
@@ -275,6 +306,21 @@ __device__ __forceinline__ uint32_t cell_of(const ScaleDev& g, float x, float y,
     return (((uint32_t)b * g.dims[2] + iz) * g.dims[1] + iy) * g.dims[0] + ix;
 }
 
+// Bit `cell` of a bitmap store: its unit and its place in it.
+__device__ __forceinline__ uint32_t unit_of(uint32_t cell, uint32_t& pos) {
+    const uint32_t u = cell / kUnitCells;
+    pos = cell - u * kUnitCells;
+    return u;
+}
+
+// Set bits of a unit below place `pos`.
+__device__ __forceinline__ uint32_t bits_below(const uint4& q, uint32_t pos) {
+    const uint32_t part = (1u << (pos & 31u)) - 1u;
+    if (pos < 32u) return __popc(q.x & part);
+    if (pos < 64u) return __popc(q.x) + __popc(q.y & part);
+    return __popc(q.x) + __popc(q.y) + __popc(q.z & part);
+}
+
 // Marks the cells of one point in both scales' stores: one fire-and-forget reduction each (OR into
 // the bit word, ADD into the cell's point count).
 __device__ __forceinline__ void mark_point(const ScaleDev& s0, const ScaleDev& s1, float x, float y, float z, int b) {
@@ -285,8 +331,21 @@ __device__ __forceinline__ void mark_point(const ScaleDev& s0, const ScaleDev& s
         const uint32_t cell = cell_of(g, x, y, z, b);
         if (cell == 0xFFFFFFFFu) continue;
         // Results unused: these compile to reductions, which the thread does not wait for.
-        if (g.mode == MODE_BITMAP) atomicOr(&g.store[2 * (size_t)(cell >> 5)], 1u << (cell & 31u));
-        else atomicAdd(&g.store[4 * (size_t)cell], 1u);
+        if (g.mode == MODE_BITMAP) {
+            uint32_t pos;
+            const uint32_t u = unit_of(cell, pos);
+            atomicOr(&g.store[4 * (size_t)u + (pos >> 5)], 1u << (pos & 31u));
+        } else {
+            atomicAdd(&g.store[cell], 1u);
+        }
+    }
+}
+
+__device__ __forceinline__ void reset_scan(const ScanReset& r, size_t thread, size_t nthreads) {
+    for (size_t i = thread; i < (size_t)r.n; i += nthreads) r.words[i] = 0u;
+    if (thread == 0 && r.totals[0]) {
+        *reinterpret_cast<int4*>(r.totals[0]) = make_int4(0, 0, 0, 0);
+        *reinterpret_cast<int4*>(r.totals[1]) = make_int4(0, 0, 0, 0);
     }
 }
 

@@ -164,6 +164,7 @@ struct PrArgs {
     ScaleDev s0, s1;      // kMark: the voxel grids whose cells the points mark
     float4* bev;          // kMark: BEV image to zero (bev_n4 float4), or null
     size_t bev_n4;
+    ScanReset reset;      // kMark: state of the rank scan to zero
 };
 
 // grid = (tiles per frame, B); tiles never straddle frames.  kMark: the kernel also does the
@@ -211,10 +212,13 @@ __global__ void __launch_bounds__(kThreads) project_route_kernel(const __grid_co
     }
     __syncthreads();
     if (t < a.rp.E) a.tile_counts[((size_t)b * a.tiles + tile) * a.rp.E + t] = hist[t];
-    if (kMark && a.bev) {
-        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (kMark) {
         const size_t cta = (size_t)blockIdx.y * gridDim.x + blockIdx.x, nthreads = (size_t)gridDim.x * gridDim.y * kThreads;
-        for (size_t i = cta * kThreads + t; i < a.bev_n4; i += nthreads) __stcs(a.bev + i, z);
+        reset_scan(a.reset, cta * kThreads + t, nthreads);
+        if (a.bev) {
+            const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (size_t i = cta * kThreads + t; i < a.bev_n4; i += nthreads) __stcs(a.bev + i, z);
+        }
     }
 }
 
@@ -670,6 +674,8 @@ int launch_project_route(emc2_bridge* h, int b0, int B, int N, const float* d_po
     pa.frame0 = b0;
     pa.s0 = h->scale[0]; pa.s1 = h->scale[1];
     pa.bev = nullptr; pa.bev_n4 = 0;
+    pa.reset = scan_reset(h);
+    if (!mark || b0 > 0) { pa.reset.n = 0; pa.reset.totals[0] = pa.reset.totals[1] = nullptr; }
     if (mark && d_bev_to_zero && bev_frames > 0) {
         const size_t bev_n = (size_t)bev_frames * c.point_floats * h->scale[1].dims[1] * h->scale[1].dims[0];
         if (bev_n & 3) {

@@ -5,15 +5,15 @@
 // frame, in ascending m.
 //
 // A neighbour is found in O(1): the scale's direct-addressed cell store (all zero between calls)
-// is filled from the list, {32 cell bits, row of the word's first voxel} per 32 cells for large
+// is filled from the list, {96 cell bits, row of the unit's first voxel} per 96 cells for large
 // grids, the row + 1 per cell for small ones.  Because the list is in cell order, a voxel's row is
-// the word's first row plus the number of set bits below it.
-//   rb_mark   every voxel sets its cell; the first voxel of a word stores its row there
+// the unit's first row plus the number of set bits below it.
+//   rb_mark   every voxel sets its cell; the first voxel of a unit stores its row there
 //   rb_count  27 look-ups per voxel -> neighbour bits per voxel, pair counts per (offset, tile)
 //   rb_scan   one CTA per offset: exclusive prefix sum of its counts over the tiles, and its total
 //   rb_fill   offsets[28] from the totals; every tile ranks its pairs per offset with warp ballots
 //             and writes them
-//   rb_clear  the touched words of the store go back to zero
+//   rb_clear  the touched units of the store go back to zero
 #include "bridge_internal.cuh"
 
 namespace emc2 {
@@ -69,11 +69,13 @@ __global__ void __launch_bounds__(kThreads) rb_mark_kernel(const __grid_constant
         if (cell == 0xFFFFFFFFu) return;
     }
     if (a.g.mode == MODE_BITMAP) {
-        uint32_t* word = a.g.store + 2 * (size_t)(cell >> 5);
-        atomicOr(word, 1u << (cell & 31u));
-        if (m == 0 || before == 0xFFFFFFFFu || (before >> 5) != (cell >> 5)) word[1] = (uint32_t)m;
+        uint32_t pos;
+        const uint32_t u = unit_of(cell, pos);
+        uint32_t* unit = a.g.store + 4 * (size_t)u;
+        atomicOr(unit + (pos >> 5), 1u << (pos & 31u));
+        if (m == 0 || before == 0xFFFFFFFFu || before / kUnitCells != u) unit[3] = (uint32_t)m;
     } else {
-        a.g.store[4 * (size_t)cell] = (uint32_t)m + 1u;
+        a.g.store[cell] = (uint32_t)m + 1u;
     }
 }
 
@@ -84,14 +86,14 @@ __global__ void __launch_bounds__(kThreads) rb_clear_kernel(const __grid_constan
     const int4 c = a.coords[m];
     const uint32_t cell = cell_at(a, c.x, c.y, c.z, c.w);
     if (cell == 0xFFFFFFFFu) return;
-    if (a.g.mode == MODE_BITMAP) *reinterpret_cast<uint2*>(a.g.store + 2 * (size_t)(cell >> 5)) = make_uint2(0u, 0u);
-    else a.g.store[4 * (size_t)cell] = 0u;
+    if (a.g.mode == MODE_BITMAP) reinterpret_cast<uint4*>(a.g.store)[cell / kUnitCells] = make_uint4(0u, 0u, 0u, 0u);
+    else a.g.store[cell] = 0u;
 }
 
-// Row of the voxel at bit `pos` of a {bits, first row} pair, -1 if the bit is clear.
-__device__ __forceinline__ int row_in_word(const uint2 pr, uint32_t pos) {
-    const uint32_t bit = 1u << pos;
-    return (pr.x & bit) ? (int)(pr.y + __popc(pr.x & (bit - 1u))) : -1;
+// Row of the voxel at place `pos` of a unit, -1 if its bit is clear.
+__device__ __forceinline__ int row_in_unit(const uint4& q, uint32_t pos) {
+    const uint32_t word = pos < 32u ? q.x : pos < 64u ? q.y : q.z;
+    return (word >> (pos & 31u)) & 1u ? (int)(q.w + bits_below(q, pos)) : -1;
 }
 
 // Where a voxel sits: its cell, the cell strides and which of its 3 x 3 x 3 neighbours the grid has.
@@ -114,23 +116,25 @@ __device__ __forceinline__ Site site_of(const RbArgs& a, const int4 c) {
 
 // Rows of the three x-neighbours (dx = -1, 0, 1) at (dz, dy) = (j / 3 - 1, j % 3 - 1) of a valid
 // site, -1 where there is none; only the ones in `want3` (bit dx + 1) are looked up.  The three
-// share a bitmap word unless they straddle a word boundary: one load, rarely two.
+// share a unit of the bitmap unless they straddle its boundary: one load, rarely two.
 __device__ __forceinline__ void neighbours3(const ScaleDev& g, const Site& s, int j, uint32_t want3, int r[3]) {
     const int dz = j / 3 - 1, dy = j % 3 - 1;
     r[0] = r[1] = r[2] = -1;
     if (!want3 || !s.okz[dz + 1] || !s.oky[dy + 1]) return;
     const uint32_t mid = s.cell + (uint32_t)dz * s.sz + (uint32_t)dy * s.sy;   // wraps like the signed sum
     if (g.mode == MODE_BITMAP) {
-        const uint2* words = reinterpret_cast<const uint2*>(g.store);
-        const uint32_t w = mid >> 5, pos = mid & 31u;
-        const uint2 pr = words[w];
-        if (want3 & 2u) r[1] = row_in_word(pr, pos);
-        if (s.okx[0] && (want3 & 1u)) r[0] = pos > 0 ? row_in_word(pr, pos - 1) : row_in_word(words[w - 1], 31);
-        if (s.okx[2] && (want3 & 4u)) r[2] = pos < 31 ? row_in_word(pr, pos + 1) : row_in_word(words[w + 1], 0);
+        const uint4* units = reinterpret_cast<const uint4*>(g.store);
+        uint32_t pos;
+        const uint32_t u = unit_of(mid, pos);
+        const uint4 q = units[u];
+        if (want3 & 2u) r[1] = row_in_unit(q, pos);
+        if (s.okx[0] && (want3 & 1u)) r[0] = pos > 0 ? row_in_unit(q, pos - 1) : row_in_unit(units[u - 1], kUnitCells - 1);
+        if (s.okx[2] && (want3 & 4u))
+            r[2] = pos < kUnitCells - 1 ? row_in_unit(q, pos + 1) : row_in_unit(units[u + 1], 0);
     } else {
 #pragma unroll
         for (int i = 0; i < 3; ++i)
-            if (s.okx[i] && ((want3 >> i) & 1u)) r[i] = (int)g.store[4 * (size_t)(mid + i - 1)] - 1;
+            if (s.okx[i] && ((want3 >> i) & 1u)) r[i] = (int)g.store[mid + i - 1] - 1;
     }
 }
 
@@ -141,17 +145,22 @@ __device__ __forceinline__ uint32_t exist3(const ScaleDev& g, const Site& s, int
     const uint32_t mid = s.cell + (uint32_t)dz * s.sz + (uint32_t)dy * s.sy;
     const uint32_t inside = (s.okx[0] ? 1u : 0u) | 2u | (s.okx[2] ? 4u : 0u);
     if (g.mode == MODE_BITMAP) {
-        const uint32_t w = mid >> 5, pos = mid & 31u;
-        // 34-bit window: the word's 32 cells with one cell of the words before and after it
-        unsigned long long window = (unsigned long long)g.store[2 * (size_t)w] << 1;
-        if (pos == 0 && s.okx[0]) window |= g.store[2 * (size_t)(w - 1)] >> 31;
-        if (pos == 31 && s.okx[2]) window |= (unsigned long long)(g.store[2 * (size_t)(w + 1)] & 1u) << 33;
-        return (uint32_t)(window >> pos) & inside;
+        const uint4* units = reinterpret_cast<const uint4*>(g.store);
+        uint32_t pos;
+        const uint32_t u = unit_of(mid, pos);
+        const uint4 q = units[u];
+        uint32_t three;                            // bits pos - 1, pos, pos + 1
+        if (pos == 0) three = (q.x & 3u) << 1 | (s.okx[0] ? units[u - 1].z >> 31 : 0u);
+        else if (pos == kUnitCells - 1) three = (q.z >> 30) | (s.okx[2] ? (units[u + 1].x & 1u) << 2 : 0u);
+        else if (pos <= 32u) three = __funnelshift_r(q.x, q.y, pos - 1);
+        else if (pos <= 64u) three = __funnelshift_r(q.y, q.z, pos - 33);
+        else three = q.z >> (pos - 65);
+        return three & inside;
     }
     uint32_t three = 0;
 #pragma unroll
     for (int i = 0; i < 3; ++i)
-        if (s.okx[i] && g.store[4 * (size_t)(mid + i - 1)]) three |= 1u << i;
+        if (s.okx[i] && g.store[mid + i - 1]) three |= 1u << i;
     return three;
 }
 

@@ -2,19 +2,17 @@
 // and means, BEV scatter (Sec. 3.1 preprocessing; BEV for the 2D expert of Sec. 3.3).
 //
 // Dedup is direct-addressed, with no sort and no hash probing.  Large grids keep one bit per
-// cell: the store is an array of {32 cell bits, rank} pairs in cell order.  Grids small enough
-// keep one record {point count, rank, rank among cells over the cap, -} per cell.  "Rank" is
-// the number of occupied cells before this word / cell in ascending (b, z, y, x) order, which
-// is the canonical voxel order, so a point finds its voxel row with ONE 8- or 16-byte load plus
-// a popcount, and no sort is ever needed.
+// cell: the store is an array of units {96 cell bits, rank} in cell order.  Grids small enough
+// keep one word per cell, its point count.  "Rank" is the number of occupied cells before this
+// unit / cell in ascending (b, z, y, x) order, which is the canonical voxel order, so a point finds
+// its voxel row with ONE 16- or 4-byte load plus a popcount, and no sort is ever needed.
 //
 //   vox_mark      every point marks its two cells with one fire-and-forget reduction each;
 //                 the same launch zeroes the BEV image.
-//   vox_count,    the rank scan, three launches: counts per 1 KB group of the store, prefix sums
-//   vox_prefix,   of the per-CTA totals, then the exclusive prefix sums (the parallel prefix-sum
-//   vox_rank      index search of Sec. 3.6) are written into the rank fields and the occupied
-//                 cell ids listed in that order; accumulators are cleared and the bookkeeping of
-//                 cells over the cap is laid out.
+//   vox_count,    the rank scan, two launches: voxels per tile of the store, then the exclusive prefix
+//   vox_rank      sums (the parallel prefix-sum index search of Sec. 3.6) are written into the rank
+//                 fields and the occupied cell ids listed in that order; the bookkeeping of cells over
+//                 the cap is laid out.
 //   vox_accum     every point looks its rank up, writes point_voxel and adds itself to its
 //                 voxels' accumulators with two fp32 vector reductions (offsets from the cell
 //                 corner, the other channels, the count).
@@ -53,30 +51,16 @@ __device__ __forceinline__ Slot slot_of(const ScaleDev& g, uint32_t cell, long l
         return s;
     }
     if (g.mode == MODE_BITMAP) {
-        const uint2 pr = *reinterpret_cast<const uint2*>(g.store + 2 * (size_t)(cell >> 5));
-        s.m = (int)(pr.y + __popc(pr.x & ((1u << (cell & 31u)) - 1u)));
+        uint32_t pos;
+        const uint32_t u = unit_of(cell, pos);
+        const uint4 q = reinterpret_cast<const uint4*>(g.store)[u];
+        s.m = (int)(q.w + bits_below(q, pos));
     } else {
-        const uint4 q = *reinterpret_cast<const uint4*>(g.store + 4 * (size_t)cell);
-        s.m = (int)q.y;
-        if (g.cap > 0 && (int)q.x > g.cap) s.j = (int)q.z;
+        const uint32_t w = g.store[cell];
+        if (w & kOverCap) s.j = (int)(w & ~kOverCap);
+        else s.m = (int)w;
     }
     return s;
-}
-
-// Exclusive scan of three counters across the warp; warp totals in tot[].
-__device__ __forceinline__ void warp_excl_scan3(int v[3], int tot[3]) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        int x = v[k];
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int y = __shfl_up_sync(0xFFFFFFFFu, x, d);
-            if (lane >= d) x += y;
-        }
-        tot[k] = __shfl_sync(0xFFFFFFFFu, x, 31);
-        v[k] = x - v[k];
-    }
 }
 
 // Lower corner of cell i along one axis; both per-point and per-voxel code use this value.
@@ -86,8 +70,9 @@ __device__ __forceinline__ float cell_corner(float mn, float vs, int i) { return
 template <int C>
 __global__ void __launch_bounds__(kThreads)
 vox_mark_kernel(const float* __restrict__ pts, long long total, int N, ScaleDev s0, ScaleDev s1,
-                float4* bev, size_t bev_n4) {
+                float4* bev, size_t bev_n4, ScanReset reset) {
     __shared__ __align__(16) float sp[kBigTile * C];
+    reset_scan(reset, (size_t)blockIdx.x * kThreads + threadIdx.x, (size_t)gridDim.x * kThreads);
     // The BEV image is zeroed here, spread over the whole grid, so it costs no extra launch.
     if (bev) {
         const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -113,292 +98,222 @@ vox_mark_kernel(const float* __restrict__ pts, long long total, int N, ScaleDev 
 // ------------------------------------------------------------------ pass 2: ranks
 struct ScanArgs {
     ScaleDev s[2];
-    uint32_t ngroups_used[2];   // 1 KB groups covering this call's B frames
     int capacity[2];
+    int32_t* counts[2];         // table stores: the kept points of every voxel go straight to the output
     int32_t* num_voxels;
     int* status;
-    int* cta_tot;               // [ctas0 + ctas1][3] voxels, cells over the cap and their points per CTA
-    int* cta_base;              // same shape: exclusive prefix sums inside each scale
-    int* unit_list;             // [ctas0 + ctas1] per scale: the CTAs of vox_count that found voxels, ascending
-    int ctas0, ctas1;           // CTAs of vox_count / vox_rank serving scale 0 and scale 1
+    int tiles[2];               // 8 KB tiles covering this call's B frames
+    ScanState st;
 };
 
-// One lane owns one 32-byte sector of the store: four {bits, rank} pairs or two cell records;
-// a warp owns a 1 KB group.
-struct Sector {
-    uint4 a, b;
-};
-
-__device__ __forceinline__ Sector load_sector(const uint32_t* store, uint32_t group, int lane) {
-    const uint4* p = reinterpret_cast<const uint4*>(store) + ((size_t)group * 32 + lane) * 2;
-    Sector s;
-    s.a = p[0];
-    s.b = p[1];
-    return s;
-}
-
-// Occupied cells, cells over the cap and points in cells over the cap of one sector.
-__device__ __forceinline__ void sector_stats(const ScaleDev& g, const Sector& s, int v[3]) {
-    if (g.mode == MODE_BITMAP) {
-        v[0] += __popc(s.a.x) + __popc(s.a.z) + __popc(s.b.x) + __popc(s.b.z);
-    } else {
-        const int n0 = (int)s.a.x, n1 = (int)s.b.x;
-        v[0] += (n0 > 0) + (n1 > 0);
-        if (g.cap > 0) {
-            if (n0 > g.cap) { v[1] += 1; v[2] += n0; }
-            if (n1 > g.cap) { v[1] += 1; v[2] += n1; }
-        }
-    }
-}
-
-// Ranks and cell list of one group of a BITMAP store: a lane owns one 32-byte sector, i.e. four
-// {bits, rank} words = 128 consecutive cells.  One warp scan of the lanes' popcounts places every
-// word; each lane then lists its own cells (a handful in all but the densest groups) with plain
-// stores that nothing waits for.  base0 = voxels before the group.
-__device__ __forceinline__ void rank_group_bitmap(const ScaleDev& g, uint32_t grp, Sector x, int base0, int lane) {
-    const uint32_t bw[4] = {x.a.x, x.a.z, x.b.x, x.b.z};
-    const int c = __popc(bw[0]) + __popc(bw[1]) + __popc(bw[2]) + __popc(bw[3]);
-    int inc = c;
+// Two launches.
+//   vox_count   streams the store once, a CTA per four 8 KB tiles: voxels per tile, their sum per 128 tiles,
+//               and a list of the tiles that hold any (most of a fine grid is empty space).
+//   vox_rank    a CTA per listed tile finds the voxels before it (sums of whole groups of 128 tiles plus
+//               those of its own group: a load or two per thread), ranks its units or cells and lists the
+//               occupied cells in rank order.
+// vox_count is bound by the streaming read (every cell of the grid is looked at), vox_rank by the latency of
+// its three dependent round trips and by the few tiles on the ground plane that hold most voxels: a thread
+// has one sector of 32 bytes, and a warp lists the cells of its 32 sectors together.
+__device__ __forceinline__ uint32_t warp_incl_scan(uint32_t x) {
+    const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-        const int y = __shfl_up_sync(0xFFFFFFFFu, inc, d);
-        if (lane >= d) inc += y;
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, d);
+        if (lane >= d) x += y;
     }
-    if (c == 0) return;
-    int m = base0 + inc - c;
-    const uint32_t word0 = (grp * 32u + lane) * 4u;
-    uint32_t rk[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        rk[i] = (uint32_t)m;
-        uint32_t bits = bw[i];
-        while (bits) {
-            const int bit = __ffs(bits) - 1;
-            bits &= bits - 1;
-            g.cell_list[m++] = (word0 + i) * 32u + bit;
-        }
-    }
-    x.a.y = rk[0]; x.a.w = rk[1]; x.b.y = rk[2]; x.b.w = rk[3];
-    uint4* p = reinterpret_cast<uint4*>(g.store) + ((size_t)grp * 32 + lane) * 2;
-    p[0] = x.a;
-    p[1] = x.b;
+    return x;
 }
 
-// Ranks, cell list and over-cap bookkeeping of one group of a TABLE store (two cell records per
-// lane).  base[] = voxels, cells over the cap and points in such cells before the group.
-__device__ __forceinline__ void rank_group_table(const ScaleDev& g, uint32_t grp, Sector x, const int base[3], int lane) {
-    int run[3] = {0, 0, 0}, gtot[3];
-    sector_stats(g, x, run);
-    const bool mine = run[0] > 0;
-    warp_excl_scan3(run, gtot);                   // run[] = exclusive offsets inside the group
-    if (!mine) return;
-    int m = base[0] + run[0];
-    int j = base[1] + run[1], off = base[2] + run[2];
-    const uint32_t cell0 = (grp * 32u + lane) * 2u;
-    x.a.y = (uint32_t)m; x.a.z = (uint32_t)j;
-    const int n0 = (int)x.a.x, n1 = (int)x.b.x;
-    const bool o0 = g.cap > 0 && n0 > g.cap, o1 = g.cap > 0 && n1 > g.cap;
-    if (o0) {
-        g.ovf_vox[j] = m; g.ovf_off[j] = off; g.ovf_cell[j] = cell0; g.ovf_cursor[(size_t)j * kCursorStride] = 0;
-        j += 1; off += n0;
-    }
-    if (n0 > 0) g.cell_list[m++] = cell0 | (o0 ? 0x80000000u : 0u);
-    x.b.y = (uint32_t)m; x.b.z = (uint32_t)j;
-    if (o1) {
-        g.ovf_vox[j] = m; g.ovf_off[j] = off; g.ovf_cell[j] = cell0 + 1u; g.ovf_cursor[(size_t)j * kCursorStride] = 0;
-    }
-    if (n1 > 0) g.cell_list[m] = (cell0 + 1u) | (o1 ? 0x80000000u : 0u);
-    uint4* p = reinterpret_cast<uint4*>(g.store) + ((size_t)grp * 32 + lane) * 2;
-    p[0] = x.a;
-    p[1] = x.b;
+// Occupied cells of a sector: two units or eight cells.
+__device__ __forceinline__ uint32_t sector_voxels(bool bitmap, const uint4& p, const uint4& q) {
+    if (bitmap) return __popc(p.x) + __popc(p.y) + __popc(p.z) + __popc(q.x) + __popc(q.y) + __popc(q.z);
+    return (p.x != 0u) + (p.y != 0u) + (p.z != 0u) + (p.w != 0u) + (q.x != 0u) + (q.y != 0u) + (q.z != 0u) + (q.w != 0u);
 }
 
-// The rank scan is three plain launches, each a few memory round trips deep, so that it keeps its
-// pace when it runs beside kernels that saturate the memory system (a deep chain of dependent loads
-// stretches with the latency of every hop).  A CTA owns 32 consecutive groups of one scale, a warp
-// four of them.
-//   vox_count   streams the store once: per-group counts into group_info, per-CTA totals.
-//   vox_prefix  one CTA per scale: exclusive prefix sums of the CTA totals, the scale's totals, the
-//               number of voxels and the capacity / consistency checks.
-//   vox_rank    a warp turns its CTA's 32 group counts into group bases with one warp scan, loads
-//               only its occupied groups (all at once), writes their ranks and lists their cells in
-//               rank order: the parallel prefix-sum index search of Sec. 3.6.  Also clears the
-//               accumulators of the voxels found.
-constexpr int kGroupsPerWarp = 4;
-constexpr int kGroupsPerCta = kGroupsPerWarp * (kThreads / 32);
-static_assert(kGroupsPerCta == 32, "vox_rank_kernel scans one group count per lane");
+constexpr int kScanSectors = (int)(kScanTileBytes / 32);          // 32-byte sectors per tile
+static_assert(kScanSectors == kThreads, "vox_count_kernel gives a thread one sector of each of its tiles");
 
-__global__ void __launch_bounds__(kThreads) vox_count_kernel(ScanArgs a) {
+__global__ void __launch_bounds__(kThreads) vox_count_kernel(const __grid_constant__ ScanArgs a) {
     constexpr int kWarps = kThreads / 32;
-    __shared__ int wtot[kWarps][3];
-    const int sc = (int)blockIdx.x >= a.ctas0 ? 1 : 0;
-    const uint32_t cta = blockIdx.x - (sc ? a.ctas0 : 0);
-    const ScaleDev& g = a.s[sc];
+    __shared__ uint32_t s_warp[kCountTiles][kWarps];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const uint32_t ng = a.ngroups_used[sc];
-    const uint32_t g0 = cta * kGroupsPerCta + warp * kGroupsPerWarp;
-    Sector x[kGroupsPerWarp];
+    int tile0 = (int)blockIdx.x * kCountTiles;
+    const int sc = tile0 < a.tiles[1] ? 1 : 0;
+    if (!sc) tile0 -= a.tiles[1];
+    const ScaleDev& g = a.s[sc];
+    const uint4* p = reinterpret_cast<const uint4*>(g.store) + ((size_t)tile0 * kScanSectors + t) * 2;
+    uint4 x[kCountTiles][2];
 #pragma unroll
-    for (int u = 0; u < kGroupsPerWarp; ++u) {
-        x[u].a = x[u].b = make_uint4(0u, 0u, 0u, 0u);
-        if (g0 + u < ng) {
-            const uint4* p = reinterpret_cast<const uint4*>(g.store) + ((size_t)(g0 + u) * 32 + lane) * 2;
-            x[u].a = __ldcs(p);                   // streaming: most of the store is empty, keep it out of L2
-            x[u].b = __ldcs(p + 1);
-        }
+    for (int u = 0; u < kCountTiles; ++u) {
+        x[u][0] = p[u * kScanSectors * 2];
+        x[u][1] = p[u * kScanSectors * 2 + 1];
     }
-    int carry[3] = {0, 0, 0};
 #pragma unroll
-    for (int u = 0; u < kGroupsPerWarp; ++u) {
-        int s[3] = {0, 0, 0};
-        sector_stats(g, x[u], s);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) s[k] = warp_sum(s[k]);
-        if (lane == 0 && g0 + u < ng) g.group_info[g0 + u] = make_int4(s[0], s[1], s[2], 0);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) carry[k] += s[k];
-    }
-    if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) wtot[warp][k] = carry[k];
+    for (int u = 0; u < kCountTiles; ++u) {
+        const uint32_t n = __reduce_add_sync(0xFFFFFFFFu, sector_voxels(g.mode == MODE_BITMAP, x[u][0], x[u][1]));
+        if (lane == 0) s_warp[u][warp] = n;
     }
     __syncthreads();
-    if (t < 3) {
-        int v = 0;
-        for (int w = 0; w < kWarps; ++w) v += wtot[w][t];
-        a.cta_tot[(size_t)blockIdx.x * 3 + t] = v;
+    if (t < kCountTiles) {
+        uint32_t n = 0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) n += s_warp[t][w];
+        a.st.tile_voxels[sc][tile0 + t] = n;
+        // One ticket per CTA: tickets on one address are served one after another (about 10 ns each).
+        constexpr unsigned kAll = (1u << kCountTiles) - 1u;
+        const unsigned some = __ballot_sync(kAll, n != 0u);
+        const uint32_t sum = __reduce_add_sync(kAll, n);          // the CTA's tiles are all in one group
+        uint32_t at = 0;
+        if (some && t == 0) {
+            atomicAdd(&a.st.group_voxels[sc][tile0 / kTilesPerGroup], sum);
+            at = atomicAdd(a.st.listed, (uint32_t)__popc(some));
+        }
+        at = __shfl_sync(kAll, at, 0) + __popc(some & ((1u << t) - 1u));
+        if (n) a.st.list[at] = (uint32_t)(tile0 + t) | (sc ? 0x80000000u : 0u);
     }
 }
 
-constexpr int kPrefixThreads = 1024;
+constexpr int kRankThreads = kScanSectors, kRankCtas = 6;
 
-// grid = 2: CTA sc scans the CTA totals of scale sc.  It also lists the CTAs that found any voxel
-// (most of a fine grid is empty space), so that the ranking pass only visits those.
-__global__ void __launch_bounds__(kPrefixThreads) vox_prefix_kernel(ScanArgs a) {
-    constexpr int kWarps = kPrefixThreads / 32;
-    __shared__ int wsum[4][kWarps];
-    __shared__ int tot[4];
-    const int sc = blockIdx.x;
-    const ScaleDev& g = a.s[sc];
-    if (g.design) return;                         // ranked by another design: its totals stand
-    const int first = sc ? a.ctas0 : 0, n = sc ? a.ctas1 : a.ctas0;
+__global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const __grid_constant__ ScanArgs a) {
+    constexpr int kWarps = kRankThreads / 32;
+    __shared__ uint32_t s_before[kWarps], s_warp[kWarps];
+    __shared__ int s_over[2];                             // cells over the cap and their points: sum, then base
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int per = (n + kPrefixThreads - 1) / kPrefixThreads;
-    const int lo = min(n, t * per), hi = min(n, lo + per);
-    const int* src = a.cta_tot + (size_t)first * 3;
-    int* dst = a.cta_base + (size_t)first * 3;
-    int run[4] = {0, 0, 0, 0};                    // voxels, cells over the cap, their points, CTAs with voxels
-    for (int i = lo; i < hi; ++i) {
+    const uint32_t listed = *a.st.listed;
+    uint32_t entry = blockIdx.x < listed ? a.st.list[blockIdx.x] : 0u, next = 0u;
+    // Voxels of both scales, and this CTA's share of their accumulators cleared: a few tiles hold most of the
+    // voxels, so the clearing is not tied to the tiles.  Done here, just before they are added to, it also brings
+    // them into L2 (cleared after use by vox_finalize, vox_accum took 48 instead of 43 us on four nuScenes-shaped
+    // frames and vox_finalize 40 instead of 37).
+    uint32_t all[2] = {0u, 0u};
 #pragma unroll
-        for (int k = 0; k < 3; ++k) run[k] += src[(size_t)i * 3 + k];
-        run[3] += src[(size_t)i * 3] > 0;
-    }
+    for (int v = 0; v < 2; ++v)
+        for (int i = t; i * kTilesPerGroup < a.tiles[v]; i += kRankThreads) all[v] += a.st.group_voxels[v][i];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {                 // run[] becomes exclusive inside the warp
-        int x = run[k];
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int y = __shfl_up_sync(0xFFFFFFFFu, x, d);
-            if (lane >= d) x += y;
-        }
-        if (lane == 31) wsum[k][warp] = x;
-        run[k] = x - run[k];
-    }
-    __syncthreads();
-    if (warp < 4) {                               // warp k scans the warp totals of counter k
-        int x = wsum[warp][lane];
-        const int v = x;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int y = __shfl_up_sync(0xFFFFFFFFu, x, d);
-            if (lane >= d) x += y;
-        }
-        wsum[warp][lane] = x - v;
-        if (lane == 31) tot[warp] = x;
+    for (int v = 0; v < 2; ++v) {
+        all[v] = __reduce_add_sync(0xFFFFFFFFu, all[v]);
+        if (lane == 0) (v ? s_warp : s_before)[warp] = all[v];
     }
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 4; ++k) run[k] += wsum[k][warp];
-    for (int i = lo; i < hi; ++i) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) dst[(size_t)i * 3 + k] = run[k];
-        const int v0 = src[(size_t)i * 3];
-        if (v0 > 0) a.unit_list[first + run[3]++] = i;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) run[k] += src[(size_t)i * 3 + k];
-    }
-    if (t == 0) {
-        // More voxels, cells over the cap or points in them than a call's points allow: the store was
-        // not all zero when the call began (two calls on one handle at once).  Nothing is ranked or
-        // listed then; the scale reports no voxels and the handle's status becomes an internal error.
-        const bool dirty = (uint32_t)tot[0] > g.max_list || (uint32_t)tot[1] > g.max_ovf || (uint32_t)tot[2] > g.max_list;
-        g.totals[0] = dirty ? 0 : tot[0]; g.totals[1] = dirty ? 0 : tot[1]; g.totals[2] = dirty ? 0 : tot[2];
-        g.totals[3] = dirty ? 0 : tot[3];         // CTAs the ranking pass has to visit
-        a.num_voxels[sc] = dirty ? 0 : tot[0];
+    for (int v = 0; v < 2; ++v) all[v] = __reduce_add_sync(0xFFFFFFFFu, lane < kWarps ? (v ? s_warp : s_before)[lane] : 0u);
+    if (blockIdx.x == 0 && t < 2 && !a.s[t].design) {
+        // More voxels than a call's points allow: the store was not all zero when the call began (two
+        // calls on one handle at once).  The scale then reports no voxels and the handle's status
+        // becomes an internal error; rows past the lists are not written anywhere.
+        const ScaleDev& g = a.s[t];
+        const uint32_t n = t ? all[1] : all[0];
+        const bool dirty = n > g.max_list;
+        g.totals[0] = dirty ? 0 : (int)n;
+        a.num_voxels[t] = dirty ? 0 : (int)n;
         if (dirty) atomicOr(a.status, kStatusDirtyStore);
-        else if (tot[0] > a.capacity[sc]) atomicOr(a.status, kStatusCapacity);
+        else if ((int)n > a.capacity[t]) atomicOr(a.status, kStatusCapacity);
     }
-}
-
-// A fixed grid: every CTA first clears its share of the accumulators of the voxels found (two
-// 16-byte halves per voxel), then takes the listed units (32 groups of one scale) in turn.
-__global__ void __launch_bounds__(kThreads, 5) vox_rank_kernel(ScanArgs a) {
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int n0 = a.s[0].totals[3], n1 = a.s[1].totals[3];
-    const int v0 = a.s[0].totals[0], v1 = a.s[1].totals[0];
     {
+        const size_t n0 = (size_t)min(all[0], a.s[0].max_list) * a.s[0].acc_f4, n1 = (size_t)min(all[1], a.s[1].max_list) * a.s[1].acc_f4;
         const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-        const size_t c0 = 2 * (size_t)v0, c1 = 2 * (size_t)v1;
-        for (size_t i = (size_t)blockIdx.x * kThreads + t; i < c0 + c1; i += (size_t)gridDim.x * kThreads) {
-            if (i < c0) a.s[0].acc[i] = z; else a.s[1].acc[i - c0] = z;
-        }
+        for (size_t i = (size_t)blockIdx.x * kRankThreads + t; i < n0; i += (size_t)gridDim.x * kRankThreads) a.s[0].acc[i] = z;
+        for (size_t i = (size_t)blockIdx.x * kRankThreads + t; i < n1; i += (size_t)gridDim.x * kRankThreads) a.s[1].acc[i] = z;
     }
-    for (int u = blockIdx.x; u < n0 + n1; u += gridDim.x) {
-        const int sc = u >= n0 ? 1 : 0;
+    __syncthreads();
+    for (uint32_t k = blockIdx.x; k < listed; k += gridDim.x, entry = next) {
+        if (k + gridDim.x < listed) next = a.st.list[k + gridDim.x];
+        const int sc = (int)(entry >> 31), tile = (int)(entry & 0x7FFFFFFFu);
         const ScaleDev& g = a.s[sc];
-        const int first = sc ? a.ctas0 : 0;
-        const uint32_t cta = (uint32_t)a.unit_list[first + (sc ? u - n0 : u)];
-        const uint32_t ng = a.ngroups_used[sc];
-        const uint32_t gc = cta * kGroupsPerCta;
-        int pre[3] = {0, 0, 0}, ctot[3];
-        if (gc + lane < ng) {
-            const int4 info = g.group_info[gc + lane];
-            pre[0] = info.x; pre[1] = info.y; pre[2] = info.z;
-        }
-        int base[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) base[k] = a.cta_base[(size_t)(first + cta) * 3 + k];
-        const unsigned occupied = __ballot_sync(0xFFFFFFFFu, pre[0] > 0);
         const bool bitmap = g.mode == MODE_BITMAP;
-        // The unit's occupied groups are dealt to the warps round-robin (a unit in open space has a few,
-        // one on the ground plane all 32); a warp requests all of its groups before it ranks any.
-        const int nocc = __popc(occupied);
-        int gidx[kGroupsPerWarp];
-        Sector x[kGroupsPerWarp];
+        const uint32_t sector = (uint32_t)tile * kScanSectors + t;
+        uint4* const at = reinterpret_cast<uint4*>(g.store) + (size_t)sector * 2;
+        uint4 p = at[0], q = at[1];
+        // Voxels before the tile: groups before its group, tiles of its group before it.
+        const int group = tile / kTilesPerGroup, in_group = tile % kTilesPerGroup;
+        uint32_t before = 0;
+        if (t < in_group) before = a.st.tile_voxels[sc][group * kTilesPerGroup + t];
+        for (int i = kRankThreads - 1 - t; i < group; i += kRankThreads) before += a.st.group_voxels[sc][i];
+        before = __reduce_add_sync(0xFFFFFFFFu, before);
+        const uint32_t c = sector_voxels(bitmap, p, q);
+        const uint32_t inc = warp_incl_scan(c);
+        if (lane == 31) { s_before[warp] = before; s_warp[warp] = inc; }
+        if (t < 2) s_over[t] = 0;
+        __syncthreads();
+        const uint32_t base = __reduce_add_sync(0xFFFFFFFFu, lane < kWarps ? s_before[lane] : 0u);
+        const uint32_t own = lane < kWarps ? s_warp[lane] : 0u;
+        uint32_t m = base + __reduce_add_sync(0xFFFFFFFFu, lane < warp ? own : 0u) + inc - c;
+        // Cells over the cap take the next places among such cells, and their points the next slots of
+        // the index list, in any order: one ticket per tile.
+        uint32_t j = 0, off = 0;
+        if (!bitmap && g.cap > 0) {
+            const uint32_t n[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+            uint32_t cells = 0, points = 0;
 #pragma unroll
-        for (int i = 0; i < kGroupsPerWarp; ++i) {
-            const int k = warp + i * (kThreads / 32);
-            gidx[i] = k < nocc ? (int)__fns(occupied, 0, k + 1) : -1;
-            if (gidx[i] >= 0) x[i] = load_sector(g.store, gc + gidx[i], lane);
+            for (int i = 0; i < 8; ++i)
+                if (n[i] > (uint32_t)g.cap) { cells += 1; points += n[i]; }
+            if (__any_sync(0xFFFFFFFFu, cells != 0)) {
+                const uint32_t ic = warp_incl_scan(cells), ip = warp_incl_scan(points);
+                int wc = 0, wp = 0;                       // the warp's share starts here inside the tile's
+                if (lane == 31) { wc = atomicAdd(&s_over[0], (int)ic); wp = atomicAdd(&s_over[1], (int)ip); }
+                j = (uint32_t)__shfl_sync(0xFFFFFFFFu, wc, 31) + ic - cells;
+                off = (uint32_t)__shfl_sync(0xFFFFFFFFu, wp, 31) + ip - points;
+            }
+            __syncthreads();
+            if (t == 0 && s_over[0] > 0) {
+                const unsigned long long add = ((unsigned long long)(uint32_t)s_over[0] << 32) | (uint32_t)s_over[1];
+                const unsigned long long first = atomicAdd(reinterpret_cast<unsigned long long*>(g.totals + 2), add);
+                s_over[0] = (int)(first >> 32); s_over[1] = (int)(uint32_t)first;
+            }
+            __syncthreads();
+            j += (uint32_t)s_over[0];
+            off += (uint32_t)s_over[1];
         }
-        warp_excl_scan3(pre, ctot);               // pre[] = what the unit's groups before this lane's group hold
+        if (bitmap) {
+            const uint32_t w[6] = {p.x, p.y, p.z, q.x, q.y, q.z};
+            if (c != 0u) {
+                p.w = m;
+                q.w = m + __popc(p.x) + __popc(p.y) + __popc(p.z);
+                at[0] = p;
+                at[1] = q;
+            }
+            uint32_t cell = sector * (2u * kUnitCells);
 #pragma unroll
-        for (int i = 0; i < kGroupsPerWarp; ++i) {
-            if (gidx[i] < 0) break;
-            int gb[3];
+            for (int i = 0; i < 6; ++i, cell += 32u) {
+                for (uint32_t bits = w[i]; bits; bits &= bits - 1u, ++m)
+                    if (m < g.max_list) g.cell_list[m] = cell + (uint32_t)__ffs(bits) - 1u;
+            }
+        } else {
+            if (c != 0u) {
+                const uint32_t cell = sector * 8u;
+                uint32_t n[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
 #pragma unroll
-            for (int k = 0; k < 3; ++k) gb[k] = base[k] + __shfl_sync(0xFFFFFFFFu, pre[k], gidx[i]);
-            if (bitmap) rank_group_bitmap(g, gc + gidx[i], x[i], gb[0], lane);
-            else rank_group_table(g, gc + gidx[i], x[i], gb, lane);
+                for (int i = 0; i < 8; ++i) {
+                    if (n[i] == 0u) continue;
+                    const bool over = g.cap > 0 && n[i] > (uint32_t)g.cap;
+                    if (m < (uint32_t)a.capacity[sc]) a.counts[sc][m] = over ? g.cap : (int)n[i];
+                    if (m < g.max_list) g.cell_list[m] = over ? (cell + i) | kOverCap : cell + i;
+                    if (over) {
+                        if (j < g.max_ovf && off + n[i] <= g.max_list) {
+                            g.ovf_vox[j] = (int)m; g.ovf_off[j] = (int)off; g.ovf_cell[j] = cell + i;
+                            g.ovf_cursor[(size_t)j * kCursorStride] = 0;
+                        }
+                        off += n[i];
+                        n[i] = kOverCap | j++;
+                    } else {
+                        n[i] = m;
+                    }
+                    ++m;
+                }
+                at[0] = make_uint4(n[0], n[1], n[2], n[3]);
+                at[1] = make_uint4(n[4], n[5], n[6], n[7]);
+            }
         }
+        __syncthreads();                                  // the shared counters are used again
     }
 }
 
 // ------------------------------------------------------------------ pass 3: accumulate
 struct AccumArgs {
     ScaleDev s[2];
-    uint32_t ngroups_used[2];
-    int capacity[2];
+    int capacity[2];            // at most max_list
     int32_t* coords[2];
     int32_t* counts[2];
     int32_t* point_voxel[2];
@@ -408,7 +323,8 @@ struct AccumArgs {
 
 // Per-voxel accumulator, 32 bytes of fp32: {sum dx, sum dy, sum dz, sum ch3}, {sum ch4, count, -, -},
 // where d* are offsets from the cell's lower corner, so that those sums stay small.  Two vector
-// reductions per point and scale.  A sum of n terms carries a relative error of at most n * 2^-24
+// reductions per point and scale; a table store's voxels have their counts already, so there the second
+// one only adds ch4, and with four channels there is neither a second reduction nor a second half.  A sum of n terms carries a relative error of at most n * 2^-24
 // (far less in practice, since the roundings do not line up).
 template <int C>
 __global__ void __launch_bounds__(kThreads)
@@ -469,9 +385,10 @@ vox_accum_kernel(const float* __restrict__ pts, long long total, int N, AccumArg
             const float dx = __fsub_rn(sp[t * C], cell_corner(g.mn[0], g.vs[0], cx[sc][i]));
             const float dy = __fsub_rn(sp[t * C + 1], cell_corner(g.mn[1], g.vs[1], cy[sc][i]));
             const float dz = __fsub_rn(sp[t * C + 2], cell_corner(g.mn[2], g.vs[2], cz[sc][i]));
-            float4* row = g.acc + 2 * (size_t)s.m;
+            float4* row = g.acc + (size_t)s.m * g.acc_f4;
             atomicAdd(row, make_float4(dx, dy, dz, sp[t * C + 3]));
-            atomicAdd(reinterpret_cast<float2*>(row + 1), make_float2(C > 4 ? sp[t * C + 4] : 0.0f, 1.0f));
+            if (g.mode == MODE_BITMAP) atomicAdd(reinterpret_cast<float2*>(row + 1), make_float2(C > 4 ? sp[t * C + 4] : 0.0f, 1.0f));
+            else if (C > 4) atomicAdd(reinterpret_cast<float*>(row + 1), sp[t * C + 4]);
         }
     }
 }
@@ -503,8 +420,9 @@ __global__ void __launch_bounds__(kThreads) vox_over_find_kernel(AccumArgs a, in
         }
         int j0 = 0, off0 = 0;
         if (lane == 31) {
-            j0 = atomicAdd(&g.totals[1], __popc(who));
-            off0 = atomicAdd(&g.totals[2], inc);
+            const unsigned long long add = ((unsigned long long)__popc(who) << 32) | (uint32_t)inc;
+            const unsigned long long at = atomicAdd(reinterpret_cast<unsigned long long*>(g.totals + 2), add);
+            j0 = (int)(at >> 32); off0 = (int)(uint32_t)at;
         }
         j0 = __shfl_sync(0xFFFFFFFFu, j0, 31);
         off0 = __shfl_sync(0xFFFFFFFFu, off0, 31);
@@ -546,23 +464,30 @@ __device__ __forceinline__ void write_batch(const AccumArgs& a, int sc, int mb, 
     const int lane = threadIdx.x & 31;
     n = min(n, a.capacity[sc] - mb);              // rows past the caller's capacity are not written
     if (n <= 0) return;
-    const float4* src = g.acc + 2 * (size_t)mb;
-    if (lane < 2 * n) stage[lane] = src[lane];
-    if (lane + 32 < 2 * n) stage[lane + 32] = src[lane + 32];
-    __syncwarp();
-    const float4 a0 = stage[2 * lane], a1 = stage[2 * lane + 1];
-    __syncwarp();
     const bool active = lane < n;
     const bool table = g.mode == MODE_TABLE;
-    const uint32_t cell = table ? (entry & 0x7FFFFFFFu) : entry;
+    int cnt = table && active ? a.counts[sc][mb + lane] : 1;         // the rank scan wrote a table store's counts
+    float4 a0, a1;
+    if (g.acc_f4 == 2) {
+        const float4* src = g.acc + 2 * (size_t)mb;
+        if (lane < 2 * n) stage[lane] = __ldcg(src + lane);
+        if (lane + 32 < 2 * n) stage[lane + 32] = __ldcg(src + lane + 32);
+        __syncwarp();
+        a0 = stage[2 * lane]; a1 = stage[2 * lane + 1];
+        __syncwarp();
+    } else {
+        a0 = a1 = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (active) a0 = __ldcg(g.acc + mb + lane);
+    }
+    const uint32_t cell = table ? (entry & ~kOverCap) : entry;
     // Over the cap: a table store flags the cell in its list entry; a bitmap store has no per-cell count,
     // there vox_over_find_kernel left the voxel's place among the over-cap voxels (+ 1) in a spare word.
-    const bool over = active && ((table && (entry >> 31) != 0u) || __float_as_uint(a1.z) != 0u);
+    const bool over = active && (table ? (entry & kOverCap) != 0u : __float_as_uint(a1.z) != 0u);
     uint32_t r = cell, x, y, z;
     g.div[0].divmod(r, r, x);
     g.div[1].divmod(r, r, y);
     g.div[2].divmod(r, r, z);
-    const int cnt = over ? g.cap : (int)a1.y;
+    if (!table) cnt = over ? g.cap : (int)a1.y;
     // Offsets are below one cell size, so fp32 keeps the mean to a few 1e-7 of that size.
     const float inv = __frcp_rn((float)cnt);
     float mu[C];
@@ -573,7 +498,7 @@ __device__ __forceinline__ void write_batch(const AccumArgs& a, int sc, int mb, 
     if (C > 4) mu[4] = __fdiv_rn(a1.x, (float)cnt);
     if (active) {
         reinterpret_cast<int4*>(a.coords[sc])[mb + lane] = make_int4((int)r, (int)z, (int)y, (int)x);
-        a.counts[sc][mb + lane] = cnt;
+        if (!table) a.counts[sc][mb + lane] = cnt;
     }
     // Mean rows: the n * C floats of rows mb .. mb+n-1 are contiguous.  The row of a cell over the
     // cap is written by that cell's own warp, so a batch holding one writes its rows one by one.
@@ -611,12 +536,12 @@ vox_finalize_kernel(const float* __restrict__ pts, long long total, AccumArgs a,
         for (int sc = 0; sc < 2; ++sc) {
             const ScaleDev& g = a.s[sc];
             if (g.cap <= 0) continue;
-            const int novf = g.totals[1];
+            const int novf = min(g.totals[3], (int)g.max_ovf);
             int32_t* pv = a.point_voxel[sc];
             for (int j = warp; j < novf; j += nwarps) {
                 const int m = g.ovf_vox[j];
-                const int n = g.ovf_cursor[(size_t)j * kCursorStride];
                 const int* list = g.ovf_list + g.ovf_off[j];
+                const int n = min(g.ovf_cursor[(size_t)j * kCursorStride], (int)g.max_list - g.ovf_off[j]);
                 // Smallest index value v with #{list <= v} >= cap, by bisection on the value.
                 long long lo = -1, hi = total - 1;
                 while (hi - lo > 1) {
@@ -662,8 +587,8 @@ vox_finalize_kernel(const float* __restrict__ pts, long long total, AccumArgs a,
         return;
     }
     // Voxel rows: a warp takes 32 consecutive rows of one scale at a time, reads their cell ids
-    // from the list the rank scan wrote, writes the rows and puts the cells' store words back to
-    // zero (whole 32-byte sectors of a bitmap store: a partial write would first fetch the sector).
+    // from the list the rank scan wrote, writes the rows and puts the cells' store sectors back to
+    // zero (whole 32-byte sectors: a partial write would first fetch the sector), once per run of voxels.
     // Every warp has its own batch, so the batches' memory latencies overlap.
     __shared__ float4 s_stage[kWarps][64];
     float4* stage = s_stage[threadIdx.x >> 5];
@@ -676,14 +601,12 @@ vox_finalize_kernel(const float* __restrict__ pts, long long total, AccumArgs a,
         const ScaleDev& g = a.s[sc];
         const int n = min(32, (sc ? tot1 : tot0) - mb);
         const uint32_t entry = lane < n ? g.cell_list[mb + lane] : 0u;
-        if (lane < n && !g.design) {
-            if (g.mode == MODE_BITMAP) {
-                uint4* sp = reinterpret_cast<uint4*>(g.store + 8 * (size_t)(entry >> 7));
-                sp[0] = make_uint4(0u, 0u, 0u, 0u);
-                sp[1] = make_uint4(0u, 0u, 0u, 0u);
-            } else {
-                *reinterpret_cast<uint4*>(g.store + 4 * (size_t)(entry & 0x7FFFFFFFu)) = make_uint4(0u, 0u, 0u, 0u);
-            }
+        const uint32_t sector = g.mode == MODE_BITMAP ? entry / (2u * kUnitCells) : (entry & ~kOverCap) >> 3;
+        const uint32_t before = __shfl_up_sync(0xFFFFFFFFu, sector, 1);
+        if (lane < n && !g.design && (lane == 0 || before != sector)) {
+            uint4* sp = reinterpret_cast<uint4*>(g.store + 8 * (size_t)sector);
+            sp[0] = make_uint4(0u, 0u, 0u, 0u);
+            sp[1] = make_uint4(0u, 0u, 0u, 0u);
         }
         write_batch<C>(a, sc, mb, n, entry, stage);
     }
@@ -705,9 +628,11 @@ int run_voxelize(emc2_bridge* h, int B, int N, const float* d_points, int32_t* c
         if (sa.s[s].design) sa.s[s].mode = MODE_BITMAP;
         aa.s[s] = sa.s[s];
         const uint64_t cells = sa.s[s].design ? 0 : (uint64_t)B * h->scale[s].cells;
-        const uint64_t per_group = h->scale[s].mode == MODE_BITMAP ? kBitmapGroupCells : kTableGroupCells;
-        sa.ngroups_used[s] = aa.ngroups_used[s] = (uint32_t)((cells + per_group - 1) / per_group);
-        sa.capacity[s] = aa.capacity[s] = capacity[s];
+        const uint64_t per_tile = sa.s[s].mode == MODE_BITMAP ? kBitmapTileCells : kTableTileCells;
+        sa.tiles[s] = (int)((cells + per_tile - 1) / per_tile + kCountTiles - 1) / kCountTiles * kCountTiles;
+        sa.capacity[s] = capacity[s];
+        sa.counts[s] = d_counts[s];
+        aa.capacity[s] = (int)min((long long)capacity[s], (long long)h->scale[s].max_list);
         aa.coords[s] = d_coords[s];
         aa.counts[s] = d_counts[s];
         aa.mean[s] = d_mean[s];
@@ -716,11 +641,7 @@ int run_voxelize(emc2_bridge* h, int B, int N, const float* d_points, int32_t* c
     }
     sa.num_voxels = d_num_voxels;
     sa.status = h->d_status;
-    sa.cta_tot = h->d_scan_tot;
-    sa.cta_base = h->d_scan_base;
-    sa.unit_list = h->d_scan_units;
-    sa.ctas0 = (int)((sa.ngroups_used[0] + kGroupsPerCta - 1) / kGroupsPerCta);
-    sa.ctas1 = (int)((sa.ngroups_used[1] + kGroupsPerCta - 1) / kGroupsPerCta);
+    sa.st = h->scan;
     aa.bev = d_bev;
 
     const size_t bev_n = d_bev ? (size_t)B * C * h->scale[1].dims[1] * h->scale[1].dims[0] : 0;
@@ -733,7 +654,7 @@ int run_voxelize(emc2_bridge* h, int B, int N, const float* d_points, int32_t* c
             LaunchScope ls(h, K_VOX_MARK, st);
             vox_mark_kernel<C><<<blocks, kThreads, 0, st>>>(d_points, total, N, sa.s[0], sa.s[1],
                                                            bev_vec ? reinterpret_cast<float4*>(d_bev) : nullptr,
-                                                           bev_vec ? bev_n >> 2 : 0);
+                                                           bev_vec ? bev_n >> 2 : 0, scan_reset(h));
         }
     }
     for (int s = 0; s < 2; ++s) {
@@ -741,17 +662,15 @@ int run_voxelize(emc2_bridge* h, int B, int N, const float* d_points, int32_t* c
         const int rc = launch_dedup_arm(h, s, h->scale[s].design, B, N, d_points, capacity[s], d_num_voxels, st);
         if (rc != EMC2_OK) return rc;
     }
-    if (sa.ctas0 + sa.ctas1 > 0) {
-        LaunchScope ls(h, K_VOX_COUNT, st);
-        vox_count_kernel<<<sa.ctas0 + sa.ctas1, kThreads, 0, st>>>(sa);
-    }
-    {
-        LaunchScope ls(h, K_VOX_PREFIX, st);      // with no frames it still reports zero voxels
-        vox_prefix_kernel<<<2, kPrefixThreads, 0, st>>>(sa);
-    }
-    if (sa.ctas0 + sa.ctas1 > 0) {
+    if (total == 0) return check_cuda(h, cudaMemsetAsync(d_num_voxels, 0, 2 * sizeof(int32_t), st));   // no points: no voxels
+    const int tiles = sa.tiles[0] + sa.tiles[1];
+    if (tiles > 0) {
+        {
+            LaunchScope ls(h, K_VOX_COUNT, st);
+            vox_count_kernel<<<tiles / kCountTiles, kThreads, 0, st>>>(sa);
+        }
         LaunchScope ls(h, K_VOX_RANK, st);
-        vox_rank_kernel<<<min(sa.ctas0 + sa.ctas1, 5 * h->num_sms), kThreads, 0, st>>>(sa);
+        vox_rank_kernel<<<min(tiles, kRankCtas * h->num_sms), kRankThreads, 0, st>>>(sa);
     }
     if (total > 0) {
         LaunchScope ls(h, K_VOX_ACCUM, st);

@@ -1,0 +1,79 @@
+"""Edges of the voxel cell stores (needs a B200)."""
+from dataclasses import replace
+
+import numpy as np
+import pytest
+import torch
+
+import emc2_gen as gen
+from emc2_gen.configs import Grid
+from parity import close, np_
+
+pytestmark = pytest.mark.gpu
+
+# A store of units of 96 cells, 8 KB tiles of 49,152 cells, groups of 128 tiles; more than 2^24 cells.
+BITMAP = Grid(min=(0.0, 0.0, 0.0), voxel=(1.0, 1.0, 1.0), dims=(4099, 4099, 1))
+# A store of one word per cell, tiles of 2,048 cells.
+TABLE = Grid(min=(0.0, 0.0, 0.0), voxel=(1.0, 1.0, 1.0), dims=(257, 255, 1), max_points=3)
+
+
+def bridge_for(w):
+    import paper_2507_04123_b200 as pkg
+    return pkg.Bridge(pkg.config_from_workload(w))
+
+
+def check_voxels(w, pts, oracle, repeat=2, rules=False):
+    br = bridge_for(w)
+    d = torch.from_numpy(pts).cuda()
+    for _ in range(repeat):                                    # a second call must see clean stores
+        vox = br.voxelize(d)
+        br.status()
+        for s, g in enumerate(w.grids):
+            ref = oracle.voxelize(pts, g.min, g.voxel, g.dims, g.max_points)
+            M = ref["num_voxels"]
+            assert int(vox["num_voxels"][s]) == M
+            for k in ("coords", "counts"):
+                assert np.array_equal(np_(vox[k][s])[:M], ref[k]), (k, s)
+            assert np.array_equal(np_(vox["point_voxel"][s]), ref["point_voxel"]), s
+            ok, mx, _ = close(np_(vox["mean"][s])[:M], ref["mean"])
+            assert ok, (s, mx)
+            if rules:
+                out = br.rulebook(vox, s)
+                br.status()
+                off, rin, rout = oracle.rulebook(ref["coords"])
+                assert np.array_equal(np_(out["offsets"]), off)
+                assert np.array_equal(np_(out["rule_in"])[:off[27]], rin)
+                assert np.array_equal(np_(out["rule_out"])[:off[27]], rout)
+    br.close()
+
+
+def centres(ids, grid, C, rng):
+    ids = np.asarray(ids, np.int64)
+    x, y = ids % grid.dims[0], ids // grid.dims[0]
+    pts = np.concatenate([np.stack([x + 0.5, y + 0.5, np.full(len(ids), 0.5)], 1), rng.random((len(ids), C - 3))], 1)
+    return pts.astype(np.float32)
+
+
+@pytest.mark.parametrize("C", [4, 5])
+@pytest.mark.parametrize("which", ["edges", "full_tile", "last_cells", "one"])
+def test_units_tiles_and_groups_of_the_stores(oracle, which, C):
+    rng = np.random.default_rng(3)
+    tile, cells = 49152, BITMAP.cells
+    if which == "edges":                                       # both sides of every unit, sector, tile and group edge
+        at = [e + d for e in (0, 32, 64, 96, 192, 6144, tile, 4 * tile, 127 * tile, 128 * tile, 256 * tile, 4099 * 96)
+              for d in range(-3, 4)]
+    elif which == "full_tile":                                 # every cell of a tile and the rows above and below
+        at = list(range(tile - 4200, 2 * tile + 4200))
+    elif which == "last_cells":
+        at = list(range(cells - 300, cells))
+    else:
+        at = [cells // 2]
+    at = sorted({a for a in at if 0 <= a < cells})
+    fine = centres(rng.permutation(np.repeat(at, 2)), BITMAP, C, rng)
+    # table cells around tile edges, some of them over their cap of 3
+    few = [a for e in (0, 8, 2048, 4 * 2048, TABLE.cells) for a in range(e - 9, e + 9) if 0 <= a < TABLE.cells]
+    table = centres(rng.permutation(np.repeat(few, rng.integers(1, 7, len(few)))), TABLE, C, rng)
+    pts = rng.permutation(np.concatenate([fine, table]))[None]
+    base = gen.KITTI if C == 4 else gen.NUSCENES
+    w = replace(base.with_shape(1, pts.shape[1]), grids=(BITMAP, TABLE))
+    check_voxels(w, np.ascontiguousarray(pts), oracle, rules=which in ("edges", "last_cells"))
