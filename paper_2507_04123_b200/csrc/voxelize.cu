@@ -349,10 +349,8 @@ vox_accum_kernel(const float* __restrict__ pts, long long total, int N, AccumArg
             cx[sc][i] = cy[sc][i] = cz[sc][i] = 0;
             if (t < npts) {
                 const float x = sp[t * C], y = sp[t * C + 1], z = sp[t * C + 2];
-                const int ix = axis_cell(x, g.mn[0], g.vs[0], g.dims[0]);
-                const int iy = axis_cell(y, g.mn[1], g.vs[1], g.dims[1]);
-                const int iz = axis_cell(z, g.mn[2], g.vs[2], g.dims[2]);
-                if ((ix | iy | iz) >= 0) {
+                int ix, iy, iz;
+                if (cell_xyz(g, x, y, z, ix, iy, iz)) {
                     const int b = b0 + (i0 + t) / N;
                     cell = (((uint32_t)b * g.dims[2] + iz) * g.dims[1] + iy) * g.dims[0] + ix;
                     cx[sc][i] = ix; cy[sc][i] = iy; cz[sc][i] = iz;

@@ -1,4 +1,4 @@
-"""Edges of the voxel cell stores (needs a B200)."""
+"""Edges of the voxel cell stores and of the cell rule (needs a B200)."""
 from dataclasses import replace
 
 import numpy as np
@@ -77,3 +77,35 @@ def test_units_tiles_and_groups_of_the_stores(oracle, which, C):
     base = gen.KITTI if C == 4 else gen.NUSCENES
     w = replace(base.with_shape(1, pts.shape[1]), grids=(BITMAP, TABLE))
     check_voxels(w, np.ascontiguousarray(pts), oracle, rules=which in ("edges", "last_cells"))
+
+
+@pytest.mark.parametrize("dims", [(1408, 1600, 40), (61, 7, 3), (2_000_000, 2, 2)])
+def test_cells_of_points_on_cell_boundaries(oracle, dims):
+    """Points a few ulps around multiples of the cell size, far away, and not finite: cells as by subtract, divide, floor."""
+    rng = np.random.default_rng(5)
+    for mn, vs in (((0.0, -40.0, -3.0), (0.05, 0.05, 0.1)), ((-51.2, -51.2, -5.0), (0.075, 1.0 / 3.0, 0.2)),
+                   ((1e-3, 0.0, 0.0), (4.0, 1e-3, 1e-30)), ((0.0, 0.0, 0.0), (1e-39, 3.0, 1e30))):
+        grid = Grid(min=mn, voxel=vs, dims=dims)
+        pillars = Grid(min=mn, voxel=vs, dims=(dims[0] % 997 + 1, dims[1], 1))
+        n = 4099
+        pts = np.zeros((1, n, 4), np.float32)
+        for k in range(3):
+            lo, size = np.float32(mn[k]), np.float32(vs[k])
+            with np.errstate(over="ignore", under="ignore"):
+                v = (lo + rng.integers(-2, dims[k] + 2, n).astype(np.float32) * size).astype(np.float32)
+            for _ in range(4):
+                v = np.where(rng.random(n) < 0.5, np.nextafter(v, np.float32(rng.choice([-np.inf, np.inf]))), v)
+            pts[0, :, k] = v
+        odd = np.array([np.nan, np.inf, -np.inf, 3e38, -3e38, 1e-45, -1e-45, 0.0, -0.0, 1.2e7, 1.7e7, 3.4e7, -1.2e7], np.float32)
+        pts[0, :600, :3] = rng.choice(odd, (600, 3))
+        pts[0, 600:900, 0] = rng.choice(odd, 300)
+        w = replace(gen.KITTI.with_shape(1, n), grids=(grid, pillars))
+        br = bridge_for(w)
+        vox = br.voxelize(torch.from_numpy(pts).cuda())
+        br.status()
+        for s, g in enumerate(w.grids):
+            ref = oracle.voxelize(pts, g.min, g.voxel, g.dims, 0)
+            assert int(vox["num_voxels"][s]) == ref["num_voxels"]
+            assert np.array_equal(np_(vox["coords"][s])[:ref["num_voxels"]], ref["coords"])
+            assert np.array_equal(np_(vox["point_voxel"][s]), ref["point_voxel"])
+        br.close()
