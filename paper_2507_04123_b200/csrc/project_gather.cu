@@ -34,52 +34,104 @@ struct Projected {
     float u, v, d;      // pixel and depth in `best`; (-1, -1, depth in camera 0 or 0) if none
 };
 
-// `P` points to the frame's matrices as float4 rows in shared memory.  The visibility decision is
-// the one of the plain definition (fp32 fma chains, IEEE divide, compare), but the divide is only
-// executed where it can matter: comparing the numerators with bounds scaled by the depth settles
-// every pixel that is not within 0.01 px of an image edge, and only the chosen camera's (u, v) is
-// divided out.  A warp of scattered points therefore does not walk the divide once per camera.
-__device__ __forceinline__ Projected project_point(const float4* P, int K, float x, float y, float z,
+// Two fp32 operations per instruction (fma.rn.f32x2 and mul.rn.f32x2 of sm_100): the same roundings as the
+// scalar forms.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// A camera's matrix as the projection reads it: rows 0 and 1 side by side, for paired arithmetic.
+struct __align__(16) Camera {
+    uint64_t x, y, z, w;    // columns of rows 0 and 1
+    float4 r2;              // row 2
+};
+
+// (t0, t1) and t2: the numerators and the depth of one point, fp32 fma chains.
+__device__ __forceinline__ void chains(const Camera& c, float x, float y, float z, uint64_t& t01, float& t2) {
+    t01 = fma2(c.x, pack2(x, x), fma2(c.y, pack2(y, y), fma2(c.z, pack2(z, z), c.w)));
+    t2 = __fmaf_rn(c.r2.x, x, __fmaf_rn(c.r2.y, y, __fmaf_rn(c.r2.z, z, c.r2.w)));
+}
+
+// The visibility decision is the one of the plain definition (fp32 fma chains, IEEE divide, compare), but
+// the divide is only executed where it can matter: the distance of the numerator from the image centre,
+// compared with half the image size scaled by the depth, settles every pixel that is not within `eps` of an
+// image edge (eps is far above the roundings of these products), and only the chosen camera's (u, v) is
+// divided out.  The loop over the cameras has no branches; cameras that are left undecided are taken up
+// after it.  `cam`: the frame's K cameras in shared memory.
+// project_route_kernel is bound by instruction issue: with a test per camera in scalar arithmetic and
+// divides for the six cell indices a warp of the six-camera workload took 860 instructions, now 680 (32 frames of
+// 262,144 points: 221 -> 178 us).
+__device__ __forceinline__ Projected project_point(const Camera* cam, int K, float x, float y, float z,
                                                     int W, int H, float min_depth) {
     Projected r;
-    r.mask = 0u; r.best = -1; r.u = -1.0f; r.v = -1.0f; r.d = 0.0f;
-    float d0 = 0.0f, b0 = 0.0f, b1 = 0.0f;
     const float fw = (float)W, fh = (float)H;
-    for (int k = 0; k < K; ++k) {
-        const float4 p0 = P[3 * k], p1 = P[3 * k + 1], p2 = P[3 * k + 2];
-        const float t2 = __fmaf_rn(p2.x, x, __fmaf_rn(p2.y, y, __fmaf_rn(p2.z, z, p2.w)));
-        const float t0 = __fmaf_rn(p0.x, x, __fmaf_rn(p0.y, y, __fmaf_rn(p0.z, z, p0.w)));
-        const float t1 = __fmaf_rn(p1.x, x, __fmaf_rn(p1.y, y, __fmaf_rn(p1.z, z, p1.w)));
-        if (k == 0) d0 = t2;
-        const bool front = t2 > min_depth;        // false for NaN
-        // 0.001 < u < W - 0.01 and the like, multiplied through by the (positive) depth.
-        const float lo = t2 * 1e-3f, hx = t2 * (fw - 1e-2f), hy = t2 * (fh - 1e-2f);
-        const float ox = t2 * (fw + 1e-2f), oy = t2 * (fh + 1e-2f);
-        const bool in_sure = (t0 > lo) && (t0 < hx) && (t1 > lo) && (t1 < hy);
-        const bool out_sure = (t0 < -lo) || (t0 > ox) || (t1 < -lo) || (t1 > oy);
-        bool vis = front && in_sure;
-        if (front && !in_sure && !out_sure) {     // within a hair of an edge, or not finite: decide exactly
-            const float u = __fdiv_rn(t0, t2), v = __fdiv_rn(t1, t2);
-            vis = (u >= 0.0f) && (u < fw) && (v >= 0.0f) && (v < fh);
-        }
-        if (vis) {
-            r.mask |= 1u << k;
-            if (r.best < 0) { r.best = k; b0 = t0; b1 = t1; r.d = t2; }
+    const float cu = 0.5f * fw, cv = 0.5f * fh;
+    const float eu = 1e-2f + 1e-6f * fw, ev = 1e-2f + 1e-6f * fh;
+    const uint64_t centre = pack2(-cu, -cv), inside = pack2(cu - eu, cv - ev), outside = pack2(cu + eu, cv + ev);
+    unsigned mask = 0u, open = 0u, bit = 1u;
+#pragma unroll 2
+    for (int k = 0; k < K; ++k, bit += bit) {
+        uint64_t t01;
+        float t2, au, av, iu, iv, ou, ov;
+        chains(cam[k], x, y, z, t01, t2);
+        const uint64_t dd = pack2(t2, t2);
+        unpack2(fma2(centre, dd, t01), au, av);
+        unpack2(mul2(inside, dd), iu, iv);
+        unpack2(mul2(outside, dd), ou, ov);
+        if (t2 > min_depth) {                     // false for NaN
+            const bool in_sure = (fabsf(au) < iu) & (fabsf(av) < iv);
+            const bool out_sure = (fabsf(au) > ou) | (fabsf(av) > ov);
+            if (in_sure) mask |= bit;
+            else if (!out_sure) open |= bit;
         }
     }
-    if (r.best >= 0) {
-        r.u = __fdiv_rn(b0, r.d);
-        r.v = __fdiv_rn(b1, r.d);
+    for (; open; open &= open - 1u) {             // within a hair of an edge, or not finite: decide exactly
+        const int k = __ffs(open) - 1;
+        uint64_t t01;
+        float t0, t1, t2;
+        chains(cam[k], x, y, z, t01, t2);
+        unpack2(t01, t0, t1);
+        const float u = __fdiv_rn(t0, t2), v = __fdiv_rn(t1, t2);
+        if ((u >= 0.0f) && (u < fw) && (v >= 0.0f) && (v < fh)) mask |= 1u << k;
+    }
+    r.mask = mask;
+    r.best = __ffs(mask) - 1;
+    uint64_t t01;
+    chains(cam[max(r.best, 0)], x, y, z, t01, r.d);
+    if (mask) {
+        float t0, t1;
+        unpack2(t01, t0, t1);
+        r.u = __fdiv_rn(t0, r.d);
+        r.v = __fdiv_rn(t1, r.d);
     } else {
-        r.d = isfinite(d0) ? d0 : 0.0f;
+        r.u = -1.0f; r.v = -1.0f;
+        if (!isfinite(r.d)) r.d = 0.0f;           // depth in camera 0
     }
     return r;
 }
 
-// Copies the K 3x4 matrices of frame b into shared memory (K * 3 float4 rows).
-__device__ __forceinline__ void load_proj(const float* __restrict__ proj, int b, int K, float4* sP) {
-    const float4* src = reinterpret_cast<const float4*>(proj) + (size_t)b * K * 3;
-    for (int i = threadIdx.x; i < K * 3; i += blockDim.x) sP[i] = __ldg(src + i);
+// Copies the K 3x4 matrices of frame b into shared memory.
+__device__ __forceinline__ void load_cameras(const float* __restrict__ proj, int b, int K, Camera* cam) {
+    const float* src = proj + (size_t)b * K * 12;
+    for (int i = threadIdx.x; i < K * 12; i += blockDim.x) {
+        const int k = i / 12, r = (i % 12) / 4, c = i % 4;
+        reinterpret_cast<float*>(cam + k)[r < 2 ? 2 * c + r : 8 + c] = __ldg(src + i);
+    }
 }
 
 // CF4 > 0: Cf/4 known at compile time, blockDim.x == 16 * CF4.  CF4 == 0: any Cf, 256 threads.
@@ -88,33 +140,33 @@ __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads) project_gather_
     __shared__ __align__(16) float sp[kTile * C];
     __shared__ float suvd[kTile * 3];
     __shared__ uint4 srow[kTile];          // {tap (y0,x0) as a float4 index, clamp flags, wx, wy}
-    __shared__ float4 sP[2][EMC2_MAX_CAMERAS * 3];   // matrices of the (at most two, if N >= 256) frames of the tile
+    __shared__ Camera sP[2][EMC2_MAX_CAMERAS];       // cameras of (at most two, if N >= 256) frames of the tile
 
     const long long g0 = (long long)blockIdx.x * kTile;
     const int npts = (int)min((long long)kTile, a.total - g0);
     load_tile_f32(a.pts + g0 * C, npts * C, sp);
     const int bfirst = (int)(g0 / a.N);
     const int nframes = (int)((g0 + npts - 1) / a.N) - bfirst + 1;
-    if (nframes <= 2) {
-        load_proj(a.proj, bfirst, a.K, sP[0]);
-        if (nframes == 2) load_proj(a.proj, bfirst + 1, a.K, sP[1]);
-    }
-    __syncthreads();
-
     const int t = threadIdx.x;
     const int cf4 = CF4 > 0 ? CF4 : a.cf4;
-    if (t < npts) {
+    // Tiny frames (N < 256) can put more than two frames in a tile: two at a time then.
+    for (int f = 0; f < nframes; f += 2) {
+    if (f) __syncthreads();
+    load_cameras(a.proj, bfirst + f, a.K, sP[0]);
+    if (f + 1 < nframes) load_cameras(a.proj, bfirst + f + 1, a.K, sP[1]);
+    __syncthreads();
+    const int frame = t < npts ? (int)((g0 + t) / a.N) - bfirst - f : -1;
+    if (frame == 0 || frame == 1) {
         const float x = sp[t * C], y = sp[t * C + 1], z = sp[t * C + 2];
         const long long gi = g0 + t;
-        const int b = (int)(gi / a.N);
-        // Tiny frames (N < 256) can put more than two frames in a tile: read those from global memory.
-        const float4* P = nframes <= 2 ? sP[b - bfirst] : reinterpret_cast<const float4*>(a.proj) + (size_t)b * a.K * 3;
-        const Projected pr = project_point(P, a.K, x, y, z, a.W, a.H, a.min_depth);
+        const int b = bfirst + f + frame;
+        const Projected pr = project_point(sP[frame], a.K, x, y, z, a.W, a.H, a.min_depth);
         suvd[t * 3] = pr.u; suvd[t * 3 + 1] = pr.v; suvd[t * 3 + 2] = pr.d;
         a.vis[gi] = (uint8_t)pr.mask;
         a.cam[gi] = (int8_t)pr.best;
         const uint4 rec = tap_record(b, pr.best, pr.u, pr.v, a.K, a.Hf, a.Wf, cf4, a.inv_stride, a.offset);
         srow[t] = rec;
+    }
     }
     __syncthreads();
 
@@ -173,11 +225,11 @@ struct PrArgs {
 // points once less; the reductions are fire-and-forget and land while the projection computes.
 template <int C, bool kMark>
 __global__ void __launch_bounds__(kThreads) project_route_kernel(const __grid_constant__ PrArgs a) {
-    __shared__ float suvd[kTile * 3];
+    __shared__ __align__(16) float suvd[kTile * 3];
     __shared__ int hist[EMC2_MAX_EXPERTS];
-    __shared__ float4 sP[EMC2_MAX_CAMERAS * 3];
+    __shared__ Camera sP[EMC2_MAX_CAMERAS];
     const int b = blockIdx.y, tile = blockIdx.x, t = threadIdx.x, lane = t & 31;
-    load_proj(a.proj, b, a.K, sP);
+    load_cameras(a.proj, b, a.K, sP);
     const int i0 = tile * kTile;
     const int npts = min(kTile, a.N - i0);
     const size_t g0 = (size_t)b * a.N + i0;
@@ -205,7 +257,12 @@ __global__ void __launch_bounds__(kThreads) project_route_kernel(const __grid_co
         a.expert[g0 + t] = (uint8_t)e;
     }
     __syncthreads();
-    for (int i = t; i < npts * 3; i += kThreads) a.uvd[g0 * 3 + i] = suvd[i];
+    float* uvd = a.uvd + g0 * 3;
+    if (npts == kTile && (reinterpret_cast<uintptr_t>(uvd) & 15) == 0) {   // whole 16-byte groups, if they are aligned
+        if (t < kTile * 3 / 4) reinterpret_cast<float4*>(uvd)[t] = reinterpret_cast<const float4*>(suvd)[t];
+    } else {
+        for (int i = t; i < npts * 3; i += kThreads) uvd[i] = suvd[i];
+    }
     for (int k = 0; k < a.rp.E; ++k) {
         const unsigned m = __ballot_sync(0xFFFFFFFFu, e == k);
         if (lane == 0 && m) atomicAdd(&hist[k], __popc(m));

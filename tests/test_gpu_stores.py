@@ -1,4 +1,4 @@
-"""Edges of the voxel cell stores and of the cell rule (needs a B200)."""
+"""Edges of the voxel cell stores, of the cell rule and of the visibility test (needs a B200)."""
 from dataclasses import replace
 
 import numpy as np
@@ -108,4 +108,36 @@ def test_cells_of_points_on_cell_boundaries(oracle, dims):
             assert int(vox["num_voxels"][s]) == ref["num_voxels"]
             assert np.array_equal(np_(vox["coords"][s])[:ref["num_voxels"]], ref["coords"])
             assert np.array_equal(np_(vox["point_voxel"][s]), ref["point_voxel"])
+        br.close()
+
+
+@pytest.mark.parametrize("B,N", [(1, 1), (7, 33), (3, 255), (2, 1031)])
+def test_points_on_image_edges(oracle, B, N):
+    """Pixels within a few ulps to a few hundredths of the image edges, at every depth: mask, camera and pixel as defined."""
+    rng = np.random.default_rng(7)
+    for base in (gen.KITTI, gen.NUSCENES):
+        w = base.with_shape(B, N)
+        P = np.broadcast_to(gen.make_projection(w), (B, w.K, 3, 4)).astype(np.float32).copy()
+        pts = np.zeros((B, N, w.C), np.float32)
+        for b in range(B):
+            for i in range(N):
+                k = rng.integers(w.K)
+                d = 0.1 * 800 ** rng.random()
+                near = rng.choice([0.0, 1e-7, 1e-5, 1e-4, 1e-3, 9e-3, 1.1e-2, 2e-2]) * rng.choice([-1, 1])
+                u = rng.choice([0.0, w.img_w]) + near if rng.random() < 0.6 else rng.random() * w.img_w
+                v = rng.choice([0.0, w.img_h]) + near if rng.random() < 0.6 else rng.random() * w.img_h
+                M = P[b, k].astype(np.float64)
+                pts[b, i, :3] = np.linalg.solve(M[:, :3], np.array([u * d, v * d, d]) - M[:, 3])
+        pts[0, 0, :3] = rng.choice([np.nan, np.inf, 1e30])
+        uvd, mask, cam = oracle.project(pts, P, w.img_h, w.img_w, w.min_depth)
+        feat = rng.standard_normal((B, w.K, w.feat_h, w.feat_w, w.feat_c)).astype(np.float32)
+        want = oracle.gather(uvd, cam, feat, w.feat_stride)
+        br = bridge_for(w)
+        d = [torch.from_numpy(a).cuda() for a in (pts, P, feat)]
+        for got in (br.project_gather(*d), br.run(*d)["pg"]):
+            br.status()
+            assert np.array_equal(np_(got["vis_mask"]), mask)
+            assert np.array_equal(np_(got["cam"]), cam)
+            assert close(np_(got["uvd"]), uvd)[0]
+            assert close(np_(got["gathered"]), want)[0]
         br.close()
