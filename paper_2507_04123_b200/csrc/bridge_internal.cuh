@@ -12,6 +12,12 @@ namespace emc2 {
 
 constexpr int kTile = 256;           // points per CTA tile in the per-point kernels
 constexpr int kThreads = 256;
+
+// Threads of the kernels that move feature rows when Cf/4 = cf4 is not one of the compiled widths: as many whole
+// rows of cf4 columns as 512 threads hold (at least 256: one per point of a tile), so that every thread keeps its
+// column and no index is divided inside the loop.  Rows wider than that take the divide.
+constexpr int kMaxRowThreads = 512;
+inline int row_threads(int cf4) { return cf4 <= kTile ? kMaxRowThreads / cf4 * cf4 : kThreads; }
 // The cell stores.  Large grids: 16-byte units of 96 cell bits and the rank of the unit's first voxel, so that
 // one 128-bit load answers a look-up and the scan streams 1.33 bits per cell (a {32 bits, rank} pair per 32
 // cells streams 2: 75 instead of 50 MB for four frames of the nuScenes-shaped grid, and the scan is paid by
@@ -379,6 +385,112 @@ __device__ __forceinline__ void reset_scan(const ScanReset& r, size_t thread, si
 }
 
 __device__ __forceinline__ int warp_sum(int v) { return __reduce_add_sync(0xFFFFFFFFu, v); }
+
+// ---- stable order of a 256-point tile by expert (used by every kernel that dispatches rows)
+template <int C>
+struct TileOrder {
+    int dest[kTile];                                  // row of every point in the frame's output
+    int wcnt[kTile / 32][EMC2_MAX_EXPERTS];           // points of expert k in warp w
+    int base[EMC2_MAX_EXPERTS];                       // first row of the tile's points of expert k
+    float pts[C == 4 ? 1 : kTile * C];                // five floats per point: the point rows in expert order ...
+    int to[C == 4 ? 1 : kTile];                       // ... and the rows they go to
+};
+
+template <int C>
+struct TilePoint {
+    int e;                                            // expert, -1 past the tile
+    float f[C];
+};
+
+// What a thread needs of point i0 + t, requested before anything waits.  `tile_base`: the tile's E bases.
+template <int C>
+__device__ __forceinline__ TilePoint<C> load_tile_point(TileOrder<C>& s, const float* __restrict__ pts, const uint8_t* expert,
+                                                        const int* tile_base, size_t g0, int npts, int E) {
+    const int t = threadIdx.x, k = t - ((int)blockDim.x - EMC2_MAX_EXPERTS);
+    if (k >= 0) s.base[k] = k < E ? tile_base[k] : 0;
+    TilePoint<C> p;
+    p.e = -1;
+    if (t < npts) {
+        p.e = (int)expert[g0 + t];
+        const float* q = pts + (g0 + t) * C;
+        if (C == 4) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(q));
+            p.f[0] = v.x; p.f[1] = v.y; p.f[2] = v.z; p.f[3] = v.w;
+        } else {
+#pragma unroll
+            for (int c = 0; c < C; ++c) p.f[c] = __ldg(q + c);
+        }
+    }
+    return p;
+}
+
+// Fills s.dest, writes the permutation and moves the point rows; f0: first row of the frame, i0: first point of
+// the tile.  At least kTile threads, all of which call it; s.dest is ready on return.
+// Scattered a float at a time the rows of five floats cost 16 us of the 188 that gather_scatter_kernel took on four
+// nuScenes-shaped frames.  They are put into expert order in shared memory instead, where the rows of one expert
+// are one contiguous run of the output, and leave as whole sectors; a row of four floats is one 16-byte store.
+template <int C>
+__device__ __forceinline__ void order_tile(TileOrder<C>& s, const TilePoint<C>& p, int32_t* perm, float* pts_out, size_t f0,
+                                           int i0, int npts, int E) {
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    int rank = 0;
+    if (t < kTile) {
+        for (int k = 0; k < E; ++k) {
+            const unsigned m = __ballot_sync(0xFFFFFFFFu, p.e == k);
+            if (p.e == k) rank = __popc(m & ((1u << lane) - 1u));
+            if (lane == 0) s.wcnt[warp][k] = __popc(m);
+        }
+    }
+    __syncthreads();
+    if (t < kTile) {
+        // Lane k: the tile's points of expert k in earlier warps, and (five floats) those of smaller experts.
+        int before = 0, all = 0, start = 0;
+        if (lane < E) {
+#pragma unroll
+            for (int w = 0; w < kTile / 32; ++w) {
+                const int n = s.wcnt[w][lane];
+                if (w < warp) before += n;
+                all += n;
+            }
+        }
+        if (C != 4) {
+            int inc = all;
+#pragma unroll
+            for (int d = 1; d < EMC2_MAX_EXPERTS; d <<= 1) {
+                const int y = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+                if (lane >= d) inc += y;
+            }
+            start = __shfl_sync(0xFFFFFFFFu, inc - all, max(p.e, 0));
+        }
+        rank += __shfl_sync(0xFFFFFFFFu, before, max(p.e, 0));
+        if (t < npts) {
+            const int d = s.base[p.e] + rank;
+            s.dest[t] = d;
+            perm[f0 + d] = i0 + t;
+            if (C == 4) {
+                float* dst = pts_out + (f0 + d) * C;      // the caller's buffer may have any alignment
+                if ((reinterpret_cast<uintptr_t>(pts_out) & 15) == 0) {
+                    *reinterpret_cast<float4*>(dst) = make_float4(p.f[0], p.f[1], p.f[2], p.f[3]);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < C; ++c) dst[c] = p.f[c];
+                }
+            } else {
+#pragma unroll
+                for (int c = 0; c < C; ++c) s.pts[(start + rank) * C + c] = p.f[c];
+                s.to[start + rank] = d;
+            }
+        }
+    }
+    __syncthreads();
+    if (C != 4) {
+        float* dst = pts_out + f0 * C;
+        for (int i = t; i < npts * C; i += blockDim.x) {
+            const int r = i / C, c = i - r * C;
+            dst[(size_t)s.to[r] * C + c] = s.pts[i];
+        }
+    }
+}
 
 // ---- bilinear sampling of the channels-last feature maps (used by every kernel that blends rows)
 constexpr uint32_t kZeroRow = 0xFFFFFFFFu;

@@ -134,9 +134,9 @@ __device__ __forceinline__ void load_cameras(const float* __restrict__ proj, int
     }
 }
 
-// CF4 > 0: Cf/4 known at compile time, blockDim.x == 16 * CF4.  CF4 == 0: any Cf, 256 threads.
+// CF4 > 0: Cf/4 known at compile time, blockDim.x == 16 * CF4; else blockDim.x == row_threads(cf4).
 template <int C, int CF4>
-__global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads) project_gather_kernel(PgArgs a) {
+__global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kMaxRowThreads) project_gather_kernel(PgArgs a) {
     __shared__ __align__(16) float sp[kTile * C];
     __shared__ float suvd[kTile * 3];
     __shared__ uint4 srow[kTile];          // {tap (y0,x0) as a float4 index, clamp flags, wx, wy}
@@ -175,14 +175,11 @@ __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads) project_gather_
 
     float4* out = a.out + (size_t)g0 * cf4;
     const uint32_t dyv = (uint32_t)a.Wf * cf4;
-    if constexpr (CF4 > 0) {
-        const int c = t % CF4, r0 = t / CF4;
+    if (CF4 > 0 || cf4 <= (int)blockDim.x) {
+        const int c = t % cf4, rows = CF4 > 0 ? 16 : (int)blockDim.x / cf4;
 #pragma unroll 4
-        for (int j = 0; j < kTile / 16; ++j) {
-            const int r = r0 + 16 * j;
-            if (r >= npts) break;
-            __stcs(out + r * CF4 + c, gather_column(a.feat, srow[r], c, (uint32_t)CF4, dyv));
-        }
+        for (int r = t / cf4; r < npts; r += rows)
+            __stcs(out + r * cf4 + c, gather_column(a.feat, srow[r], c, (uint32_t)cf4, dyv));
     } else {
         const int items = npts * cf4;
         for (int i = t; i < items; i += blockDim.x) {
@@ -294,72 +291,53 @@ struct GsArgs {
     float inv_stride, offset;
 };
 
-// CF4 > 0: Cf/4 known at compile time, blockDim.x == 16 * CF4.  CF4 == 0: any Cf, 256 threads.
+// CF4 > 0: Cf/4 known at compile time, blockDim.x == kGsRows<CF4> * CF4; else blockDim.x == row_threads(cf4).
+// Bound by the memory system's writes: two rows of 4 Cf bytes per point, 384 MB each on four nuScenes-shaped
+// frames.  A plain kernel writes those bytes in 113 us, this one in 177 with its taps (188 before the point rows
+// left in expert order; 158 of those without the taps).  Neither more rows in flight per thread, nor fewer
+// resident warps, nor other cache policies of the stores move it; a persistent grid writes 10 % slower than
+// tiles in launch order.
+// Rows at a time: 512 threads where registers allow four such CTAs, so that a tile is through sooner: 64 channels
+// 112 -> 109 us on the KITTI-shaped batch and 15 -> 11 us on one small frame, 128 channels 90 -> 83 us; 80
+// channels take 16 rows (320 threads) because 24 or 32 leave fewer warps resident (177 -> 181 and 191 us).
+template <int CF4> constexpr int kGsRows = CF4 == 16 ? 32 : 16;
+
 template <int C, int CF4>
-__global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads) gather_scatter_kernel(const __grid_constant__ GsArgs a) {
+__global__ void __launch_bounds__(CF4 > 0 ? kGsRows<CF4> * CF4 : kMaxRowThreads) gather_scatter_kernel(const __grid_constant__ GsArgs a) {
+    constexpr int kRows = kGsRows<CF4>;
     __shared__ uint4 srow[kTile];
-    __shared__ int sdest[kTile];
-    __shared__ int wcnt[kTile / 32][EMC2_MAX_EXPERTS];
-    const int b = blockIdx.y, tile = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    __shared__ TileOrder<C> order;
+    const int b = blockIdx.y, tile = blockIdx.x, t = threadIdx.x;
     const int i0 = tile * kTile;
     const int npts = min(kTile, a.N - i0);
     const size_t f0 = (size_t)b * a.N;        // first row of the frame
     const size_t g0 = f0 + i0;
     const int cf4 = CF4 > 0 ? CF4 : a.cf4;
-    // The tile's bases are requested first, together with the points' records: nothing below waits for
-    // a second round trip to memory before the rows start to move.
-    __shared__ int tbase[EMC2_MAX_EXPERTS];
-    if (t >= (int)blockDim.x - EMC2_MAX_EXPERTS) {
-        const int k = t - ((int)blockDim.x - EMC2_MAX_EXPERTS);
-        if (k < a.E) tbase[k] = a.tile_base[((size_t)b * a.tiles + tile) * a.E + k];
-    }
-
-    // Stable rank inside the tile by ballots per expert, and the tap record of every point.
-    int e = -1, rank = 0;
-    if (t < kTile) {
-        if (t < npts) {
-            e = (int)a.expert[g0 + t];
-            const float u = a.uvd[(g0 + t) * 3], v = a.uvd[(g0 + t) * 3 + 1];
-            srow[t] = tap_record(b, (int)a.cam[g0 + t], u, v, a.K, a.Hf, a.Wf, cf4, a.inv_stride, a.offset);
-        }
-        for (int k = 0; k < a.E; ++k) {
-            const unsigned m = __ballot_sync(0xFFFFFFFFu, e == k);
-            if (e == k) rank = __popc(m & ((1u << lane) - 1u));
-            if (lane == 0) wcnt[warp][k] = __popc(m);
-        }
-    }
-    __syncthreads();
+    // Everything the tile needs is requested first: nothing below waits for a second round trip to memory
+    // before the rows start to move.
+    float u = 0.f, v = 0.f;
+    int cam = -1;
     if (t < npts) {
-        int before = 0;
-        for (int w = 0; w < warp; ++w) before += wcnt[w][e];
-        const int d = tbase[e] + before + rank;
-        sdest[t] = d;
-        a.perm[f0 + d] = i0 + t;
+        u = a.uvd[(g0 + t) * 3];
+        v = a.uvd[(g0 + t) * 3 + 1];
+        cam = (int)a.cam[g0 + t];
     }
-    __syncthreads();
-
-    // Point rows: the tile's source floats are contiguous.
-    const float* psrc = a.pts + g0 * C;
-    float* pdst = a.pts_out + f0 * C;
-    for (int i = t; i < npts * C; i += blockDim.x) {
-        const int r = i / C, c = i - r * C;
-        pdst[(size_t)sdest[r] * C + c] = __ldg(psrc + i);
-    }
-    // Feature rows: 16 rows x Cf/4 columns of threads; blended once, stored at both places (the
-    // rows in point order only if the caller wants them).
+    const TilePoint<C> p = load_tile_point<C>(order, a.pts, a.expert, a.tile_base + ((size_t)b * a.tiles + tile) * a.E, g0, npts, a.E);
+    if (t < npts) srow[t] = tap_record(b, cam, u, v, a.K, a.Hf, a.Wf, cf4, a.inv_stride, a.offset);
+    order_tile<C>(order, p, a.perm, a.pts_out, f0, i0, npts, a.E);
+    // Feature rows: blockDim.x / (Cf/4) rows x Cf/4 columns of threads; blended once, stored at both places
+    // (the rows in point order only if the caller wants them).
     const bool keep = a.gathered != nullptr;
     float4* out = a.gathered + g0 * cf4;
     float4* fdst = a.feat_out + f0 * cf4;
     const uint32_t dyv = (uint32_t)a.Wf * cf4;
-    if constexpr (CF4 > 0) {
-        const int c = t % CF4, r0 = t / CF4;
+    if (CF4 > 0 || cf4 <= (int)blockDim.x) {
+        const int c = t % cf4, rows = CF4 > 0 ? kRows : (int)blockDim.x / cf4;
 #pragma unroll 4
-        for (int j = 0; j < kTile / 16; ++j) {
-            const int r = r0 + 16 * j;
-            if (r >= npts) break;
-            const float4 o = gather_column(a.feat, srow[r], c, (uint32_t)CF4, dyv);
-            if (keep) __stcs(out + r * CF4 + c, o);
-            __stcs(fdst + (size_t)sdest[r] * CF4 + c, o);
+        for (int r = t / cf4; r < npts; r += rows) {
+            const float4 o = gather_column(a.feat, srow[r], c, (uint32_t)cf4, dyv);
+            if (keep) __stcs(out + r * cf4 + c, o);
+            __stcs(fdst + (size_t)order.dest[r] * cf4 + c, o);
         }
     } else {
         const int items = npts * cf4;
@@ -367,7 +345,7 @@ __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads) gather_scatter_
             const int r = i / cf4, c = i - r * cf4;
             const float4 o = gather_column(a.feat, srow[r], c, (uint32_t)cf4, dyv);
             if (keep) __stcs(out + i, o);
-            __stcs(fdst + (size_t)sdest[r] * cf4 + c, o);
+            __stcs(fdst + (size_t)order.dest[r] * cf4 + c, o);
         }
     }
 }
@@ -611,9 +589,9 @@ void launch_gs(emc2_bridge* h, const GsArgs& a, dim3 grid, cudaStream_t st) {
         if (a.cf4 == 20) { gather_scatter_bulk_kernel<C, 20, false><<<grid, 16 * 20, 0, st>>>(a); return; }
     }
     switch (a.cf4) {
-        case 16: gather_scatter_kernel<C, 16><<<grid, 16 * 16, 0, st>>>(a); break;
-        case 20: gather_scatter_kernel<C, 20><<<grid, 16 * 20, 0, st>>>(a); break;
-        default: gather_scatter_kernel<C, 0><<<grid, kThreads, 0, st>>>(a); break;
+        case 16: gather_scatter_kernel<C, 16><<<grid, kGsRows<16> * 16, 0, st>>>(a); break;
+        case 20: gather_scatter_kernel<C, 20><<<grid, kGsRows<20> * 20, 0, st>>>(a); break;
+        default: gather_scatter_kernel<C, 0><<<grid, row_threads(a.cf4), 0, st>>>(a); break;
     }
 }
 
@@ -686,7 +664,7 @@ void launch_c(emc2_bridge* h, const PgArgs& a, int tiles, cudaStream_t st) {
     switch (a.cf4) {
         case 16: project_gather_kernel<C, 16><<<tiles, 16 * 16, 0, st>>>(a); break;
         case 20: project_gather_kernel<C, 20><<<tiles, 16 * 20, 0, st>>>(a); break;
-        default: project_gather_kernel<C, 0><<<tiles, kThreads, 0, st>>>(a); break;
+        default: project_gather_kernel<C, 0><<<tiles, row_threads(a.cf4), 0, st>>>(a); break;
     }
 }
 

@@ -163,83 +163,59 @@ struct ScatterArgs {
     int N, tiles, E, cf4;
 };
 
-// CF4 > 0: Cf/4 known at compile time, blockDim.x == 16 * CF4.  CF4 == 0: any Cf, 256 threads.
+// CF4 > 0: Cf/4 known at compile time, blockDim.x == 16 * CF4; else blockDim.x == row_threads(cf4).
 template <int C, int CF4>
-__global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads) dispatch_scatter_kernel(ScatterArgs a) {
-    __shared__ int sdest[kTile];
-    __shared__ int wcnt[kTile / 32][EMC2_MAX_EXPERTS];
-    const int b = blockIdx.y, tile = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+__global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kMaxRowThreads) dispatch_scatter_kernel(ScatterArgs a) {
+    __shared__ TileOrder<C> order;
+    const int b = blockIdx.y, tile = blockIdx.x, t = threadIdx.x;
     const int i0 = tile * kTile;
     const int npts = min(kTile, a.N - i0);
     const size_t f0 = (size_t)b * a.N;        // first row of the frame
     const size_t g0 = f0 + i0;
     const int cf4 = CF4 > 0 ? CF4 : a.cf4;
-
-    // Stable rank inside the tile: ballots per expert (warps past the tile only take part in
-    // the barriers).
-    int e = -1, rank = 0;
-    if (t < kTile) {
-        e = t < npts ? (int)a.expert[g0 + t] : -1;
-        for (int k = 0; k < a.E; ++k) {
-            const unsigned m = __ballot_sync(0xFFFFFFFFu, e == k);
-            if (e == k) rank = __popc(m & ((1u << lane) - 1u));
-            if (lane == 0) wcnt[warp][k] = __popc(m);
-        }
-    }
-    __syncthreads();
-    if (t < npts) {
-        int before = 0;
-        for (int w = 0; w < warp; ++w) before += wcnt[w][e];
-        const int d = a.tile_base[((size_t)b * a.tiles + tile) * a.E + e] + before + rank;
-        sdest[t] = d;
-        a.perm[f0 + d] = i0 + t;
-    }
-    __syncthreads();
-
-    // Point rows: the tile's source floats are contiguous.
-    const float* psrc = a.pts + g0 * C;
-    float* pdst = a.pts_out + f0 * C;
-    for (int i = t; i < npts * C; i += blockDim.x) {
-        const int r = i / C, c = i - r * C;
-        pdst[(size_t)sdest[r] * C + c] = __ldg(psrc + i);
-    }
-    // Feature rows: 16 rows x Cf/4 columns of threads; each thread keeps its column, reads
+    const TilePoint<C> p = load_tile_point<C>(order, a.pts, a.expert, a.tile_base + ((size_t)b * a.tiles + tile) * a.E, g0, npts, a.E);
+    order_tile<C>(order, p, a.perm, a.pts_out, f0, i0, npts, a.E);
+    // Feature rows: blockDim.x / (Cf/4) rows x Cf/4 columns of threads; each thread keeps its column, reads
     // eight rows (eight independent 128-bit streaming loads), then writes them to their slots.
     const float4* fsrc = a.feat + g0 * cf4;
     float4* fdst = a.feat_out + f0 * cf4;
-    if constexpr (CF4 > 0) {
-        const int c = t % CF4, r0 = t / CF4;
-#pragma unroll
-        for (int j0 = 0; j0 < kTile / 16; j0 += 8) {
+    if (CF4 > 0 || cf4 <= (int)blockDim.x) {
+        const int c = t % cf4, rows = CF4 > 0 ? 16 : (int)blockDim.x / cf4;
+        for (int r0 = t / cf4; r0 < npts; r0 += 8 * rows) {
             float4 v[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                const int r = r0 + 16 * (j0 + u);
-                if (r < npts) v[u] = __ldcs(fsrc + r * CF4 + c);
+                const int r = r0 + u * rows;
+                if (r < npts) v[u] = __ldcs(fsrc + r * cf4 + c);
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                const int r = r0 + 16 * (j0 + u);
-                if (r < npts) __stcs(fdst + (size_t)sdest[r] * CF4 + c, v[u]);
+                const int r = r0 + u * rows;
+                if (r < npts) __stcs(fdst + (size_t)order.dest[r] * cf4 + c, v[u]);
             }
         }
     } else {
         const int items = npts * cf4;
         for (int i = t; i < items; i += blockDim.x) {
             const int r = i / cf4, c = i - r * cf4;
-            __stcs(fdst + (size_t)sdest[r] * cf4 + c, __ldcs(fsrc + i));
+            __stcs(fdst + (size_t)order.dest[r] * cf4 + c, __ldcs(fsrc + i));
         }
+    }
+}
+
+template <int C>
+void launch_scatter_kernel(const ScatterArgs& a, dim3 grid, cudaStream_t st) {
+    switch (a.cf4) {
+        case 16: dispatch_scatter_kernel<C, 16><<<grid, 16 * 16, 0, st>>>(a); break;
+        case 20: dispatch_scatter_kernel<C, 20><<<grid, 16 * 20, 0, st>>>(a); break;
+        default: dispatch_scatter_kernel<C, 0><<<grid, row_threads(a.cf4), 0, st>>>(a); break;
     }
 }
 
 template <int C>
 void launch_scatter(emc2_bridge* h, const ScatterArgs& a, dim3 grid, cudaStream_t st) {
     LaunchScope ls(h, K_DISPATCH_SCATTER, st);
-    switch (a.cf4) {
-        case 16: dispatch_scatter_kernel<C, 16><<<grid, 16 * 16, 0, st>>>(a); break;
-        case 20: dispatch_scatter_kernel<C, 20><<<grid, 16 * 20, 0, st>>>(a); break;
-        default: dispatch_scatter_kernel<C, 0><<<grid, kThreads, 0, st>>>(a); break;
-    }
+    launch_scatter_kernel<C>(a, grid, st);
 }
 
 }  // namespace
@@ -419,16 +395,7 @@ extern "C" int emc2_route_dispatch_static(const emc2_config_t* config, int32_t B
             sa.tile_base = tile_base; sa.perm = d_perm; sa.pts_out = d_points_out;
             sa.feat_out = reinterpret_cast<float4*>(d_feat_out);
             sa.N = N; sa.tiles = tiles; sa.E = E; sa.cf4 = c.feat_c / 4;
-            const int threads = sa.cf4 == 16 ? 256 : sa.cf4 == 20 ? 320 : kThreads;
-            if (c.point_floats == 4) {
-                if (sa.cf4 == 16) dispatch_scatter_kernel<4, 16><<<grid, threads, 0, st>>>(sa);
-                else if (sa.cf4 == 20) dispatch_scatter_kernel<4, 20><<<grid, threads, 0, st>>>(sa);
-                else dispatch_scatter_kernel<4, 0><<<grid, threads, 0, st>>>(sa);
-            } else {
-                if (sa.cf4 == 16) dispatch_scatter_kernel<5, 16><<<grid, threads, 0, st>>>(sa);
-                else if (sa.cf4 == 20) dispatch_scatter_kernel<5, 20><<<grid, threads, 0, st>>>(sa);
-                else dispatch_scatter_kernel<5, 0><<<grid, threads, 0, st>>>(sa);
-            }
+            if (c.point_floats == 4) launch_scatter_kernel<4>(sa, grid, st); else launch_scatter_kernel<5>(sa, grid, st);
         }
         if (cudaGetLastError() != cudaSuccess) rc = EMC2_ERR_CUDA;
     }

@@ -1,4 +1,4 @@
-"""Edges of the voxel cell stores, of the cell rule and of the visibility test (needs a B200)."""
+"""Edges of the voxel cell stores, the cell rule, the visibility test and the row kernels (needs a B200)."""
 from dataclasses import replace
 
 import numpy as np
@@ -140,4 +140,28 @@ def test_points_on_image_edges(oracle, B, N):
             assert np.array_equal(np_(got["cam"]), cam)
             assert close(np_(got["uvd"]), uvd)[0]
             assert close(np_(got["gathered"]), want)[0]
+        br.close()
+
+
+@pytest.mark.parametrize("cf", [4, 32, 64, 68, 80, 128, 256, 1020, 1024, 1028])
+def test_row_widths_of_the_row_kernels(oracle, cf):
+    """Compiled widths, whole rows per CTA, and rows wider than a CTA; ragged tiles, four and five floats per point,
+    dispatched point rows in a buffer of any alignment."""
+    for base, B, N in ((gen.KITTI, 2, 259), (gen.NUSCENES, 1, 517)):
+        w = replace(base.with_shape(B, N), img_h=64, img_w=96, feat_stride=8, feat_c=cf)
+        batch = gen.make_batch(w)
+        ref = oracle.bridge(w, batch)
+        d = {k: torch.from_numpy(v).cuda() for k, v in batch.items()}
+        br = bridge_for(w)
+        odd = torch.zeros(B * N * w.C + 1, device="cuda")[1:].view(B, N, w.C)      # 4 bytes past a 16-byte boundary
+        for step in (br.run, br.run_staged):
+            bufs = step(d["points"], d["proj"], d["feat"])
+            bufs["rd"]["points_out"] = odd.zero_()
+            bufs = step(d["points"], d["proj"], d["feat"], bufs)
+            br.status()
+            rd = bufs["rd"]
+            assert np.array_equal(np_(rd["perm"]), ref["perm"]) and np.array_equal(np_(rd["offsets"]), ref["offsets"])
+            assert np.array_equal(np_(rd["points_out"]).view(np.uint32), ref["points_out"].view(np.uint32))
+            assert close(np_(rd["feat_out"]), ref["feat_out"])[0]
+            assert close(np_(bufs["pg"]["gathered"]), ref["gathered"])[0]
         br.close()
