@@ -187,8 +187,8 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out) {
     const size_t o_vif_part = plan.take(((size_t)h->vif_scan_blocks + 1) * sizeof(int));
     const size_t rb_tiles = (maxpts + kTile - 1) / kTile;
     const size_t o_rb_bits = plan.take(maxpts * sizeof(uint32_t));
-    const size_t o_rb_counts = plan.take(27 * rb_tiles * sizeof(int));
-    const size_t o_rb_base = plan.take((27 * rb_tiles + 27) * sizeof(int));
+    const size_t o_rb_counts = plan.take(13 * rb_tiles * sizeof(int));
+    const size_t o_rb_base = plan.take((13 * rb_tiles + 13) * sizeof(int));
     h->max_tiles = (c.max_points + kTile - 1) / kTile;
     const size_t tile_ints = (size_t)c.max_batch * h->max_tiles * c.num_experts;
     const size_t o_tc = plan.take(tile_ints * sizeof(int));

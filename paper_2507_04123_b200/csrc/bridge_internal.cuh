@@ -191,7 +191,7 @@ struct emc2_bridge {
     int* d_vif_part = nullptr;     // [vif_scan_blocks]
     int vif_scan_blocks = 0;
     uint32_t* d_rb_bits = nullptr;  // emc2_rulebook: [max points] neighbour bits per voxel
-    int* d_rb_counts = nullptr;    // [27][voxel tiles] pairs per (offset, tile), and their prefix sums
+    int* d_rb_counts = nullptr;    // [13][voxel tiles] pairs per (offset, tile), and their prefix sums
     int* d_rb_base = nullptr;
     int max_tiles = 0;
     int tune[EMC2_TUNE_KNOBS] = {0, 1, 0, 0, 0};   // emc2_bridge_set_tuning

@@ -9,10 +9,17 @@
 // grids, the row + 1 per cell for small ones.  Because the list is in cell order, a voxel's row is
 // the unit's first row plus the number of set bits below it.
 //   rb_mark   every voxel sets its cell; the first voxel of a unit stores its row there
-//   rb_count  27 look-ups per voxel -> neighbour bits per voxel, pair counts per (offset, tile)
+//   rb_count  13 neighbours per voxel -> neighbour bits per voxel, pair counts per (offset, tile)
 //   rb_scan   one CTA per offset: exclusive prefix sum of its counts over the tiles, and its total
 //   rb_fill   offsets[28] from the totals; every tile ranks its pairs per offset with warp ballots
 //             and writes them
+// Only the 13 offsets k < 13, whose neighbour comes before the voxel in the list, are looked up.  The
+// neighbour at offset 26 - k is the opposite one, and adding a fixed step of cells keeps the order of the
+// list, so the pairs of offset 26 - k are those of offset k in the same order with in and out exchanged;
+// offset 13 pairs every voxel with itself.  The three x-neighbours of a (dz, dy) have consecutive rows: one
+// look-up gives the first, and the neighbour at dx = -1 in the voxel's own row is the voxel before it.
+// Both passes are bound by instruction issue: with 27 look-ups each they took 28 and 62 us for 894 k voxels
+// with 4.8 M pairs (B200).
 //   rb_clear  the touched units of the store go back to zero
 #include "bridge_internal.cuh"
 
@@ -21,7 +28,7 @@ namespace {
 
 constexpr int kStatusCapacity = 1;
 constexpr int kStatusBadList = 4;
-constexpr int kOffsets = 27;
+constexpr int kOffsets = 27, kHalf = 13;
 constexpr int kRbScanThreads = 1024;
 
 struct RbArgs {
@@ -31,9 +38,9 @@ struct RbArgs {
     int capacity, max_batch;
     int tiles;                   // ceil(capacity / kTile)
     uint32_t* nbr_bits;          // [capacity] bit k: the neighbour at offset k exists
-    int* tile_counts;            // [27][tiles]
-    int* tile_base;              // [27][tiles] exclusive prefix sum of tile_counts along the tiles
-    int* offset_pairs;           // [27] pairs per offset
+    int* tile_counts;            // [13][tiles]
+    int* tile_base;              // [13][tiles] exclusive prefix sum of tile_counts along the tiles
+    int* offset_pairs;           // [13] pairs per offset
     int32_t* offsets;            // [28]
     int32_t* rule_in;
     int32_t* rule_out;
@@ -90,12 +97,6 @@ __global__ void __launch_bounds__(kThreads) rb_clear_kernel(const __grid_constan
     else a.g.store[cell] = 0u;
 }
 
-// Row of the voxel at place `pos` of a unit, -1 if its bit is clear.
-__device__ __forceinline__ int row_in_unit(const uint4& q, uint32_t pos) {
-    const uint32_t word = pos < 32u ? q.x : pos < 64u ? q.y : q.z;
-    return (word >> (pos & 31u)) & 1u ? (int)(q.w + bits_below(q, pos)) : -1;
-}
-
 // Where a voxel sits: its cell, the cell strides and which of its 3 x 3 x 3 neighbours the grid has.
 struct Site {
     uint32_t cell, sy, sz;
@@ -114,28 +115,17 @@ __device__ __forceinline__ Site site_of(const RbArgs& a, const int4 c) {
     return s;
 }
 
-// Rows of the three x-neighbours (dx = -1, 0, 1) at (dz, dy) = (j / 3 - 1, j % 3 - 1) of a valid
-// site, -1 where there is none; only the ones in `want3` (bit dx + 1) are looked up.  The three
-// share a unit of the bitmap unless they straddle its boundary: one load, rarely two.
-__device__ __forceinline__ void neighbours3(const ScaleDev& g, const Site& s, int j, uint32_t want3, int r[3]) {
+// Row of the first of the x-neighbours `three` (bit dx + 1, at least one) at (dz, dy) = (j / 3 - 1, j % 3 - 1).
+__device__ __forceinline__ int first_row(const ScaleDev& g, const Site& s, int j, uint32_t three) {
     const int dz = j / 3 - 1, dy = j % 3 - 1;
-    r[0] = r[1] = r[2] = -1;
-    if (!want3 || !s.okz[dz + 1] || !s.oky[dy + 1]) return;
     const uint32_t mid = s.cell + (uint32_t)dz * s.sz + (uint32_t)dy * s.sy;   // wraps like the signed sum
-    if (g.mode == MODE_BITMAP) {
-        const uint4* units = reinterpret_cast<const uint4*>(g.store);
-        uint32_t pos;
-        const uint32_t u = unit_of(mid, pos);
-        const uint4 q = units[u];
-        if (want3 & 2u) r[1] = row_in_unit(q, pos);
-        if (s.okx[0] && (want3 & 1u)) r[0] = pos > 0 ? row_in_unit(q, pos - 1) : row_in_unit(units[u - 1], kUnitCells - 1);
-        if (s.okx[2] && (want3 & 4u))
-            r[2] = pos < kUnitCells - 1 ? row_in_unit(q, pos + 1) : row_in_unit(units[u + 1], 0);
-    } else {
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-            if (s.okx[i] && ((want3 >> i) & 1u)) r[i] = (int)g.store[mid + i - 1] - 1;
-    }
+    if (g.mode == MODE_TABLE) return (int)g.store[mid + (uint32_t)__ffs(three) - 2u] - 1;
+    const uint4* units = reinterpret_cast<const uint4*>(g.store);
+    // Look-up at the first neighbour's own unit: a unit without voxels has no rank.
+    uint32_t pos;
+    const uint32_t u = unit_of(mid + (uint32_t)__ffs(three) - 2u, pos);
+    const uint4 q = units[u];
+    return (int)(q.w + bits_below(q, pos));
 }
 
 // Which of the three x-neighbours at (dz, dy) exist (bit dx + 1), for a valid site.
@@ -165,27 +155,28 @@ __device__ __forceinline__ uint32_t exist3(const ScaleDev& g, const Site& s, int
 }
 
 __global__ void __launch_bounds__(kThreads) rb_count_kernel(const __grid_constant__ RbArgs a) {
-    __shared__ int wcount[kThreads / 32][kOffsets];
+    __shared__ int wcount[kThreads / 32][kHalf];
     const int M = voxels_in_list(a);
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int m = blockIdx.x * kTile + t;
     uint32_t bits = 0;
     if (m < M) {
-        const int4 c = a.coords[m];
+        const int4 c = a.coords[m], p = a.coords[max(m - 1, 0)];
         const Site s = site_of(a, c);
         if (s.cell != 0xFFFFFFFFu) {
 #pragma unroll
-            for (int j = 0; j < 9; ++j) bits |= exist3(a.g, s, j) << (3 * j);
+            for (int j = 0; j < 4; ++j) bits |= exist3(a.g, s, j) << (3 * j);
+            if (m > 0 && p.x == c.x && p.y == c.y && p.z == c.z && p.w + 1 == c.w) bits |= 1u << 12;
         }
     }
     if (m < a.capacity) a.nbr_bits[m] = bits;
 #pragma unroll
-    for (int k = 0; k < kOffsets; ++k) {
+    for (int k = 0; k < kHalf; ++k) {
         const unsigned b = __ballot_sync(0xFFFFFFFFu, (bits >> k) & 1u);
         if (lane == 0) wcount[warp][k] = __popc(b);
     }
     __syncthreads();
-    if (t < kOffsets) {
+    if (t < kHalf) {
         int sum = 0;
 #pragma unroll
         for (int w = 0; w < kThreads / 32; ++w) sum += wcount[w][t];
@@ -235,23 +226,24 @@ __global__ void __launch_bounds__(kRbScanThreads) rb_scan_kernel(const __grid_co
     if (t == 0) a.offset_pairs[blockIdx.x] = s_carry;
 }
 
-__global__ void __launch_bounds__(kThreads, 6) rb_fill_kernel(const __grid_constant__ RbArgs a) {
-    __shared__ int wcount[kThreads / 32][kOffsets];   // pairs per warp, then where the warp's pairs start
+__global__ void __launch_bounds__(kThreads) rb_fill_kernel(const __grid_constant__ RbArgs a) {
+    __shared__ int wcount[kThreads / 32][kHalf];      // pairs per warp, then where the warp's pairs start
     __shared__ int s_start[kOffsets + 1];             // offsets[]
     const int M = voxels_in_list(a);
     if (blockIdx.x > 0 && blockIdx.x * kTile >= M) return;   // CTA 0 always writes offsets[]
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int m = blockIdx.x * kTile + t;
     // Loads that depend on nothing go first.
-    const int tile_start = t < kOffsets ? a.tile_base[(size_t)t * a.tiles + blockIdx.x] : 0;
-    const int own = t < kOffsets ? a.offset_pairs[t] : 0;
+    const int tile_start = t < kHalf ? a.tile_base[(size_t)t * a.tiles + blockIdx.x] : 0;
+    int own = 0;
+    if (t < kOffsets) own = t == kHalf ? max(M, 0) : a.offset_pairs[min(t, kOffsets - 1 - t)];
     int4 c = make_int4(0, 0, 0, 0);
     uint32_t bits = 0u;
     if (m < M) {
         c = a.coords[m];
         bits = a.nbr_bits[m];
     }
-    if (warp == 0) {                                   // offsets[] from the 27 totals
+    if (warp == 0) {                                   // offsets[] from the totals
         int inc = own;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
@@ -261,13 +253,13 @@ __global__ void __launch_bounds__(kThreads, 6) rb_fill_kernel(const __grid_const
         if (lane <= kOffsets) s_start[lane] = inc - own;
     }
 #pragma unroll
-    for (int k = 0; k < kOffsets; ++k) {
+    for (int k = 0; k < kHalf; ++k) {
         const unsigned b = __ballot_sync(0xFFFFFFFFu, (bits >> k) & 1u);
         if (lane == 0) wcount[warp][k] = __popc(b);
     }
     __syncthreads();
-    if (t < kOffsets) {
-        int run = s_start[t] + tile_start;
+    if (t < kHalf) {                                   // places inside the segment
+        int run = tile_start;
 #pragma unroll
         for (int w = 0; w < kThreads / 32; ++w) {
             const int n = wcount[w][t];
@@ -282,22 +274,30 @@ __global__ void __launch_bounds__(kThreads, 6) rb_fill_kernel(const __grid_const
     __syncthreads();
     const Site s = site_of(a, c);                      // bits == 0 for rows outside the list or the grid
     const unsigned below = (1u << lane) - 1u;
+    int first[4];
 #pragma unroll
-    for (int j = 0; j < 9; ++j) {
-        int r[3];
-        neighbours3(a.g, s, j, (bits >> (3 * j)) & 7u, r);
+    for (int j = 0; j < 4; ++j) {
+        const uint32_t three = (bits >> (3 * j)) & 7u;
+        first[j] = three ? first_row(a.g, s, j, three) : 0;
+    }
+    auto put = [&](int pos, int in, int out) {
+        if ((long long)pos < a.pair_capacity) {
+            a.rule_in[pos] = in;
+            a.rule_out[pos] = out;
+        }
+    };
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const int k = 3 * j + i;
-            const bool has = (bits >> k) & 1u;
-            const unsigned b = __ballot_sync(0xFFFFFFFFu, has);
-            const int pos = wcount[warp][k] + __popc(b & below);
-            if (has && (long long)pos < a.pair_capacity) {
-                a.rule_in[pos] = r[i];
-                a.rule_out[pos] = m;
-            }
+    for (int k = 0; k < kHalf; ++k) {
+        const bool has = (bits >> k) & 1u;
+        const unsigned b = __ballot_sync(0xFFFFFFFFu, has);
+        if (has) {
+            const int at = wcount[warp][k] + __popc(b & below);
+            const int n = k == 12 ? m - 1 : first[k / 3] + __popc((bits >> (k / 3 * 3)) & ((1u << (k % 3)) - 1u));
+            put(s_start[k] + at, n, m);
+            put(s_start[kOffsets - 1 - k] + at, m, n);
         }
     }
+    if (m < M) put(s_start[kHalf] + m, m, m);
 }
 
 }  // namespace
@@ -315,7 +315,7 @@ int launch_rulebook(emc2_bridge* h, int scale, int capacity, const int32_t* d_co
     a.nbr_bits = h->d_rb_bits;
     a.tile_counts = h->d_rb_counts;
     a.tile_base = h->d_rb_base;
-    a.offset_pairs = h->d_rb_base + (size_t)kOffsets * a.tiles;
+    a.offset_pairs = h->d_rb_base + (size_t)kHalf * a.tiles;
     a.offsets = d_rule_offsets; a.rule_in = d_rule_in; a.rule_out = d_rule_out;
     a.pair_capacity = pair_capacity;
     a.status = h->d_status;
@@ -330,7 +330,7 @@ int launch_rulebook(emc2_bridge* h, int scale, int capacity, const int32_t* d_co
     }
     {
         LaunchScope ls(h, K_RB_SCAN, st);
-        rb_scan_kernel<<<kOffsets, kRbScanThreads, 0, st>>>(a);
+        rb_scan_kernel<<<kHalf, kRbScanThreads, 0, st>>>(a);
     }
     {
         LaunchScope ls(h, K_RB_FILL, st);
