@@ -597,48 +597,67 @@ void launch_gs(emc2_bridge* h, const GsArgs& a, dim3 grid, cudaStream_t st) {
 
 // ------------------------------------------------------------------ planar -> channels-last
 // Per map the planar data is a Cf x P matrix (P = Hf * Wf pixels) and the channels-last data its
-// transpose.  A CTA moves a tile of 64 channels x 128 pixels through shared memory:
-//   in   one warp per channel row, 32 consecutive pixels (128 B) per instruction;
-//   out  a warp instruction covers 4 pixels x 32 channels: eight lanes store 128 contiguous bytes
-//        of one pixel's row.  With a row stride of 129 words the column reads from the tile
-//        (bank = channel + pixel mod 32) are conflict-free.
-constexpr int kClChan = 64, kClPix = 128, kClStride = kClPix + 1;
+// transpose.  A CTA moves `chan` channels x 64 pixels through shared memory; with up to 128 channels that is all
+// of them, so what it writes is one contiguous block.
+//   in   one warp per channel row, 32 consecutive pixels (128 B) per instruction; a thread requests ten of its
+//        words before it waits for any;
+//   out  a warp instruction covers 8 pixels x 16 channels, 64 contiguous bytes of a pixel's row per four lanes.
+//        With a row stride of 66 words the column reads from the tile (bank = 2 * channel + pixel mod 32) are
+//        conflict-free.
+// Bound by the memory system (each byte is read and written once).  A tile of 64 channels x 128 pixels, which gives
+// 80 channels a second CTA for 16 of them, took 82 us for 24 maps of 80 x 113 x 200 (174 MB); this takes 63.
+constexpr int kClPix = 64, kClStride = kClPix + 2, kClMaxChan = 128, kClBatch = 10;
 
 __global__ void __launch_bounds__(256)
-channels_last_kernel(const float* __restrict__ planar, float* __restrict__ last, int Cf, int P, int ptiles) {
-    __shared__ float tile[kClChan][kClStride];
+channels_last_kernel(const float* __restrict__ planar, float* __restrict__ last, int Cf, int P, int ptiles, int chan) {
+    extern __shared__ float tile[];                         // [chan][kClStride]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t m = blockIdx.x / ptiles;
     const int p0 = (int)(blockIdx.x - m * ptiles) * kClPix;
-    const int c0 = blockIdx.y * kClChan;
-    const int nc = min(kClChan, Cf - c0);
+    const int c0 = blockIdx.y * chan;
+    const int nc = min(chan, Cf - c0);
     const float* src = planar + (m * Cf + c0) * (size_t)P + p0;
-    for (int c = warp; c < nc; c += 8) {
+    // Item i of a warp: half (i & 1) of channel row warp + 8 * (i >> 1).
+    const bool in[2] = {p0 + lane < P, p0 + 32 + lane < P};
+    const int items = 2 * ((nc - warp + 7) / 8);
+    for (int i0 = 0; i0 < items; i0 += kClBatch) {
+        float v[kClBatch];
 #pragma unroll
-        for (int j = 0; j < kClPix / 32; ++j) {
-            const int q = lane + 32 * j;
-            tile[c][q] = p0 + q < P ? __ldcs(src + (size_t)c * P + q) : 0.f;
+        for (int u = 0; u < kClBatch; ++u) {
+            const int c = warp + 8 * ((i0 + u) >> 1), half = u & 1;
+            v[u] = c < nc && in[half] ? __ldcs(src + (size_t)c * P + 32 * half + lane) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < kClBatch; ++u) {
+            const int c = warp + 8 * ((i0 + u) >> 1);
+            if (c < nc) tile[c * kClStride + 32 * (u & 1) + lane] = v[u];
         }
     }
     __syncthreads();
     float* dst = last + (m * P + p0) * (size_t)Cf + c0;
-    const int halves = (nc + 31) / 32;                      // 32-channel halves of the tile
-    const int c = 4 * (lane & 7), dq = lane >> 3;
-    for (int job = warp; job < halves * (kClPix / 4); job += 8) {
-        const int cc = c + 32 * (job % halves), q = 4 * (job / halves) + dq;
-        if (cc >= nc || p0 + q >= P) continue;              // Cf % 4 == 0: a whole float4 or none
-        const float4 v = make_float4(tile[cc][q], tile[cc + 1][q], tile[cc + 2][q], tile[cc + 3][q]);
-        __stcs(reinterpret_cast<float4*>(dst + (size_t)q * Cf + cc), v);
+    const int q8 = lane >> 2, cq = 4 * (lane & 3);          // pixel of a group of 8, channel of a group of 16
+    const int quads = (nc + 15) / 16;
+    for (int job = warp; job < quads * (kClPix / 8); job += 8) {
+        const int g = job / quads;                          // consecutive jobs share their pixels
+        const int c = cq + 16 * (job - g * quads), q = 8 * g + q8;
+        if (c >= nc || p0 + q >= P) continue;               // Cf % 4 == 0: a whole float4 or none
+        const float* col = tile + c * kClStride + q;
+        __stcs(reinterpret_cast<float4*>(dst + (size_t)q * Cf + c),
+               make_float4(col[0], col[kClStride], col[2 * kClStride], col[3 * kClStride]));
     }
 }
 
 // ------------------------------------------------------------------ Multiscale Pooling (Sec. 3.5)
 // One thread per (pooled texel, float4 column); grid = (columns of a pooled row, pooled rows,
 // maps).  Consecutive threads read consecutive columns of the same input rows, so every load
-// covers whole 256/320-byte rows.  Streams the maps once.
+// covers whole 256/320-byte rows.  Streams the maps once.  PW: window size known at compile time
+// (2 and 4: all texels of a whole window are requested at once; 60 -> 40 us for 24 maps of 113 x 200 x 80 at
+// p = 2), 0 = any.  The sum is rows outer, columns inner for every size.
+template <int PW>
 __global__ void __launch_bounds__(kThreads)
 pool_features_kernel(const float4* __restrict__ feat, float4* __restrict__ pooled, int Hf, int Wf, int Hp, int Wp,
-                     int cf4, int p) {
+                     int cf4, int pw) {
+    const int p = PW > 0 ? PW : pw;
     const int ic = blockIdx.x * kThreads + threadIdx.x;     // I * cf4 + c
     if (ic >= Wp * cf4) return;
     const int I = ic / cf4, c = ic - I * cf4;
@@ -646,12 +665,24 @@ pool_features_kernel(const float4* __restrict__ feat, float4* __restrict__ poole
     const size_t m = blockIdx.z;                            // map index b * K + k
     const int j0 = J * p, j1 = min(Hf, j0 + p), i0 = I * p, i1 = min(Wf, i0 + p);
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int j = j0; j < j1; ++j) {
-        const float4* row = feat + ((m * Hf + j) * Wf + i0) * cf4 + c;
+    auto add = [&](const float4& v) { s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w; };
+    const float4* corner = feat + ((m * Hf + j0) * Wf + i0) * cf4 + c;
+    if (PW > 0 && j1 - j0 == p && i1 - i0 == p) {
+        constexpr int kW = PW > 0 ? PW : 1;
+        float4 v[kW][kW];
+#pragma unroll
+        for (int j = 0; j < kW; ++j)
+#pragma unroll
+            for (int x = 0; x < kW; ++x) v[j][x] = __ldcs(corner + ((size_t)j * Wf + x) * cf4);
+#pragma unroll
+        for (int j = 0; j < kW; ++j)
+#pragma unroll
+            for (int x = 0; x < kW; ++x) add(v[j][x]);
+    } else {
+        for (int j = 0; j < j1 - j0; ++j) {
+            const float4* row = corner + (size_t)j * Wf * cf4;
 #pragma unroll 4
-        for (int x = 0; x < i1 - i0; ++x) {
-            const float4 v = __ldcs(row + (size_t)x * cf4);
-            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+            for (int x = 0; x < i1 - i0; ++x) add(__ldcs(row + (size_t)x * cf4));
         }
     }
     const float inv = 1.0f / (float)((j1 - j0) * (i1 - i0));
@@ -766,11 +797,12 @@ int launch_channels_last(emc2_bridge* h, int B, const float* d_planar, float* d_
     const long long P = (long long)c.feat_h * c.feat_w;
     const long long ptiles = (P + kClPix - 1) / kClPix;
     const long long ctas = (long long)B * c.num_cameras * ptiles;
-    const int ct = (c.feat_c + kClChan - 1) / kClChan;
+    const int ct = (c.feat_c + kClMaxChan - 1) / kClMaxChan;
+    const int chan = ((c.feat_c + ct - 1) / ct + 3) / 4 * 4;
     if (P > 0x7FFFFFFFLL || ctas > 0x7FFFFFFFLL || ct > 65535) return EMC2_ERR_INVALID_ARG;
     LaunchScope ls(h, K_CHANNELS_LAST, st);
-    const dim3 grid((unsigned)ctas, ct);
-    channels_last_kernel<<<grid, 256, 0, st>>>(d_planar, d_feat, c.feat_c, (int)P, (int)ptiles);
+    const dim3 grid((unsigned)ctas, (c.feat_c + chan - 1) / chan);
+    channels_last_kernel<<<grid, 256, (size_t)chan * kClStride * sizeof(float), st>>>(d_planar, d_feat, c.feat_c, (int)P, (int)ptiles, chan);
     return check_cuda(h, cudaGetLastError());
 }
 
@@ -781,9 +813,9 @@ int launch_pool_features(emc2_bridge* h, int B, int p, const float* d_feat, floa
     const dim3 grid((Wp * cf4 + kThreads - 1) / kThreads, Hp, B * c.num_cameras);
     {
         LaunchScope ls(h, K_POOL_FEATURES, st);
-        pool_features_kernel<<<grid, kThreads, 0, st>>>(reinterpret_cast<const float4*>(d_feat),
-                                                        reinterpret_cast<float4*>(d_pooled), c.feat_h, c.feat_w, Hp,
-                                                        Wp, cf4, p);
+        auto kernel = p == 2 ? pool_features_kernel<2> : p == 4 ? pool_features_kernel<4> : pool_features_kernel<0>;
+        kernel<<<grid, kThreads, 0, st>>>(reinterpret_cast<const float4*>(d_feat), reinterpret_cast<float4*>(d_pooled),
+                                          c.feat_h, c.feat_w, Hp, Wp, cf4, p);
     }
     return check_cuda(h, cudaGetLastError());
 }

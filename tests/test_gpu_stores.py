@@ -165,3 +165,20 @@ def test_row_widths_of_the_row_kernels(oracle, cf):
             assert close(np_(rd["feat_out"]), ref["feat_out"])[0]
             assert close(np_(bufs["pg"]["gathered"]), ref["gathered"])[0]
         br.close()
+
+
+@pytest.mark.parametrize("cf", [4, 12, 64, 80, 128, 132, 260])
+@pytest.mark.parametrize("hw", [(1, 3), (8, 8), (9, 63), (13, 65)])
+def test_map_layout_and_pooling_at_tile_edges(oracle, cf, hw):
+    h, wd = hw
+    w = replace(gen.KITTI.with_shape(2, 16), img_h=8 * h, img_w=8 * wd, feat_stride=8, feat_c=cf)
+    rng = np.random.default_rng(cf)
+    planar = rng.standard_normal((2, 1, cf, h, wd)).astype(np.float32)
+    br = bridge_for(w)
+    last = br.features_channels_last(torch.from_numpy(planar).cuda())
+    want = oracle.channels_last(planar)
+    assert np.array_equal(np_(last), want)
+    for p in (1, 2, 3, 4, 8):
+        assert close(np_(br.pool_features(last, p)), oracle.pool(want, p))[0]
+    br.status()
+    br.close()
