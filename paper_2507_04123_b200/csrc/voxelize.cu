@@ -25,7 +25,7 @@
 // Writes and reductions that land in one 32-byte sector are served one after another by the
 // L2 (about 10 ns each on B200), so nothing here funnels many points into a shared flag or
 // counter: the only contended words are the cells themselves.  The cost of a call follows the
-// occupied groups, not the grid volume, except for one streaming read of the store.
+// occupied tiles, not the grid volume, except for one streaming read of the store.
 #include "bridge_internal.cuh"
 
 namespace emc2 {
@@ -294,6 +294,8 @@ __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const
                         if (j < g.max_ovf && off + n[i] <= g.max_list) {
                             g.ovf_vox[j] = (int)m; g.ovf_off[j] = (int)off; g.ovf_cell[j] = cell + i;
                             g.ovf_cursor[(size_t)j * kCursorStride] = 0;
+                        } else {
+                            atomicOr(a.status, kStatusDirtyStore);
                         }
                         off += n[i];
                         n[i] = kOverCap | j++;
@@ -534,7 +536,10 @@ vox_finalize_kernel(const float* __restrict__ pts, long long total, AccumArgs a,
         for (int sc = 0; sc < 2; ++sc) {
             const ScaleDev& g = a.s[sc];
             if (g.cap <= 0) continue;
-            const int novf = min(g.totals[3], (int)g.max_ovf);
+            // More of them, or more points in them, than this call's points allow: a store that was not all zero
+            // (the status says so); the lists then hold nothing that can be used.
+            const bool dirty = g.totals[0] == 0 || (uint32_t)g.totals[2] > g.max_list || (uint32_t)g.totals[3] > g.max_ovf;
+            const int novf = dirty ? 0 : g.totals[3];
             int32_t* pv = a.point_voxel[sc];
             for (int j = warp; j < novf; j += nwarps) {
                 const int m = g.ovf_vox[j];
