@@ -238,6 +238,28 @@ int launch_route_dispatch(emc2_bridge* h, int B, int N, const float* d_points, c
                           const float* d_gathered, uint8_t* d_expert, int32_t* d_offsets, int32_t* d_perm,
                           float* d_points_out, float* d_feat_out, cudaStream_t st);
 
+#ifdef __CUDACC__
+// Launches a kernel that may be set up while its predecessor in the stream still drains (programmatic dependent
+// launch); for kernels that follow another kernel of the same call on the same stream.  Every kernel launched this
+// way calls await_predecessor() before it touches memory and, when its own work is done, release_successor().
+// Released earlier, the successor's CTAs would hold places on the SMs that the kernels of the other stream need.
+// us per call: one small frame 35 -> 30, stage calls with occlusion 155 -> 140, voxels and rulebooks 261 -> 239 (B200).
+template <typename... P, typename... A>
+inline void launch_chained(void (*kernel)(P...), dim3 grid, unsigned threads, size_t shared, cudaStream_t st, const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = shared;
+    cfg.stream = st;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+#endif
+
 inline ScanReset scan_reset(const emc2_bridge* h) {
     ScanReset r;
     r.words = h->scan.group_voxels[0];
@@ -285,6 +307,11 @@ int launch_scan_gather_scatter(emc2_bridge* h, int b0, int B, int N, const float
 
 // ---------------------------------------------------------------- device helpers
 #ifdef __CUDACC__
+
+// See launch_chained.  What the predecessors in the stream wrote is visible after the first call; the second one
+// lets the successor be set up (it waits for the end of this kernel all the same).
+__device__ __forceinline__ void await_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void release_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Loads `nfloats` consecutive floats starting at a 16-byte aligned address into shared
 // memory with 128-bit loads (scalar loads for a ragged tail).

@@ -40,6 +40,7 @@ __device__ __forceinline__ size_t cell_and_depth(const OcclArgs& a, const float4
 
 template <int C, bool TEST>
 __global__ void __launch_bounds__(kThreads) occl_kernel(const __grid_constant__ OcclArgs a) {
+    await_predecessor();
     const long long i = (long long)blockIdx.x * kThreads + threadIdx.x;
     if (i >= a.total) return;
     unsigned m = a.vis[i] & ((1u << a.K) - 1u);            // cameras the handle has
@@ -64,11 +65,13 @@ __global__ void __launch_bounds__(kThreads) occl_kernel(const __grid_constant__ 
         a.occ[i] = (uint8_t)occ;
         a.clear[i] = (uint8_t)(m & ~occ);
     }
+    release_successor();
 }
 
 __global__ void __launch_bounds__(kThreads) occl_fill_kernel(uint32_t* zbuf, size_t n) {
     for (size_t i = (size_t)blockIdx.x * kThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kThreads)
         zbuf[i] = 0x7F800000u;                      // +infinity
+    release_successor();
 }
 
 }  // namespace
@@ -92,13 +95,13 @@ int launch_occlusion(emc2_bridge* h, int B, int N, const float* d_points, const 
         const unsigned blocks = (unsigned)((a.total + kThreads - 1) / kThreads);
         {
             LaunchScope ls(h, K_OCCL_SPLAT, st);
-            if (c.point_floats == 4) occl_kernel<4, false><<<blocks, kThreads, 0, st>>>(a);
-            else occl_kernel<5, false><<<blocks, kThreads, 0, st>>>(a);
+            if (c.point_floats == 4) launch_chained(occl_kernel<4, false>, blocks, kThreads, 0, st, a);
+            else launch_chained(occl_kernel<5, false>, blocks, kThreads, 0, st, a);
         }
         {
             LaunchScope ls(h, K_OCCL_TEST, st);
-            if (c.point_floats == 4) occl_kernel<4, true><<<blocks, kThreads, 0, st>>>(a);
-            else occl_kernel<5, true><<<blocks, kThreads, 0, st>>>(a);
+            if (c.point_floats == 4) launch_chained(occl_kernel<4, true>, blocks, kThreads, 0, st, a);
+            else launch_chained(occl_kernel<5, true>, blocks, kThreads, 0, st, a);
         }
     }
     return check_cuda(h, cudaGetLastError());

@@ -274,6 +274,7 @@ __global__ void __launch_bounds__(kThreads) project_route_kernel(const __grid_co
             for (size_t i = cta * kThreads + t; i < a.bev_n4; i += nthreads) __stcs(a.bev + i, z);
         }
     }
+    release_successor();
 }
 
 struct GsArgs {
@@ -304,6 +305,7 @@ template <int CF4> constexpr int kGsRows = CF4 == 16 ? 32 : 16;
 
 template <int C, int CF4>
 __global__ void __launch_bounds__(CF4 > 0 ? kGsRows<CF4> * CF4 : kMaxRowThreads) gather_scatter_kernel(const __grid_constant__ GsArgs a) {
+    await_predecessor();
     constexpr int kRows = kGsRows<CF4>;
     __shared__ uint4 srow[kTile];
     __shared__ TileOrder<C> order;
@@ -348,6 +350,7 @@ __global__ void __launch_bounds__(CF4 > 0 ? kGsRows<CF4> * CF4 : kMaxRowThreads)
             __stcs(fdst + (size_t)order.dest[r] * cf4 + c, o);
         }
     }
+    release_successor();
 }
 
 // ---- the same pass with the rows staged in shared memory and written by bulk asynchronous copies
@@ -376,6 +379,7 @@ __device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy
 // kBoth: also stage and bulk-copy the rows in point order; otherwise those are stored from registers.
 template <int C, int CF4, bool kBoth>
 __global__ void __launch_bounds__(16 * CF4) gather_scatter_bulk_kernel(const __grid_constant__ GsArgs a) {
+    await_predecessor();
     constexpr int kSub = 32, kBufs = 2, kWarpsTile = kTile / 32;
     __shared__ __align__(128) float4 stage[kBufs][kBoth ? 2 : 1][kSub * CF4];   // [buffer][expert order, point order]
     __shared__ uint4 srow[kTile];
@@ -514,6 +518,7 @@ __device__ __forceinline__ F8 gather_column8(const float* __restrict__ feat, con
 
 template <int C, int CF8>
 __global__ void __launch_bounds__(32 * CF8) gather_scatter_wide_kernel(const __grid_constant__ GsArgs a) {
+    await_predecessor();
     __shared__ uint4 srow[kTile];
     __shared__ int sdest[kTile];
     __shared__ int wcnt[kTile / 32][EMC2_MAX_EXPERTS];
@@ -570,6 +575,7 @@ __global__ void __launch_bounds__(32 * CF8) gather_scatter_wide_kernel(const __g
         if (keep) stcs8(out + (size_t)r * (8 * CF8) + 8 * c, o);
         stcs8(fdst + (size_t)sdest[r] * (8 * CF8) + 8 * c, o);
     }
+    release_successor();
 }
 
 
@@ -578,20 +584,20 @@ void launch_gs(emc2_bridge* h, const GsArgs& a, dim3 grid, cudaStream_t st) {
     LaunchScope ls(h, K_GATHER_SCATTER, st);
     const int mode = h->tune[EMC2_TUNE_ROW_STORE];
     if (mode == 1 && a.E < 31) {
-        if (a.cf4 == 16) { gather_scatter_bulk_kernel<C, 16, true><<<grid, 16 * 16, 0, st>>>(a); return; }
-        if (a.cf4 == 20) { gather_scatter_bulk_kernel<C, 20, true><<<grid, 16 * 20, 0, st>>>(a); return; }
+        if (a.cf4 == 16) { launch_chained(gather_scatter_bulk_kernel<C, 16, true>, grid, 16 * 16, 0, st, a); return; }
+        if (a.cf4 == 20) { launch_chained(gather_scatter_bulk_kernel<C, 20, true>, grid, 16 * 20, 0, st, a); return; }
     } else if (mode == 3 && ((reinterpret_cast<uintptr_t>(a.feat) | reinterpret_cast<uintptr_t>(a.gathered) |
                               reinterpret_cast<uintptr_t>(a.feat_out)) & 31) == 0) {
-        if (a.cf4 == 16) { gather_scatter_wide_kernel<C, 8><<<grid, 32 * 8, 0, st>>>(a); return; }
-        if (a.cf4 == 20) { gather_scatter_wide_kernel<C, 10><<<grid, 32 * 10, 0, st>>>(a); return; }
+        if (a.cf4 == 16) { launch_chained(gather_scatter_wide_kernel<C, 8>, grid, 32 * 8, 0, st, a); return; }
+        if (a.cf4 == 20) { launch_chained(gather_scatter_wide_kernel<C, 10>, grid, 32 * 10, 0, st, a); return; }
     } else if (mode == 2) {
-        if (a.cf4 == 16) { gather_scatter_bulk_kernel<C, 16, false><<<grid, 16 * 16, 0, st>>>(a); return; }
-        if (a.cf4 == 20) { gather_scatter_bulk_kernel<C, 20, false><<<grid, 16 * 20, 0, st>>>(a); return; }
+        if (a.cf4 == 16) { launch_chained(gather_scatter_bulk_kernel<C, 16, false>, grid, 16 * 16, 0, st, a); return; }
+        if (a.cf4 == 20) { launch_chained(gather_scatter_bulk_kernel<C, 20, false>, grid, 16 * 20, 0, st, a); return; }
     }
     switch (a.cf4) {
-        case 16: gather_scatter_kernel<C, 16><<<grid, kGsRows<16> * 16, 0, st>>>(a); break;
-        case 20: gather_scatter_kernel<C, 20><<<grid, kGsRows<20> * 20, 0, st>>>(a); break;
-        default: gather_scatter_kernel<C, 0><<<grid, row_threads(a.cf4), 0, st>>>(a); break;
+        case 16: launch_chained(gather_scatter_kernel<C, 16>, grid, kGsRows<16> * 16, 0, st, a); break;
+        case 20: launch_chained(gather_scatter_kernel<C, 20>, grid, kGsRows<20> * 20, 0, st, a); break;
+        default: launch_chained(gather_scatter_kernel<C, 0>, grid, row_threads(a.cf4), 0, st, a); break;
     }
 }
 

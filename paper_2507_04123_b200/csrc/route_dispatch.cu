@@ -74,6 +74,7 @@ __global__ void __launch_bounds__(kThreads) route_hist_kernel(const __grid_const
         if (tile0 + u < a.tiles && k < a.E)
             a.tile_counts[((size_t)b * a.tiles + tile0 + u) * a.E + k] = hist[u][k];
     }
+    release_successor();
 }
 
 template <int C>
@@ -90,6 +91,7 @@ constexpr int kScanThreads = 1024;
 __global__ void __launch_bounds__(kScanThreads)
 route_scan_kernel(const int* __restrict__ tile_counts, int* __restrict__ tile_base, int32_t* offsets,
                   int tiles, int E, int N) {
+    await_predecessor();
     constexpr int kWarps = kScanThreads / 32;
     __shared__ int wsum[EMC2_MAX_EXPERTS][kWarps];
     __shared__ int etot[EMC2_MAX_EXPERTS + 1];
@@ -150,6 +152,7 @@ route_scan_kernel(const int* __restrict__ tile_counts, int* __restrict__ tile_ba
             }
         }
     }
+    release_successor();
 }
 
 struct ScatterArgs {
@@ -166,6 +169,7 @@ struct ScatterArgs {
 // CF4 > 0: Cf/4 known at compile time, blockDim.x == 16 * CF4; else blockDim.x == row_threads(cf4).
 template <int C, int CF4>
 __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kMaxRowThreads) dispatch_scatter_kernel(ScatterArgs a) {
+    await_predecessor();
     __shared__ TileOrder<C> order;
     const int b = blockIdx.y, tile = blockIdx.x, t = threadIdx.x;
     const int i0 = tile * kTile;
@@ -201,14 +205,15 @@ __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kMaxRowThreads) dispatch_
             __stcs(fdst + (size_t)order.dest[r] * cf4 + c, __ldcs(fsrc + i));
         }
     }
+    release_successor();
 }
 
 template <int C>
 void launch_scatter_kernel(const ScatterArgs& a, dim3 grid, cudaStream_t st) {
     switch (a.cf4) {
-        case 16: dispatch_scatter_kernel<C, 16><<<grid, 16 * 16, 0, st>>>(a); break;
-        case 20: dispatch_scatter_kernel<C, 20><<<grid, 16 * 20, 0, st>>>(a); break;
-        default: dispatch_scatter_kernel<C, 0><<<grid, row_threads(a.cf4), 0, st>>>(a); break;
+        case 16: launch_chained(dispatch_scatter_kernel<C, 16>, grid, 16 * 16, 0, st, a); break;
+        case 20: launch_chained(dispatch_scatter_kernel<C, 20>, grid, 16 * 20, 0, st, a); break;
+        default: launch_chained(dispatch_scatter_kernel<C, 0>, grid, row_threads(a.cf4), 0, st, a); break;
     }
 }
 
@@ -260,7 +265,7 @@ int launch_scene_route(emc2_bridge* h, int B, const int32_t* d_offsets, const ui
 void launch_route_scan(emc2_bridge* h, int b0, int B, int tiles, int N, int32_t* d_offsets, cudaStream_t st) {
     LaunchScope ls(h, K_ROUTE_SCAN, st);
     const size_t t0 = (size_t)b0 * tiles * h->cfg.num_experts;
-    route_scan_kernel<<<B, kScanThreads, 0, st>>>(h->d_tile_counts + t0, h->d_tile_base + t0, d_offsets, tiles,
+    launch_chained(route_scan_kernel, B, kScanThreads, 0, st, h->d_tile_counts + t0, h->d_tile_base + t0, d_offsets, tiles,
                                                   h->cfg.num_experts, N);
 }
 
@@ -283,7 +288,7 @@ int launch_route_dispatch(emc2_bridge* h, int B, int N, const float* d_points, c
     }
     {
         LaunchScope ls(h, K_ROUTE_SCAN, st);
-        route_scan_kernel<<<B, kScanThreads, 0, st>>>(h->d_tile_counts, h->d_tile_base, d_offsets, tiles, E, N);
+        launch_chained(route_scan_kernel, B, kScanThreads, 0, st, h->d_tile_counts, h->d_tile_base, d_offsets, tiles, E, N);
     }
     if (tiles > 0) {
         ScatterArgs sa;
@@ -388,7 +393,7 @@ extern "C" int emc2_route_dispatch_static(const emc2_config_t* config, int32_t B
             for (int k = 0; k < 16; ++k) ra.lut[k] = c.lut[k >> 3][k & 7];
             if (c.point_floats == 4) launch_hist<4>(ra, B, st); else launch_hist<5>(ra, B, st);
         }
-        route_scan_kernel<<<B, kScanThreads, 0, st>>>(tile_counts, tile_base, d_offsets, tiles, E, N);
+        launch_chained(route_scan_kernel, B, kScanThreads, 0, st, tile_counts, tile_base, d_offsets, tiles, E, N);
         if (tiles > 0) {
             ScatterArgs sa;
             sa.pts = d_points; sa.feat = reinterpret_cast<const float4*>(d_gathered); sa.expert = d_expert;

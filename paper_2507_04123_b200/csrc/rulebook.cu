@@ -84,9 +84,11 @@ __global__ void __launch_bounds__(kThreads) rb_mark_kernel(const __grid_constant
     } else {
         a.g.store[cell] = (uint32_t)m + 1u;
     }
+    release_successor();
 }
 
 __global__ void __launch_bounds__(kThreads) rb_clear_kernel(const __grid_constant__ RbArgs a) {
+    await_predecessor();
     const int M = voxels_in_list(a);
     const int m = blockIdx.x * kThreads + threadIdx.x;
     if (m >= M) return;
@@ -95,6 +97,7 @@ __global__ void __launch_bounds__(kThreads) rb_clear_kernel(const __grid_constan
     if (cell == 0xFFFFFFFFu) return;
     if (a.g.mode == MODE_BITMAP) reinterpret_cast<uint4*>(a.g.store)[cell / kUnitCells] = make_uint4(0u, 0u, 0u, 0u);
     else a.g.store[cell] = 0u;
+    release_successor();
 }
 
 // Where a voxel sits: its cell, the cell strides and which of its 3 x 3 x 3 neighbours the grid has.
@@ -155,6 +158,7 @@ __device__ __forceinline__ uint32_t exist3(const ScaleDev& g, const Site& s, int
 }
 
 __global__ void __launch_bounds__(kThreads) rb_count_kernel(const __grid_constant__ RbArgs a) {
+    await_predecessor();
     __shared__ int wcount[kThreads / 32][kHalf];
     const int M = voxels_in_list(a);
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -182,11 +186,13 @@ __global__ void __launch_bounds__(kThreads) rb_count_kernel(const __grid_constan
         for (int w = 0; w < kThreads / 32; ++w) sum += wcount[w][t];
         a.tile_counts[(size_t)t * a.tiles + blockIdx.x] = sum;
     }
+    release_successor();
 }
 
 // CTA k: exclusive prefix sum of offset k's counts over the tiles, 4096 entries per round, and the
 // offset's pair total.  The totals become offsets[28] in rb_fill.
 __global__ void __launch_bounds__(kRbScanThreads) rb_scan_kernel(const __grid_constant__ RbArgs a) {
+    await_predecessor();
     __shared__ int wsum[kRbScanThreads / 32];
     __shared__ int s_carry;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -224,9 +230,11 @@ __global__ void __launch_bounds__(kRbScanThreads) rb_scan_kernel(const __grid_co
         __syncthreads();
     }
     if (t == 0) a.offset_pairs[blockIdx.x] = s_carry;
+    release_successor();
 }
 
 __global__ void __launch_bounds__(kThreads) rb_fill_kernel(const __grid_constant__ RbArgs a) {
+    await_predecessor();
     __shared__ int wcount[kThreads / 32][kHalf];      // pairs per warp, then where the warp's pairs start
     __shared__ int s_start[kOffsets + 1];             // offsets[]
     const int M = voxels_in_list(a);
@@ -298,6 +306,7 @@ __global__ void __launch_bounds__(kThreads) rb_fill_kernel(const __grid_constant
         }
     }
     if (m < M) put(s_start[kHalf] + m, m, m);
+    release_successor();
 }
 
 }  // namespace
@@ -326,19 +335,19 @@ int launch_rulebook(emc2_bridge* h, int scale, int capacity, const int32_t* d_co
     }
     {
         LaunchScope ls(h, K_RB_COUNT, st);
-        rb_count_kernel<<<blocks, kThreads, 0, st>>>(a);
+        launch_chained(rb_count_kernel, blocks, kThreads, 0, st, a);
     }
     {
         LaunchScope ls(h, K_RB_SCAN, st);
-        rb_scan_kernel<<<kHalf, kRbScanThreads, 0, st>>>(a);
+        launch_chained(rb_scan_kernel, kHalf, kRbScanThreads, 0, st, a);
     }
     {
         LaunchScope ls(h, K_RB_FILL, st);
-        rb_fill_kernel<<<blocks, kThreads, 0, st>>>(a);
+        launch_chained(rb_fill_kernel, blocks, kThreads, 0, st, a);
     }
     {
         LaunchScope ls(h, K_RB_CLEAR, st);
-        rb_clear_kernel<<<blocks, kThreads, 0, st>>>(a);
+        launch_chained(rb_clear_kernel, blocks, kThreads, 0, st, a);
     }
     return check_cuda(h, cudaGetLastError());
 }

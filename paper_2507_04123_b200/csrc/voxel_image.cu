@@ -105,6 +105,7 @@ __global__ void __launch_bounds__(kThreads) vif_scan_kernel(VifArgs a) {
 }
 
 __global__ void __launch_bounds__(kThreads) vif_fill_kernel(VifArgs a) {
+    await_predecessor();
     if (*a.bad) return;
     const int M = voxels_in_use(a);
     for (long long i = (long long)blockIdx.x * kThreads + threadIdx.x; i < a.total; i += (long long)gridDim.x * kThreads) {
@@ -129,11 +130,13 @@ __global__ void __launch_bounds__(kThreads) vif_fill_kernel(VifArgs a) {
         if (a.vis) a.list[pos] = entry;
         else a.recs[pos] = rec;
     }
+    release_successor();
 }
 
 // CF4 > 0: Cf/4 known at compile time, blockDim.x == 16 * CF4.  CF4 == 0: any Cf, 256 threads.
 template <int CF4>
 __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads) vif_mean_kernel(VifArgs a) {
+    await_predecessor();
     if (*a.bad) return;
     const int M = voxels_in_use(a);
     const int cf4 = CF4 > 0 ? CF4 : a.cf4;
@@ -188,6 +191,7 @@ __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads) vif_mean_kernel
             if (c == 0) a.vox_cnt[mm[u]] = seen[u];
         }
     }
+    release_successor();
 }
 
 // Mean of the p x p window of map texels that pooled texel (ty, tx) of map `map` stands for, column c:
@@ -229,6 +233,7 @@ __device__ __forceinline__ float4 pooled_column(const VifArgs& a, const uint4& r
 // kPooled: the taps are window means of the unpooled maps (emc2_voxel_image_pooled).
 template <int CF4, bool kPooled>
 __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads) vif_sample_kernel(VifArgs a) {
+    await_predecessor();
     if (*a.bad) return;
     const int M = voxels_in_use(a);
     const int cf4 = CF4 > 0 ? CF4 : a.cf4;
@@ -288,6 +293,7 @@ __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads) vif_sample_kern
             if (c == 0) a.vox_cnt[mm[u]] = seen[u];
         }
     }
+    release_successor();
 }
 
 }  // namespace
@@ -340,25 +346,25 @@ int launch_voxel_image(emc2_bridge* h, int B, int N, int capacity, const int32_t
     {
         LaunchScope ls(h, K_VIF_FILL, st);
         const int blocks = (int)min((long long)h->num_sms * 16, (a.total + kThreads - 1) / kThreads);
-        vif_fill_kernel<<<blocks, kThreads, 0, st>>>(a);
+        launch_chained(vif_fill_kernel, blocks, kThreads, 0, st, a);
     }
     const int blocks = (int)min((long long)h->num_sms * 16, ((long long)a.capacity + 15) / 16);
     if (d_gathered) {
         LaunchScope ls(h, K_VIF_MEAN, st);
         switch (a.cf4) {
-            case 16: vif_mean_kernel<16><<<blocks, 16 * 16, 0, st>>>(a); break;
-            case 20: vif_mean_kernel<20><<<blocks, 16 * 20, 0, st>>>(a); break;
-            default: vif_mean_kernel<0><<<blocks, kThreads, 0, st>>>(a); break;
+            case 16: launch_chained(vif_mean_kernel<16>, blocks, 16 * 16, 0, st, a); break;
+            case 20: launch_chained(vif_mean_kernel<20>, blocks, 16 * 20, 0, st, a); break;
+            default: launch_chained(vif_mean_kernel<0>, blocks, kThreads, 0, st, a); break;
         }
     } else {
         LaunchScope ls(h, K_VIF_SAMPLE, st);
         if (pool > 1) {
-            vif_sample_kernel<0, true><<<blocks, kThreads, 0, st>>>(a);
+            launch_chained(vif_sample_kernel<0, true>, blocks, kThreads, 0, st, a);
         } else {
             switch (a.cf4) {
-                case 16: vif_sample_kernel<16, false><<<blocks, 16 * 16, 0, st>>>(a); break;
-                case 20: vif_sample_kernel<20, false><<<blocks, 16 * 20, 0, st>>>(a); break;
-                default: vif_sample_kernel<0, false><<<blocks, kThreads, 0, st>>>(a); break;
+                case 16: launch_chained(vif_sample_kernel<16, false>, blocks, 16 * 16, 0, st, a); break;
+                case 20: launch_chained(vif_sample_kernel<20, false>, blocks, 16 * 20, 0, st, a); break;
+                default: launch_chained(vif_sample_kernel<0, false>, blocks, kThreads, 0, st, a); break;
             }
         }
     }

@@ -93,6 +93,7 @@ vox_mark_kernel(const float* __restrict__ pts, long long total, int N, ScaleDev 
         const float x = sp[t * C], y = sp[t * C + 1], z = sp[t * C + 2];
         mark_point(s0, s1, x, y, z, b0 + (i0 + t) / N);
     }
+    release_successor();
 }
 
 // ------------------------------------------------------------------ pass 2: ranks
@@ -135,6 +136,7 @@ constexpr int kScanSectors = (int)(kScanTileBytes / 32);          // 32-byte sec
 static_assert(kScanSectors == kThreads, "vox_count_kernel gives a thread one sector of each of its tiles");
 
 __global__ void __launch_bounds__(kThreads) vox_count_kernel(const __grid_constant__ ScanArgs a) {
+    await_predecessor();
     constexpr int kWarps = kThreads / 32;
     __shared__ uint32_t s_warp[kCountTiles][kWarps];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -172,11 +174,13 @@ __global__ void __launch_bounds__(kThreads) vox_count_kernel(const __grid_consta
         at = __shfl_sync(kAll, at, 0) + __popc(some & ((1u << t) - 1u));
         if (n) a.st.list[at] = (uint32_t)(tile0 + t) | (sc ? 0x80000000u : 0u);
     }
+    release_successor();
 }
 
 constexpr int kRankThreads = kScanSectors, kRankCtas = 6;
 
 __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const __grid_constant__ ScanArgs a) {
+    await_predecessor();
     constexpr int kWarps = kRankThreads / 32;
     __shared__ uint32_t s_before[kWarps], s_warp[kWarps];
     __shared__ int s_over[2];                             // cells over the cap and their points: sum, then base
@@ -310,6 +314,7 @@ __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const
         }
         __syncthreads();                                  // the shared counters are used again
     }
+    release_successor();
 }
 
 // ------------------------------------------------------------------ pass 3: accumulate
@@ -331,6 +336,7 @@ struct AccumArgs {
 template <int C>
 __global__ void __launch_bounds__(kThreads)
 vox_accum_kernel(const float* __restrict__ pts, long long total, int N, AccumArgs a) {
+    await_predecessor();
     __shared__ __align__(16) float sp[kBigTile * C];
     const long long g0 = (long long)blockIdx.x * kBigTile;
     const int npts = (int)min((long long)kBigTile, total - g0);
@@ -391,6 +397,7 @@ vox_accum_kernel(const float* __restrict__ pts, long long total, int N, AccumArg
             else if (C > 4) atomicAdd(reinterpret_cast<float*>(row + 1), sp[t * C + 4]);
         }
     }
+    release_successor();
 }
 
 // ------------------------------------------------------------------ per-voxel cap on a bitmap scale
@@ -403,6 +410,7 @@ vox_accum_kernel(const float* __restrict__ pts, long long total, int N, AccumArg
 //                   voxel's list.
 // vox_finalize then keeps the `cap` lowest indices of every list exactly as for a table scale.
 __global__ void __launch_bounds__(kThreads) vox_over_find_kernel(AccumArgs a, int sc) {
+    await_predecessor();
     const ScaleDev& g = a.s[sc];
     const int lane = threadIdx.x & 31;
     const int M = min(g.totals[0], a.capacity[sc]);
@@ -434,11 +442,13 @@ __global__ void __launch_bounds__(kThreads) vox_over_find_kernel(AccumArgs a, in
         g.ovf_cursor[(size_t)j * kCursorStride] = 0;
         reinterpret_cast<uint32_t*>(g.acc + 2 * (size_t)m + 1)[2] = (uint32_t)j + 1u;
     }
+    release_successor();
 }
 
 template <int C>
 __global__ void __launch_bounds__(kThreads)
 vox_over_fill_kernel(const float* __restrict__ pts, long long total, int N, AccumArgs a, int sc) {
+    await_predecessor();
     const ScaleDev& g = a.s[sc];
     for (long long i = (long long)blockIdx.x * kThreads + threadIdx.x; i < total; i += (long long)gridDim.x * kThreads) {
         const float* p = pts + i * C;
@@ -451,6 +461,7 @@ vox_over_fill_kernel(const float* __restrict__ pts, long long total, int N, Accu
         const uint32_t pos = (uint32_t)(g.ovf_off[j] + tk);
         if (pos < g.max_list) g.ovf_list[pos] = (int)i;
     }
+    release_successor();
 }
 
 // ------------------------------------------------------------------ pass 4: rows, BEV, cleanup
@@ -528,6 +539,7 @@ __device__ __forceinline__ void write_batch(const AccumArgs& a, int sc, int mb, 
 template <int C>
 __global__ void __launch_bounds__(kThreads)
 vox_finalize_kernel(const float* __restrict__ pts, long long total, AccumArgs a, int ovf_blocks) {
+    await_predecessor();
     constexpr int kWarps = kThreads / 32;
     const int lane = threadIdx.x & 31;
     if ((int)blockIdx.x < ovf_blocks) {
@@ -613,6 +625,7 @@ vox_finalize_kernel(const float* __restrict__ pts, long long total, AccumArgs a,
         }
         write_batch<C>(a, sc, mb, n, entry, stage);
     }
+    release_successor();
 }
 
 template <int C>
@@ -670,24 +683,26 @@ int run_voxelize(emc2_bridge* h, int B, int N, const float* d_points, int32_t* c
     if (tiles > 0) {
         {
             LaunchScope ls(h, K_VOX_COUNT, st);
-            vox_count_kernel<<<tiles / kCountTiles, kThreads, 0, st>>>(sa);
+            // In the one-call path the first kernel of the side stream: its predecessor is on another stream.
+            if (marked) vox_count_kernel<<<tiles / kCountTiles, kThreads, 0, st>>>(sa);
+            else launch_chained(vox_count_kernel, tiles / kCountTiles, kThreads, 0, st, sa);
         }
         LaunchScope ls(h, K_VOX_RANK, st);
-        vox_rank_kernel<<<min(tiles, kRankCtas * h->num_sms), kRankThreads, 0, st>>>(sa);
+        launch_chained(vox_rank_kernel, min(tiles, kRankCtas * h->num_sms), kRankThreads, 0, st, sa);
     }
     if (total > 0) {
         LaunchScope ls(h, K_VOX_ACCUM, st);
-        vox_accum_kernel<C><<<ptiles, kThreads, 0, st>>>(d_points, total, N, aa);
+        launch_chained(vox_accum_kernel<C>, ptiles, kThreads, 0, st, d_points, total, N, aa);
     }
     for (int s = 0; s < 2 && total > 0; ++s) {
         if (aa.s[s].mode != MODE_BITMAP || h->scale[s].cap <= 0) continue;
         {
             LaunchScope ls(h, K_VOX_OVER_FIND, st);
-            vox_over_find_kernel<<<4 * h->num_sms, kThreads, 0, st>>>(aa, s);
+            launch_chained(vox_over_find_kernel, 4 * h->num_sms, kThreads, 0, st, aa, s);
         }
         {
             LaunchScope ls(h, K_VOX_OVER_FILL, st);
-            vox_over_fill_kernel<C><<<(int)min((long long)8 * h->num_sms, (total + kThreads - 1) / kThreads), kThreads, 0, st>>>(
+            launch_chained(vox_over_fill_kernel<C>, (int)min((long long)8 * h->num_sms, (total + kThreads - 1) / kThreads), kThreads, 0, st, 
                 d_points, total, N, aa, s);
         }
     }
@@ -696,7 +711,7 @@ int run_voxelize(emc2_bridge* h, int B, int N, const float* d_points, int32_t* c
         const int ovf_blocks = any_cap ? 2 * h->num_sms : 0;    // CTAs that serve cells over the cap
         const int vox_blocks = (int)min((long long)h->num_sms * 8, (2 * total + 32 * 8 - 1) / (32 * 8) + 1);
         LaunchScope ls(h, K_VOX_FINALIZE, st);
-        vox_finalize_kernel<C><<<ovf_blocks + vox_blocks, kThreads, 0, st>>>(d_points, total, aa, ovf_blocks);
+        launch_chained(vox_finalize_kernel<C>, ovf_blocks + vox_blocks, kThreads, 0, st, d_points, total, aa, ovf_blocks);
     }
     return check_cuda(h, cudaGetLastError());
 }
