@@ -296,14 +296,13 @@ int launch_scene_route(emc2_bridge* h, int B, const int32_t* d_offsets, const ui
 void launch_route_scan(emc2_bridge* h, int b0, int B, int tiles, int N, int32_t* d_offsets, cudaStream_t st);
 // Stages 2 - 4 in one pass over the feature rows (the one-call path), in two parts: projection +
 // routing per point (which, with `d_bev_to_zero`/`mark`, also marks the voxel cells of both scales
-// and zeroes the BEV image, so that stage 1 reads the points once less), then offsets + rows.
+// and zeroes the BEV image, so that stage 1 reads the points once less), then, after launch_route_scan, the rows.
 int launch_project_route(emc2_bridge* h, int b0, int B, int N, const float* d_points, const float* d_proj,
                          float* d_uvd, uint8_t* d_vis_mask, int8_t* d_cam, uint8_t* d_expert, bool mark,
                          float* d_bev_to_zero, int bev_frames, cudaStream_t st);
-int launch_scan_gather_scatter(emc2_bridge* h, int b0, int B, int N, const float* d_points, const float* d_feat,
-                               const float* d_uvd, const int8_t* d_cam, float* d_gathered, const uint8_t* d_expert,
-                               int32_t* d_offsets, int32_t* d_perm, float* d_points_out, float* d_feat_out,
-                               cudaStream_t st);
+int launch_gather_scatter(emc2_bridge* h, int b0, int B, int N, const float* d_points, const float* d_feat,
+                          const float* d_uvd, const int8_t* d_cam, float* d_gathered, const uint8_t* d_expert,
+                          int32_t* d_perm, float* d_points_out, float* d_feat_out, cudaStream_t st);
 
 // ---------------------------------------------------------------- device helpers
 #ifdef __CUDACC__

@@ -770,17 +770,15 @@ int launch_project_route(emc2_bridge* h, int b0, int B, int N, const float* d_po
     return check_cuda(h, cudaGetLastError());
 }
 
-int launch_scan_gather_scatter(emc2_bridge* h, int b0, int B, int N, const float* d_points, const float* d_feat,
-                               const float* d_uvd, const int8_t* d_cam, float* d_gathered, const uint8_t* d_expert,
-                               int32_t* d_offsets, int32_t* d_perm, float* d_points_out, float* d_feat_out,
-                               cudaStream_t st) {
+int launch_gather_scatter(emc2_bridge* h, int b0, int B, int N, const float* d_points, const float* d_feat,
+                          const float* d_uvd, const int8_t* d_cam, float* d_gathered, const uint8_t* d_expert,
+                          int32_t* d_perm, float* d_points_out, float* d_feat_out, cudaStream_t st) {
     const emc2_config_t& c = h->cfg;
     if (B == 0) return EMC2_OK;
     const int tiles = (N + kTile - 1) / kTile;
     const dim3 grid(tiles > 0 ? tiles : 1, B);
     const int E = c.num_experts;
     const size_t p0 = (size_t)b0 * N, t0 = (size_t)b0 * tiles * E;
-    launch_route_scan(h, b0, B, tiles, N, d_offsets + (size_t)b0 * (E + 1), st);
     if (tiles > 0) {
         GsArgs ga;
         ga.pts = d_points + p0 * c.point_floats; ga.uvd = d_uvd + p0 * 3; ga.cam = d_cam + p0; ga.expert = d_expert + p0;
