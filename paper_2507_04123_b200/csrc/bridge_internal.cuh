@@ -242,6 +242,9 @@ int launch_route_dispatch(emc2_bridge* h, int B, int N, const float* d_points, c
 // Launches a kernel that may be set up while its predecessor in the stream still drains (programmatic dependent
 // launch); for kernels that follow another kernel of the same call on the same stream.  Every kernel launched this
 // way calls await_predecessor() before it touches memory and, when its own work is done, release_successor().
+// Such a kernel can be resident while its predecessor still writes: what a kernel of the same call writes is read
+// through plain pointers, never through `const __restrict__` ones or __ldg, whose loads the compiler may move ahead
+// of the wait.  The call's own inputs are complete before the first kernel of a call, which is launched plainly.
 // Released earlier, the successor's CTAs would hold places on the SMs that the kernels of the other stream need.
 // us per call: one small frame 35 -> 30, stage calls with occlusion 155 -> 140, voxels and rulebooks 261 -> 239 (B200).
 template <typename... P, typename... A>

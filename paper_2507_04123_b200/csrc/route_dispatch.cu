@@ -88,9 +88,10 @@ constexpr int kScanThreads = 1024;
 // One CTA of 1024 threads per frame.  Every thread owns a run of consecutive tiles and loads all
 // their counts up front; per expert, a CTA-wide exclusive scan of the run totals gives the run's
 // base, the expert totals give the frame's offsets, and the bases are written in one sweep.
+// The counts may still be in the making while this kernel is set up (see launch_chained), so they are
+// not declared read-only; a tile's counts are loaded together before its bases are stored.
 __global__ void __launch_bounds__(kScanThreads)
-route_scan_kernel(const int* __restrict__ tile_counts, int* __restrict__ tile_base, int32_t* offsets,
-                  int tiles, int E, int N) {
+route_scan_kernel(const int* tile_counts, int* tile_base, int32_t* offsets, int tiles, int E, int N) {
     await_predecessor();
     constexpr int kWarps = kScanThreads / 32;
     __shared__ int wsum[EMC2_MAX_EXPERTS][kWarps];
@@ -144,11 +145,15 @@ route_scan_kernel(const int* __restrict__ tile_counts, int* __restrict__ tile_ba
     for (int e = 0; e < EMC2_MAX_EXPERTS; ++e)
         if (e < E) run[e] += etot[e] + wsum[e][warp];
     for (int i = lo; i < hi; ++i) {
+        int n[EMC2_MAX_EXPERTS];
+#pragma unroll
+        for (int e = 0; e < EMC2_MAX_EXPERTS; ++e)
+            if (e < E) n[e] = cnt[(size_t)i * E + e];
 #pragma unroll
         for (int e = 0; e < EMC2_MAX_EXPERTS; ++e) {
             if (e < E) {
                 base[(size_t)i * E + e] = run[e];
-                run[e] += cnt[(size_t)i * E + e];
+                run[e] += n[e];
             }
         }
     }
