@@ -10,7 +10,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libemc2_bridge.so")
 SOURCES = ["bridge.cu", "voxelize.cu", "project_gather.cu", "route_dispatch.cu", "voxel_image.cu", "occlusion.cu", "rulebook.cu", "dedup_arms.cu"]
-HEADERS = [os.path.join(CSRC, "bridge_internal.cuh"), os.path.join(ROOT, "include", "emc2_bridge.h")]
+HEADERS = [os.path.join(CSRC, "bridge_internal.cuh"), os.path.join(CSRC, "rules.cuh"), os.path.join(ROOT, "include", "emc2_bridge.h")]
 
 
 def nvcc_command(verbose_ptxas: bool = False):

@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "emc2_bridge.h"
+#include "rules.cuh"
 
 namespace emc2 {
 
@@ -122,8 +123,8 @@ struct ScaleDev {
     int design;             // dedup design of this scale: 0 = this direct-addressed store, 1 = hash, 2 = sort
                             // (dedup_arms.cu); with 1 or 2 the store is not used and rows come from point_rank
     const int* point_rank;  // design != 0: [points of the call] row of every point's voxel, -1 if outside
-    int* totals;            // [0] voxels, [2] points in cells over the cap, [3] cells over the cap ([2] and [3] are
-                            // one 64-bit ticket counter)
+    int* totals;            // [0] voxels, [1] not 0: the lists of cells over the cap are not used (refuse_lists),
+                            // [2] points in cells over the cap, [3] cells over the cap (one 64-bit ticket counter)
 };
 
 // Routing tables as the kernels take them (Sec. 3.2 distance rule, per point with visibility).

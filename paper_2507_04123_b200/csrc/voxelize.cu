@@ -177,6 +177,13 @@ __global__ void __launch_bounds__(kThreads) vox_count_kernel(const __grid_consta
     release_successor();
 }
 
+// More cells over the cap, or more points in them, than a call's points allow: the store was not all zero when the
+// call began.  The scale's lists are not used then; vox_finalize reports no voxels for it.
+__device__ __forceinline__ void refuse_lists(const ScaleDev& g, int* status) {
+    atomicOr(&g.totals[1], 1);
+    atomicOr(status, kStatusDirtyStore);
+}
+
 constexpr int kRankThreads = kScanSectors, kRankCtas = 6;
 
 __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const __grid_constant__ ScanArgs a) {
@@ -247,26 +254,35 @@ __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const
         // Cells over the cap take the next places among such cells, and their points the next slots of
         // the index list, in any order: one ticket per tile.
         uint32_t j = 0, off = 0;
+        bool list_over = false;
         if (!bitmap && g.cap > 0) {
             const uint32_t n[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
             uint32_t cells = 0, points = 0;
 #pragma unroll
             for (int i = 0; i < 8; ++i)
-                if (n[i] > (uint32_t)g.cap) { cells += 1; points += n[i]; }
+                if (n[i] > (uint32_t)g.cap) { cells += 1; points += clamp_points(n[i]); }
             if (__any_sync(0xFFFFFFFFu, cells != 0)) {
+                points = clamp_points(points);
                 const uint32_t ic = warp_incl_scan(cells), ip = warp_incl_scan(points);
                 int wc = 0, wp = 0;                       // the warp's share starts here inside the tile's
-                if (lane == 31) { wc = atomicAdd(&s_over[0], (int)ic); wp = atomicAdd(&s_over[1], (int)ip); }
+                if (lane == 31) { wc = atomicAdd(&s_over[0], (int)ic); wp = atomicAdd(&s_over[1], (int)clamp_points(ip)); }
                 j = (uint32_t)__shfl_sync(0xFFFFFFFFu, wc, 31) + ic - cells;
                 off = (uint32_t)__shfl_sync(0xFFFFFFFFu, wp, 31) + ip - points;
             }
             __syncthreads();
             if (t == 0 && s_over[0] > 0) {
-                const unsigned long long add = ((unsigned long long)(uint32_t)s_over[0] << 32) | (uint32_t)s_over[1];
-                const unsigned long long first = atomicAdd(reinterpret_cast<unsigned long long*>(g.totals + 2), add);
-                s_over[0] = (int)(first >> 32); s_over[1] = (int)(uint32_t)first;
+                const uint32_t tc = (uint32_t)s_over[0], tp = (uint32_t)s_over[1];
+                unsigned long long first = 0;
+                bool fits = tp <= g.max_list;
+                if (fits) {
+                    first = atomicAdd(reinterpret_cast<unsigned long long*>(g.totals + 2), (unsigned long long)over_ticket(tc, tp));
+                    fits = over_fits(first, tc, tp, g.max_ovf, g.max_list);
+                }
+                if (!fits) refuse_lists(g, a.status);
+                s_over[0] = fits ? (int)(first >> 32) : -1; s_over[1] = (int)(uint32_t)first;
             }
             __syncthreads();
+            list_over = s_over[0] >= 0;
             j += (uint32_t)s_over[0];
             off += (uint32_t)s_over[1];
         }
@@ -291,16 +307,12 @@ __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     if (n[i] == 0u) continue;
-                    const bool over = g.cap > 0 && n[i] > (uint32_t)g.cap;
+                    const bool over = list_over && n[i] > (uint32_t)g.cap;
                     if (m < (uint32_t)a.capacity[sc]) a.counts[sc][m] = over ? g.cap : (int)n[i];
                     if (m < g.max_list) g.cell_list[m] = over ? (cell + i) | kOverCap : cell + i;
                     if (over) {
-                        if (j < g.max_ovf && off + n[i] <= g.max_list) {
-                            g.ovf_vox[j] = (int)m; g.ovf_off[j] = (int)off; g.ovf_cell[j] = cell + i;
-                            g.ovf_cursor[(size_t)j * kCursorStride] = 0;
-                        } else {
-                            atomicOr(a.status, kStatusDirtyStore);
-                        }
+                        g.ovf_vox[j] = (int)m; g.ovf_off[j] = (int)off; g.ovf_cell[j] = cell + i;
+                        g.ovf_cursor[(size_t)j * kCursorStride] = 0;
                         off += n[i];
                         n[i] = kOverCap | j++;
                     } else {
@@ -326,6 +338,8 @@ struct AccumArgs {
     int32_t* point_voxel[2];
     float* mean[2];
     float* bev;
+    int32_t* num_voxels;
+    int* status;
 };
 
 // Per-voxel accumulator, 32 bytes of fp32: {sum dx, sum dy, sum dz, sum ch3}, {sum ch4, count, -, -},
@@ -427,17 +441,22 @@ __global__ void __launch_bounds__(kThreads) vox_over_find_kernel(AccumArgs a, in
             if (lane >= d) inc += y;
         }
         int j0 = 0, off0 = 0;
-        if (lane == 31) {
-            const unsigned long long add = ((unsigned long long)__popc(who) << 32) | (uint32_t)inc;
-            const unsigned long long at = atomicAdd(reinterpret_cast<unsigned long long*>(g.totals + 2), add);
-            j0 = (int)(at >> 32); off0 = (int)(uint32_t)at;
+        if (lane == 31) {                         // sums of at most 32 counts of at most 2^24
+            const uint32_t cells = (uint32_t)__popc(who), points = (uint32_t)inc;
+            unsigned long long at = 0;
+            bool fits = points <= g.max_list;
+            if (fits) {
+                at = atomicAdd(reinterpret_cast<unsigned long long*>(g.totals + 2), (unsigned long long)over_ticket(cells, points));
+                fits = over_fits(at, cells, points, g.max_ovf, g.max_list);
+            }
+            if (!fits) refuse_lists(g, a.status);     // never with this batch's own counts
+            j0 = fits ? (int)(at >> 32) : -1; off0 = (int)(uint32_t)at;
         }
         j0 = __shfl_sync(0xFFFFFFFFu, j0, 31);
         off0 = __shfl_sync(0xFFFFFFFFu, off0, 31);
-        if (!over) continue;
+        if (!over || j0 < 0) continue;
         const int j = j0 + __popc(who & ((1u << lane) - 1u));
         const int off = off0 + inc - n;
-        if ((uint32_t)j >= g.max_ovf || (uint32_t)(off + n) > g.max_list) continue;   // cannot happen with this batch's counts
         g.ovf_vox[j] = m; g.ovf_off[j] = off; g.ovf_cell[j] = g.cell_list[m];
         g.ovf_cursor[(size_t)j * kCursorStride] = 0;
         reinterpret_cast<uint32_t*>(g.acc + 2 * (size_t)m + 1)[2] = (uint32_t)j + 1u;
@@ -548,15 +567,15 @@ vox_finalize_kernel(const float* __restrict__ pts, long long total, AccumArgs a,
         for (int sc = 0; sc < 2; ++sc) {
             const ScaleDev& g = a.s[sc];
             if (g.cap <= 0) continue;
-            // More of them, or more points in them, than this call's points allow: a store that was not all zero
-            // (the status says so); the lists then hold nothing that can be used.
-            const bool dirty = g.totals[0] == 0 || (uint32_t)g.totals[2] > g.max_list || (uint32_t)g.totals[3] > g.max_ovf;
-            const int novf = dirty ? 0 : g.totals[3];
+            const bool refused = g.totals[0] == 0 || g.totals[1] != 0;        // see refuse_lists
+            if (refused && g.totals[1] != 0 && warp == 0 && lane == 0) a.num_voxels[sc] = 0;
+            const int novf = refused ? 0 : min(g.totals[3], (int)g.max_ovf);
             int32_t* pv = a.point_voxel[sc];
             for (int j = warp; j < novf; j += nwarps) {
                 const int m = g.ovf_vox[j];
-                const int* list = g.ovf_list + g.ovf_off[j];
-                const int n = min(g.ovf_cursor[(size_t)j * kCursorStride], (int)g.max_list - g.ovf_off[j]);
+                const uint32_t start = (uint32_t)g.ovf_off[j];
+                const int* list = g.ovf_list + start;
+                const int n = start < g.max_list ? min(g.ovf_cursor[(size_t)j * kCursorStride], (int)(g.max_list - start)) : 0;
                 // Smallest index value v with #{list <= v} >= cap, by bisection on the value.
                 long long lo = -1, hi = total - 1;
                 while (hi - lo > 1) {
@@ -571,6 +590,7 @@ vox_finalize_kernel(const float* __restrict__ pts, long long total, AccumArgs a,
                 for (int k = 0; k < C; ++k) acc[k] = 0.0;
                 for (int i = lane; i < n; i += 32) {
                     const int v = list[i];
+                    if ((unsigned long long)v >= (unsigned long long)total) continue;   // never a point of this call
                     const bool keep = v <= hi;
                     if (pv) pv[v] = keep ? m : -1;
                     if (keep) {
@@ -583,7 +603,7 @@ vox_finalize_kernel(const float* __restrict__ pts, long long total, AccumArgs a,
 #pragma unroll
                     for (int d = 16; d > 0; d >>= 1) acc[k] += __shfl_xor_sync(0xFFFFFFFFu, acc[k], d);
                 }
-                if (lane < C && m < a.capacity[sc]) {
+                if (lane < C && (unsigned)m < (unsigned)a.capacity[sc]) {
                     double v = 0.0;
 #pragma unroll
                     for (int k = 0; k < C; ++k) v = lane == k ? acc[k] : v;
@@ -659,6 +679,8 @@ int run_voxelize(emc2_bridge* h, int B, int N, const float* d_points, int32_t* c
     sa.status = h->d_status;
     sa.st = h->scan;
     aa.bev = d_bev;
+    aa.num_voxels = d_num_voxels;
+    aa.status = h->d_status;
 
     const size_t bev_n = d_bev ? (size_t)B * C * h->scale[1].dims[1] * h->scale[1].dims[0] : 0;
     const bool bev_vec = (bev_n & 3) == 0;

@@ -1,0 +1,87 @@
+"""The index arithmetic of csrc/rules.cuh, compiled for the host (CPU)."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2507_04123_b200", "csrc")
+
+SHIM = r"""
+#include "rules.cuh"
+using namespace emc2;
+extern "C" {
+uint32_t clamp(uint32_t n) { return clamp_points(n); }
+int fits(uint64_t first, uint32_t cells, uint32_t points, uint32_t max_ovf, uint32_t max_list) {
+    return over_fits(first, cells, points, max_ovf, max_list);
+}
+uint64_t ticket(uint32_t cells, uint32_t points) { return over_ticket(cells, points); }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    d = tmp_path_factory.mktemp("rules")
+    src, lib = str(d / "shim.cpp"), str(d / "librules.so")
+    with open(src, "w") as f:
+        f.write(SHIM)
+    subprocess.run(["g++", "-std=c++17", "-O2", "-Wall", "-Werror", "-ffp-contract=off", "-fsanitize=undefined",
+                    "-fno-sanitize-recover=undefined", "-fPIC", "-shared", "-I", CSRC, "-o", lib, src], check=True)
+    so = ctypes.CDLL(lib)
+    u32, u64 = ctypes.c_uint32, ctypes.c_uint64
+    so.clamp.restype, so.clamp.argtypes = u32, [u32]
+    so.fits.restype, so.fits.argtypes = ctypes.c_int, [u64, u32, u32, u32, u32]
+    so.ticket.restype, so.ticket.argtypes = u64, [u32, u32]
+    return so
+
+
+def test_point_sums_of_a_tile_never_wrap_and_never_pass_for_small_ones(rules):
+    """2,048 words of a tile, summed as the rank scan does (8 per thread, 32 threads per warp, 8 warps), whatever they hold."""
+    rng = np.random.default_rng(0)
+    words = np.array([33, 1 << 24, (1 << 24) + 1, 0x80000000, 0x80000001, 0x80000005, 0xFFFFFFFF], np.uint64)
+    for most in (1, 300000, 1 << 24):
+        for trial in range(60):
+            n = np.full(2048, 33, np.uint64) if trial == 0 else rng.choice(words[: 1 + trial % len(words)], 2048)
+            n[rng.random(2048) < rng.random()] = 0
+            threads = [sum(rules.clamp(int(v)) for v in t) for t in n.reshape(-1, 8)]
+            assert max(threads) < 1 << 31
+            warps = [sum(rules.clamp(v) for v in w) for w in np.reshape(threads, (-1, 32)).tolist()]
+            assert max(warps) < 1 << 31
+            tile = sum(rules.clamp(v) for v in warps)
+            assert tile < 1 << 31
+            true = int(n.sum())
+            assert (tile > most) == (true > most)
+            if true <= most:
+                assert tile == true
+
+
+def test_tickets_that_do_not_fit_are_found(rules):
+    """A run of tickets is refused from the first one on that leaves the lists, also where 32-bit sums would wrap."""
+    rng = np.random.default_rng(1)
+    for max_list, max_ovf in ((300000, 9092), (1 << 24, 508401), (1, 2), (96, 4)):
+        for _ in range(200):
+            counter, cells, points, refused = 0, 0, 0, False
+            for _ in range(60):
+                c = int(rng.integers(1, 2049))
+                p = int(rng.choice([c, min(33 * c, max_list), max_list, int(rng.integers(0, max_list + 1))]))
+                p = min(p, max_list)
+                first = counter
+                counter = (counter + rules.ticket(c, p)) % (1 << 64)
+                cells, points = cells + c, points + p
+                ok = bool(rules.fits(first, c, p, max_ovf, max_list))
+                if not refused:
+                    assert ok == (cells <= max_ovf and points <= max_list)
+                refused = refused or not ok
+                if ok:                                      # in bounds whatever came before
+                    assert (first >> 32) + c <= max_ovf and (first & 0xFFFFFFFF) + p <= max_list
+            assert refused == (cells > max_ovf or points > max_list)
+
+
+def test_leftover_words_do_not_make_a_small_sum(rules):
+    """Two leftover words {over the cap, place 1} and {over the cap, place 5} add up to 6 in 32 bits."""
+    words = [0x80000001, 0x80000005]
+    assert sum(words) % (1 << 32) == 6
+    assert sum(rules.clamp(w) for w in words) > 1 << 24
+    assert not rules.fits(rules.ticket(0, 0x80000001), 1, 0x80000005, 1000, 300000)
