@@ -212,11 +212,11 @@ __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const
     for (int v = 0; v < 2; ++v) all[v] = __reduce_add_sync(0xFFFFFFFFu, lane < kWarps ? (v ? s_warp : s_before)[lane] : 0u);
     if (blockIdx.x == 0 && t < 2 && !a.s[t].design) {
         // More voxels than a call's points allow: the store was not all zero when the call began (two
-        // calls on one handle at once).  The scale then reports no voxels and the handle's status
-        // becomes an internal error; rows past the lists are not written anywhere.
+        // calls on one handle at once).  The scale is then not ranked and reports no voxels, and the
+        // handle's status becomes an internal error.
         const ScaleDev& g = a.s[t];
         const uint32_t n = t ? all[1] : all[0];
-        const bool dirty = n > g.max_list;
+        const bool dirty = !voxels_possible(n, g.max_list);
         g.totals[0] = dirty ? 0 : (int)n;
         a.num_voxels[t] = dirty ? 0 : (int)n;
         if (dirty) atomicOr(a.status, kStatusDirtyStore);
@@ -233,6 +233,7 @@ __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const
         if (k + gridDim.x < listed) next = a.st.list[k + gridDim.x];
         const int sc = (int)(entry >> 31), tile = (int)(entry & 0x7FFFFFFFu);
         const ScaleDev& g = a.s[sc];
+        if (!voxels_possible(sc ? all[1] : all[0], g.max_list)) continue;
         const bool bitmap = g.mode == MODE_BITMAP;
         const uint32_t sector = (uint32_t)tile * kScanSectors + t;
         uint4* const at = reinterpret_cast<uint4*>(g.store) + (size_t)sector * 2;

@@ -85,3 +85,13 @@ def test_leftover_words_do_not_make_a_small_sum(rules):
     assert sum(words) % (1 << 32) == 6
     assert sum(rules.clamp(w) for w in words) > 1 << 24
     assert not rules.fits(rules.ticket(0, 0x80000001), 1, 0x80000005, 1000, 300000)
+
+
+def test_a_scale_with_more_voxels_than_points_is_not_ranked():
+    """vox_rank leaves such a scale's tiles before it writes a rank, a list entry or one of the caller's counts."""
+    text = open(os.path.join(CSRC, "voxelize.cu")).read()
+    body = text[text.index("vox_rank_kernel("):text.index("pass 3: accumulate")]
+    loop = body[body.index("k < listed"):]
+    guard = loop.index("if (!voxels_possible(sc ? all[1] : all[0], g.max_list)) continue;")
+    for write in ("a.counts[sc][m] =", "g.cell_list[m] =", "at[0] =", "atomicAdd("):
+        assert guard < loop.index(write), write
