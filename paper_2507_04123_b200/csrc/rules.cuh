@@ -15,6 +15,10 @@ namespace emc2 {
 // ---- voxels found by the rank scan: at most one per point of a call, or the store was not all zero when it began
 EMC2_RULE bool voxels_possible(uint32_t voxels, uint32_t max_list) { return voxels <= max_list; }
 
+// The scan covers whole tiles, which can reach past the call's last frame; a cell found there was left over as well,
+// and the caller's BEV image has no such frame.
+EMC2_RULE bool frame_in_call(uint32_t frame, uint32_t frames) { return frame < frames; }
+
 // ---- cells over the per-voxel cap (rank scan of a table store)
 // A tile sums the points of its cells over the cap and takes one 64-bit ticket for them, {cells, points} before the
 // tile.  In a store that was not all zero a word can hold anything, and a sum that wrapped would pass for a small

@@ -339,6 +339,7 @@ struct AccumArgs {
     int32_t* point_voxel[2];
     float* mean[2];
     float* bev;
+    uint32_t frames;            // B
     int32_t* num_voxels;
     int* status;
 };
@@ -545,7 +546,7 @@ __device__ __forceinline__ void write_batch(const AccumArgs& a, int sc, int mb, 
 #pragma unroll
         for (int k = 0; k < C; ++k) rows[lane * C + k] = mu[k];
     }
-    if (sc == 1 && a.bev && active && !over) {
+    if (sc == 1 && a.bev && active && !over && frame_in_call(r, a.frames)) {
         const size_t plane = (size_t)g.dims[1] * g.dims[0];
         float* dst = a.bev + (size_t)r * C * plane + (size_t)y * g.dims[0] + x;
 #pragma unroll
@@ -615,7 +616,7 @@ vox_finalize_kernel(const float* __restrict__ pts, long long total, AccumArgs a,
                         g.div[0].divmod(r, r, x);
                         g.div[1].divmod(r, r, y);
                         const size_t plane = (size_t)g.dims[1] * g.dims[0];
-                        a.bev[((size_t)r * C + lane) * plane + (size_t)y * g.dims[0] + x] = mu;
+                        if (frame_in_call(r, a.frames)) a.bev[((size_t)r * C + lane) * plane + (size_t)y * g.dims[0] + x] = mu;
                     }
                 }
             }
@@ -680,6 +681,7 @@ int run_voxelize(emc2_bridge* h, int B, int N, const float* d_points, int32_t* c
     sa.status = h->d_status;
     sa.st = h->scan;
     aa.bev = d_bev;
+    aa.frames = (uint32_t)B;
     aa.num_voxels = d_num_voxels;
     aa.status = h->d_status;
 

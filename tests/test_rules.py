@@ -1,6 +1,7 @@
 """The index arithmetic of csrc/rules.cuh, compiled for the host (CPU)."""
 import ctypes
 import os
+import re
 import subprocess
 
 import numpy as np
@@ -95,3 +96,13 @@ def test_a_scale_with_more_voxels_than_points_is_not_ranked():
     guard = loop.index("if (!voxels_possible(sc ? all[1] : all[0], g.max_list)) continue;")
     for write in ("a.counts[sc][m] =", "g.cell_list[m] =", "at[0] =", "atomicAdd("):
         assert guard < loop.index(write), write
+
+
+def test_the_bev_image_is_written_for_frames_of_the_call_only():
+    """A pillar scan's tiles cover cells of frames past the call's last one: every write into the image tests the frame."""
+    text = open(os.path.join(CSRC, "voxelize.cu")).read()
+    code = text[text.index("vox_accum_kernel("):text.index("int run_voxelize")]
+    spots = [m.start() for m in re.finditer(r"a\.bev\[|dst = a\.bev \+", code)]
+    assert len(spots) == 2
+    for at in spots:
+        assert "frame_in_call(r, a.frames)" in code[at - 300:at]
