@@ -150,9 +150,8 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out) {
         for (int k = 0; k < 3; ++k) {
             d.mn[k] = g.min[k]; d.vs[k] = g.voxel[k]; d.dims[k] = g.dims[k];
             d.div[k] = make_fast_div((uint32_t)g.dims[k]);
-            const float inv = 1.0f / g.voxel[k];
-            d.inv[k] = std::isnormal(inv) ? inv : NAN;
-            d.margin[k] = 4e-7f * (float)(g.dims[k] + 2);
+            d.inv[k] = axis_inverse(g.voxel[k]);
+            d.margin[k] = axis_margin(g.dims[k]);
         }
         d.cap = g.max_points;
         d.design = 0;

@@ -100,7 +100,7 @@ struct ScaleDev {
     float mn[3];
     float vs[3];
     float inv[3];           // 1 / vs in fp32 (NaN where that is not a normal number) and how far from an integer
-    float margin[3];        // a product with it decides the cell without a divide, see cell_xyz
+    float margin[3];        // a product with it decides the cell without a divide, see cell_by_product
     int dims[3];            // Gx, Gy, Gz
     FastDiv div[3];         // division by Gx, Gy, Gz
     int cap;                // 0 = none
@@ -324,44 +324,6 @@ __device__ __forceinline__ void load_tile_f32(const float* __restrict__ src, int
     float4* d4 = reinterpret_cast<float4*>(smem);
     for (int i = threadIdx.x; i < nvec; i += blockDim.x) d4[i] = __ldg(s4 + i);
     for (int i = (nvec << 2) + threadIdx.x; i < nfloats; i += blockDim.x) smem[i] = __ldg(src + i);
-}
-
-// Cell index along one axis: one fp32 subtract, one IEEE fp32 divide, floor.  -1 if outside.
-__device__ __forceinline__ int axis_cell(float p, float mn, float vs, int dim) {
-    float q = __fdiv_rn(__fsub_rn(p, mn), vs);
-    float f = floorf(q);
-    // NaN fails both comparisons; +-inf fails one of them.
-    if (!(f >= 0.0f) || !(f < (float)dim)) return -1;
-    return (int)f;
-}
-
-// The same along all three axes; true if inside the grid.
-// A divide is a subroutine of some twenty instructions and every point needs six, in two kernels, so it is
-// only executed where it can matter.  q = d * RN(1 / vs) and RN(d / vs) differ by at most 3 * 2^-24 of their
-// value (one rounding each of the reciprocal, the product and the quotient): unless q lies within
-// `margin` = 4e-7 * (cells of the axis + 2) of an integer, both have the same floor, or both are outside.
-// Adding 1.5 * 2^23 leaves the nearest integer in the low bits of the sum (values too large for that come out
-// as no index of the axis, or exactly on an integer); zero, tiny and non-finite values fail the test of the
-// margin.
-__device__ __forceinline__ bool cell_xyz(const ScaleDev& g, float x, float y, float z, int& ix, int& iy, int& iz) {
-    constexpr float kMagic = 12582912.0f;
-    const float p[3] = {x, y, z};
-    int c[3];
-    bool sure = true;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const float q = __fmul_rn(__fsub_rn(p[k], g.mn[k]), g.inv[k]);
-        const float t = __fadd_rn(q, kMagic);
-        const float e = __fsub_rn(q, __fsub_rn(t, kMagic));       // q minus the nearest integer
-        sure &= fabsf(e) > g.margin[k];
-        c[k] = __float_as_int(t) - __float_as_int(kMagic) + (__float_as_int(e) >> 31);
-    }
-    if (!sure) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) c[k] = axis_cell(p[k], g.mn[k], g.vs[k], g.dims[k]);
-    }
-    ix = c[0]; iy = c[1]; iz = c[2];
-    return ((unsigned)ix < (unsigned)g.dims[0]) & ((unsigned)iy < (unsigned)g.dims[1]) & ((unsigned)iz < (unsigned)g.dims[2]);
 }
 
 // Cell id of a point inside the whole batch, or 0xFFFFFFFF if outside the grid.

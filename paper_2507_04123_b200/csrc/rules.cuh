@@ -2,7 +2,9 @@
 // exercise these lines and not a copy of them.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
+#include <cstring>
 
 #ifdef __CUDACC__
 #define EMC2_RULE __host__ __device__ __forceinline__
@@ -11,6 +13,78 @@
 #endif
 
 namespace emc2 {
+
+// ---- fp32 operations with one rounding each, never contracted (host: built without contraction)
+#ifdef __CUDA_ARCH__
+__device__ __forceinline__ float sub1(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float add1(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float mul1(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float div1(float a, float b) { return __fdiv_rn(a, b); }
+__device__ __forceinline__ uint32_t bits_of(float a) { return __float_as_uint(a); }
+#else
+inline float sub1(float a, float b) { return a - b; }
+inline float add1(float a, float b) { return a + b; }
+inline float mul1(float a, float b) { return a * b; }
+inline float div1(float a, float b) { return a / b; }
+inline uint32_t bits_of(float a) { uint32_t u; std::memcpy(&u, &a, sizeof u); return u; }
+#endif
+
+// ---- cell of a point
+// Cell index along one axis: one fp32 subtract, one IEEE fp32 divide, floor.  -1 if outside.
+EMC2_RULE int axis_cell(float p, float mn, float vs, int dim) {
+    const float f = floorf(div1(sub1(p, mn), vs));
+    // NaN fails both comparisons; +-inf fails one of them.
+    if (!(f >= 0.0f) || !(f < (float)dim)) return -1;
+    return (int)f;
+}
+
+// 1 / vs in fp32 (NaN where that is not a normal number) and how far from an integer a product with it decides the
+// cell without a divide, see cell_by_product.
+inline float axis_inverse(float vs) {
+    const float inv = 1.0f / vs;
+    return std::isnormal(inv) ? inv : NAN;
+}
+inline float axis_margin(int dim) { return 4e-7f * (float)(dim + 2); }
+
+// The cell along all three axes by a multiplication each; true where that provably decides it.  G has the arrays mn,
+// vs, inv, margin and dims of the axes.  A divide is a subroutine of some twenty instructions and every point needs six, in two kernels, so it is
+// only executed where it can matter.  q = d * RN(1 / vs) and RN(d / vs) differ by at most 3 * 2^-24 of their
+// value (one rounding each of the reciprocal, the product and the quotient): unless q lies within
+// `margin` = 4e-7 * (cells of the axis + 2) of an integer, both have the same floor, or both are outside.
+// Adding 1.5 * 2^23 leaves the nearest integer in the low bits of the sum (values too large for that come out
+// as no index of the axis, or exactly on an integer); zero, tiny and non-finite values fail the test of the
+// margin.  The bits are subtracted modulo 2^32: those of a negative sum come out as no index of the axis.
+template <class G>
+EMC2_RULE bool cell_by_product(const G& g, const float p[3], uint32_t c[3]) {
+    constexpr float kMagic = 12582912.0f;
+    bool sure = true;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int k = 0; k < 3; ++k) {
+        const float q = mul1(sub1(p[k], g.mn[k]), g.inv[k]);
+        const float t = add1(q, kMagic);
+        const float e = sub1(q, sub1(t, kMagic));                 // q minus the nearest integer
+        sure &= fabsf(e) > g.margin[k];
+        c[k] = bits_of(t) - bits_of(kMagic) - (bits_of(e) >> 31);
+    }
+    return sure;
+}
+
+// Cell of a point as by subtract, divide, floor; true if inside the grid.
+template <class G>
+EMC2_RULE bool cell_xyz(const G& g, float x, float y, float z, int& ix, int& iy, int& iz) {
+    const float p[3] = {x, y, z};
+    uint32_t c[3];
+    if (!cell_by_product(g, p, c)) {
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+        for (int k = 0; k < 3; ++k) c[k] = (uint32_t)axis_cell(p[k], g.mn[k], g.vs[k], g.dims[k]);
+    }
+    ix = (int)c[0]; iy = (int)c[1]; iz = (int)c[2];
+    return (c[0] < (uint32_t)g.dims[0]) & (c[1] < (uint32_t)g.dims[1]) & (c[2] < (uint32_t)g.dims[2]);
+}
 
 // ---- voxels found by the rank scan: at most one per point of a call, or the store was not all zero when it began
 EMC2_RULE bool voxels_possible(uint32_t voxels, uint32_t max_list) { return voxels <= max_list; }

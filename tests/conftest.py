@@ -1,4 +1,6 @@
+import ctypes
 import os
+import subprocess
 import sys
 
 import pytest
@@ -17,3 +19,19 @@ def oracle():
     import oracle as _oracle
     _oracle.build()
     return _oracle
+
+
+@pytest.fixture(scope="session")
+def rules(tmp_path_factory):
+    """The index arithmetic of csrc/rules.cuh compiled for the host; undefined behaviour ends the process."""
+    lib = str(tmp_path_factory.mktemp("rules") / "librules.so")
+    subprocess.run(["g++", "-std=c++17", "-O2", "-Wall", "-Werror", "-ffp-contract=off", "-fsanitize=undefined",
+                    "-fno-sanitize-recover=undefined", "-fPIC", "-shared",
+                    "-I", os.path.join(ROOT, "paper_2507_04123_b200", "csrc"),
+                    "-o", lib, os.path.join(ROOT, "tests", "rules_shim.cpp")], check=True)
+    so = ctypes.CDLL(lib)
+    u32, u64 = ctypes.c_uint32, ctypes.c_uint64
+    so.clamp.restype, so.clamp.argtypes = u32, [u32]
+    so.fits.restype, so.fits.argtypes = ctypes.c_int, [u64, u32, u32, u32, u32]
+    so.ticket.restype, so.ticket.argtypes = u64, [u32, u32]
+    return so

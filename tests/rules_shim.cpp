@@ -1,0 +1,38 @@
+// csrc/rules.cuh for the CPU tests: its functions behind a C interface.
+#include "rules.cuh"
+
+using namespace emc2;
+
+struct Axes {
+    float mn[3], vs[3], inv[3], margin[3];
+    int dims[3];
+};
+
+extern "C" {
+
+uint32_t clamp(uint32_t n) { return clamp_points(n); }
+int fits(uint64_t first, uint32_t cells, uint32_t points, uint32_t max_ovf, uint32_t max_list) {
+    return over_fits(first, cells, points, max_ovf, max_list);
+}
+uint64_t ticket(uint32_t cells, uint32_t points) { return over_ticket(cells, points); }
+
+// Cells of n points (x, y, z), -1 -1 -1 outside the grid; returns for how many of them no divide was needed.
+int cells(const float* pts, int n, const float* mn, const float* vs, const int* dims, int* out) {
+    Axes g;
+    for (int k = 0; k < 3; ++k) {
+        g.mn[k] = mn[k]; g.vs[k] = vs[k]; g.dims[k] = dims[k];
+        g.inv[k] = axis_inverse(vs[k]);
+        g.margin[k] = axis_margin(dims[k]);
+    }
+    int sure = 0;
+    for (int i = 0; i < n; ++i) {
+        int c[3];
+        uint32_t by_product[3];
+        const bool in = cell_xyz(g, pts[3 * i], pts[3 * i + 1], pts[3 * i + 2], c[0], c[1], c[2]);
+        for (int k = 0; k < 3; ++k) out[3 * i + k] = in ? c[k] : -1;
+        sure += cell_by_product(g, pts + 3 * i, by_product);
+    }
+    return sure;
+}
+
+}  // extern "C"

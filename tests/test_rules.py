@@ -1,41 +1,10 @@
 """The index arithmetic of csrc/rules.cuh, compiled for the host (CPU)."""
-import ctypes
 import os
 import re
-import subprocess
 
 import numpy as np
-import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2507_04123_b200", "csrc")
-
-SHIM = r"""
-#include "rules.cuh"
-using namespace emc2;
-extern "C" {
-uint32_t clamp(uint32_t n) { return clamp_points(n); }
-int fits(uint64_t first, uint32_t cells, uint32_t points, uint32_t max_ovf, uint32_t max_list) {
-    return over_fits(first, cells, points, max_ovf, max_list);
-}
-uint64_t ticket(uint32_t cells, uint32_t points) { return over_ticket(cells, points); }
-}
-"""
-
-
-@pytest.fixture(scope="module")
-def rules(tmp_path_factory):
-    d = tmp_path_factory.mktemp("rules")
-    src, lib = str(d / "shim.cpp"), str(d / "librules.so")
-    with open(src, "w") as f:
-        f.write(SHIM)
-    subprocess.run(["g++", "-std=c++17", "-O2", "-Wall", "-Werror", "-ffp-contract=off", "-fsanitize=undefined",
-                    "-fno-sanitize-recover=undefined", "-fPIC", "-shared", "-I", CSRC, "-o", lib, src], check=True)
-    so = ctypes.CDLL(lib)
-    u32, u64 = ctypes.c_uint32, ctypes.c_uint64
-    so.clamp.restype, so.clamp.argtypes = u32, [u32]
-    so.fits.restype, so.fits.argtypes = ctypes.c_int, [u64, u32, u32, u32, u32]
-    so.ticket.restype, so.ticket.argtypes = u64, [u32, u32]
-    return so
 
 
 def test_point_sums_of_a_tile_never_wrap_and_never_pass_for_small_ones(rules):
