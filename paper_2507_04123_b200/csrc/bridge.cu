@@ -371,7 +371,7 @@ static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_poi
             rc2 = launch_project_route(h, 0, B, N, d_points, d_proj, d_uvd, d_vis_mask, d_cam, d_expert, false, nullptr, 0, st);
         const int tiles = (N + kTile - 1) / kTile;
         if (rc2 == EMC2_OK) {
-            launch_route_scan(h, 0, half0, tiles, N, d_offsets, st);
+            launch_route_scan(h, 0, half0, tiles, N, d_offsets, N > 0, st);
             if (h_feat) {
                 const emc2_config_t& c = h->cfg;
                 const size_t bytes = (size_t)B * c.num_cameras * c.feat_h * c.feat_w * c.feat_c * sizeof(float);
@@ -381,14 +381,14 @@ static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_poi
         }
         if (rc2 == EMC2_OK)
             rc2 = launch_gather_scatter(h, 0, half0, N, d_points, d_feat, d_uvd, d_cam, d_gathered, d_expert, d_perm,
-                                        d_points_out, d_feat_out, st);
+                                        d_points_out, d_feat_out, !h_feat, st);
         if (rc2 == EMC2_OK && half0 < B) {
             e = cudaStreamWaitEvent(st, h->ev_half, 0);
             if (e != cudaSuccess) rc2 = check_cuda(h, e);
             else {
-                launch_route_scan(h, half0, B - half0, tiles, N, d_offsets + (size_t)half0 * (h->cfg.num_experts + 1), st);
+                launch_route_scan(h, half0, B - half0, tiles, N, d_offsets + (size_t)half0 * (h->cfg.num_experts + 1), false, st);
                 rc2 = launch_gather_scatter(h, half0, B - half0, N, d_points, d_feat, d_uvd, d_cam, d_gathered, d_expert,
-                                            d_perm, d_points_out, d_feat_out, st);
+                                            d_perm, d_points_out, d_feat_out, true, st);
             }
         }
     }

@@ -248,8 +248,10 @@ int launch_route_dispatch(emc2_bridge* h, int B, int N, const float* d_points, c
 // of the wait.  The call's own inputs are complete before the first kernel of a call, which is launched plainly.
 // Released earlier, the successor's CTAs would hold places on the SMs that the kernels of the other stream need.
 // us per call: one small frame 35 -> 30, stage calls with occlusion 155 -> 140, voxels and rulebooks 261 -> 239 (B200).
+// `chained` false: an ordinary launch, for a kernel that follows a copy or an event wait, or that can be the first of
+// its call.
 template <typename... P, typename... A>
-inline void launch_chained(void (*kernel)(P...), dim3 grid, unsigned threads, size_t shared, cudaStream_t st, const A&... args) {
+inline void launch_kernel(bool chained, void (*kernel)(P...), dim3 grid, unsigned threads, size_t shared, cudaStream_t st, const A&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
@@ -259,8 +261,13 @@ inline void launch_chained(void (*kernel)(P...), dim3 grid, unsigned threads, si
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = chained ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
+template <typename... P, typename... A>
+inline void launch_chained(void (*kernel)(P...), dim3 grid, unsigned threads, size_t shared, cudaStream_t st, const A&... args) {
+    launch_kernel(true, kernel, grid, threads, shared, st, args...);
 }
 #endif
 
@@ -297,7 +304,8 @@ int launch_pool_features(emc2_bridge* h, int B, int p, const float* d_feat, floa
 int launch_scene_route(emc2_bridge* h, int B, const int32_t* d_offsets, const uint8_t* priority, int min_points,
                        int32_t* d_scene_expert, cudaStream_t st);
 // Tile histograms (handle scratch) of frames [b0, b0 + B) -> d_offsets (of frame b0 on) and tile bases.
-void launch_route_scan(emc2_bridge* h, int b0, int B, int tiles, int N, int32_t* d_offsets, cudaStream_t st);
+// `chained` (here and below): the call's previous work on `st` is one kernel, see launch_chained.
+void launch_route_scan(emc2_bridge* h, int b0, int B, int tiles, int N, int32_t* d_offsets, bool chained, cudaStream_t st);
 // Stages 2 - 4 in one pass over the feature rows (the one-call path), in two parts: projection +
 // routing per point (which, with `d_bev_to_zero`/`mark`, also marks the voxel cells of both scales
 // and zeroes the BEV image, so that stage 1 reads the points once less), then, after launch_route_scan, the rows.
@@ -306,7 +314,7 @@ int launch_project_route(emc2_bridge* h, int b0, int B, int N, const float* d_po
                          float* d_bev_to_zero, int bev_frames, cudaStream_t st);
 int launch_gather_scatter(emc2_bridge* h, int b0, int B, int N, const float* d_points, const float* d_feat,
                           const float* d_uvd, const int8_t* d_cam, float* d_gathered, const uint8_t* d_expert,
-                          int32_t* d_perm, float* d_points_out, float* d_feat_out, cudaStream_t st);
+                          int32_t* d_perm, float* d_points_out, float* d_feat_out, bool chained, cudaStream_t st);
 
 // ---------------------------------------------------------------- device helpers
 #ifdef __CUDACC__

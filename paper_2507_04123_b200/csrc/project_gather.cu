@@ -580,24 +580,24 @@ __global__ void __launch_bounds__(32 * CF8) gather_scatter_wide_kernel(const __g
 
 
 template <int C>
-void launch_gs(emc2_bridge* h, const GsArgs& a, dim3 grid, cudaStream_t st) {
+void launch_gs(emc2_bridge* h, const GsArgs& a, dim3 grid, bool chained, cudaStream_t st) {
     LaunchScope ls(h, K_GATHER_SCATTER, st);
     const int mode = h->tune[EMC2_TUNE_ROW_STORE];
     if (mode == 1 && a.E < 31) {
-        if (a.cf4 == 16) { launch_chained(gather_scatter_bulk_kernel<C, 16, true>, grid, 16 * 16, 0, st, a); return; }
-        if (a.cf4 == 20) { launch_chained(gather_scatter_bulk_kernel<C, 20, true>, grid, 16 * 20, 0, st, a); return; }
+        if (a.cf4 == 16) { launch_kernel(chained, gather_scatter_bulk_kernel<C, 16, true>, grid, 16 * 16, 0, st, a); return; }
+        if (a.cf4 == 20) { launch_kernel(chained, gather_scatter_bulk_kernel<C, 20, true>, grid, 16 * 20, 0, st, a); return; }
     } else if (mode == 3 && ((reinterpret_cast<uintptr_t>(a.feat) | reinterpret_cast<uintptr_t>(a.gathered) |
                               reinterpret_cast<uintptr_t>(a.feat_out)) & 31) == 0) {
-        if (a.cf4 == 16) { launch_chained(gather_scatter_wide_kernel<C, 8>, grid, 32 * 8, 0, st, a); return; }
-        if (a.cf4 == 20) { launch_chained(gather_scatter_wide_kernel<C, 10>, grid, 32 * 10, 0, st, a); return; }
+        if (a.cf4 == 16) { launch_kernel(chained, gather_scatter_wide_kernel<C, 8>, grid, 32 * 8, 0, st, a); return; }
+        if (a.cf4 == 20) { launch_kernel(chained, gather_scatter_wide_kernel<C, 10>, grid, 32 * 10, 0, st, a); return; }
     } else if (mode == 2) {
-        if (a.cf4 == 16) { launch_chained(gather_scatter_bulk_kernel<C, 16, false>, grid, 16 * 16, 0, st, a); return; }
-        if (a.cf4 == 20) { launch_chained(gather_scatter_bulk_kernel<C, 20, false>, grid, 16 * 20, 0, st, a); return; }
+        if (a.cf4 == 16) { launch_kernel(chained, gather_scatter_bulk_kernel<C, 16, false>, grid, 16 * 16, 0, st, a); return; }
+        if (a.cf4 == 20) { launch_kernel(chained, gather_scatter_bulk_kernel<C, 20, false>, grid, 16 * 20, 0, st, a); return; }
     }
     switch (a.cf4) {
-        case 16: launch_chained(gather_scatter_kernel<C, 16>, grid, kGsRows<16> * 16, 0, st, a); break;
-        case 20: launch_chained(gather_scatter_kernel<C, 20>, grid, kGsRows<20> * 20, 0, st, a); break;
-        default: launch_chained(gather_scatter_kernel<C, 0>, grid, row_threads(a.cf4), 0, st, a); break;
+        case 16: launch_kernel(chained, gather_scatter_kernel<C, 16>, grid, kGsRows<16> * 16, 0, st, a); break;
+        case 20: launch_kernel(chained, gather_scatter_kernel<C, 20>, grid, kGsRows<20> * 20, 0, st, a); break;
+        default: launch_kernel(chained, gather_scatter_kernel<C, 0>, grid, row_threads(a.cf4), 0, st, a); break;
     }
 }
 
@@ -772,7 +772,7 @@ int launch_project_route(emc2_bridge* h, int b0, int B, int N, const float* d_po
 
 int launch_gather_scatter(emc2_bridge* h, int b0, int B, int N, const float* d_points, const float* d_feat,
                           const float* d_uvd, const int8_t* d_cam, float* d_gathered, const uint8_t* d_expert,
-                          int32_t* d_perm, float* d_points_out, float* d_feat_out, cudaStream_t st) {
+                          int32_t* d_perm, float* d_points_out, float* d_feat_out, bool chained, cudaStream_t st) {
     const emc2_config_t& c = h->cfg;
     if (B == 0) return EMC2_OK;
     const int tiles = (N + kTile - 1) / kTile;
@@ -791,7 +791,7 @@ int launch_gather_scatter(emc2_bridge* h, int b0, int B, int N, const float* d_p
         ga.cf4 = c.feat_c / 4;
         ga.inv_stride = 1.0f / (float)c.feat_stride;
         ga.offset = c.feat_offset;
-        if (c.point_floats == 4) launch_gs<4>(h, ga, grid, st); else launch_gs<5>(h, ga, grid, st);
+        if (c.point_floats == 4) launch_gs<4>(h, ga, grid, chained, st); else launch_gs<5>(h, ga, grid, chained, st);
     }
     return check_cuda(h, cudaGetLastError());
 }

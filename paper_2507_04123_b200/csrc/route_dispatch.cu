@@ -267,11 +267,11 @@ int launch_scene_route(emc2_bridge* h, int B, const int32_t* d_offsets, const ui
     return check_cuda(h, cudaGetLastError());
 }
 
-void launch_route_scan(emc2_bridge* h, int b0, int B, int tiles, int N, int32_t* d_offsets, cudaStream_t st) {
+void launch_route_scan(emc2_bridge* h, int b0, int B, int tiles, int N, int32_t* d_offsets, bool chained, cudaStream_t st) {
     LaunchScope ls(h, K_ROUTE_SCAN, st);
     const size_t t0 = (size_t)b0 * tiles * h->cfg.num_experts;
-    launch_chained(route_scan_kernel, B, kScanThreads, 0, st, h->d_tile_counts + t0, h->d_tile_base + t0, d_offsets, tiles,
-                                                  h->cfg.num_experts, N);
+    launch_kernel(chained, route_scan_kernel, B, kScanThreads, 0, st, h->d_tile_counts + t0, h->d_tile_base + t0, d_offsets, tiles,
+                  h->cfg.num_experts, N);
 }
 
 int launch_route_dispatch(emc2_bridge* h, int B, int N, const float* d_points, const uint8_t* d_vis_mask,
@@ -293,7 +293,7 @@ int launch_route_dispatch(emc2_bridge* h, int B, int N, const float* d_points, c
     }
     {
         LaunchScope ls(h, K_ROUTE_SCAN, st);
-        launch_chained(route_scan_kernel, B, kScanThreads, 0, st, h->d_tile_counts, h->d_tile_base, d_offsets, tiles, E, N);
+        launch_kernel(tiles > 0, route_scan_kernel, B, kScanThreads, 0, st, h->d_tile_counts, h->d_tile_base, d_offsets, tiles, E, N);
     }
     if (tiles > 0) {
         ScatterArgs sa;
@@ -398,7 +398,7 @@ extern "C" int emc2_route_dispatch_static(const emc2_config_t* config, int32_t B
             for (int k = 0; k < 16; ++k) ra.lut[k] = c.lut[k >> 3][k & 7];
             if (c.point_floats == 4) launch_hist<4>(ra, B, st); else launch_hist<5>(ra, B, st);
         }
-        launch_chained(route_scan_kernel, B, kScanThreads, 0, st, tile_counts, tile_base, d_offsets, tiles, E, N);
+        launch_kernel(tiles > 0, route_scan_kernel, B, kScanThreads, 0, st, tile_counts, tile_base, d_offsets, tiles, E, N);
         if (tiles > 0) {
             ScatterArgs sa;
             sa.pts = d_points; sa.feat = reinterpret_cast<const float4*>(d_gathered); sa.expert = d_expert;

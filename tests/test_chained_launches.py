@@ -11,9 +11,9 @@ def sources():
 
 
 def chained_kernels():
-    """{kernel: (parameters, body)} of every kernel that is launched through launch_chained."""
+    """{kernel: (parameters, body)} of every kernel that can be launched through launch_chained."""
     text = "\n".join(sources().values())
-    names = set(re.findall(r"launch_chained\(\s*(\w+_kernel)\b", text))
+    names = set(re.findall(r"launch_(?:chained\(|kernel\([^,()]*,)\s*(\w+_kernel)\b", text))
     found = {}
     for name in names:
         m = re.search(r"__global__[^;{]*?\b" + name + r"\s*\(([^)]*)\)\s*\{(.*?)\n\}", text, re.S)

@@ -1,0 +1,138 @@
+"""Calls captured into CUDA graphs: which launches are chained to their predecessor, and replays on new frames (needs a B200)."""
+from dataclasses import replace
+
+import numpy as np
+import pytest
+import torch
+
+import emc2_gen as gen
+from parity import compare_bridge, to_dev
+
+pytestmark = pytest.mark.gpu
+rt = pytest.importorskip("cuda.bindings.runtime")
+
+
+def bridge_for(w, **kw):
+    import paper_2507_04123_b200 as pkg
+    return pkg.Bridge(pkg.config_from_workload(w, **kw))
+
+
+def captured(call):
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    return graph
+
+
+def chained_launches(graph):
+    """Checks that every chained launch follows exactly one node, a kernel; returns how many there are."""
+    def ok(res):
+        assert res[0] == rt.cudaError_t.cudaSuccess, res[0]
+        return res[1:]
+
+    g = rt.cudaGraph_t(init_value=graph.raw_cuda_graph())
+    n = ok(rt.cudaGraphGetEdges_v2(g))[-1]
+    tails, heads, data, n = ok(rt.cudaGraphGetEdges_v2(g, n))
+    kernel = rt.cudaGraphNodeType.cudaGraphNodeTypeKernel
+    before = {}
+    for a, b in zip(tails, heads):
+        before.setdefault(int(b), []).append(a)
+    found = 0
+    for a, b, d in zip(tails, heads, data):
+        if int(d.type) == int(rt.cudaGraphDependencyType.cudaGraphDependencyTypeProgrammatic):
+            found += 1
+            assert ok(rt.cudaGraphNodeGetType(a))[0] == kernel and ok(rt.cudaGraphNodeGetType(b))[0] == kernel
+            assert len(before[int(b)]) == 1
+    return found
+
+
+def test_host_frame_replays_from_a_graph(oracle):
+    """The row pass follows the copy of the feature maps there; page-locked buffers, refilled before each replay."""
+    w = gen.KITTI.with_shape(2, 20001)
+    frames = [gen.make_batch(w, frames=[2 * i, 2 * i + 1]) for i in range(2)]
+    br = bridge_for(w)
+    host = {k: torch.from_numpy(v.copy()).pin_memory() for k, v in frames[0].items()}
+    staging = {k: torch.zeros_like(v, device="cuda") for k, v in host.items()}
+    d = to_dev(frames[0])
+    bufs = br.run(d["points"], d["proj"], d["feat"])
+    h_off = torch.zeros((w.B, w.num_experts + 1), dtype=torch.int32).pin_memory()
+    h_nv = torch.zeros((2,), dtype=torch.int32).pin_memory()
+    torch.cuda.synchronize()
+    graph = captured(lambda: br.run_host(host, staging, bufs, h_off, h_nv))
+    assert chained_launches(graph) >= 3
+    for batch in (frames[1], frames[0]):
+        for k, v in batch.items():
+            host[k].copy_(torch.from_numpy(v))
+            staging[k].fill_(float("nan"))
+        bufs["rd"]["feat_out"].fill_(-1.0)
+        graph.replay()
+        torch.cuda.synchronize()
+        br.status()
+        ref = oracle.bridge(w, batch)
+        compare_bridge(w, ref, bufs)
+        assert np.array_equal(h_off.numpy(), ref["offsets"])
+        assert h_nv.tolist() == [ref["vox0"]["num_voxels"], ref["vox1"]["num_voxels"]]
+    del graph
+    br.close()
+
+
+@pytest.mark.parametrize("B", [2, 3])
+@pytest.mark.parametrize("tuning", [{}, {"split_batch": 1}, {"mark_in_projection": 0}, {"dedup_pillars": 1},
+                                    {"dedup_fine": 2, "dedup_pillars": 2}])
+def test_one_call_replays_from_a_graph_under_every_tuning(oracle, tuning, B):
+    """split_batch: the second half's route scan follows a wait for the other stream."""
+    w = gen.NUSCENES.with_shape(B, 7001)
+    w = replace(w, img_h=180, img_w=320)
+    frames = [gen.make_batch(w, frames=list(range(B * i, B * i + B))) for i in range(2)]
+    for overlap in (True, False):
+        br = bridge_for(w)
+        br.set_overlap(overlap)
+        for knob, value in tuning.items():
+            br.set_tuning(knob, value)
+        d = to_dev(frames[0])
+        bufs = br.run(d["points"], d["proj"], d["feat"])
+        torch.cuda.synchronize()
+        graph = captured(lambda: br.run(d["points"], d["proj"], d["feat"], bufs))
+        assert chained_launches(graph) >= 3
+        for batch in (frames[1], frames[0]):
+            for k, v in batch.items():
+                d[k].copy_(torch.from_numpy(v))
+            bufs["rd"]["feat_out"].fill_(-1.0)
+            bufs["vox"]["num_voxels"].fill_(-1)
+            graph.replay()
+            torch.cuda.synchronize()
+            br.status()
+            compare_bridge(w, oracle.bridge(w, batch), bufs)
+        del graph
+        br.close()
+
+
+def test_stage_calls_and_calls_without_points_in_a_graph():
+    """With N = 0 the route scan is the first kernel of its call: nothing is chained to what the stream held before."""
+    w = gen.KITTI.with_shape(2, 1000)
+    br = bridge_for(w)
+    d = to_dev(gen.make_batch(w))
+    bufs = br.run_staged(d["points"], d["proj"], d["feat"])
+    torch.cuda.synchronize()
+    graph = captured(lambda: br.run_staged(d["points"], d["proj"], d["feat"], bufs))
+    assert chained_launches(graph) >= 4
+    del graph
+    none = br.run(d["points"][:, :0].contiguous(), d["proj"], d["feat"])
+    rd = none["rd"]
+    torch.cuda.synchronize()
+    for call in (lambda: br.run(d["points"][:, :0].contiguous(), d["proj"], d["feat"], none),
+                 lambda: br.route_dispatch(d["points"][:, :0].contiguous(), none["pg"]["vis_mask"], none["pg"]["gathered"], out=rd)):
+        rd["offsets"].fill_(-1)
+        torch.cuda.synchronize()
+
+        def kernel_first():
+            bufs["pg"]["uvd"].fill_(0.0)                    # a kernel of the caller's right before the call
+            call()
+
+        graph = captured(kernel_first)
+        assert chained_launches(graph) == 0
+        graph.replay()
+        torch.cuda.synchronize()
+        assert not rd["offsets"].any()
+        del graph
+    br.close()
