@@ -125,22 +125,25 @@ __device__ __forceinline__ Projected project_point(const Camera* cam, int K, flo
     return r;
 }
 
-// Copies the K 3x4 matrices of frame b into shared memory.
-__device__ __forceinline__ void load_cameras(const float* __restrict__ proj, int b, int K, Camera* cam) {
+// Copies the 3x4 matrices of `frames` frames of K cameras, from frame b on, into shared memory.
+__device__ __forceinline__ void load_cameras(const float* __restrict__ proj, int b, int frames, int K, Camera* cam) {
     const float* src = proj + (size_t)b * K * 12;
-    for (int i = threadIdx.x; i < K * 12; i += blockDim.x) {
+    for (int i = threadIdx.x; i < frames * K * 12; i += blockDim.x) {
         const int k = i / 12, r = (i % 12) / 4, c = i % 4;
         reinterpret_cast<float*>(cam + k)[r < 2 ? 2 * c + r : 8 + c] = __ldg(src + i);
     }
 }
 
 // CF4 > 0: Cf/4 known at compile time, blockDim.x == 16 * CF4; else blockDim.x == row_threads(cf4).
-template <int C, int CF4>
+// kFrames: most frames that the points of a tile belong to, see frames_of_tile: two but for frames of fewer than 255
+// points, whose cameras are all staged at once (32 frames of 8 points through 6 cameras: 31 us with the cameras of two
+// frames at a time in turn, 10.3 with every point reading its own from global memory, 9.8 this way).
+template <int C, int CF4, int kFrames = 2>
 __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kMaxRowThreads) project_gather_kernel(PgArgs a) {
     __shared__ __align__(16) float sp[kTile * C];
     __shared__ float suvd[kTile * 3];
     __shared__ uint4 srow[kTile];          // {tap (y0,x0) as a float4 index, clamp flags, wx, wy}
-    __shared__ Camera sP[2][EMC2_MAX_CAMERAS];       // cameras of (at most two, if N >= 256) frames of the tile
+    __shared__ Camera sP[kFrames * EMC2_MAX_CAMERAS];      // cameras of the tile's frames
 
     const long long g0 = (long long)blockIdx.x * kTile;
     const int npts = (int)min((long long)kTile, a.total - g0);
@@ -149,24 +152,18 @@ __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kMaxRowThreads) project_g
     const int nframes = (int)((g0 + npts - 1) / a.N) - bfirst + 1;
     const int t = threadIdx.x;
     const int cf4 = CF4 > 0 ? CF4 : a.cf4;
-    // Tiny frames (N < 256) can put more than two frames in a tile: two at a time then.
-    for (int f = 0; f < nframes; f += 2) {
-    if (f) __syncthreads();
-    load_cameras(a.proj, bfirst + f, a.K, sP[0]);
-    if (f + 1 < nframes) load_cameras(a.proj, bfirst + f + 1, a.K, sP[1]);
+    load_cameras(a.proj, bfirst, nframes, a.K, sP);
     __syncthreads();
-    const int frame = t < npts ? (int)((g0 + t) / a.N) - bfirst - f : -1;
-    if (frame == 0 || frame == 1) {
+    if (t < npts) {
         const float x = sp[t * C], y = sp[t * C + 1], z = sp[t * C + 2];
         const long long gi = g0 + t;
-        const int b = bfirst + f + frame;
-        const Projected pr = project_point(sP[frame], a.K, x, y, z, a.W, a.H, a.min_depth);
+        const int b = (int)(gi / a.N);
+        const Projected pr = project_point(sP + (b - bfirst) * a.K, a.K, x, y, z, a.W, a.H, a.min_depth);
         suvd[t * 3] = pr.u; suvd[t * 3 + 1] = pr.v; suvd[t * 3 + 2] = pr.d;
         a.vis[gi] = (uint8_t)pr.mask;
         a.cam[gi] = (int8_t)pr.best;
         const uint4 rec = tap_record(b, pr.best, pr.u, pr.v, a.K, a.Hf, a.Wf, cf4, a.inv_stride, a.offset);
         srow[t] = rec;
-    }
     }
     __syncthreads();
 
@@ -226,7 +223,7 @@ __global__ void __launch_bounds__(kThreads) project_route_kernel(const __grid_co
     __shared__ int hist[EMC2_MAX_EXPERTS];
     __shared__ Camera sP[EMC2_MAX_CAMERAS];
     const int b = blockIdx.y, tile = blockIdx.x, t = threadIdx.x, lane = t & 31;
-    load_cameras(a.proj, b, a.K, sP);
+    load_cameras(a.proj, b, 1, a.K, sP);
     const int i0 = tile * kTile;
     const int npts = min(kTile, a.N - i0);
     const size_t g0 = (size_t)b * a.N + i0;
@@ -698,6 +695,10 @@ pool_features_kernel(const float4* __restrict__ feat, float4* __restrict__ poole
 template <int C>
 void launch_c(emc2_bridge* h, const PgArgs& a, int tiles, cudaStream_t st) {
     LaunchScope ls(h, K_PROJECT_GATHER, st);
+    if (frames_of_tile(a.total / a.N, a.N) > 2) {
+        project_gather_kernel<C, 0, EMC2_MAX_BATCH><<<tiles, row_threads(a.cf4), 0, st>>>(a);
+        return;
+    }
     switch (a.cf4) {
         case 16: project_gather_kernel<C, 16><<<tiles, 16 * 16, 0, st>>>(a); break;
         case 20: project_gather_kernel<C, 20><<<tiles, 16 * 20, 0, st>>>(a); break;

@@ -86,6 +86,12 @@ EMC2_RULE bool cell_xyz(const G& g, float x, float y, float z, int& ix, int& iy,
     return (c[0] < (uint32_t)g.dims[0]) & (c[1] < (uint32_t)g.dims[1]) & (c[2] < (uint32_t)g.dims[2]);
 }
 
+// ---- frames that kTile = 256 consecutive points of a batch of B frames of N can belong to, at most
+inline long long frames_of_tile(long long B, long long N) {
+    const long long most = (256 - 2) / N + 2;      // a last point of one frame, then whole frames
+    return B < most ? B : most;
+}
+
 // ---- voxels found by the rank scan: at most one per point of a call, or the store was not all zero when it began
 EMC2_RULE bool voxels_possible(uint32_t voxels, uint32_t max_list) { return voxels <= max_list; }
 

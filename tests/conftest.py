@@ -34,4 +34,5 @@ def rules(tmp_path_factory):
     so.clamp.restype, so.clamp.argtypes = u32, [u32]
     so.fits.restype, so.fits.argtypes = ctypes.c_int, [u64, u32, u32, u32, u32]
     so.ticket.restype, so.ticket.argtypes = u64, [u32, u32]
+    so.tile_frames.restype, so.tile_frames.argtypes = ctypes.c_int64, [ctypes.c_int64, ctypes.c_int64]
     return so

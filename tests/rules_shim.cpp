@@ -14,6 +14,7 @@ uint32_t clamp(uint32_t n) { return clamp_points(n); }
 int fits(uint64_t first, uint32_t cells, uint32_t points, uint32_t max_ovf, uint32_t max_list) {
     return over_fits(first, cells, points, max_ovf, max_list);
 }
+int64_t tile_frames(int64_t B, int64_t N) { return frames_of_tile(B, N); }
 uint64_t ticket(uint32_t cells, uint32_t points) { return over_ticket(cells, points); }
 
 // Cells of n points (x, y, z), -1 -1 -1 outside the grid; returns for how many of them no divide was needed.

@@ -111,7 +111,7 @@ def test_cells_of_points_on_cell_boundaries(oracle, dims):
         br.close()
 
 
-@pytest.mark.parametrize("B,N", [(1, 1), (7, 33), (3, 255), (2, 1031)])
+@pytest.mark.parametrize("B,N", [(1, 1), (7, 33), (3, 255), (2, 1031), (32, 1), (32, 9), (5, 254)])
 def test_points_on_image_edges(oracle, B, N):
     """Pixels within a few ulps to a few hundredths of the image edges, at every depth: mask, camera and pixel as defined."""
     rng = np.random.default_rng(7)

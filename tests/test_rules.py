@@ -75,3 +75,16 @@ def test_the_bev_image_is_written_for_frames_of_the_call_only():
     assert len(spots) == 2
     for at in spots:
         assert "frame_in_call(r, a.frames)" in code[at - 300:at]
+
+
+def test_frames_of_a_tile(rules):
+    """256 consecutive points from any multiple of 256 on lie in no more frames than the rule says, and the rule is met."""
+    for N in list(range(1, 300)) + [511, 512, 513, 1000]:
+        for B in (1, 2, 3, 4, 7, 31, 32):
+            total = B * N
+            spans = [(min(g + 255, total - 1) // N) - g // N + 1 for g in range(0, total, 256)]
+            most = rules.tile_frames(B, N)
+            assert max(spans) <= most <= B
+            if most > 2:
+                assert N < 255
+    assert rules.tile_frames(32, 1) == 32 and rules.tile_frames(32, 255) == 2 and rules.tile_frames(32, 254) == 3
