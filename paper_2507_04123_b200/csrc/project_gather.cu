@@ -600,53 +600,73 @@ void launch_gs(emc2_bridge* h, const GsArgs& a, dim3 grid, bool chained, cudaStr
 
 // ------------------------------------------------------------------ planar -> channels-last
 // Per map the planar data is a Cf x P matrix (P = Hf * Wf pixels) and the channels-last data its
-// transpose.  A CTA moves `chan` channels x 64 pixels through shared memory; with up to 128 channels that is all
-// of them, so what it writes is one contiguous block.
-//   in   one warp per channel row, 32 consecutive pixels (128 B) per instruction; a thread requests ten of its
-//        words before it waits for any;
+// transpose.  A CTA moves `chan` channels x kPix pixels through shared memory.
+//   in   one warp per channel row, 32 consecutive pixels (128 B) per instruction; a thread requests ten or twelve of
+//        its words before it waits for any;
 //   out  a warp instruction covers 8 pixels x 16 channels, 64 contiguous bytes of a pixel's row per four lanes.
-//        With a row stride of 66 words the column reads from the tile (bank = 2 * channel + pixel mod 32) are
+//        With a row stride of kPix + 2 words the column reads from the tile (bank = 2 * channel + pixel mod 32) are
 //        conflict-free.
-// Bound by the memory system (each byte is read and written once).  A tile of 64 channels x 128 pixels, which gives
-// 80 channels a second CTA for 16 of them, took 82 us for 24 maps of 80 x 113 x 200 (174 MB); this takes 63.
-constexpr int kClPix = 64, kClStride = kClPix + 2, kClMaxChan = 128, kClBatch = 10;
+// Bound by the memory system (each byte is read and written once).  The tile, measured on 12 maps of 113 x 200
+// texels (us per call; 64 x 128 pixels, ragged at the last channels, is what every width took once):
+//   channels                          8      32     48     64     80     96    128    192    256    512
+//   64 x 128 pixels, ragged         10.3   14.5   19.1   27.4   41.5   49.7   57.9   88.4    111    220
+//   all (at most 128) x 64 pixels   12.8   15.4   21.7   27.1   33.3   46.5   62.0   90.7    119    234
+//   64 x 64 pixels                  12.8   14.8   21.2   27.2   37.4   49.8   51.7   76.3   98.8    194
+//   all (at most 64) x 128 pixels    9.0   14.8   18.9   29.6   35.9   53.6   57.9   90.6    119    236
+// So: 128 pixels up to 48 channels, where a tile of 64 is too little work for a CTA; chunks of 64 channels where they
+// divide the width, whole sectors of the rows in small tiles; else as few CTAs per row as 128 channels allow, so that
+// no CTA is left with a few channels.
+constexpr int kClMaxChan = 128;
+template <int kPix> constexpr int kClStride = kPix + 2;
 
+struct ClTile {
+    int pix, chan;
+};
+
+inline ClTile channels_last_tile(int Cf) {
+    if (Cf <= 48) return {128, Cf};
+    if (Cf % 64 == 0) return {64, 64};
+    const int ctas = (Cf + kClMaxChan - 1) / kClMaxChan;
+    return {64, ((Cf + ctas - 1) / ctas + 3) / 4 * 4};
+}
+
+template <int kPix>
 __global__ void __launch_bounds__(256)
 channels_last_kernel(const float* __restrict__ planar, float* __restrict__ last, int Cf, int P, int ptiles, int chan) {
-    extern __shared__ float tile[];                         // [chan][kClStride]
+    constexpr int kStride = kClStride<kPix>, kParts = kPix / 32, kBatch = kParts == 2 ? 10 : 12;
+    extern __shared__ float tile[];                         // [chan][kStride]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t m = blockIdx.x / ptiles;
-    const int p0 = (int)(blockIdx.x - m * ptiles) * kClPix;
+    const int p0 = (int)(blockIdx.x - m * ptiles) * kPix;
     const int c0 = blockIdx.y * chan;
     const int nc = min(chan, Cf - c0);
     const float* src = planar + (m * Cf + c0) * (size_t)P + p0;
-    // Item i of a warp: half (i & 1) of channel row warp + 8 * (i >> 1).
-    const bool in[2] = {p0 + lane < P, p0 + 32 + lane < P};
-    const int items = 2 * ((nc - warp + 7) / 8);
-    for (int i0 = 0; i0 < items; i0 += kClBatch) {
-        float v[kClBatch];
+    // Item i of a warp: part i % kParts of channel row warp + 8 * (i / kParts).
+    const int items = kParts * ((nc - warp + 7) / 8);
+    for (int i0 = 0; i0 < items; i0 += kBatch) {
+        float v[kBatch];
 #pragma unroll
-        for (int u = 0; u < kClBatch; ++u) {
-            const int c = warp + 8 * ((i0 + u) >> 1), half = u & 1;
-            v[u] = c < nc && in[half] ? __ldcs(src + (size_t)c * P + 32 * half + lane) : 0.f;
+        for (int u = 0; u < kBatch; ++u) {
+            const int c = warp + 8 * ((i0 + u) / kParts), q = 32 * (u % kParts) + lane;
+            v[u] = c < nc && p0 + q < P ? __ldcs(src + (size_t)c * P + q) : 0.f;
         }
 #pragma unroll
-        for (int u = 0; u < kClBatch; ++u) {
-            const int c = warp + 8 * ((i0 + u) >> 1);
-            if (c < nc) tile[c * kClStride + 32 * (u & 1) + lane] = v[u];
+        for (int u = 0; u < kBatch; ++u) {
+            const int c = warp + 8 * ((i0 + u) / kParts), q = 32 * (u % kParts) + lane;
+            if (c < nc) tile[c * kStride + q] = v[u];
         }
     }
     __syncthreads();
     float* dst = last + (m * P + p0) * (size_t)Cf + c0;
     const int q8 = lane >> 2, cq = 4 * (lane & 3);          // pixel of a group of 8, channel of a group of 16
     const int quads = (nc + 15) / 16;
-    for (int job = warp; job < quads * (kClPix / 8); job += 8) {
+    for (int job = warp; job < quads * (kPix / 8); job += 8) {
         const int g = job / quads;                          // consecutive jobs share their pixels
         const int c = cq + 16 * (job - g * quads), q = 8 * g + q8;
         if (c >= nc || p0 + q >= P) continue;               // Cf % 4 == 0: a whole float4 or none
-        const float* col = tile + c * kClStride + q;
+        const float* col = tile + c * kStride + q;
         __stcs(reinterpret_cast<float4*>(dst + (size_t)q * Cf + c),
-               make_float4(col[0], col[kClStride], col[2 * kClStride], col[3 * kClStride]));
+               make_float4(col[0], col[kStride], col[2 * kStride], col[3 * kStride]));
     }
 }
 
@@ -800,14 +820,19 @@ int launch_gather_scatter(emc2_bridge* h, int b0, int B, int N, const float* d_p
 int launch_channels_last(emc2_bridge* h, int B, const float* d_planar, float* d_feat, cudaStream_t st) {
     const emc2_config_t& c = h->cfg;
     const long long P = (long long)c.feat_h * c.feat_w;
-    const long long ptiles = (P + kClPix - 1) / kClPix;
+    const ClTile tile = channels_last_tile(c.feat_c);
+    const long long ptiles = (P + tile.pix - 1) / tile.pix;
     const long long ctas = (long long)B * c.num_cameras * ptiles;
-    const int ct = (c.feat_c + kClMaxChan - 1) / kClMaxChan;
-    const int chan = ((c.feat_c + ct - 1) / ct + 3) / 4 * 4;
+    const int ct = (c.feat_c + tile.chan - 1) / tile.chan;
     if (P > 0x7FFFFFFFLL || ctas > 0x7FFFFFFFLL || ct > 65535) return EMC2_ERR_INVALID_ARG;
     LaunchScope ls(h, K_CHANNELS_LAST, st);
-    const dim3 grid((unsigned)ctas, (c.feat_c + chan - 1) / chan);
-    channels_last_kernel<<<grid, 256, (size_t)chan * kClStride * sizeof(float), st>>>(d_planar, d_feat, c.feat_c, (int)P, (int)ptiles, chan);
+    const dim3 grid((unsigned)ctas, ct);
+    if (tile.pix == 128)
+        channels_last_kernel<128><<<grid, 256, (size_t)tile.chan * kClStride<128> * sizeof(float), st>>>(
+            d_planar, d_feat, c.feat_c, (int)P, (int)ptiles, tile.chan);
+    else
+        channels_last_kernel<64><<<grid, 256, (size_t)tile.chan * kClStride<64> * sizeof(float), st>>>(
+            d_planar, d_feat, c.feat_c, (int)P, (int)ptiles, tile.chan);
     return check_cuda(h, cudaGetLastError());
 }
 

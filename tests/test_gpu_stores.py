@@ -167,8 +167,8 @@ def test_row_widths_of_the_row_kernels(oracle, cf):
         br.close()
 
 
-@pytest.mark.parametrize("cf", [4, 12, 64, 80, 128, 132, 260])
-@pytest.mark.parametrize("hw", [(1, 3), (8, 8), (9, 63), (13, 65)])
+@pytest.mark.parametrize("cf", [4, 12, 48, 52, 64, 80, 128, 132, 192, 260])
+@pytest.mark.parametrize("hw", [(1, 3), (8, 8), (9, 63), (13, 65), (1, 127), (3, 43), (11, 13)])
 def test_map_layout_and_pooling_at_tile_edges(oracle, cf, hw):
     h, wd = hw
     w = replace(gen.KITTI.with_shape(2, 16), img_h=8 * h, img_w=8 * wd, feat_stride=8, feat_c=cf)
