@@ -569,9 +569,9 @@ vox_finalize_kernel(const float* __restrict__ pts, long long total, AccumArgs a,
         for (int sc = 0; sc < 2; ++sc) {
             const ScaleDev& g = a.s[sc];
             if (g.cap <= 0) continue;
-            const bool refused = g.totals[0] == 0 || g.totals[1] != 0;        // see refuse_lists
-            if (refused && g.totals[1] != 0 && warp == 0 && lane == 0) a.num_voxels[sc] = 0;
-            const int novf = refused ? 0 : min(g.totals[3], (int)g.max_ovf);
+            const int4 tot = *reinterpret_cast<const int4*>(g.totals);
+            if (tot.y != 0 && warp == 0 && lane == 0) a.num_voxels[sc] = 0;   // see refuse_lists
+            const int novf = tot.x == 0 || tot.y != 0 ? 0 : min(tot.w, (int)g.max_ovf);
             int32_t* pv = a.point_voxel[sc];
             for (int j = warp; j < novf; j += nwarps) {
                 const int m = g.ovf_vox[j];
@@ -592,9 +592,9 @@ vox_finalize_kernel(const float* __restrict__ pts, long long total, AccumArgs a,
                 for (int k = 0; k < C; ++k) acc[k] = 0.0;
                 for (int i = lane; i < n; i += 32) {
                     const int v = list[i];
-                    if ((unsigned long long)v >= (unsigned long long)total) continue;   // never a point of this call
-                    const bool keep = v <= hi;
-                    if (pv) pv[v] = keep ? m : -1;
+                    const bool mine = (unsigned)v < (unsigned)total;      // always, with this call's own lists
+                    const bool keep = mine && v <= hi;
+                    if (pv && mine) pv[v] = keep ? m : -1;
                     if (keep) {
 #pragma unroll
                         for (int k = 0; k < C; ++k) acc[k] += (double)pts[(size_t)v * C + k];
