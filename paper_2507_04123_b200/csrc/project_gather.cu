@@ -642,18 +642,21 @@ channels_last_kernel(const float* __restrict__ planar, float* __restrict__ last,
     const int nc = min(chan, Cf - c0);
     const float* src = planar + (m * Cf + c0) * (size_t)P + p0;
     // Item i of a warp: part i % kParts of channel row warp + 8 * (i / kParts).
+    bool in[kParts];
+#pragma unroll
+    for (int i = 0; i < kParts; ++i) in[i] = p0 + 32 * i + lane < P;
     const int items = kParts * ((nc - warp + 7) / 8);
     for (int i0 = 0; i0 < items; i0 += kBatch) {
         float v[kBatch];
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
-            const int c = warp + 8 * ((i0 + u) / kParts), q = 32 * (u % kParts) + lane;
-            v[u] = c < nc && p0 + q < P ? __ldcs(src + (size_t)c * P + q) : 0.f;
+            const int c = warp + 8 * ((i0 + u) / kParts), part = u % kParts;
+            v[u] = c < nc && in[part] ? __ldcs(src + (size_t)c * P + 32 * part + lane) : 0.f;
         }
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
-            const int c = warp + 8 * ((i0 + u) / kParts), q = 32 * (u % kParts) + lane;
-            if (c < nc) tile[c * kStride + q] = v[u];
+            const int c = warp + 8 * ((i0 + u) / kParts);
+            if (c < nc) tile[c * kStride + 32 * (u % kParts) + lane] = v[u];
         }
     }
     __syncthreads();
