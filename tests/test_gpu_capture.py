@@ -1,4 +1,5 @@
 """Calls captured into CUDA graphs: which launches are chained to their predecessor, and replays on new frames (needs a B200)."""
+import ctypes
 from dataclasses import replace
 
 import numpy as np
@@ -9,7 +10,6 @@ import emc2_gen as gen
 from parity import compare_bridge, to_dev
 
 pytestmark = pytest.mark.gpu
-rt = pytest.importorskip("cuda.bindings.runtime")
 
 
 def bridge_for(w, **kw):
@@ -26,23 +26,24 @@ def captured(call):
 
 def chained_launches(graph):
     """Checks that every chained launch follows exactly one node, a kernel; returns how many there are."""
-    def ok(res):
-        assert res[0] == rt.cudaError_t.cudaSuccess, res[0]
-        return res[1:]
+    cu = ctypes.CDLL("libcuda.so.1")
+    g, n = ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t(0)
+    assert cu.cuGraphGetEdges_v2(g, None, None, None, ctypes.byref(n)) == 0
+    tails, heads = (ctypes.c_void_p * n.value)(), (ctypes.c_void_p * n.value)()
+    edges = (ctypes.c_uint8 * 8 * n.value)()               # CUgraphEdgeData: from_port, to_port, type, 5 reserved bytes
+    assert cu.cuGraphGetEdges_v2(g, tails, heads, edges, ctypes.byref(n)) == 0
 
-    g = rt.cudaGraph_t(init_value=graph.raw_cuda_graph())
-    n = ok(rt.cudaGraphGetEdges_v2(g))[-1]
-    tails, heads, data, n = ok(rt.cudaGraphGetEdges_v2(g, n))
-    kernel = rt.cudaGraphNodeType.cudaGraphNodeTypeKernel
-    before = {}
-    for a, b in zip(tails, heads):
-        before.setdefault(int(b), []).append(a)
+    def is_kernel(node):
+        kind = ctypes.c_int(-1)
+        assert cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        return kind.value == 0                               # CU_GRAPH_NODE_TYPE_KERNEL
+
     found = 0
-    for a, b, d in zip(tails, heads, data):
-        if int(d.type) == int(rt.cudaGraphDependencyType.cudaGraphDependencyTypeProgrammatic):
+    for i in range(n.value):
+        if edges[i][2] == 1:                                 # CU_GRAPH_DEPENDENCY_TYPE_PROGRAMMATIC
             found += 1
-            assert ok(rt.cudaGraphNodeGetType(a))[0] == kernel and ok(rt.cudaGraphNodeGetType(b))[0] == kernel
-            assert len(before[int(b)]) == 1
+            assert is_kernel(tails[i]) and is_kernel(heads[i])
+            assert list(heads).count(heads[i]) == 1
     return found
 
 
