@@ -16,9 +16,15 @@ constexpr int kThreads = 256;
 
 // Threads of the kernels that move feature rows when Cf/4 = cf4 is not one of the compiled widths: as many whole
 // rows of cf4 columns as 512 threads hold (at least 256: one per point of a tile), so that every thread keeps its
-// column and no index is divided inside the loop.  Rows wider than that take the divide.
+// column and no index is divided inside the loop.  Rows wider than that take the divide.  Rows of an odd number of
+// columns are half a sector off at every other row: up to 1 KB an even number of them is taken, so that a CTA's
+// stores stay on sectors (132 channels, 1,800 tiles: project_gather 47.7 -> 44.7 us; 36: 23.1 -> 22.0; 52: 27.2 -> 25.1).
 constexpr int kMaxRowThreads = 512;
-inline int row_threads(int cf4) { return cf4 <= kTile ? kMaxRowThreads / cf4 * cf4 : kThreads; }
+inline int row_threads(int cf4) {
+    if (cf4 > kTile) return kThreads;
+    const int rows = kMaxRowThreads / cf4;
+    return (cf4 <= 64 && (cf4 & 1) ? rows & ~1 : rows) * cf4;
+}
 // The cell stores.  Large grids: 16-byte units of 96 cell bits and the rank of the unit's first voxel, so that
 // one 128-bit load answers a look-up and the scan streams 1.33 bits per cell (a {32 bits, rank} pair per 32
 // cells streams 2: 75 instead of 50 MB for four frames of the nuScenes-shaped grid, and the scan is paid by

@@ -134,12 +134,16 @@ __device__ __forceinline__ void load_cameras(const float* __restrict__ proj, int
     }
 }
 
-// CF4 > 0: Cf/4 known at compile time, blockDim.x == 16 * CF4; else blockDim.x == row_threads(cf4).
+// CF4 > 0: Cf/4 known at compile time, blockDim.x == 16 * CF4; else blockDim.x == row_threads(cf4), with 40 registers
+// (three CTAs per SM; left to itself the compiler takes 32 and the rows lose their loads in flight: 256 channels,
+// 1,800 tiles of mostly visible points: 127 -> 136 us).  Rows of more than 1 KB and an odd number of columns are the
+// one case where whole rows can lose against one divide per float4, which kept all stores on sectors: 260 channels,
+// 1,800 tiles: 99 against 87 us where few points are visible, 156 against 169 where most are.
 // kFrames: most frames that the points of a tile belong to, see frames_of_tile: two but for frames of fewer than 255
 // points, whose cameras are all staged at once (32 frames of 8 points through 6 cameras: 31 us with the cameras of two
 // frames at a time in turn, 10.3 with every point reading its own from global memory, 9.8 this way).
 template <int C, int CF4, int kFrames = 2>
-__global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kMaxRowThreads) project_gather_kernel(PgArgs a) {
+__global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kMaxRowThreads, CF4 > 0 ? 0 : 3) project_gather_kernel(PgArgs a) {
     __shared__ __align__(16) float sp[kTile * C];
     __shared__ float suvd[kTile * 3];
     __shared__ uint4 srow[kTile];          // {tap (y0,x0) as a float4 index, clamp flags, wx, wy}

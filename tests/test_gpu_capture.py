@@ -83,7 +83,7 @@ def test_host_frame_replays_from_a_graph(oracle):
 def test_one_call_replays_from_a_graph_under_every_tuning(oracle, tuning, B):
     """split_batch: the second half's route scan follows a wait for the other stream."""
     w = gen.NUSCENES.with_shape(B, 7001)
-    w = replace(w, img_h=180, img_w=320)
+    w = replace(w, img_h=180, img_w=320, cameras=tuple(replace(c, fx=200.0, fy=200.0, cx=160.0, cy=90.0) for c in w.cameras))
     frames = [gen.make_batch(w, frames=list(range(B * i, B * i + B))) for i in range(2)]
     for overlap in (True, False):
         br = bridge_for(w)

@@ -47,6 +47,12 @@ def check_voxels(w, pts, oracle, repeat=2, rules=False):
     br.close()
 
 
+def small_images(w, h, wd):
+    """The workload with images of h x wd pixels, the cameras' axes in their middle and about 77 degrees wide."""
+    cams = tuple(replace(c, fx=0.63 * wd, fy=0.63 * wd, cx=wd / 2, cy=h / 2) for c in w.cameras)
+    return replace(w, img_h=h, img_w=wd, feat_stride=8, cameras=cams)
+
+
 def centres(ids, grid, C, rng):
     ids = np.asarray(ids, np.int64)
     x, y = ids % grid.dims[0], ids // grid.dims[0]
@@ -143,14 +149,15 @@ def test_points_on_image_edges(oracle, B, N):
         br.close()
 
 
-@pytest.mark.parametrize("cf", [4, 32, 64, 68, 80, 128, 256, 1020, 1024, 1028])
+@pytest.mark.parametrize("cf", [4, 32, 36, 64, 68, 80, 128, 132, 252, 256, 260, 1020, 1024, 1028])
 def test_row_widths_of_the_row_kernels(oracle, cf):
     """Compiled widths, whole rows per CTA, and rows wider than a CTA; ragged tiles, four and five floats per point,
     dispatched point rows in a buffer of any alignment."""
     for base, B, N in ((gen.KITTI, 2, 259), (gen.NUSCENES, 1, 517)):
-        w = replace(base.with_shape(B, N), img_h=64, img_w=96, feat_stride=8, feat_c=cf)
+        w = replace(small_images(base.with_shape(B, N), 64, 96), feat_c=cf)
         batch = gen.make_batch(w)
         ref = oracle.bridge(w, batch)
+        assert 0.1 < (ref["cam"] >= 0).mean() < 1
         d = {k: torch.from_numpy(v).cuda() for k, v in batch.items()}
         br = bridge_for(w)
         odd = torch.zeros(B * N * w.C + 1, device="cuda")[1:].view(B, N, w.C)      # 4 bytes past a 16-byte boundary
