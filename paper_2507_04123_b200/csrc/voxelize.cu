@@ -556,9 +556,10 @@ __device__ __forceinline__ void write_batch(const AccumArgs& a, int sc, int mb, 
 
 // CTAs [0, ovf_blocks) serve cells over the cap, one warp per cell: the `cap` lowest point
 // indices are kept (keep-first-by-index), summed in fp64 and written as the voxel's mean; all of
-// the cell's points get their point_voxel entry.  The other CTAs write the voxel rows.
+// the cell's points get their point_voxel entry.  The other CTAs write the voxel rows.  Six CTAs per SM, 40
+// registers: with 47, five, four nuScenes-shaped frames took 39.4 instead of 37.8 us.
 template <int C>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 6)
 vox_finalize_kernel(const float* __restrict__ pts, long long total, AccumArgs a, int ovf_blocks) {
     await_predecessor();
     constexpr int kWarps = kThreads / 32;
