@@ -181,8 +181,8 @@ int emc2_bridge_run(emc2_bridge_t* bridge, int32_t B, int32_t N, const float* d_
  * points, calibration and image features arrive on the host): enqueues, on `cuda_stream`, the copies
  * of h_points [B, N, C], h_proj [B, K, 3, 4] and h_feat [B, K, Hf, Wf, Cf] into the caller's device
  * buffers d_points, d_proj, d_feat (the maps last, beside the work that does not need them) and
- * emc2_bridge_run on them with the same outputs, then the copies of d_offsets [B, E+1] and d_num_voxels [2] into h_offsets and h_num_voxels (either may be
- * NULL: not copied).  Nothing is synchronised: the host buffers must stay valid and unchanged until
+ * emc2_bridge_run on them with the same outputs, then the copies of d_offsets [B, E+1] and
+ * d_num_voxels [2] into h_offsets and h_num_voxels (either may be NULL: not copied).  Nothing is synchronised: the host buffers must stay valid and unchanged until
  * the stream has passed the call; the copies are asynchronous only for page-locked host memory
  * (which stream capture requires).  A
  * caller who alternates between two handles, streams and buffer sets overlaps one frame's copies with

@@ -253,7 +253,8 @@ int launch_route_dispatch(emc2_bridge* h, int B, int N, const float* d_points, c
 // through plain pointers, never through `const __restrict__` ones or __ldg, whose loads the compiler may move ahead
 // of the wait.  The call's own inputs are complete before the first kernel of a call, which is launched plainly.
 // Released earlier, the successor's CTAs would hold places on the SMs that the kernels of the other stream need.
-// us per call: one small frame 35 -> 30, stage calls with occlusion 155 -> 140, voxels and rulebooks 261 -> 239 (B200).
+// us per call queued behind others: one small frame 35 -> 30, stage calls with occlusion 155 -> 140, voxels and rulebooks
+// 261 -> 239 (B200).  A call on an idle GPU gains less: there the host's enqueuing of its kernels and events sets the pace.
 // `chained` false: an ordinary launch, for a kernel that follows a copy or an event wait, or that can be the first of
 // its call.
 template <typename... P, typename... A>

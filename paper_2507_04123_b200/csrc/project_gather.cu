@@ -73,9 +73,10 @@ __device__ __forceinline__ void chains(const Camera& c, float x, float y, float 
 // image edge (eps is far above the roundings of these products), and only the chosen camera's (u, v) is
 // divided out.  The loop over the cameras has no branches; cameras that are left undecided are taken up
 // after it.  `cam`: the frame's K cameras in shared memory.
-// project_route_kernel is bound by instruction issue: with a test per camera in scalar arithmetic and
-// divides for the six cell indices a warp of the six-camera workload took 860 instructions, now 680 (32 frames of
-// 262,144 points: 221 -> 178 us).
+// A warp of the six-camera workload took 860 instructions with a test per camera in scalar arithmetic and divides for
+// the six cell indices, now 680.  That shows in project_route_kernel where instruction issue bounds it: 32 frames of
+// 262,144 points 222 -> 179 us, eight KITTI-shaped frames 33.9 -> 31.2.  On four nuScenes-shaped frames it does not
+// (43.9 and 44.3 us): there the kernel waits for the marks, whose sectors of the cell store are not in L2.
 __device__ __forceinline__ Projected project_point(const Camera* cam, int K, float x, float y, float z,
                                                     int W, int H, float min_depth) {
     Projected r;
@@ -294,14 +295,22 @@ struct GsArgs {
 };
 
 // CF4 > 0: Cf/4 known at compile time, blockDim.x == kGsRows<CF4> * CF4; else blockDim.x == row_threads(cf4).
-// Bound by the memory system's writes: two rows of 4 Cf bytes per point, 384 MB each on four nuScenes-shaped
-// frames.  A plain kernel writes those bytes in 113 us, this one in 177 with its taps (188 before the point rows
-// left in expert order; 158 of those without the taps).  Neither more rows in flight per thread, nor fewer
-// resident warps, nor other cache policies of the stores move it; a persistent grid writes 10 % slower than
-// tiles in launch order.
-// Rows at a time: 512 threads where registers allow four such CTAs, so that a tile is through sooner: 64 channels
-// 112 -> 109 us on the KITTI-shaped batch and 15 -> 11 us on one small frame, 128 channels 90 -> 83 us; 80
-// channels take 16 rows (320 threads) because 24 or 32 leave fewer warps resident (177 -> 181 and 191 us).
+// Two rows of 4 Cf bytes per point are written, 384 MB each on four nuScenes-shaped frames.  A plain kernel writes
+// those bytes in 113 us, this one takes 176 with its taps (188 before the point rows left in expert order; 158 of those
+// without the taps).  No unit of the chip is busy all the time; what the tap reads and the two streams of writes cost
+// beyond the writes alone is how they interleave.  More resident warps do not move it, nor do more rows in flight per
+// thread or other cache policies of the stores; a persistent grid writes 10 % slower than tiles in launch order.
+// Rows at a time, with the registers the compiler takes or is held to, and the time alone (us):
+//   80 channels, 4 x 300,000 points, C = 5        64 channels, 8 x 120,000 points, C = 4
+//     16 rows, 42 registers, 40 warps   176         32 rows, 40 registers, 48 warps   108
+//     16 rows, 32 registers, 50 warps   179         32 rows, 32 registers, 64 warps   109
+//     16 rows, 32 registers, 60 warps   182         32 rows, 56 registers, 32 warps   115
+//     24 rows, 40 registers, 45 warps   174         16 rows, 40 registers, 48 warps   111
+//     24 rows, 32 registers, 60 warps   178         16 rows, 32 registers, 64 warps   113
+//     32 rows, 40 registers, 40 warps   187         16 rows, 56 registers, 32 warps   109
+// (32 registers spill a word; as a step the rows of 80 channels differ by 1 %.)  One small frame of 64 channels: 32 rows
+// 10.7 us, 16 rows 12.7: a tile is through sooner.  Other widths take as many rows as 512 threads hold (128 channels: 90
+// -> 83 us).
 template <int CF4> constexpr int kGsRows = CF4 == 16 ? 32 : 16;
 
 template <int C, int CF4>
