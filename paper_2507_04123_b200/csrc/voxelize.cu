@@ -558,6 +558,11 @@ __device__ __forceinline__ void write_batch(const AccumArgs& a, int sc, int mb, 
 // indices are kept (keep-first-by-index), summed in fp64 and written as the voxel's mean; all of
 // the cell's points get their point_voxel entry.  The other CTAs write the voxel rows.  Six CTAs per SM, 40
 // registers: with 47, five, four nuScenes-shaped frames took 39.4 instead of 37.8 us.
+// A warp takes some twenty steps to bisect a cell's indices, each of which waited for the list to come from L2 again: it
+// keeps the first 256 of them in registers (the densest cells of the dense frame have about 300).  One dense frame: the
+// kernel 19.0 -> 12.7 us, the call 76.3 -> 70.5; four nuScenes-shaped frames: the kernel 38.0 -> 34.9.
+constexpr int kHeld = 8;
+
 template <int C>
 __global__ void __launch_bounds__(kThreads, 6)
 vox_finalize_kernel(const float* __restrict__ pts, long long total, AccumArgs a, int ovf_blocks) {
@@ -579,12 +584,24 @@ vox_finalize_kernel(const float* __restrict__ pts, long long total, AccumArgs a,
                 const uint32_t start = (uint32_t)g.ovf_off[j];
                 const int* list = g.ovf_list + start;
                 const int n = start < g.max_list ? min(g.ovf_cursor[(size_t)j * kCursorStride], (int)(g.max_list - start)) : 0;
-                // Smallest index value v with #{list <= v} >= cap, by bisection on the value.
-                long long lo = -1, hi = total - 1;
+                // Smallest index value v with #{list <= v} >= cap, by bisection on the value, between the smallest
+                // and the largest of the list.
+                int held[kHeld];
+                int lo = 0x7FFFFFFF, hi = -1;
+#pragma unroll
+                for (int u = 0; u < kHeld; ++u) {
+                    held[u] = 32 * u + lane < n ? list[32 * u + lane] : 0x7FFFFFFF;
+                    if (32 * u + lane < n) { lo = min(lo, held[u]); hi = max(hi, held[u]); }
+                }
+                for (int i = 32 * kHeld + lane; i < n; i += 32) { lo = min(lo, list[i]); hi = max(hi, list[i]); }
+                lo = __reduce_min_sync(0xFFFFFFFFu, lo) - 1;
+                hi = __reduce_max_sync(0xFFFFFFFFu, hi);
                 while (hi - lo > 1) {
-                    const long long mid = lo + (hi - lo) / 2;
+                    const int mid = lo + (hi - lo) / 2;
                     int c = 0;
-                    for (int i = lane; i < n; i += 32) c += list[i] <= mid;
+#pragma unroll
+                    for (int u = 0; u < kHeld; ++u) c += held[u] <= mid;
+                    for (int i = 32 * kHeld + lane; i < n; i += 32) c += list[i] <= mid;
                     c = warp_sum(c);
                     if (c >= g.cap) hi = mid; else lo = mid;
                 }

@@ -189,3 +189,16 @@ def test_map_layout_and_pooling_at_tile_edges(oracle, cf, hw):
         assert close(np_(br.pool_features(last, p)), oracle.pool(want, p))[0]
     br.status()
     br.close()
+
+
+@pytest.mark.parametrize("cap", [1, 3, 32, 255, 256, 257, 300])
+def test_cells_over_the_cap_by_the_length_of_their_lists(oracle, cap):
+    """Lists around 32 and 256 entries, which a warp holds in registers, and longer ones; the first and the last points of
+    the call among them, on both kinds of store."""
+    rng = np.random.default_rng(cap)
+    sizes = [cap, cap + 1, 31, 32, 33, 255, 256, 257, 288, 289, 600, 1025]
+    for grids in ((BITMAP, replace(TABLE, max_points=cap)), (replace(BITMAP, max_points=cap), replace(TABLE, max_points=cap))):
+        at = np.repeat([97 * i for i in range(len(sizes))], sizes)
+        cells = np.concatenate([[0], rng.permutation(at[1:-1]), [at[-1]]])       # cell 0 has point 0, the last cell the last point
+        pts = centres(cells, TABLE, 4, rng)[None]
+        check_voxels(replace(gen.KITTI.with_shape(1, pts.shape[1]), grids=grids), pts, oracle)
