@@ -138,8 +138,6 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out) {
 
     if (cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, config->device) != cudaSuccess ||
         h->num_sms < 1) { delete h; return EMC2_ERR_CUDA; }
-    h->vif_scan_blocks = voxel_image_scan_max_blocks();
-    if (h->vif_scan_blocks < 1) { delete h; return EMC2_ERR_CUDA; }
 
     // Plan the slab: everything the stage calls need, allocated once.
     SlabPlan plan;
@@ -183,7 +181,7 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out) {
     const size_t o_vif_cursor = plan.take(maxpts * sizeof(int));
     const size_t o_vif_list = plan.take(maxpts * sizeof(int));
     const size_t o_vif_recs = plan.take(maxpts * sizeof(uint4));
-    const size_t o_vif_part = plan.take(((size_t)h->vif_scan_blocks + 1) * sizeof(int));
+    const size_t o_vif_part = plan.take(3 * sizeof(int));
     const size_t rb_tiles = (maxpts + kTile - 1) / kTile;
     const size_t o_rb_bits = plan.take(maxpts * sizeof(uint32_t));
     const size_t o_rb_counts = plan.take(13 * rb_tiles * sizeof(int));

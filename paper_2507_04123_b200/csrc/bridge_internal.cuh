@@ -195,8 +195,7 @@ struct emc2_bridge {
     int* d_vif_cursor = nullptr;
     int* d_vif_list = nullptr;
     uint4* d_vif_recs = nullptr;   // emc2_voxel_image_sampled: [max points] tap records in list order
-    int* d_vif_part = nullptr;     // [vif_scan_blocks]
-    int vif_scan_blocks = 0;
+    int* d_vif_part = nullptr;     // list slots given out (64 bits, zero between calls), flag of bad counts
     uint32_t* d_rb_bits = nullptr;  // emc2_rulebook: [max points] neighbour bits per voxel
     int* d_rb_counts = nullptr;    // [13][voxel tiles] pairs per (offset, tile), and their prefix sums
     int* d_rb_base = nullptr;
@@ -298,7 +297,6 @@ inline RouteParams route_params(const emc2_bridge* h) {
 int launch_occlusion(emc2_bridge* h, int B, int N, const float* d_points, const float* d_proj,
                      const uint8_t* d_vis_mask, int cell, float margin, uint32_t* d_zbuf, uint8_t* d_occ_mask,
                      uint8_t* d_clear_mask, cudaStream_t st);
-int voxel_image_scan_max_blocks();
 int launch_voxel_image(emc2_bridge* h, int B, int N, int capacity, const int32_t* d_point_voxel,
                        const int32_t* d_counts, const int32_t* d_num_voxels, const uint8_t* d_vis_mask,
                        const float* d_gathered, const float* d_uvd, const int8_t* d_cam, const float* d_feat,

@@ -4,20 +4,17 @@
 // points that some camera sees.
 //
 // Rows are 256/320 bytes: adding them up with reductions would cost twenty 16-byte requests per
-// point.  Instead the points are listed per voxel and each voxel reads its points' rows whole:
-//   vif_scan   cooperative launch: exclusive prefix sum of the voxels' kept-point counts (the
-//              prefix-sum indexing of Sec. 3.6) -> start of every voxel's list; cursors cleared.
-//   vif_fill   every kept point takes a ticket in its voxel's list (one atomic with return).
+// point.  Instead the visible points are listed per voxel and each voxel reads its points' rows whole:
+//   vif_scan   exclusive prefix sums of the voxels' kept-point counts (the prefix-sum indexing of Sec. 3.6) -> start
+//              of every voxel's list.  The sums go over 4096 voxels; a CTA takes their part of the list array with one
+//              ticket, so that no pass over all the counts has to come first.
+//   vif_fill   every kept point that a camera sees takes a ticket in its voxel's list (one atomic with return).
 //   vif_mean   16 voxels x Cf/4 columns of threads per CTA: a voxel's threads walk its list and
-//              read each visible point's row with one contiguous 128-bit load per thread.
+//              read each listed point's row with one contiguous 128-bit load per thread.
 //   vif_sample the same, but the rows are blended from the feature maps on the spot
 //              (emc2_voxel_image_sampled: no [points, Cf] buffer at all); for it vif_fill stores
 //              each listed point's tap record (16 bytes) in place of its index.
-#include <cooperative_groups.h>
-
 #include "bridge_internal.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace emc2 {
 namespace {
@@ -38,11 +35,11 @@ struct VifArgs {
     float4* vox_img;            // [capacity, cf4]
     int32_t* vox_cnt;           // [capacity]
     int* start;                 // [capacity] first list slot of each voxel
-    int* cursor;                // [capacity]
-    int* list;                  // [total] point indices; bitwise complement for points no camera sees
+    int* cursor;                // [capacity] next free list slot of each voxel
+    int* list;                  // [total] point indices
     uint4* recs;                // [total] vif_sample: tap record of every listed point, in list order
-    int* part;                  // [gridDim.x]
-    int* bad;                   // set by vif_scan when counts[] add up to more than there are points
+    unsigned long long* taken;  // list slots given out by vif_scan; zero between calls
+    int* bad;                   // counts[] add up to more than there are points
     int* status;
     long long total;
     int capacity, cf4;
@@ -50,84 +47,89 @@ struct VifArgs {
 
 __device__ __forceinline__ int voxels_in_use(const VifArgs& a) { return min(*a.num_voxels, a.capacity); }
 
-// Every thread owns a run of consecutive voxels.  CTA totals, grid barrier, then the prefix.
-__global__ void __launch_bounds__(kThreads) vif_scan_kernel(VifArgs a) {
+// A warp has kScanRows * 32 consecutive voxels, a CTA eight times as many and one ticket: tickets on one address are
+// served one after another (about 10 ns each).  As a cooperative launch that summed all counts before any start was known
+// this took 14.3 us for the lists of four nuScenes-shaped frames (mean of both scales, by events), now 10.7; the fill, which
+// looked the start up and listed invisible points as well, 26.9, now 22.7; both scales together 300.7 -> 282.1 us.
+constexpr int kScanRows = 16, kScanVoxels = kThreads * kScanRows;
+
+__global__ void __launch_bounds__(kThreads) vif_scan_kernel(const __grid_constant__ VifArgs a) {
     __shared__ int wsum[kThreads / 32];
-    __shared__ int s_base;
-    cg::grid_group grid = cg::this_grid();
+    __shared__ long long s_base;
     const int M = voxels_in_use(a);
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const long long nthreads = (long long)gridDim.x * kThreads;
-    const int per = (int)((M + nthreads - 1) / nthreads);
-    const long long lo64 = ((long long)blockIdx.x * kThreads + t) * per;
-    const int lo = (int)min((long long)M, lo64), hi = (int)min((long long)M, lo64 + per);
+    if ((long long)blockIdx.x * kScanVoxels >= M) return;
+    const int m0 = blockIdx.x * kScanVoxels + warp * (32 * kScanRows) + lane;
     // Sums saturate at one more than the points of the call (at most 2^24 + 1): they cannot wrap, and
     // counts[] that add up to more than the points are still seen as such.
     const int limit = (int)min(a.total, (long long)1 << 24) + 1;
-    auto count_of = [&](int m) { return min(max(a.counts[m], 0), limit); };
-    int sum = 0;
-    for (int m = lo; m < hi; ++m) sum = min(sum + count_of(m), limit);
-    int inc = sum;
+    int n[kScanRows];
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int y = __shfl_up_sync(0xFFFFFFFFu, inc, d);
-        if (lane >= d) inc = min(inc + y, limit);
+    for (int j = 0; j < kScanRows; ++j) n[j] = m0 + 32 * j < M ? min(max(a.counts[m0 + 32 * j], 0), limit) : 0;
+    int carry = 0;
+#pragma unroll
+    for (int j = 0; j < kScanRows; ++j) {                 // n[j]: slots of the warp's voxels before this one
+        int inc = n[j];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int y = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+            if (lane >= d) inc += y;                      // 32 terms of at most 2^24 + 1
+        }
+        n[j] = carry + inc - n[j];
+        carry = min(carry + __shfl_sync(0xFFFFFFFFu, inc, 31), limit);
     }
-    if (lane == 31) wsum[warp] = inc;
+    if (lane == 0) wsum[warp] = carry;
     __syncthreads();
-    int before = 0, cta_total = 0;
+    int before = 0, all = 0;
+#pragma unroll
     for (int w = 0; w < kThreads / 32; ++w) {
-        if (w < warp) before = min(before + wsum[w], limit);
-        cta_total = min(cta_total + wsum[w], limit);
+        if (w < warp) before += wsum[w];
+        all += wsum[w];
     }
-    if (t == 0) a.part[blockIdx.x] = cta_total;
-    grid.sync();
-    if (warp == 0) {
-        int v = 0;
-        for (int c = lane; c < (int)blockIdx.x; c += 32) v = min(v + a.part[c], limit);
-        v = min(warp_sum(v), limit);                      // 32 terms of at most 2^24 + 1
-        if (lane == 0) s_base = v;
-    }
+    if (t == 0) s_base = (long long)atomicAdd(a.taken, (unsigned long long)all);
     __syncthreads();
-    // counts[] that add up to more than the points of the call are not the voxelizer's counts for this
-    // batch: the lists would not fit the list array, so the later kernels do nothing.
-    if (blockIdx.x == gridDim.x - 1 && t == 0) {
-        const int inconsistent = (long long)s_base + cta_total > a.total ? 1 : 0;
-        *a.bad = inconsistent;
-        if (inconsistent) atomicOr(a.status, 4);
+    const long long base = s_base + before;               // exact whenever the counts are consistent
+#pragma unroll
+    for (int j = 0; j < kScanRows; ++j) {
+        if (m0 + 32 * j >= M) break;
+        const int at = (int)min(base + n[j], (long long)limit);
+        a.start[m0 + 32 * j] = at;
+        a.cursor[m0 + 32 * j] = at;
     }
-    int run = min(s_base + before, limit) + inc - sum;      // exact whenever the counts are consistent
-    for (int m = lo; m < hi; ++m) {
-        a.start[m] = run;
-        a.cursor[m] = 0;
-        run = min(run + count_of(m), limit);
-    }
+    release_successor();
 }
 
-__global__ void __launch_bounds__(kThreads) vif_fill_kernel(VifArgs a) {
+__global__ void __launch_bounds__(kThreads) vif_fill_kernel(const __grid_constant__ VifArgs a) {
     await_predecessor();
-    if (*a.bad) return;
+    // counts[] that add up to more than the points of the call are not the voxelizer's counts for this
+    // batch: the lists would not fit the list array, so nothing is listed and the next kernel does nothing.
+    const bool bad = *a.taken > (unsigned long long)a.total;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *a.bad = bad ? 1 : 0;
+        if (bad) atomicOr(a.status, 4);
+    }
+    if (bad) return;
     const int M = voxels_in_use(a);
     for (long long i = (long long)blockIdx.x * kThreads + threadIdx.x; i < a.total; i += (long long)gridDim.x * kThreads) {
         const int m = a.pv[i];
         if (m < 0 || m >= M) continue;
         // What goes into the list first (its loads do not wait for the ticket), then the ticket.
-        int entry = 0;
         uint4 rec = make_uint4(kZeroRow, 0u, 0u, 0u);
         if (a.vis) {
-            entry = a.vis[i] ? (int)i : ~(int)i;
+            if (!a.vis[i]) continue;
         } else {                                        // rows will be blended from the maps: keep the taps
             // pooled: the record addresses a TEXEL of the pooled map (not a float4 of a row), see pooled_column
             rec = a.pool > 1 ? tap_record((int)(i / a.N), (int)a.cam[i], a.uvd[3 * i], a.uvd[3 * i + 1], a.K, a.Hp, a.Wp, 1,
                                           a.inv_stride, a.offset)
                              : tap_record((int)(i / a.N), (int)a.cam[i], a.uvd[3 * i], a.uvd[3 * i + 1], a.K, a.Hf, a.Wf,
                                           a.cf4, a.inv_stride, a.offset);
+            if (rec.x == kZeroRow) continue;
         }
-        const int pos = a.start[m] + atomicAdd(&a.cursor[m], 1);
+        const int pos = atomicAdd(&a.cursor[m], 1);
         // Inside the list whenever counts[] are the kept-point counts of pv[] (the voxelizer's outputs
         // for this batch); anything else must not index out of range.
         if ((unsigned)pos >= (unsigned)a.total) continue;
-        if (a.vis) a.list[pos] = entry;
+        if (a.vis) a.list[pos] = (int)i;
         else a.recs[pos] = rec;
     }
     release_successor();
@@ -137,6 +139,7 @@ __global__ void __launch_bounds__(kThreads) vif_fill_kernel(VifArgs a) {
 template <int CF4>
 __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads) vif_mean_kernel(VifArgs a) {
     await_predecessor();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.taken = 0ull;     // for the next call; nothing reads it any more
     if (*a.bad) return;
     const int M = voxels_in_use(a);
     const int cf4 = CF4 > 0 ? CF4 : a.cf4;
@@ -153,7 +156,7 @@ __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads) vif_mean_kernel
         for (int u = 0; u < 2; ++u) {
             const bool ok = mm[u] < M;
             s0[u] = ok ? a.start[mm[u]] : 0;
-            n[u] = ok ? min(a.counts[mm[u]], a.cursor[mm[u]]) : 0;   // never past what this call appended
+            n[u] = ok ? min(a.counts[mm[u]], a.cursor[mm[u]] - s0[u]) : 0;   // never past what this call appended
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u) first[u] = n[u] > 0 ? a.list[s0[u]] : -1;
@@ -234,6 +237,7 @@ __device__ __forceinline__ float4 pooled_column(const VifArgs& a, const uint4& r
 template <int CF4, bool kPooled>
 __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads) vif_sample_kernel(VifArgs a) {
     await_predecessor();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.taken = 0ull;     // for the next call; nothing reads it any more
     if (*a.bad) return;
     const int M = voxels_in_use(a);
     const int cf4 = CF4 > 0 ? CF4 : a.cf4;
@@ -249,7 +253,7 @@ __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads) vif_sample_kern
         for (int u = 0; u < 2; ++u) {
             const bool ok = mm[u] < M;
             s0[u] = ok ? a.start[mm[u]] : 0;
-            n[u] = ok ? min(a.counts[mm[u]], a.cursor[mm[u]]) : 0;   // never past what this call appended
+            n[u] = ok ? min(a.counts[mm[u]], a.cursor[mm[u]] - s0[u]) : 0;   // never past what this call appended
             acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
         // The first entries of the two voxels together, then the rest of each list, two at a time;
@@ -298,14 +302,6 @@ __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads) vif_sample_kern
 
 }  // namespace
 
-int voxel_image_scan_max_blocks() {
-    int dev = 0, sms = 0, per_sm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, vif_scan_kernel, kThreads, 0) != cudaSuccess) return 0;
-    return sms * min(per_sm, 2);
-}
-
 // d_gathered != null: rows are read from it and d_vis_mask says which points count; else rows are
 // sampled from d_feat at d_uvd in camera d_cam, and a point counts iff its camera is >= 0.
 int launch_voxel_image(emc2_bridge* h, int B, int N, int capacity, const int32_t* d_point_voxel,
@@ -327,9 +323,10 @@ int launch_voxel_image(emc2_bridge* h, int B, int N, int capacity, const int32_t
         a.offset = cfg.feat_offset + 0.5f * (float)(pool - 1) * (float)cfg.feat_stride;
     }
     a.vox_img = reinterpret_cast<float4*>(d_vox_img); a.vox_cnt = d_vox_img_count;
-    a.start = h->d_vif_start; a.cursor = h->d_vif_cursor; a.list = h->d_vif_list; a.part = h->d_vif_part;
+    a.start = h->d_vif_start; a.cursor = h->d_vif_cursor; a.list = h->d_vif_list;
     a.recs = h->d_vif_recs;
-    a.bad = h->d_vif_part + h->vif_scan_blocks;
+    a.taken = reinterpret_cast<unsigned long long*>(h->d_vif_part);
+    a.bad = h->d_vif_part + 2;
     a.status = h->d_status;
     a.total = (long long)B * N;
     a.capacity = (int)min((long long)capacity, a.total);   // a voxel holds at least one point
@@ -338,10 +335,7 @@ int launch_voxel_image(emc2_bridge* h, int B, int N, int capacity, const int32_t
     if (a.cf4 > kThreads) return EMC2_ERR_INVALID_ARG;      // a feature row must fit one CTA
     {
         LaunchScope ls(h, K_VIF_SCAN, st);
-        void* args[] = {&a};
-        cudaError_t e = cudaLaunchCooperativeKernel((const void*)vif_scan_kernel, dim3(h->vif_scan_blocks),
-                                                    dim3(kThreads), args, 0, st);
-        if (e != cudaSuccess) return check_cuda(h, e);
+        vif_scan_kernel<<<(a.capacity + kScanVoxels - 1) / kScanVoxels, kThreads, 0, st>>>(a);
     }
     {
         LaunchScope ls(h, K_VIF_FILL, st);
