@@ -174,6 +174,8 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out) {
     const size_t tiles[2] = {h->scale[0].tiles, h->scale[1].tiles};
     const size_t groups[2] = {(tiles[0] + kTilesPerGroup - 1) / kTilesPerGroup, (tiles[1] + kTilesPerGroup - 1) / kTilesPerGroup};
     const size_t o_tiles = plan.take((tiles[0] + tiles[1]) * sizeof(uint32_t));
+    const size_t marked[2] = {(tiles[0] + 31) / 32, (tiles[1] + 31) / 32};
+    const size_t o_marked = plan.take((marked[0] + marked[1]) * sizeof(uint32_t));
     const size_t o_list = plan.take((tiles[0] + tiles[1]) * sizeof(uint32_t));
     h->scan_reset_words = (int)(groups[0] + groups[1] + 1);
     const size_t o_groups = plan.take((size_t)h->scan_reset_words * sizeof(uint32_t));
@@ -214,6 +216,8 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out) {
     h->scan.tile_voxels[0] = reinterpret_cast<uint32_t*>(base + o_tiles);
     h->scan.tile_voxels[1] = h->scan.tile_voxels[0] + tiles[0];
     h->scan.list = reinterpret_cast<uint32_t*>(base + o_list);
+    h->scan.marked[0] = reinterpret_cast<uint32_t*>(base + o_marked);
+    h->scan.marked[1] = h->scan.marked[0] + marked[0];
     h->scan.group_voxels[0] = reinterpret_cast<uint32_t*>(base + o_groups);
     h->scan.group_voxels[1] = h->scan.group_voxels[0] + groups[0];
     h->scan.listed = h->scan.group_voxels[1] + groups[1];
@@ -346,8 +350,9 @@ static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_poi
     // With two or more frames the batch is taken in two halves: the rows of the first half start to
     // move as soon as ITS points are projected, while the second half is projected on the side stream.
     const int half0 = fused_mark && h->overlap && B >= 2 && h->tune[EMC2_TUNE_SPLIT_BATCH] != 0 ? B / 2 : B;
+    const TileMarks marks = tile_marks(h, B, N);
     if (fused_mark)
-        rc = launch_project_route(h, 0, half0, N, d_points, d_proj, d_uvd, d_vis_mask, d_cam, d_expert, true, d_bev, B, st);
+        rc = launch_project_route(h, 0, half0, N, d_points, d_proj, d_uvd, d_vis_mask, d_cam, d_expert, true, d_bev, B, marks, st);
     if (rc == EMC2_OK && h->overlap) {
         e = cudaEventRecord(h->ev_fork, st);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(h->side, h->ev_fork, 0);
@@ -355,7 +360,7 @@ static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_poi
     }
     if (rc == EMC2_OK && half0 < B) {
         rc = launch_project_route(h, half0, B - half0, N, d_points, d_proj, d_uvd, d_vis_mask, d_cam, d_expert, true,
-                                  nullptr, 0, h->side);
+                                  nullptr, 0, marks, h->side);
         if (rc == EMC2_OK) {
             e = cudaEventRecord(h->ev_half, h->side);
             if (e != cudaSuccess) rc = check_cuda(h, e);
@@ -366,7 +371,7 @@ static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_poi
                              d_bev, vox_st, fused_mark);
     if (rc == EMC2_OK && rc2 == EMC2_OK && B > 0) {
         if (!fused_mark)
-            rc2 = launch_project_route(h, 0, B, N, d_points, d_proj, d_uvd, d_vis_mask, d_cam, d_expert, false, nullptr, 0, st);
+            rc2 = launch_project_route(h, 0, B, N, d_points, d_proj, d_uvd, d_vis_mask, d_cam, d_expert, false, nullptr, 0, marks, st);
         const int tiles = (N + kTile - 1) / kTile;
         if (rc2 == EMC2_OK) {
             launch_route_scan(h, 0, half0, tiles, N, d_offsets, N > 0, st);

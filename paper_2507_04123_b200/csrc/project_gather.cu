@@ -219,6 +219,7 @@ struct PrArgs {
     float4* bev;          // kMark: BEV image to zero (bev_n4 float4), or null
     size_t bev_n4;
     ScanReset reset;      // kMark: state of the rank scan to zero
+    TileMarks marks;      // kMark
 };
 
 // grid = (tiles per frame, B); tiles never straddle frames.  kMark: the kernel also does the
@@ -226,7 +227,7 @@ struct PrArgs {
 // is zeroed, spread over the grid), so that stage 1 starts from marked stores and reads the
 // points once less; the reductions are fire-and-forget and land while the projection computes.
 template <int C, bool kMark>
-__global__ void __launch_bounds__(kThreads) project_route_kernel(const __grid_constant__ PrArgs a) {
+__global__ void __launch_bounds__(kThreads, 8) project_route_kernel(const __grid_constant__ PrArgs a) {
     __shared__ __align__(16) float suvd[kTile * 3];
     __shared__ int hist[EMC2_MAX_EXPERTS];
     __shared__ Camera sP[EMC2_MAX_CAMERAS];
@@ -236,6 +237,9 @@ __global__ void __launch_bounds__(kThreads) project_route_kernel(const __grid_co
     const int npts = min(kTile, a.N - i0);
     const size_t g0 = (size_t)b * a.N + i0;
     if (t < EMC2_MAX_EXPERTS) hist[t] = 0;
+    __shared__ FrameTiles tiles;
+    const bool marks = kMark && a.marks.marked[0] != nullptr;
+    if (marks) begin_tiles(tiles, a.s0, a.s1, (uint32_t)(a.frame0 + b));
     __syncthreads();
     int e = -1;
     if (t < npts) {
@@ -247,7 +251,11 @@ __global__ void __launch_bounds__(kThreads) project_route_kernel(const __grid_co
         } else {
             x = __ldg(p); y = __ldg(p + 1); z = __ldg(p + 2);
         }
-        if (kMark) mark_point(a.s0, a.s1, x, y, z, a.frame0 + b);
+        if (kMark) {
+            int at[2];
+            mark_point(a.s0, a.s1, x, y, z, a.frame0 + b, at);
+            if (marks) note_tiles(tiles, at);
+        }
         const Projected pr = project_point(sP, a.K, x, y, z, a.W, a.H, a.min_depth);
         suvd[t * 3] = pr.u; suvd[t * 3 + 1] = pr.v; suvd[t * 3 + 2] = pr.d;
         a.vis[g0 + t] = (uint8_t)pr.mask;
@@ -271,6 +279,7 @@ __global__ void __launch_bounds__(kThreads) project_route_kernel(const __grid_co
     }
     __syncthreads();
     if (t < a.rp.E) a.tile_counts[((size_t)b * a.tiles + tile) * a.rp.E + t] = hist[t];
+    if (marks) publish_tiles(tiles, a.marks);
     if (kMark) {
         const size_t cta = (size_t)blockIdx.y * gridDim.x + blockIdx.x, nthreads = (size_t)gridDim.x * gridDim.y * kThreads;
         reset_scan(a.reset, cta * kThreads + t, nthreads);
@@ -775,7 +784,7 @@ int launch_project_gather(emc2_bridge* h, int B, int N, const float* d_points, c
 // zeroes the BEV image of that many frames.
 int launch_project_route(emc2_bridge* h, int b0, int B, int N, const float* d_points, const float* d_proj,
                          float* d_uvd, uint8_t* d_vis_mask, int8_t* d_cam, uint8_t* d_expert, bool mark,
-                         float* d_bev_to_zero, int bev_frames, cudaStream_t st) {
+                         float* d_bev_to_zero, int bev_frames, const TileMarks& marks, cudaStream_t st) {
     const emc2_config_t& c = h->cfg;
     const int tiles = (N + kTile - 1) / kTile;
     if (B == 0 || tiles == 0) return EMC2_OK;
@@ -792,6 +801,7 @@ int launch_project_route(emc2_bridge* h, int b0, int B, int N, const float* d_po
     pa.s0 = h->scale[0]; pa.s1 = h->scale[1];
     pa.bev = nullptr; pa.bev_n4 = 0;
     pa.reset = scan_reset(h);
+    pa.marks = marks;
     if (!mark || b0 > 0) { pa.reset.n = 0; pa.reset.totals[0] = pa.reset.totals[1] = nullptr; }
     if (mark && d_bev_to_zero && bev_frames > 0) {
         const size_t bev_n = (size_t)bev_frames * c.point_floats * h->scale[1].dims[1] * h->scale[1].dims[0];

@@ -35,4 +35,9 @@ def rules(tmp_path_factory):
     so.fits.restype, so.fits.argtypes = ctypes.c_int, [u64, u32, u32, u32, u32]
     so.ticket.restype, so.ticket.argtypes = u64, [u32, u32]
     so.tile_frames.restype, so.tile_frames.argtypes = ctypes.c_int64, [ctypes.c_int64, ctypes.c_int64]
+    for f in (so.first_word, so.words_of_frame):
+        f.restype, f.argtypes = u32, [u32, u32, u32]
+    so.most_words.restype, so.most_words.argtypes = u32, [u32, u32]
+    so.four_bits.restype, so.four_bits.argtypes = u32, [u32]
+    so.notes.argtypes = [u64, u64, ctypes.c_int, ctypes.c_int]
     return so

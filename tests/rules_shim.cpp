@@ -15,6 +15,11 @@ int fits(uint64_t first, uint32_t cells, uint32_t points, uint32_t max_ovf, uint
     return over_fits(first, cells, points, max_ovf, max_list);
 }
 int64_t tile_frames(int64_t B, int64_t N) { return frames_of_tile(B, N); }
+uint32_t first_word(uint32_t b, uint32_t cells, uint32_t per) { return frame_first_word(b, cells, per); }
+uint32_t words_of_frame(uint32_t b, uint32_t cells, uint32_t per) { return frame_words(b, cells, per); }
+uint32_t most_words(uint32_t cells, uint32_t per) { return most_frame_words(cells, per); }
+uint32_t four_bits(uint32_t bytes) { return bits_of_bytes(bytes); }
+int notes(uint64_t bytes, uint64_t words, int B, int N) { return keeps_notes(bytes, words, B, N); }
 uint64_t ticket(uint32_t cells, uint32_t points) { return over_ticket(cells, points); }
 
 // Cells of n points (x, y, z), -1 -1 -1 outside the grid; returns for how many of them no divide was needed.

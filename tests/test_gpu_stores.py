@@ -7,7 +7,7 @@ import torch
 
 import emc2_gen as gen
 from emc2_gen.configs import Grid
-from parity import close, np_
+from parity import close, compare_bridge, np_, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -202,3 +202,32 @@ def test_cells_over_the_cap_by_the_length_of_their_lists(oracle, cap):
         cells = np.concatenate([[0], rng.permutation(at[1:-1]), [at[-1]]])       # cell 0 has point 0, the last cell the last point
         pts = centres(cells, TABLE, 4, rng)[None]
         check_voxels(replace(gen.KITTI.with_shape(1, pts.shape[1]), grids=grids), pts, oracle)
+
+
+@pytest.mark.parametrize("base,B,N,cap", [(gen.KITTI, 2, 1001, 0), (gen.KITTI, 9, 257, 0), (gen.KITTI, 32, 33, 0),
+                                          (gen.NUSCENES, 3, 777, 0), (gen.DENSE, 3, 30000, 0), (gen.NUSCENES, 5, 20000, 3),
+                                          (gen.KITTI, 3, 1, 0)], ids=lambda v: getattr(v, "name", str(v)))
+def test_calls_that_note_the_tiles_they_mark(oracle, base, B, N, cap):
+    """Only noted tiles are counted: frames that share a word of notes, the first and last cells of frames among the points,
+    both kinds of store over their caps; notes are cleared for the next call, which has other points or fewer frames."""
+    w = base.with_shape(B, N)
+    w = replace(w, grids=(replace(w.grids[0], max_points=cap), w.grids[1]), feat_c=4)
+    frames = [gen.make_batch(w, frames=[B * i + k for k in range(B)]) for i in range(2)]
+    for g, at in zip(w.grids, (0, -1)):                        # a point in the first cell and one in the last
+        centre = [[m + 0.5 * v for m, v in zip(g.min, g.voxel)], [m + (d - 0.5) * v for m, v, d in zip(g.min, g.voxel, g.dims)]]
+        frames[0]["points"][:, at, :3] = np.float32(centre[at])
+    refs = [oracle.bridge(w, f) for f in frames]
+    for step in ("run", "run_staged"):
+        br = bridge_for(w)
+        for i in (0, 1, 0):
+            d = to_dev(frames[i])
+            bufs = getattr(br, step)(d["points"], d["proj"], d["feat"])
+            br.status()
+            compare_bridge(w, refs[i], bufs)
+        w1 = w.with_shape(1, N)
+        one = {k: np.ascontiguousarray(v[:1]) for k, v in frames[1].items()}
+        d = to_dev(one)
+        compare_bridge(w1, oracle.bridge(w1, one), getattr(br, step)(d["points"], d["proj"], d["feat"]))
+        d = to_dev(frames[1])
+        compare_bridge(w, refs[1], getattr(br, step)(d["points"], d["proj"], d["feat"]))
+        br.close()

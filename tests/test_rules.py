@@ -88,3 +88,27 @@ def test_frames_of_a_tile(rules):
             if most > 2:
                 assert N < 255
     assert rules.tile_frames(32, 1) == 32 and rules.tile_frames(32, 255) == 2 and rules.tile_frames(32, 254) == 3
+
+
+def test_noted_tiles_of_a_frame_have_a_place(rules):
+    """Every tile of a frame lies in the words the rule gives, frames that share a word included, and no frame has more."""
+    for per in (49152, 2048):
+        for cells in (1, 47, 2048, 49152, 49153, 220000, 262144, 1 << 20, 74_638_240, 90_112_000):
+            most = rules.most_words(cells, per)
+            for b in range(0, min(32, (1 << 32) // cells)):
+                first, n = rules.first_word(b, cells, per), rules.words_of_frame(b, cells, per)
+                assert first == b * cells // per // 32 and first + n - 1 == ((b + 1) * cells - 1) // per // 32
+                assert 1 <= n <= most
+
+
+def test_four_bytes_become_four_bits(rules):
+    for v in range(16):
+        assert rules.four_bits(sum((v >> k & 1) << (8 * k) for k in range(4))) == v
+
+
+def test_calls_that_keep_notes(rules):
+    kitti, nuscenes = 15_018_656 + 880_000, 12_439_696 + 1_048_576
+    for frame, words in ((kitti, 64), (nuscenes, 55)):
+        assert not rules.notes(frame, words, 1, 1000)
+        assert rules.notes(frame, words, 2, 1) and rules.notes(frame, words, 32, 1 << 17)
+        assert not rules.notes(frame, words, 32, (1 << 17) + 1) and not rules.notes(frame, 73, 32, 1000)
