@@ -235,6 +235,7 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out) {
     int prio_lo = 0, prio_hi = 0;
     e = cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, prio_hi);
+    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->rows, cudaStreamNonBlocking, prio_lo);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_half, cudaEventDisableTiming);
@@ -342,11 +343,15 @@ static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_poi
     DeviceGuard guard(h->cfg.device);
     if (!guard.ok) return EMC2_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    cudaStream_t vox_st = h->overlap ? h->side : st;
     cudaError_t e = cudaSuccess;
     // One pass over the points serves the projection, the routing and the voxelizer's marking; the
-    // rest of stage 1 then runs on the side stream beside the row traffic of stages 2 - 4.
+    // rest of stage 1 then runs beside the row traffic of stages 2 - 4, one of the two on a stream of the handle.
     const bool fused_mark = rc2 == EMC2_OK && B > 0 && N > 0 && h->tune[EMC2_TUNE_MARK_IN_PROJECTION] != 0;
+    const size_t row_bytes = (size_t)B * N * h->cfg.feat_c * sizeof(float) * (d_gathered ? 2 : 1);
+    const bool rows_aside = fused_mark && h->overlap && !h_feat && h->tune[EMC2_TUNE_SPLIT_BATCH] == 0 &&
+                            rows_on_other_stream((uint64_t)B * N, row_bytes, d_gathered != nullptr);
+    const cudaStream_t other = rows_aside ? h->rows : h->side;
+    const cudaStream_t vox_st = h->overlap && !rows_aside ? other : st, row_st = rows_aside ? other : st;
     // With two or more frames the batch is taken in two halves: the rows of the first half start to
     // move as soon as ITS points are projected, while the second half is projected on the side stream.
     const int half0 = fused_mark && h->overlap && B >= 2 && h->tune[EMC2_TUNE_SPLIT_BATCH] != 0 ? B / 2 : B;
@@ -355,7 +360,7 @@ static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_poi
         rc = launch_project_route(h, 0, half0, N, d_points, d_proj, d_uvd, d_vis_mask, d_cam, d_expert, true, d_bev, B, marks, st);
     if (rc == EMC2_OK && h->overlap) {
         e = cudaEventRecord(h->ev_fork, st);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(h->side, h->ev_fork, 0);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(other, h->ev_fork, 0);
         if (e != cudaSuccess) return check_cuda(h, e);
     }
     if (rc == EMC2_OK && half0 < B) {
@@ -368,13 +373,13 @@ static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_poi
     }
     if (rc == EMC2_OK)
         rc = launch_voxelize(h, B, N, d_points, d_coords, d_counts, d_mean, d_point_voxel, capacity, d_num_voxels,
-                             d_bev, vox_st, fused_mark);
+                             d_bev, vox_st, fused_mark, rows_aside);
     if (rc == EMC2_OK && rc2 == EMC2_OK && B > 0) {
         if (!fused_mark)
             rc2 = launch_project_route(h, 0, B, N, d_points, d_proj, d_uvd, d_vis_mask, d_cam, d_expert, false, nullptr, 0, marks, st);
         const int tiles = (N + kTile - 1) / kTile;
         if (rc2 == EMC2_OK) {
-            launch_route_scan(h, 0, half0, tiles, N, d_offsets, N > 0, st);
+            launch_route_scan(h, 0, half0, tiles, N, d_offsets, N > 0 && !rows_aside, row_st);
             if (h_feat) {
                 const emc2_config_t& c = h->cfg;
                 const size_t bytes = (size_t)B * c.num_cameras * c.feat_h * c.feat_w * c.feat_c * sizeof(float);
@@ -384,7 +389,7 @@ static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_poi
         }
         if (rc2 == EMC2_OK)
             rc2 = launch_gather_scatter(h, 0, half0, N, d_points, d_feat, d_uvd, d_cam, d_gathered, d_expert, d_perm,
-                                        d_points_out, d_feat_out, !h_feat, st);
+                                        d_points_out, d_feat_out, !h_feat, row_st);
         if (rc2 == EMC2_OK && half0 < B) {
             e = cudaStreamWaitEvent(st, h->ev_half, 0);
             if (e != cudaSuccess) rc2 = check_cuda(h, e);
@@ -395,9 +400,9 @@ static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_poi
             }
         }
     }
-    // Join even after an error, so that `cuda_stream` never runs ahead of stage 1.
+    // Join even after an error, so that `cuda_stream` never runs ahead of the other stream.
     if (h->overlap) {
-        e = cudaEventRecord(h->ev_join, h->side);
+        e = cudaEventRecord(h->ev_join, other);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(st, h->ev_join, 0);
     }
     if (rc != EMC2_OK) return rc;
@@ -618,6 +623,7 @@ int emc2_bridge_destroy(emc2_bridge_t* h) {
     if (h->ev_join) cudaEventDestroy(h->ev_join);
     if (h->ev_half) cudaEventDestroy(h->ev_half);
     if (h->side) cudaStreamDestroy(h->side);
+    if (h->rows) cudaStreamDestroy(h->rows);
     if (h->slab && cudaFree(h->slab) != cudaSuccess) rc = EMC2_ERR_CUDA;
     if (h->arm.slab && cudaFree(h->arm.slab) != cudaSuccess) rc = EMC2_ERR_CUDA;
     delete h;

@@ -211,7 +211,8 @@ struct emc2_bridge {
     emc2::DedupArm arm;
     int num_sms = 0;               // multiprocessors of the handle's device
     bool overlap = true;           // emc2_bridge_run puts stage 1 on `side`
-    cudaStream_t side = nullptr;   // stream of stage 1 inside emc2_bridge_run
+    cudaStream_t side = nullptr;   // stream of stage 1 inside emc2_bridge_run ...
+    cudaStream_t rows = nullptr;   // ... or, in small calls, of the rows
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_half = nullptr;
     int last_cuda_error = 0;
     bool profiling = false;
@@ -236,11 +237,12 @@ struct LaunchScope {
 int check_cuda(emc2_bridge* h, cudaError_t e);
 
 // `marked`: the cells of this batch are already marked and the BEV image zeroed (by the projection
-// kernel of the one-call path); the marking pass is then skipped.
+// kernel of the one-call path); the marking pass is then skipped.  `chained`: that kernel is the call's previous work on
+// `st`, see launch_chained.
 int launch_voxelize(emc2_bridge* h, int B, int N, const float* d_points, int32_t* const d_coords[2],
                     int32_t* const d_counts[2], float* const d_mean[2], int32_t* const d_point_voxel[2],
                     const int32_t capacity[2], int32_t* d_num_voxels, float* d_bev, cudaStream_t st,
-                    bool marked = false);
+                    bool marked = false, bool chained = false);
 int dedup_arm_alloc(emc2_bridge* h);
 int launch_dedup_arm(emc2_bridge* h, int s, int design, int B, int N, const float* d_points, int capacity,
                      int32_t* d_num_voxels, cudaStream_t st);

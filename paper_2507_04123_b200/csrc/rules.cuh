@@ -92,6 +92,18 @@ inline long long frames_of_tile(long long B, long long N) {
     return B < most ? B : most;
 }
 
+// ---- which branch of a call of all stages stays on the caller's stream
+// Stage 1 is a chain of four kernels.  In a small call it is the longer branch and waiting for another stream, at its begin
+// and at the end of the call, costs more than it can hide: the rows go to the other stream instead.  In a large call the
+// rows are the longer branch, and stage 1, which shares the chip with them, needs its stream's priority.
+// `row_bytes`: feature rows written.  us per call, rows on the caller's stream / stage 1 on it: one frame of 120,000 points,
+// 64 channels, dispatched rows only (31 MB) 37.7 / 28.9; 3 x 33,333 x 80 channels (64 MB) 53.8 / 50.5, 8 x 16,384 (84 MB)
+// 93.5 / 86.9, one of 240,000 (154 MB) 75.3 / 72.2; but 4 x 120,000 x 64 channels (246 MB) 97.0 / 103.1, one of 480,000 with
+// dispatched rows only (123 MB) 67.6 / 69.8.
+inline bool rows_on_other_stream(uint64_t points, uint64_t row_bytes, bool both_rows) {
+    return points <= 320000 && row_bytes <= (both_rows ? 160000000u : 96000000u);
+}
+
 // ---- notes of the tiles of a store that the marking pass touched: a bit per tile, 32 tiles to a word
 // Words that hold the tiles of frame b, for frames of `cells` cells and tiles of `per_tile` cells: the first, how many, and
 // at most how many of any frame.

@@ -710,7 +710,7 @@ vox_finalize_kernel(const float* __restrict__ pts, long long total, AccumArgs a,
 template <int C>
 int run_voxelize(emc2_bridge* h, int B, int N, const float* d_points, int32_t* const d_coords[2],
                  int32_t* const d_counts[2], float* const d_mean[2], int32_t* const d_point_voxel[2],
-                 const int32_t capacity[2], int32_t* d_num_voxels, float* d_bev, cudaStream_t st, bool marked) {
+                 const int32_t capacity[2], int32_t* d_num_voxels, float* d_bev, cudaStream_t st, bool marked, bool chained) {
     const long long total = (long long)B * N;
     const int ptiles = (int)((total + kThreads - 1) / kThreads);   // one point per thread (two measured 1 - 3 % slower per step)
     ScanArgs sa;
@@ -767,11 +767,11 @@ int run_voxelize(emc2_bridge* h, int B, int N, const float* d_points, int32_t* c
     if (tiles > 0) {
         {
             LaunchScope ls(h, K_VOX_COUNT, st);
-            // In the one-call path the first kernel of the side stream: its predecessor is on another stream.
+            // In the one-call path its predecessor can be on another stream.
             if (keeps_tile_marks(h, B, N))
-                launch_kernel(!marked, vox_count_marked_kernel, min(tiles / kCountTiles, 8 * h->num_sms), kThreads, 0, st, sa);
+                launch_kernel(!marked || chained, vox_count_marked_kernel, min(tiles / kCountTiles, 8 * h->num_sms), kThreads, 0, st, sa);
             else
-                launch_kernel(!marked, vox_count_kernel, tiles / kCountTiles, kThreads, 0, st, sa);
+                launch_kernel(!marked || chained, vox_count_kernel, tiles / kCountTiles, kThreads, 0, st, sa);
         }
         LaunchScope ls(h, K_VOX_RANK, st);
         launch_chained(vox_rank_kernel, min(tiles, kRankCtas * h->num_sms), kRankThreads, 0, st, sa);
@@ -806,12 +806,12 @@ int run_voxelize(emc2_bridge* h, int B, int N, const float* d_points, int32_t* c
 
 int launch_voxelize(emc2_bridge* h, int B, int N, const float* d_points, int32_t* const d_coords[2],
                     int32_t* const d_counts[2], float* const d_mean[2], int32_t* const d_point_voxel[2],
-                    const int32_t capacity[2], int32_t* d_num_voxels, float* d_bev, cudaStream_t st, bool marked) {
+                    const int32_t capacity[2], int32_t* d_num_voxels, float* d_bev, cudaStream_t st, bool marked, bool chained) {
     if (h->cfg.point_floats == 4)
         return run_voxelize<4>(h, B, N, d_points, d_coords, d_counts, d_mean, d_point_voxel, capacity,
-                               d_num_voxels, d_bev, st, marked);
+                               d_num_voxels, d_bev, st, marked, chained);
     return run_voxelize<5>(h, B, N, d_points, d_coords, d_counts, d_mean, d_point_voxel, capacity,
-                           d_num_voxels, d_bev, st, marked);
+                           d_num_voxels, d_bev, st, marked, chained);
 }
 
 }  // namespace emc2

@@ -108,6 +108,37 @@ def test_one_call_replays_from_a_graph_under_every_tuning(oracle, tuning, B):
         br.close()
 
 
+@pytest.mark.parametrize("cf,rows", [(64, True), (1024, True), (1024, False)])
+def test_either_branch_of_a_call_beside_the_callers_stream(oracle, cf, rows):
+    """Small calls put the rows on the other stream, calls of many row bytes stage 1: directly, and from a graph."""
+    w = replace(gen.KITTI.with_shape(1, 24001), feat_c=cf)
+    frames = [gen.make_batch(w, frames=[i]) for i in range(2)]
+    br = bridge_for(w)
+    d = to_dev(frames[0])
+    bufs = br.run(d["points"], d["proj"], d["feat"])
+    gathered = bufs["pg"]["gathered"]
+    if not rows:
+        bufs["pg"]["gathered"] = None
+    torch.cuda.synchronize()
+    graph = captured(lambda: br.run(d["points"], d["proj"], d["feat"], bufs))
+    assert chained_launches(graph) >= 4
+    for call in (lambda: br.run(d["points"], d["proj"], d["feat"], bufs), graph.replay):
+        for batch in (frames[1], frames[0]):
+            ref = oracle.bridge(w, batch)
+            for k, v in batch.items():
+                d[k].copy_(torch.from_numpy(v))
+            for t in (bufs["rd"]["feat_out"], bufs["vox"]["bev"], gathered):
+                t.fill_(-1.0)
+            call()
+            torch.cuda.synchronize()
+            br.status()
+            shown = {**bufs, "pg": {**bufs["pg"], "gathered": gathered if rows else torch.from_numpy(ref["gathered"])}}
+            compare_bridge(w, ref, shown)
+            assert rows or bool((gathered == -1.0).all())
+    del graph
+    br.close()
+
+
 def test_stage_calls_and_calls_without_points_in_a_graph():
     """With N = 0 the route scan is the first kernel of its call: nothing is chained to what the stream held before."""
     w = gen.KITTI.with_shape(2, 1000)
