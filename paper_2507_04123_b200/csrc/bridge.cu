@@ -239,6 +239,8 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out) {
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_half, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_copy, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_scan, cudaEventDisableTiming);
     if (e != cudaSuccess) { emc2_bridge_destroy(h); return EMC2_ERR_CUDA; }
     *out = h;
     return EMC2_OK;
@@ -313,15 +315,24 @@ int emc2_route_dispatch(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_p
                                  d_points_out, d_feat_out, static_cast<cudaStream_t>(cuda_stream));
 }
 
-// emc2_bridge_run; `h_feat` not null: the feature maps are in host memory and are copied into d_feat just before the
-// rows need them, so that the copy, the longest part of a frame from the host, runs beside stage 1 (one KITTI-shaped
-// frame: 246 -> 233 us per call).
+// What emc2_bridge_run_host adds to emc2_bridge_run.
+struct HostEnds {
+    const float* feat;          // feature maps in host memory
+    int32_t* offsets;           // where the results go, or null
+    int32_t* num_voxels;
+};
+
+// emc2_bridge_run; with `host`, the feature maps are copied into d_feat first.  Their copy is the longest part of a frame
+// from the host: it has a stream of its own (h->rows, after the copies of the points, so that the bus does not pause for
+// the projection), only the rows wait for it, and the copies of the results go beside the rows.  One KITTI-shaped frame:
+// 246 us per call with the maps copied first, 223 with all copies in turn on the caller's stream, 208 so; its 9.4 MB alone
+// take 177 on the bus.
 static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_points, const float* d_proj,
                     float* d_feat, int32_t* const d_coords[2], int32_t* const d_counts[2],
                     float* const d_mean[2], int32_t* const d_point_voxel[2], const int32_t capacity[2],
                     int32_t* d_num_voxels, float* d_bev, float* d_uvd, uint8_t* d_vis_mask, int8_t* d_cam,
                     float* d_gathered, uint8_t* d_expert, int32_t* d_offsets, int32_t* d_perm,
-                    float* d_points_out, float* d_feat_out, const float* h_feat, void* cuda_stream) {
+                    float* d_points_out, float* d_feat_out, const HostEnds* host, void* cuda_stream) {
     // The stage calls validate before they enqueue anything; a host-detected error in stage 2 or
     // 3 - 4 leaves stage 1 enqueued, exactly as three separate calls would.
     if (!h) return EMC2_ERR_INVALID_ARG;
@@ -348,7 +359,7 @@ static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_poi
     // rest of stage 1 then runs beside the row traffic of stages 2 - 4, one of the two on a stream of the handle.
     const bool fused_mark = rc2 == EMC2_OK && B > 0 && N > 0 && h->tune[EMC2_TUNE_MARK_IN_PROJECTION] != 0;
     const size_t row_bytes = (size_t)B * N * h->cfg.feat_c * sizeof(float) * (d_gathered ? 2 : 1);
-    const bool rows_aside = fused_mark && h->overlap && !h_feat && h->tune[EMC2_TUNE_SPLIT_BATCH] == 0 &&
+    const bool rows_aside = fused_mark && h->overlap && !host && h->tune[EMC2_TUNE_SPLIT_BATCH] == 0 &&
                             rows_on_other_stream((uint64_t)B * N, row_bytes, d_gathered != nullptr);
     const cudaStream_t other = rows_aside ? h->rows : h->side;
     const cudaStream_t vox_st = h->overlap && !rows_aside ? other : st, row_st = rows_aside ? other : st;
@@ -356,6 +367,14 @@ static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_poi
     // move as soon as ITS points are projected, while the second half is projected on the side stream.
     const int half0 = fused_mark && h->overlap && B >= 2 && h->tune[EMC2_TUNE_SPLIT_BATCH] != 0 ? B / 2 : B;
     const TileMarks marks = tile_marks(h, B, N);
+    const cudaStream_t copy_st = h->overlap ? h->rows : st;
+    const size_t feat_bytes = (size_t)B * h->cfg.num_cameras * h->cfg.feat_h * h->cfg.feat_w * h->cfg.feat_c * sizeof(float);
+    const bool early_copy = host && rc2 == EMC2_OK && B > 0 && h->overlap;
+    if (early_copy) {
+        e = cudaEventRecord(h->ev_copy, st);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(copy_st, h->ev_copy, 0);
+        if (e != cudaSuccess) rc2 = check_cuda(h, e);
+    }
     if (fused_mark)
         rc = launch_project_route(h, 0, half0, N, d_points, d_proj, d_uvd, d_vis_mask, d_cam, d_expert, true, d_bev, B, marks, st);
     if (rc == EMC2_OK && h->overlap) {
@@ -380,16 +399,21 @@ static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_poi
         const int tiles = (N + kTile - 1) / kTile;
         if (rc2 == EMC2_OK) {
             launch_route_scan(h, 0, half0, tiles, N, d_offsets, N > 0 && !rows_aside, row_st);
-            if (h_feat) {
-                const emc2_config_t& c = h->cfg;
-                const size_t bytes = (size_t)B * c.num_cameras * c.feat_h * c.feat_w * c.feat_c * sizeof(float);
-                e = cudaMemcpyAsync(d_feat, h_feat, bytes, cudaMemcpyHostToDevice, st);
+            if (early_copy) {
+                // Enqueued after the kernels: from memory that is not page-locked the host copies while they run.
+                e = cudaEventRecord(h->ev_scan, st);
+                if (e == cudaSuccess) e = cudaMemcpyAsync(d_feat, host->feat, feat_bytes, cudaMemcpyHostToDevice, copy_st);
+                if (e == cudaSuccess) e = cudaEventRecord(h->ev_copy, copy_st);
+                if (e == cudaSuccess) e = cudaStreamWaitEvent(st, h->ev_copy, 0);
+                if (e != cudaSuccess) rc2 = check_cuda(h, e);
+            } else if (host) {
+                e = cudaMemcpyAsync(d_feat, host->feat, feat_bytes, cudaMemcpyHostToDevice, st);
                 if (e != cudaSuccess) rc2 = check_cuda(h, e);
             }
         }
         if (rc2 == EMC2_OK)
             rc2 = launch_gather_scatter(h, 0, half0, N, d_points, d_feat, d_uvd, d_cam, d_gathered, d_expert, d_perm,
-                                        d_points_out, d_feat_out, !h_feat, row_st);
+                                        d_points_out, d_feat_out, !host, row_st);
         if (rc2 == EMC2_OK && half0 < B) {
             e = cudaStreamWaitEvent(st, h->ev_half, 0);
             if (e != cudaSuccess) rc2 = check_cuda(h, e);
@@ -399,6 +423,24 @@ static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_poi
                                             d_perm, d_points_out, d_feat_out, true, st);
             }
         }
+    }
+    // The results go back beside the rows; their copies are enqueued last, because a copy into memory that is not
+    // page-locked makes the host wait.
+    if (host && rc == EMC2_OK && rc2 == EMC2_OK) {
+        if (host->offsets && d_offsets && B > 0) {
+            if (early_copy) e = cudaStreamWaitEvent(copy_st, h->ev_scan, 0);
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(host->offsets, d_offsets, (size_t)B * (h->cfg.num_experts + 1) * sizeof(int32_t),
+                                    cudaMemcpyDeviceToHost, copy_st);
+        }
+        if (e == cudaSuccess && host->num_voxels)
+            e = cudaMemcpyAsync(host->num_voxels, d_num_voxels, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, vox_st);
+        if (e != cudaSuccess) rc2 = check_cuda(h, e);
+    }
+    if (early_copy) {
+        e = cudaEventRecord(h->ev_copy, copy_st);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(st, h->ev_copy, 0);
+        if (e != cudaSuccess && rc2 == EMC2_OK) rc2 = check_cuda(h, e);
     }
     // Join even after an error, so that `cuda_stream` never runs ahead of the other stream.
     if (h->overlap) {
@@ -525,15 +567,9 @@ int emc2_bridge_run_host(emc2_bridge_t* h, int32_t B, int32_t N, const float* h_
         if (e == cudaSuccess) e = cudaMemcpyAsync(d_proj, h_proj, prj, cudaMemcpyHostToDevice, st);
         if (e != cudaSuccess) return check_cuda(h, e);
     }
-    rc = run_bridge(h, B, N, d_points, d_proj, d_feat, d_coords, d_counts, d_mean, d_point_voxel, capacity, d_num_voxels, d_bev,
-                      d_uvd, d_vis_mask, d_cam, d_gathered, d_expert, d_offsets, d_perm, d_points_out, d_feat_out, h_feat, cuda_stream);
-    if (rc != EMC2_OK) return rc;
-    if (h_offsets && d_offsets && B > 0)
-        e = cudaMemcpyAsync(h_offsets, d_offsets, (size_t)B * (c.num_experts + 1) * sizeof(int32_t),
-                            cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && h_num_voxels && d_num_voxels)
-        e = cudaMemcpyAsync(h_num_voxels, d_num_voxels, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, st);
-    return check_cuda(h, e);
+    const HostEnds host = {h_feat, h_offsets, h_num_voxels};
+    return run_bridge(h, B, N, d_points, d_proj, d_feat, d_coords, d_counts, d_mean, d_point_voxel, capacity, d_num_voxels, d_bev,
+                      d_uvd, d_vis_mask, d_cam, d_gathered, d_expert, d_offsets, d_perm, d_points_out, d_feat_out, &host, cuda_stream);
 }
 
 int emc2_features_channels_last(emc2_bridge_t* h, int32_t B, const float* d_planar, float* d_feat,
@@ -622,6 +658,8 @@ int emc2_bridge_destroy(emc2_bridge_t* h) {
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
     if (h->ev_join) cudaEventDestroy(h->ev_join);
     if (h->ev_half) cudaEventDestroy(h->ev_half);
+    if (h->ev_copy) cudaEventDestroy(h->ev_copy);
+    if (h->ev_scan) cudaEventDestroy(h->ev_scan);
     if (h->side) cudaStreamDestroy(h->side);
     if (h->rows) cudaStreamDestroy(h->rows);
     if (h->slab && cudaFree(h->slab) != cudaSuccess) rc = EMC2_ERR_CUDA;

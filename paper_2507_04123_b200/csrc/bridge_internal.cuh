@@ -212,8 +212,8 @@ struct emc2_bridge {
     int num_sms = 0;               // multiprocessors of the handle's device
     bool overlap = true;           // emc2_bridge_run puts stage 1 on `side`
     cudaStream_t side = nullptr;   // stream of stage 1 inside emc2_bridge_run ...
-    cudaStream_t rows = nullptr;   // ... or, in small calls, of the rows
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_half = nullptr;
+    cudaStream_t rows = nullptr;   // ... or, in small calls, of the rows; of the maps' copy in emc2_bridge_run_host
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_half = nullptr, ev_copy = nullptr, ev_scan = nullptr;
     int last_cuda_error = 0;
     bool profiling = false;
     int64_t launches[emc2::K_KINDS] = {0};

@@ -77,6 +77,36 @@ def test_host_frame_replays_from_a_graph(oracle):
     br.close()
 
 
+@pytest.mark.parametrize("overlap", [True, False])
+@pytest.mark.parametrize("pinned", [True, False])
+def test_host_frames_one_behind_another(oracle, overlap, pinned):
+    """The maps are copied on a stream of their own: not before an earlier call's rows have read the last ones, and the results
+    are back when the caller's stream is through."""
+    w = gen.KITTI.with_shape(2, 20001)
+    frames = [gen.make_batch(w, frames=[2 * i, 2 * i + 1]) for i in range(3)]
+    br = bridge_for(w)
+    br.set_overlap(overlap)
+    d = to_dev(frames[0])
+    buffers = [br.run(d["points"], d["proj"], d["feat"]) for _ in frames]
+    hosts = [{k: torch.from_numpy(v.copy()) for k, v in f.items()} for f in frames]
+    if pinned:
+        hosts = [{k: v.pin_memory() for k, v in h.items()} for h in hosts]
+    staging = {k: torch.zeros_like(v, device="cuda") for k, v in hosts[0].items()}
+    results = [(torch.zeros((w.B, w.num_experts + 1), dtype=torch.int32).pin_memory(), torch.zeros((2,), dtype=torch.int32).pin_memory())
+               for _ in frames]
+    torch.cuda.synchronize()
+    for host, bufs, res in zip(hosts, buffers, results):       # all enqueued before the first is through
+        br.run_host(host, staging, bufs, *res)
+    torch.cuda.current_stream().synchronize()
+    for batch, bufs, (off, nv) in zip(frames, buffers, results):
+        ref = oracle.bridge(w, batch)
+        assert np.array_equal(off.numpy(), ref["offsets"])
+        assert nv.tolist() == [ref["vox0"]["num_voxels"], ref["vox1"]["num_voxels"]]
+        compare_bridge(w, ref, bufs)
+    br.status()
+    br.close()
+
+
 @pytest.mark.parametrize("B", [2, 3])
 @pytest.mark.parametrize("tuning", [{}, {"split_batch": 1}, {"mark_in_projection": 0}, {"dedup_pillars": 1},
                                     {"dedup_fine": 2, "dedup_pillars": 2}])
