@@ -162,10 +162,11 @@ int emc2_route_dispatch(emc2_bridge_t* bridge, int32_t B, int32_t N, const float
  * every feature row is blended once and stored both at its row of d_gathered and at its slot of
  * d_feat_out, so the rows are not read back.  The pass over the points that
  * projects and routes them also marks their voxel cells, so stage 1 reads the points once less.
- * The rest of stage 1 does not depend on stages 2 - 4, so the library runs it on a stream of its own
- * (created with the handle, highest priority) beside them: it starts once that first pass, and with it
- * the work already queued on `cuda_stream`, has finished, and `cuda_stream` waits for it before the
- * call's work counts as complete.  Seen from
+ * The rest of stage 1 does not depend on stages 2 - 4, so the library runs it beside them, on a stream
+ * of its own (created with the handle, highest priority); in small calls, where stage 1 is the longer
+ * branch, it stays on `cuda_stream` and the rows go to another stream of the handle (lowest priority).
+ * The other stream starts once that first pass, and with it the work already queued on `cuda_stream`,
+ * has finished, and `cuda_stream` waits for it before the call's work counts as complete.  Seen from
  * `cuda_stream` the call therefore behaves like the three calls, only shorter.  No allocation,
  * no host synchronisation.  d_gathered may be NULL for a caller who consumes only the dispatched
  * rows (d_feat_out with d_perm): the rows in point order are then not stored, which saves their
@@ -182,7 +183,8 @@ int emc2_bridge_run(emc2_bridge_t* bridge, int32_t B, int32_t N, const float* d_
  * of h_points [B, N, C], h_proj [B, K, 3, 4] and h_feat [B, K, Hf, Wf, Cf] into the caller's device
  * buffers d_points, d_proj, d_feat (the maps last, beside the work that does not need them) and
  * emc2_bridge_run on them with the same outputs, then the copies of d_offsets [B, E+1] and
- * d_num_voxels [2] into h_offsets and h_num_voxels (either may be NULL: not copied).  Nothing is synchronised: the host buffers must stay valid and unchanged until
+ * d_num_voxels [2] into h_offsets and h_num_voxels (either may be NULL: not copied).  The copies of the feature
+ * maps and of the results run on streams of the handle, ordered like the kernels.  Nothing is synchronised: the host buffers must stay valid and unchanged until
  * the stream has passed the call; the copies are asynchronous only for page-locked host memory
  * (which stream capture requires).  A
  * caller who alternates between two handles, streams and buffer sets overlaps one frame's copies with
@@ -304,7 +306,7 @@ int emc2_occlusion(emc2_bridge_t* bridge, int32_t B, int32_t N, const float* d_p
 int emc2_scene_route(emc2_bridge_t* bridge, int32_t B, const int32_t* d_offsets, const uint8_t* priority,
                      int32_t min_points, int32_t* d_scene_expert, void* cuda_stream);
 
-/* Turns the side stream of emc2_bridge_run off (0) or on (non-zero, the default).  Off, every
+/* Turns the handle's own streams in emc2_bridge_run off (0) or on (non-zero, the default).  Off, every
  * kernel of the call is enqueued on `cuda_stream` itself, one after another: for callers that
  * want no second stream, and for timing kernels one at a time. */
 int emc2_bridge_set_overlap(emc2_bridge_t* bridge, int enable);
