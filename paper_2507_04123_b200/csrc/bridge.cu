@@ -419,9 +419,14 @@ static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_poi
             if (e != cudaSuccess) rc2 = check_cuda(h, e);
             else {
                 launch_route_scan(h, half0, B - half0, tiles, N, d_offsets + (size_t)half0 * (h->cfg.num_experts + 1), false, st);
+                if (early_copy) {                         // the copy of the offsets takes those of both halves
+                    e = cudaEventRecord(h->ev_scan, st);
+                    if (e != cudaSuccess) rc2 = check_cuda(h, e);
+                }
+            }
+            if (rc2 == EMC2_OK)
                 rc2 = launch_gather_scatter(h, half0, B - half0, N, d_points, d_feat, d_uvd, d_cam, d_gathered, d_expert,
                                             d_perm, d_points_out, d_feat_out, true, st);
-            }
         }
     }
     // The results go back beside the rows; their copies are enqueued last, because a copy into memory that is not

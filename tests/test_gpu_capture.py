@@ -108,6 +108,45 @@ def test_host_frames_one_behind_another(oracle, overlap, pinned):
 
 
 @pytest.mark.parametrize("B", [2, 3])
+@pytest.mark.parametrize("tuning", [{}, {"split_batch": 1}, {"mark_in_projection": 0}, {"split_batch": 1, "mark_in_projection": 0},
+                                    {"dedup_fine": 2, "dedup_pillars": 1}], ids=str)
+def test_host_frame_under_every_tuning(oracle, tuning, B):
+    """The results are copied after the kernels that write them, whichever frames those are launched for: directly and from
+    a graph, with nothing of an earlier call in the buffers."""
+    w = gen.KITTI.with_shape(B, 20001)
+    frames = [gen.make_batch(w, frames=list(range(B * i, B * i + B))) for i in range(2)]
+    for overlap in (True, False):
+        br = bridge_for(w)
+        br.set_overlap(overlap)
+        for knob, value in tuning.items():
+            br.set_tuning(knob, value)
+        host = {k: torch.from_numpy(v.copy()).pin_memory() for k, v in frames[0].items()}
+        staging = {k: torch.zeros_like(v, device="cuda") for k, v in host.items()}
+        d = to_dev(frames[0])
+        bufs = br.run(d["points"], d["proj"], d["feat"])
+        h_off = torch.zeros((B, w.num_experts + 1), dtype=torch.int32).pin_memory()
+        h_nv = torch.zeros((2,), dtype=torch.int32).pin_memory()
+        torch.cuda.synchronize()
+        graph = captured(lambda: br.run_host(host, staging, bufs, h_off, h_nv))
+        for call in (lambda: br.run_host(host, staging, bufs, h_off, h_nv), graph.replay):
+            for batch in (frames[1], frames[0]):
+                for k, v in batch.items():
+                    host[k].copy_(torch.from_numpy(v))
+                for t in (h_off, h_nv, bufs["rd"]["offsets"], bufs["vox"]["num_voxels"], bufs["rd"]["feat_out"]):
+                    t.fill_(-1)
+                torch.cuda.synchronize()
+                call()
+                torch.cuda.synchronize()
+                br.status()
+                ref = oracle.bridge(w, batch)
+                assert np.array_equal(h_off.numpy(), ref["offsets"])
+                assert h_nv.tolist() == [ref["vox0"]["num_voxels"], ref["vox1"]["num_voxels"]]
+                compare_bridge(w, ref, bufs)
+        del graph
+        br.close()
+
+
+@pytest.mark.parametrize("B", [2, 3])
 @pytest.mark.parametrize("tuning", [{}, {"split_batch": 1}, {"mark_in_projection": 0}, {"dedup_pillars": 1},
                                     {"dedup_fine": 2, "dedup_pillars": 2}])
 def test_one_call_replays_from_a_graph_under_every_tuning(oracle, tuning, B):
