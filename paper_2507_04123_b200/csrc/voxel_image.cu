@@ -200,14 +200,25 @@ __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads) vif_mean_kernel
 // Mean of the p x p window of map texels that pooled texel (ty, tx) of map `map` stands for, column c:
 // the same sum, in the same order, as pool_features_kernel (rows outer, columns inner, one multiply by
 // the reciprocal of the texel count), so the value is the pooled map's, bit for bit.
+template <int PW>
 __device__ __forceinline__ float4 window_mean(const VifArgs& a, uint32_t map, int ty, int tx, int c, int cf4) {
-    const int j0 = ty * a.pool, j1 = min(a.Hf, j0 + a.pool), i0 = tx * a.pool, i1 = min(a.Wf, i0 + a.pool);
+    const int p = PW > 0 ? PW : a.pool;
+    const int j0 = ty * p, j1 = min(a.Hf, j0 + p), i0 = tx * p, i1 = min(a.Wf, i0 + p);
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int j = j0; j < j1; ++j) {
-        const float4* row = a.feat + (((size_t)map * a.Hf + j) * a.Wf + i0) * cf4 + c;
-        for (int x = 0; x < i1 - i0; ++x) {
-            const float4 v = __ldg(row + (size_t)x * cf4);
-            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+    auto add = [&](const float4& v) { s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w; };
+    const float4* row = a.feat + (((size_t)map * a.Hf + j0) * a.Wf + i0) * cf4 + c;
+    const uint32_t step = (uint32_t)a.Wf * (uint32_t)cf4;
+    if (PW > 0) {
+#pragma unroll
+        for (int j = 0; j < PW; ++j)
+#pragma unroll
+            for (int x = 0; x < PW; ++x)
+                if (j < j1 - j0 && x < i1 - i0) add(__ldg(row + (uint32_t)j * step + (uint32_t)x * (uint32_t)cf4));
+    } else {
+        for (int j = j0; j < j1; ++j, row += step) {
+            const float4* at = row;
+#pragma unroll 4
+            for (int x = i0; x < i1; ++x, at += cf4) add(__ldg(at));
         }
     }
     const float inv = 1.0f / (float)((j1 - j0) * (i1 - i0));
@@ -215,6 +226,7 @@ __device__ __forceinline__ float4 window_mean(const VifArgs& a, uint32_t map, in
 }
 
 // gather_column on the pooled map that is never materialised: the four taps are window means.
+template <int PW>
 __device__ __forceinline__ float4 pooled_column(const VifArgs& a, const uint4& rec, int c, int cf4) {
     if (rec.x == kZeroRow) return make_float4(0.f, 0.f, 0.f, 0.f);
     uint32_t t = rec.x;
@@ -223,10 +235,10 @@ __device__ __forceinline__ float4 pooled_column(const VifArgs& a, const uint4& r
     const int y0 = (int)(t % (uint32_t)a.Hp);
     const uint32_t map = t / (uint32_t)a.Hp;
     const int x1 = x0 + (int)(rec.y & 1u), y1 = y0 + (int)((rec.y >> 1) & 1u);
-    const float4 f00 = window_mean(a, map, y0, x0, c, cf4);
-    const float4 f01 = x1 != x0 ? window_mean(a, map, y0, x1, c, cf4) : f00;
-    const float4 f10 = y1 != y0 ? window_mean(a, map, y1, x0, c, cf4) : f00;
-    const float4 f11 = y1 != y0 ? (x1 != x0 ? window_mean(a, map, y1, x1, c, cf4) : f10) : f01;
+    const float4 f00 = window_mean<PW>(a, map, y0, x0, c, cf4);
+    const float4 f01 = x1 != x0 ? window_mean<PW>(a, map, y0, x1, c, cf4) : f00;
+    const float4 f10 = y1 != y0 ? window_mean<PW>(a, map, y1, x0, c, cf4) : f00;
+    const float4 f11 = y1 != y0 ? (x1 != x0 ? window_mean<PW>(a, map, y1, x1, c, cf4) : f10) : f01;
     return blend(f00, f01, f10, f11, __uint_as_float(rec.z), __uint_as_float(rec.w));
 }
 
@@ -238,9 +250,13 @@ __device__ __forceinline__ float4 pooled_column(const VifArgs& a, const uint4& r
 // length of the one after it are.  Two voxels at once without that took 283.3 us for both scales of four nuScenes-shaped
 // frames, this 273.5; 12 rows and 40 registers (48 warps instead of 40) 275.0 without, 307.8 with it (it spills); a CTA per
 // 16 voxels instead of a fixed grid 382.  Bound by the taps' way from L2 to the SMs and the requests they take in L1.
-// kPooled: the taps are window means of the unpooled maps (emc2_voxel_image_pooled).
-template <int CF4, bool kPooled>
-__global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads) vif_sample_kernel(const __grid_constant__ VifArgs a) {
+// kPool != 0: the taps are window means of the unpooled maps (emc2_voxel_image_pooled), 2: of 2 x 2 texels, known at compile
+// time, 1: of any window.  Bound by the windows' loads from L1 and L2, which want registers, so one record is taken at a
+// time: with two, as above, the compiler held to 64 registers and spilled.  us for both scales with two records and p at
+// run time / so: four nuScenes-shaped frames of 120,001 points p = 2 959 / 443, p = 4 1,578 / 1,240, p = 8 4,759 / 3,709;
+// one KITTI-shaped frame of 20,000 p = 8 209 / 152.
+template <int CF4, int kPool>
+__global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads, kPool == 1 ? 3 : 0) vif_sample_kernel(const __grid_constant__ VifArgs a) {
     await_predecessor();
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.taken = 0ull;     // for the next call; nothing reads it any more
     if (*a.bad) return;
@@ -267,14 +283,21 @@ __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads) vif_sample_kern
         int s2 = 0, n2 = 0;
         const uint4 rec1 = n1 > 0 ? a.recs[s1] : none;
         list_of(m + 2 * stride, s2, n2);
-        float4 acc = kPooled ? pooled_column(a, rec, c, cf4) : gather_column(a.feat, rec, c, (uint32_t)cf4, row_stride);
-        for (int k = 1; k < n; k += 2) {
-            const bool two = k + 1 < n;
-            const uint4 ra = a.recs[s0 + k], rb = two ? a.recs[s0 + k + 1] : none;
-            const float4 v0 = kPooled ? pooled_column(a, ra, c, cf4) : gather_column(a.feat, ra, c, (uint32_t)cf4, row_stride);
-            const float4 v1 = kPooled ? pooled_column(a, rb, c, cf4) : gather_column(a.feat, rb, c, (uint32_t)cf4, row_stride);
-            acc.x += v0.x; acc.y += v0.y; acc.z += v0.z; acc.w += v0.w;
-            if (two) { acc.x += v1.x; acc.y += v1.y; acc.z += v1.z; acc.w += v1.w; }
+        float4 acc = kPool != 0 ? pooled_column<kPool == 1 ? 0 : kPool>(a, rec, c, cf4) : gather_column(a.feat, rec, c, (uint32_t)cf4, row_stride);
+        if (kPool != 0) {
+            for (int k = 1; k < n; ++k) {
+                const float4 v = pooled_column<kPool == 1 ? 0 : kPool>(a, a.recs[s0 + k], c, cf4);
+                acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+            }
+        } else {
+            for (int k = 1; k < n; k += 2) {
+                const bool two = k + 1 < n;
+                const uint4 ra = a.recs[s0 + k], rb = two ? a.recs[s0 + k + 1] : none;
+                const float4 v0 = gather_column(a.feat, ra, c, (uint32_t)cf4, row_stride);
+                const float4 v1 = gather_column(a.feat, rb, c, (uint32_t)cf4, row_stride);
+                acc.x += v0.x; acc.y += v0.y; acc.z += v0.z; acc.w += v0.w;
+                if (two) { acc.x += v1.x; acc.y += v1.y; acc.z += v1.z; acc.w += v1.w; }
+            }
         }
         if (n > 1) {
             const float inv = 1.0f / (float)n;
@@ -340,12 +363,12 @@ int launch_voxel_image(emc2_bridge* h, int B, int N, int capacity, const int32_t
     } else {
         LaunchScope ls(h, K_VIF_SAMPLE, st);
         if (pool > 1) {
-            launch_chained(vif_sample_kernel<0, true>, blocks, kThreads, 0, st, a);
+            launch_chained(pool == 2 ? vif_sample_kernel<0, 2> : vif_sample_kernel<0, 1>, blocks, kThreads, 0, st, a);
         } else {
             switch (a.cf4) {
-                case 16: launch_chained(vif_sample_kernel<16, false>, blocks, 16 * 16, 0, st, a); break;
-                case 20: launch_chained(vif_sample_kernel<20, false>, blocks, 16 * 20, 0, st, a); break;
-                default: launch_chained(vif_sample_kernel<0, false>, blocks, kThreads, 0, st, a); break;
+                case 16: launch_chained(vif_sample_kernel<16, 0>, blocks, 16 * 16, 0, st, a); break;
+                case 20: launch_chained(vif_sample_kernel<20, 0>, blocks, 16 * 20, 0, st, a); break;
+                default: launch_chained(vif_sample_kernel<0, 0>, blocks, kThreads, 0, st, a); break;
             }
         }
     }

@@ -191,6 +191,32 @@ def test_map_layout_and_pooling_at_tile_edges(oracle, cf, hw):
     br.close()
 
 
+@pytest.mark.parametrize("p", [2, 4, 8, 16])
+@pytest.mark.parametrize("cf,hw", [(4, (13, 21)), (68, (13, 21)), (256, (13, 21)), (64, (16, 32)), (80, (7, 9))])
+def test_pooled_sampling_of_cut_windows(oracle, cf, hw, p):
+    """Windows cut by both far edges, windows larger than the map, and none cut; voxels of one, two and more points."""
+    h, wd = hw
+    base = gen.KITTI.with_shape(2, 5001)
+    cams = tuple(replace(c, fx=4.0 * wd, fy=4.0 * wd, cx=4.0 * wd, cy=4.0 * h) for c in base.cameras)
+    w = replace(base, img_h=8 * h, img_w=8 * wd, feat_stride=8, feat_c=cf, cameras=cams)
+    batch = gen.make_batch(w)
+    again = np.random.default_rng(cf).integers(0, w.N // 3, w.N)              # about three points at every place
+    batch["points"][..., :3] = batch["points"][:, again, :3]
+    d = to_dev(batch)
+    br = bridge_for(w)
+    bufs = br.run(d["points"], d["proj"], d["feat"])
+    ref = oracle.bridge(replace(w, feat_stride=8 * p, feat_offset=(p - 1) / 2 * 8), dict(batch, feat=oracle.pool(batch["feat"], p)))
+    for s in range(2):
+        M = ref[f"vox{s}"]["num_voxels"]
+        want, cnt = oracle.voxel_image(ref[f"vox{s}"]["point_voxel"], M, ref["vis_mask"], ref["gathered"])
+        assert all(int((cnt == n).sum()) > 0 for n in (0, 1, 2, 3, 4))
+        out = br.voxel_image_pooled(bufs["vox"], s, bufs["pg"]["uvd"], bufs["pg"]["cam"], d["feat"], p)
+        br.status()
+        assert np.array_equal(np_(out["vox_img_count"])[:M], cnt)
+        assert close(np_(out["vox_img"])[:M], want)[0]
+    br.close()
+
+
 @pytest.mark.parametrize("cap", [1, 3, 32, 255, 256, 257, 300])
 def test_cells_over_the_cap_by_the_length_of_their_lists(oracle, cap):
     """Lists around 32 and 256 entries, which a warp holds in registers, and longer ones; the first and the last points of

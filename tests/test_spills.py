@@ -10,7 +10,7 @@ from paper_2507_04123_b200 import build
 REPORT = re.compile(r"Compiling entry function '(\w+)'[^\n]*\n[^\n]*\n\s*(\d+) bytes stack frame, (\d+) bytes spill stores")
 
 
-@pytest.mark.parametrize("source", ["project_gather.cu"])
+@pytest.mark.parametrize("source", [s for s in build.SOURCES if s != "bridge.cu"])       # no kernels there
 def test_no_kernel_spills(source, tmp_path):
     full = build.nvcc_command(verbose_ptxas=True)
     flags = [a for a in full if a not in ("-shared", "-o", build.LIB) and not a.endswith(".cu")]
