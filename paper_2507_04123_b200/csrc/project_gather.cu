@@ -25,6 +25,7 @@ struct PgArgs {
     long long total;
     int N, K, H, W, Hf, Wf, cf4;
     float min_depth, inv_stride, offset;
+    bool stream;          // rows too many for L2: streaming stores
 };
 
 // Projection of one point into the K cameras of its frame (P: [K][3][4] row-major).
@@ -175,21 +176,24 @@ __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kMaxRowThreads, CF4 > 0 ?
     // uvd: the tile's 3*npts floats are contiguous in global memory.
     for (int i = t; i < npts * 3; i += blockDim.x) a.uvd[g0 * 3 + i] = suvd[i];
 
-    // Plain stores, not streaming ones: the dispatch reads these rows next and finds them in L2 as far as they fit (two
-    // frames of 120,001 points and 80 channels, 77 MB: dispatch_scatter 31.2 -> 26.9 us; four of 300,000, 384 MB: 131.0 ->
-    // 130.0).  This kernel does not mind (37.3 and 134 us either way; eight KITTI-shaped frames 68.3 -> 66.2).
+    // Rows that fit in L2 are stored plainly, because the dispatch reads them next: us for this kernel and the stage call of
+    // the dispatch, streaming / plain stores: one frame of 120,000 points 64 channels (31 MB) 30.7 / 29.4, 256 channels
+    // (123 MB) 89.0 / 84.0, two frames of 120,001 80 channels (77 MB) 72.8 / 69.6.  By itself this kernel loses up to 2 us,
+    // because the next stores have to write them back first (12.3 / 14.0, 38.6 / 39.4, 36.3 / 36.2).  Past L2 the plain
+    // stores only lose: 154 MB 160.1 / 161.8, 246 MB 180.7 / 182.1, 384 MB 275.3 / 276.5.
     float4* out = a.out + (size_t)g0 * cf4;
     const uint32_t dyv = (uint32_t)a.Wf * cf4;
+    auto store = [&](float4* p, const float4& v) { if (a.stream) __stcs(p, v); else *p = v; };
     if (CF4 > 0 || cf4 <= (int)blockDim.x) {
         const int c = t % cf4, rows = CF4 > 0 ? 16 : (int)blockDim.x / cf4;
 #pragma unroll 4
         for (int r = t / cf4; r < npts; r += rows)
-            out[r * cf4 + c] = gather_column(a.feat, srow[r], c, (uint32_t)cf4, dyv);
+            store(out + r * cf4 + c, gather_column(a.feat, srow[r], c, (uint32_t)cf4, dyv));
     } else {
         const int items = npts * cf4;
         for (int i = t; i < items; i += blockDim.x) {
             const int r = i / cf4, c = i - r * cf4;
-            out[i] = gather_column(a.feat, srow[r], c, (uint32_t)cf4, dyv);
+            store(out + i, gather_column(a.feat, srow[r], c, (uint32_t)cf4, dyv));
         }
     }
 }
@@ -778,6 +782,7 @@ int launch_project_gather(emc2_bridge* h, int B, int N, const float* d_points, c
     a.min_depth = c.min_depth;
     a.inv_stride = 1.0f / (float)c.feat_stride;
     a.offset = c.feat_offset;
+    a.stream = !rows_stay_in_l2((uint64_t)a.total, c.feat_c);
     const int tiles = (int)((a.total + kTile - 1) / kTile);
     if (tiles == 0) return EMC2_OK;
     if (c.point_floats == 4) launch_c<4>(h, a, tiles, st); else launch_c<5>(h, a, tiles, st);

@@ -104,6 +104,10 @@ inline bool rows_on_other_stream(uint64_t points, uint64_t row_bytes, bool both_
     return points <= 320000 && row_bytes <= (both_rows ? 160000000u : 96000000u);
 }
 
+// ---- whether the gathered rows of a call stay in L2 (126 MB) until the dispatch reads them: measured at 123 and 154 MB, see
+// project_gather_kernel
+inline bool rows_stay_in_l2(uint64_t points, uint64_t feat_c) { return points * feat_c * 4u <= (uint64_t)128 << 20; }
+
 // ---- notes of the tiles of a store that the marking pass touched: a bit per tile, 32 tiles to a word
 // Words that hold the tiles of frame b, for frames of `cells` cells and tiles of `per_tile` cells: the first, how many, and
 // at most how many of any frame.

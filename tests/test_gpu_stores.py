@@ -217,6 +217,20 @@ def test_pooled_sampling_of_cut_windows(oracle, cf, hw, p):
     br.close()
 
 
+@pytest.mark.parametrize("base,B,N,cf", [(gen.KITTI, 1, 131072, 256), (gen.KITTI, 1, 131073, 256), (gen.KITTI, 2, 66000, 260),
+                                         (gen.NUSCENES, 2, 209715, 80), (gen.NUSCENES, 2, 209716, 80)],
+                         ids=lambda v: getattr(v, "name", str(v)))
+def test_gathered_rows_on_either_side_of_l2(oracle, base, B, N, cf):
+    w = replace(base.with_shape(B, N), feat_c=cf)
+    batch = gen.make_batch(w)
+    ref = oracle.bridge(w, batch)
+    br = bridge_for(w)
+    d = to_dev(batch)
+    compare_bridge(w, ref, br.run_staged(d["points"], d["proj"], d["feat"]))
+    br.status()
+    br.close()
+
+
 @pytest.mark.parametrize("cap", [1, 3, 32, 255, 256, 257, 300])
 def test_cells_over_the_cap_by_the_length_of_their_lists(oracle, cap):
     """Lists around 32 and 256 entries, which a warp holds in registers, and longer ones; the first and the last points of

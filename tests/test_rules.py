@@ -112,3 +112,9 @@ def test_calls_that_keep_notes(rules):
         assert not rules.notes(frame, words, 1, 1000)
         assert rules.notes(frame, words, 2, 1) and rules.notes(frame, words, 32, 1 << 17)
         assert not rules.notes(frame, words, 32, (1 << 17) + 1) and not rules.notes(frame, 73, 32, 1000)
+
+
+def test_gathered_rows_that_stay_in_l2(rules):
+    for points, feat_c, stays in ((120000, 256, 1), (131072, 256, 1), (131073, 256, 0), (419430, 80, 1), (419431, 80, 0), (1, 4, 1),
+                                  (1 << 24, 1020, 0)):
+        assert rules.rows_stay(points, feat_c) == stays
