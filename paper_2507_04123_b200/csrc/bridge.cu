@@ -358,9 +358,8 @@ static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_poi
     // One pass over the points serves the projection, the routing and the voxelizer's marking; the
     // rest of stage 1 then runs beside the row traffic of stages 2 - 4, one of the two on a stream of the handle.
     const bool fused_mark = rc2 == EMC2_OK && B > 0 && N > 0 && h->tune[EMC2_TUNE_MARK_IN_PROJECTION] != 0;
-    const size_t row_bytes = (size_t)B * N * h->cfg.feat_c * sizeof(float) * (d_gathered ? 2 : 1);
     const bool rows_aside = fused_mark && h->overlap && !host && h->tune[EMC2_TUNE_SPLIT_BATCH] == 0 &&
-                            rows_on_other_stream((uint64_t)B * N, row_bytes, d_gathered != nullptr);
+                            rows_on_other_stream((uint64_t)B * N, (uint64_t)h->cfg.feat_c, d_gathered != nullptr);
     const cudaStream_t other = rows_aside ? h->rows : h->side;
     const cudaStream_t vox_st = h->overlap && !rows_aside ? other : st, row_st = rows_aside ? other : st;
     // With two or more frames the batch is taken in two halves: the rows of the first half start to

@@ -95,13 +95,22 @@ inline long long frames_of_tile(long long B, long long N) {
 // ---- which branch of a call of all stages stays on the caller's stream
 // Stage 1 is a chain of four kernels.  In a small call it is the longer branch and waiting for another stream, at its begin
 // and at the end of the call, costs more than it can hide: the rows go to the other stream instead.  In a large call the
-// rows are the longer branch, and stage 1, which shares the chip with them, needs its stream's priority.
-// `row_bytes`: feature rows written.  us per call, rows on the caller's stream / stage 1 on it: one frame of 120,000 points,
-// 64 channels, dispatched rows only (31 MB) 37.7 / 28.9; 3 x 33,333 x 80 channels (64 MB) 53.8 / 50.5, 8 x 16,384 (84 MB)
-// 93.5 / 86.9, one of 240,000 (154 MB) 75.3 / 72.2; but 4 x 120,000 x 64 channels (246 MB) 97.0 / 103.1, one of 480,000 with
-// dispatched rows only (123 MB) 67.6 / 69.8.
-inline bool rows_on_other_stream(uint64_t points, uint64_t row_bytes, bool both_rows) {
-    return points <= 320000 && row_bytes <= (both_rows ? 160000000u : 96000000u);
+// rows are the longer branch, and stage 1, which shares the chip with them, needs its stream's priority.  So they are where
+// few points have wide rows: a CTA takes the rows of 256 points in a time that grows with the channels, however few CTAs
+// there are.  us per call, rows on the caller's stream / stage 1 on it, both outputs of the rows unless said otherwise:
+//   one frame of 120,000 points, 64 channels 44.6 / 37.4, dispatched rows only 38.9 / 32.4; 3 x 33,333 x 80 channels 58.4 /
+//   53.9; 8 x 16,384 x 80 95.0 / 91.6.
+//   Bytes: one of 240,000 x 80 (154 MB) 84.0 / 81.0, of 300,000 x 64 (154 MB) 67.8 / 65.7 or, dense, 68.3 / 69.9; 4 x 100,000
+//   x 64 (205 MB) 98.9 / 104.7.  Dispatched rows only: one of 300,000 x 80 (96 MB) 83.7 / 80.3, of 480,000 x 64 (123 MB)
+//   72.8 / 75.0.
+//   Points: one of 300,000 x 64, dispatched rows only, 57.8 / 53.8, of 340,000 60.1 / 58.7, of 400,000 65.3 / 65.4; both
+//   rows of several frames cross earlier, 4 x 40,000 x 64 61.8 / 60.0, 4 x 78,000 85.0 / 87.2, but within 3 % either way.
+//   Wide rows: one of 45,000 x 128 33.2 / 35.5, of 60,000 35.0 / 36.5 (six cameras: 46.0 / 41.0), of 120,000 55.4 / 51.0; of
+//   60,000 x 192 42.5 / 45.2, of 90,000 50.4 / 51.5 (six cameras: 61.3 / 60.0); of 30,000 x 256 46.0 / 50.3, of 8,000 x 512
+//   41.3 / 75.  Dispatched rows only: of 30,000 x 192 30 / 34.2, of 60,000 34.0 / 35.2, of 90,000 41.4 / 37.8.
+inline bool rows_on_other_stream(uint64_t points, uint64_t feat_c, bool both_rows) {
+    if (feat_c >= 128 && points < feat_c * (both_rows ? 450u : 300u)) return false;
+    return points <= 320000 && points * feat_c * (both_rows ? 8u : 4u) <= (both_rows ? 160000000u : 96000000u);
 }
 
 // ---- whether the gathered rows of a call stay in L2 (126 MB) until the dispatch reads them: measured at 123 and 154 MB, see

@@ -118,3 +118,17 @@ def test_gathered_rows_that_stay_in_l2(rules):
     for points, feat_c, stays in ((120000, 256, 1), (131072, 256, 1), (131073, 256, 0), (419430, 80, 1), (419431, 80, 0), (1, 4, 1),
                                   (1 << 24, 1020, 0)):
         assert rules.rows_stay(points, feat_c) == stays
+
+
+def test_calls_whose_rows_go_to_the_other_stream(rules):
+    """Either side of the limits: points, bytes of rows, and few points with wide rows."""
+    for both, most_bytes, per_channel in ((1, 160_000_000, 450), (0, 96_000_000, 300)):
+        width = 8 if both else 4
+        for cf in (4, 64, 80, 96, 124, 128, 132, 192, 256, 512, 1024):
+            least = cf * per_channel if cf >= 128 else 0
+            most = min(320_000, most_bytes // (cf * width))
+            for n in {1, least - 1, least, least + 1, most, most + 1, 1 << 24}:
+                if n > 0:
+                    assert rules.rows_aside(n, cf, both) == (least <= n <= most), (n, cf, both)
+    assert rules.rows_aside(120_000, 64, 1) and rules.rows_aside(120_000, 64, 0) and rules.rows_aside(99_999, 128, 1)
+    assert not rules.rows_aside(8_000, 512, 1) and not rules.rows_aside(8_000, 512, 0) and not rules.rows_aside(30_000, 256, 1)
