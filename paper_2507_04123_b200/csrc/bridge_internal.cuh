@@ -421,6 +421,17 @@ struct FrameTiles {
     __align__(16) uint8_t seen[kMarkWords * 32];        // a byte per tile, scale 1 behind scale 0
 };
 
+// Shared memory for them where the kernel keeps notes.
+template <bool kNote>
+__device__ __forceinline__ FrameTiles* frame_tiles() {
+    if constexpr (kNote) {
+        __shared__ FrameTiles tiles;
+        return &tiles;
+    } else {
+        return nullptr;
+    }
+}
+
 // The caller synchronises the CTA before the first note_tiles and before publish_tiles.
 __device__ __forceinline__ void begin_tiles(FrameTiles& f, const ScaleDev& s0, const ScaleDev& s1, uint32_t b) {
     if (threadIdx.x < 2) {
