@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(CF4 > 0 ? 16 * CF4 : kThreads, kPool == 1 ? 3 
         s0 = n = 0;
         if (m < M) {
             s0 = a.start[m];
-            n = min(a.counts[m], a.cursor[m] - s0);              // never past what this call appended
+            n = max(min(a.counts[m], a.cursor[m] - s0), 0);      // never past what this call appended, none where counts[] is negative
         }
     };
     const uint4 none = make_uint4(kZeroRow, 0u, 0u, 0u);

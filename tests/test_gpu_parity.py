@@ -388,6 +388,40 @@ def test_per_voxel_fusion_with_counts_moved_between_voxels_reads_only_what_it_ap
     br.close()
 
 
+@pytest.mark.parametrize("negative", [False, True])
+def test_sampled_fusion_with_wrong_counts_reads_only_what_it_appended(b200, oracle, negative):
+    """The paths without stored rows, with counts that belong to other voxels or are negative: every row is a mean of samples
+    of this call's maps, and no count below zero is stored.  Records of two voxels can meet in one slot here, so the maps
+    have memory behind them."""
+    w = gen.KITTI.with_shape(1, 20_000)
+    batch = gen.make_batch(w)
+    br = b200.Bridge(b200.config_from_workload(w))
+    d = to_dev(batch)
+    bufs = br.run(d["points"], d["proj"], d["feat"])
+    br.status()
+    pg, vox = bufs["pg"], bufs["vox"]
+    feat = torch.ones((3,) + tuple(d["feat"].shape), device="cuda")[0]       # every sample is 1 but for rounding
+    for s in range(2):
+        M = int(vox["num_voxels"][s].item())
+        wrong = vox["counts"][s].clone()
+        if negative:
+            wrong[:M:3] = -5
+        else:
+            wrong[:M] = torch.roll(wrong[:M], 1)                             # same sum, other voxels
+        voxels = {**vox, "counts": [wrong if k == s else vox["counts"][k] for k in range(2)]}
+        for out in (br.voxel_image_sampled(voxels, s, pg["uvd"], pg["cam"], feat),
+                    br.voxel_image_pooled(voxels, s, pg["uvd"], pg["cam"], feat, 2),
+                    br.voxel_image_pooled(voxels, s, pg["uvd"], pg["cam"], feat, 4)):
+            assert br.status(raise_on_error=False) == b200.bridge.EMC2_OK
+            rows, cnt = out["vox_img"][:M], out["vox_img_count"][:M]
+            assert bool((cnt >= 0).all()) and bool((cnt <= wrong[:M].clamp(min=0)).all())
+            if negative:
+                assert bool((cnt[::3] == 0).all())
+            seen = cnt > 0
+            assert bool(((rows[seen] - 1.0).abs() < 1e-5).all()) and bool((rows[~seen] == 0.0).all())
+    br.close()
+
+
 @pytest.mark.parametrize("cid,B,N", [(2, 2, 60_000), (1, 3, 33_333), (3, 1, 150_000), (0, 1, 16_384), (2, 1, 1)])
 def test_sparse_convolution_rulebook(b200, oracle, cid, B, N):
     w = gen.workload(cid).with_shape(B, N)
