@@ -33,7 +33,10 @@ namespace emc2 {
 namespace {
 
 constexpr int kStatusCapacity = 1;
-constexpr int kStatusDirtyStore = 8;   // the cell store held more than one call's points can set
+// The cell store held more than one call's points can set, or a cell that none of them marked.  A call that keeps notes looks
+// at the noted tiles only: what two calls on one handle at once left in another tile stays there until some call marks a
+// cell of that tile, and is found, reported (on a bitmap scale, by its missing points) and cleared then.
+constexpr int kStatusDirtyStore = 8;
 
 // Where a point's cell sits in the unique list.
 struct Slot {
@@ -559,6 +562,7 @@ __device__ __forceinline__ void write_batch(const AccumArgs& a, int sc, int mb, 
     g.div[1].divmod(r, r, y);
     g.div[2].divmod(r, r, z);
     if (!table) cnt = over ? g.cap : (int)a1.y;
+    if (!table && active && cnt == 0) atomicOr(a.status, kStatusDirtyStore);     // no point of this call marked the cell
     // Offsets are below one cell size, so fp32 keeps the mean to a few 1e-7 of that size.
     const float inv = __frcp_rn((float)cnt);
     float mu[C];
