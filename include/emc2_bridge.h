@@ -21,10 +21,8 @@
  *   - Every call that takes `cuda_stream` (a cudaStream_t passed as void*,
  *     NULL = legacy default stream) only enqueues kernels.  These calls do not
  *     allocate, do not synchronise and do not touch the host except to return.
- *     Some kernels are cooperative launches (grid-wide barrier), which the
- *     device must support; emc2_bridge_create() fails otherwise.  The calls
- *     that take a handle and a stream can therefore be captured into a CUDA
- *     graph and replayed (emc2_bridge_status synchronises and cannot).
+ *     The calls that take a handle and a stream can therefore be captured into
+ *     a CUDA graph and replayed (emc2_bridge_status synchronises and cannot).
  *   - One handle serves one device and one stream at a time; it is not
  *     thread-safe.  Calls on the same handle must be ordered on the stream.
  *   - Errors are returned as negative emc2_status_t values.  Errors the host
@@ -52,11 +50,11 @@ typedef enum {
     EMC2_ERR_CUDA = -3,        /* a CUDA runtime call failed; see emc2_bridge_last_cuda_error */
     EMC2_ERR_CAPACITY = -4,    /* more unique voxels than capacity[s] (device-detected, sticky) */
     EMC2_ERR_TIMEOUT = -5,     /* reserved: a bounded device-side wait gave up.  No kernel of this library
-                                  spins on another CTA (the only grid-wide waits are the barriers of
-                                  cooperative launches), so it is never returned at present */
-    EMC2_ERR_INTERNAL = -6,    /* from emc2_bridge_status: a call found the handle's scratch in use (two
-                                  calls on one handle at once); that call's voxel outputs are void and the
-                                  handle should be destroyed */
+                                  waits for another CTA, so it is never returned at present */
+    EMC2_ERR_INTERNAL = -6,    /* from emc2_bridge_status: a call found the handle's scratch in use, or cells
+                                  marked that none of its points lies in (two calls on one handle at once);
+                                  that call's voxel outputs are void and the handle should be destroyed.  Not
+                                  every such overlap is found, nor always by the next call */
     EMC2_ERR_TOO_LARGE = -7    /* the call needs more scratch than a fixed-size scratch area holds */
 } emc2_status_t;
 
@@ -343,7 +341,7 @@ int emc2_route_dispatch_static(const emc2_config_t* config, int32_t B, int32_t N
                                float* d_feat_out, void* cuda_stream);
 
 /* Waits for `cuda_stream`, then returns and clears the sticky device status: EMC2_OK,
- * EMC2_ERR_CAPACITY, EMC2_ERR_TIMEOUT or EMC2_ERR_CUDA. */
+ * EMC2_ERR_CAPACITY, EMC2_ERR_INVALID_ARG, EMC2_ERR_INTERNAL, EMC2_ERR_TIMEOUT or EMC2_ERR_CUDA. */
 int emc2_bridge_status(emc2_bridge_t* bridge, void* cuda_stream);
 
 /* Frees scratch memory.  The caller must have synchronised the streams it used.  NULL is OK. */

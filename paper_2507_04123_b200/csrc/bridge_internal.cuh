@@ -210,7 +210,7 @@ struct emc2_bridge {
     int tune[EMC2_TUNE_KNOBS] = {0, 1, 0, 0, 0};   // emc2_bridge_set_tuning
     emc2::DedupArm arm;
     int num_sms = 0;               // multiprocessors of the handle's device
-    bool overlap = true;           // emc2_bridge_run puts stage 1 on `side`
+    bool overlap = true;           // emc2_bridge_run uses `side` and `rows`
     cudaStream_t side = nullptr;   // stream of stage 1 inside emc2_bridge_run ...
     cudaStream_t rows = nullptr;   // ... or, in small calls, of the rows; of the maps' copy in emc2_bridge_run_host
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_half = nullptr, ev_copy = nullptr, ev_scan = nullptr;

@@ -25,8 +25,8 @@
 //
 // Writes and reductions that land in one 32-byte sector are served one after another by the
 // L2 (about 10 ns each on B200), so nothing here funnels many points into a shared flag or
-// counter: the only contended words are the cells themselves.  The cost of a call follows the
-// occupied tiles, not the grid volume, except for one streaming read of the store.
+// counter: the contended words are the cells themselves and the notes of their tiles.  The cost of a call follows the
+// occupied tiles, not the grid volume, except for one streaming read of the store where no notes are kept.
 #include "bridge_internal.cuh"
 
 namespace emc2 {
@@ -122,12 +122,13 @@ struct ScanArgs {
 };
 
 // Two launches.
-//   vox_count   streams the store once, a CTA per four 8 KB tiles: voxels per tile, their sum per 128 tiles,
-//               and a list of the tiles that hold any (most of a fine grid is empty space).
+//   vox_count   voxels per 8 KB tile of the store, their sum per 128 tiles, and a list of the tiles that hold any
+//               (most of a fine grid is empty space).  One kernel streams the whole store, a CTA per four tiles; another,
+//               where the marking pass keeps notes (see keeps_notes), reads the noted tiles only.
 //   vox_rank    a CTA per listed tile finds the voxels before it (sums of whole groups of 128 tiles plus
 //               those of its own group: a load or two per thread), ranks its units or cells and lists the
 //               occupied cells in rank order.
-// vox_count is bound by the streaming read (every cell of the grid is looked at), vox_rank by the latency of
+// The counting is bound by the read of the store or of the noted tiles, vox_rank by the latency of
 // its three dependent round trips and by the few tiles on the ground plane that hold most voxels: a thread
 // has one sector of 32 bytes, and a warp lists the cells of its 32 sectors together.
 __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t x) {
@@ -200,8 +201,9 @@ __global__ void __launch_bounds__(kThreads) vox_count_kernel(const __grid_consta
 }
 
 // The same where the marking pass noted the tiles it touched: only those are looked at (vox_rank clears the notes).  A
-// fixed grid of CTAs, each with at most kThreads groups of four tiles.  Eight KITTI-shaped frames (127 MB of stores): 28 ->
-// 16 us; the marking pass of emc2_voxelize does not mind (27.1 and 27.4 us on four nuScenes-shaped frames).
+// fixed grid of CTAs, each with at most kThreads groups of four tiles.  us by events, whole stores / noted tiles: eight
+// KITTI-shaped frames (127 MB of stores) 28.3 / 15.4, while the marking pass goes from 27.5 to 38.4 and project_route, where
+// it does the marking, from 32.5 to 42.3; four of 60,000 points 18.8 / 12.7 and 14.6 / 16.2.  See keeps_notes for whole calls.
 __global__ void __launch_bounds__(kThreads) vox_count_marked_kernel(const __grid_constant__ ScanArgs a) {
     await_predecessor();
     __shared__ uint32_t s_warp[kCountTiles][kThreads / 32], s_which[kThreads];
