@@ -97,7 +97,8 @@ inline long long frames_of_tile(long long B, long long N) {
 // and at the end of the call, costs more than it can hide: the rows go to the other stream instead.  In a large call the
 // rows are the longer branch, and stage 1, which shares the chip with them, needs its stream's priority.  So they are where
 // few points have wide rows: a CTA takes the rows of 256 points in a time that grows with the channels, however few CTAs
-// there are.  us per call, rows on the caller's stream / stage 1 on it, both outputs of the rows unless said otherwise:
+// there are.  us per call, rows on the caller's stream / stage 1 on it, both outputs of the rows unless said otherwise;
+// 80 channels are nuScenes-shaped frames, other widths KITTI-shaped ones unless they have six cameras:
 //   one frame of 120,000 points, 64 channels 44.6 / 37.4, dispatched rows only 38.9 / 32.4; 3 x 33,333 x 80 channels 58.4 /
 //   53.9; 8 x 16,384 x 80 95.0 / 91.6.
 //   Bytes: one of 240,000 x 80 (154 MB) 84.0 / 81.0, of 300,000 x 64 (154 MB) 67.8 / 65.7 or, dense, 68.3 / 69.9; 4 x 100,000

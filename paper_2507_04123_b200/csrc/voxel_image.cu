@@ -249,7 +249,8 @@ __device__ __forceinline__ float4 pooled_column(const VifArgs& a, const uint4& r
 // three rounds: while the taps of one voxel are in flight, the first record of the thread's next voxel and the start and
 // length of the one after it are.  Two voxels at once without that took 283.3 us for both scales of four nuScenes-shaped
 // frames, this 273.5; 12 rows and 40 registers (48 warps instead of 40) 275.0 without, 307.8 with it (it spills); a CTA per
-// 16 voxels instead of a fixed grid 382.  Bound by the taps' way from L2 to the SMs and the requests they take in L1.
+// 16 voxels instead of a fixed grid 382.  Bound by the wait for the taps (12 of 16 cycles between a warp's instructions, at 56 %
+// occupancy); no unit is full: L1 52 %, L2 31 %, DRAM 14 %, issue 0.51 (one nuScenes-shaped frame, cold L2).
 // kPool != 0: the taps are window means of the unpooled maps (emc2_voxel_image_pooled), 2: of 2 x 2 texels, known at compile
 // time, 1: of any window.  Bound by the windows' loads from L1 and L2, which want registers, so one record is taken at a
 // time: with two, as above, the compiler held to 64 registers and spilled.  us for both scales with two records and p at
