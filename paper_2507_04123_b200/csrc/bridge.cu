@@ -174,9 +174,10 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out) {
     const size_t tiles[2] = {h->scale[0].tiles, h->scale[1].tiles};
     const size_t groups[2] = {(tiles[0] + kTilesPerGroup - 1) / kTilesPerGroup, (tiles[1] + kTilesPerGroup - 1) / kTilesPerGroup};
     const size_t o_tiles = plan.take((tiles[0] + tiles[1]) * sizeof(uint32_t));
+    const size_t o_parts = plan.take((tiles[0] + tiles[1]) * sizeof(uint4));
     const size_t marked[2] = {(tiles[0] + 31) / 32, (tiles[1] + 31) / 32};
     const size_t o_marked = plan.take((marked[0] + marked[1]) * sizeof(uint32_t));
-    const size_t o_list = plan.take((tiles[0] + tiles[1]) * sizeof(uint32_t));
+    const size_t o_list = plan.take((tiles[0] + tiles[1]) * 8 * sizeof(uint32_t));
     h->scan_reset_words = (int)(groups[0] + groups[1] + 1);
     const size_t o_groups = plan.take((size_t)h->scan_reset_words * sizeof(uint32_t));
     const size_t o_vif_start = plan.take(maxpts * sizeof(int));
@@ -215,6 +216,8 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out) {
     }
     h->scan.tile_voxels[0] = reinterpret_cast<uint32_t*>(base + o_tiles);
     h->scan.tile_voxels[1] = h->scan.tile_voxels[0] + tiles[0];
+    h->scan.tile_parts[0] = reinterpret_cast<uint4*>(base + o_parts);
+    h->scan.tile_parts[1] = h->scan.tile_parts[0] + tiles[0];
     h->scan.list = reinterpret_cast<uint32_t*>(base + o_list);
     h->scan.marked[0] = reinterpret_cast<uint32_t*>(base + o_marked);
     h->scan.marked[1] = h->scan.marked[0] + marked[0];

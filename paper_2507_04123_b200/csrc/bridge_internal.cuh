@@ -145,9 +145,10 @@ constexpr int kTilesPerGroup = 128;
 constexpr int kCountTiles = 4;  // tiles per CTA of the counting pass
 struct ScanState {
     uint32_t* tile_voxels[2];   // [tiles] voxels per tile
+    uint4* tile_parts[2];       // [tiles] voxels per eighth of a tile, 16 bits each
     uint32_t* group_voxels[2];  // [ceil(tiles / 128)] per group of tiles; zero when the scan begins
-    uint32_t* listed;           // tiles in `list`; zero when the scan begins
-    uint32_t* list;             // [tiles of both scales] tiles that hold voxels, in any order; bit 31: scale 1
+    uint32_t* listed;           // parts in `list`; zero when the scan begins
+    uint32_t* list;             // [8 * tiles of both scales] parts that hold voxels, in any order: 8 * tile + part; bit 31: scale 1
     uint32_t* marked[2];        // a bit per tile of a store: a cell of it was marked; zero between calls
     int words[2];               // words of `marked` to clear, 0 where the marking pass does not keep it
 };

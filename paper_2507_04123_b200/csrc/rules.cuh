@@ -153,16 +153,16 @@ EMC2_RULE bool voxels_possible(uint32_t voxels, uint32_t max_list) { return voxe
 EMC2_RULE bool frame_in_call(uint32_t frame, uint32_t frames) { return frame < frames; }
 
 // ---- cells over the per-voxel cap (rank scan of a table store)
-// A tile sums the points of its cells over the cap and takes one 64-bit ticket for them, {cells, points} before the
-// tile.  In a store that was not all zero a word can hold anything, and a sum that wrapped would pass for a small
-// one: every term and every partial sum of a tile is clamped to kPointsClamp, which is above the points of any call
-// (2^24), so that 2,048 cells summed by threads of 8, warps of 32 and 8 warps stay below 2^31.
+// A part of a tile sums the points of its cells over the cap and takes one 64-bit ticket for them, {cells, points} before
+// the part.  In a store that was not all zero a word can hold anything, and a sum that wrapped would pass for a small
+// one: every term and every lane's sum is clamped to kPointsClamp, which is above the points of any call
+// (2^24), so that 256 cells summed by lanes of 8 and a warp of 32 stay below 2^31.
 constexpr uint32_t kPointsClamp = 1u << 25;
 
 EMC2_RULE uint32_t clamp_points(uint32_t n) { return n < kPointsClamp ? n : kPointsClamp; }
 
-// Whether a tile with `cells` cells over the cap and `points` points in them, which took the ticket `first`, finds
-// room: the tile's index lists then lie inside [0, max_list) and its cells' places inside [0, max_ovf).  No ticket may
+// Whether a part with `cells` cells over the cap and `points` points in them, which took the ticket `first`, finds
+// room: its index lists then lie inside [0, max_list) and its cells' places inside [0, max_ovf).  No ticket may
 // be taken with points > max_list.  The first ticket that does not fit is always found, because nothing has wrapped
 // before it.
 EMC2_RULE bool over_fits(uint64_t first, uint32_t cells, uint32_t points, uint32_t max_ovf, uint32_t max_list) {

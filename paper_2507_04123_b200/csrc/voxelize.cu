@@ -122,15 +122,18 @@ struct ScanArgs {
 };
 
 // Two launches.
-//   vox_count   voxels per 8 KB tile of the store, their sum per 128 tiles, and a list of the tiles that hold any
-//               (most of a fine grid is empty space).  One kernel streams the whole store, a CTA per four tiles; another,
-//               where the marking pass keeps notes (see keeps_notes), reads the noted tiles only.
-//   vox_rank    a CTA per listed tile finds the voxels before it (sums of whole groups of 128 tiles plus
-//               those of its own group: a load or two per thread), ranks its units or cells and lists the
+//   vox_count   voxels per 8 KB tile of the store and per eighth of it (a part: 32 sectors), their sum per 128 tiles, and a
+//               list of the parts that hold any (most of a fine grid is empty space).  One kernel streams the whole store, a CTA
+//               per four tiles; another, where the marking pass keeps notes (see keeps_notes), reads the noted tiles only.
+//   vox_rank    a warp per listed part finds the voxels before it (groups of tiles before its group, tiles of the group
+//               and parts of the tile before it: a load each), ranks its units or cells and lists the
 //               occupied cells in rank order.
 // The counting is bound by the read of the store or of the noted tiles, vox_rank by the latency of
-// its three dependent round trips and by the few tiles on the ground plane that hold most voxels: a thread
-// has one sector of 32 bytes, and a warp lists the cells of its 32 sectors together.
+// its three dependent round trips and by the parts on the ground plane that hold most voxels: a lane
+// has one sector of 32 bytes, and a warp lists the cells of its 32 sectors together.  Nothing in its loop waits for another
+// warp.  By events, us, a CTA per listed tile with three barriers each / a warp per part of the listed tiles / per listed part:
+// tiny frame 12.6 / 12.9 / 10.7, eight KITTI-shaped frames 34.1 / 32.7 / 28.3, four nuScenes-shaped 34.4 / 30.8 / 30.6, 32 frames
+// of 262,144 points 152 / 137 / 125; the next part's sectors requested ahead: 29.9, 30.3, 125.
 __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t x) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
@@ -172,21 +175,35 @@ __device__ __forceinline__ void count_tiles(const ScanArgs& a, uint32_t (*s_warp
     }
     __syncthreads();
     if (t < kCountTiles) {
-        uint32_t n = 0;
+        uint32_t n = 0, pair[kWarps / 2];
 #pragma unroll
-        for (int w = 0; w < kWarps; ++w) n += s_warp[t][w];
+        for (int w = 0; w < kWarps; w += 2) {
+            n += s_warp[t][w] + s_warp[t][w + 1];
+            pair[w / 2] = s_warp[t][w] | s_warp[t][w + 1] << 16;          // a part holds at most 32 * 192 voxels
+        }
         a.st.tile_voxels[sc][tile0 + t] = n;
+        a.st.tile_parts[sc][tile0 + t] = make_uint4(pair[0], pair[1], pair[2], pair[3]);
         // One ticket per CTA: tickets on one address are served one after another (about 10 ns each).
         constexpr unsigned kAll = (1u << kCountTiles) - 1u;
-        const unsigned some = __ballot_sync(kAll, n != 0u);
-        const uint32_t sum = __reduce_add_sync(kAll, n);          // the CTA's tiles are all in one group
-        uint32_t at = 0;
-        if (some && t == 0) {
-            atomicAdd(&a.st.group_voxels[sc][tile0 / kTilesPerGroup], sum);
-            at = atomicAdd(a.st.listed, (uint32_t)__popc(some));
+        uint32_t held = 0u;                                       // a bit per part that holds voxels
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) held |= s_warp[t][w] != 0u ? 1u << w : 0u;
+        const uint32_t mine = __popc(held);
+        uint32_t at = mine;
+#pragma unroll
+        for (int d = 1; d < kCountTiles; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(kAll, at, d);
+            if (t >= d) at += y;
         }
-        at = __shfl_sync(kAll, at, 0) + __popc(some & ((1u << t) - 1u));
-        if (n) a.st.list[at] = (uint32_t)(tile0 + t) | (sc ? 0x80000000u : 0u);
+        const uint32_t sum = __reduce_add_sync(kAll, n);          // the CTA's tiles are all in one group
+        uint32_t first = 0;
+        if (t == kCountTiles - 1 && at) {
+            atomicAdd(&a.st.group_voxels[sc][tile0 / kTilesPerGroup], sum);
+            first = atomicAdd(a.st.listed, at);
+        }
+        at += __shfl_sync(kAll, first, kCountTiles - 1) - mine;
+        for (uint32_t entry = (sc ? 0x80000000u : 0u) | (uint32_t)(tile0 + t) << 3; held; held &= held - 1u)
+            a.st.list[at++] = entry | (uint32_t)__ffs(held) - 1u;
     }
 }
 
@@ -234,35 +251,47 @@ __device__ __forceinline__ void refuse_lists(const ScaleDev& g, int* status) {
     atomicOr(status, kStatusDirtyStore);
 }
 
-constexpr int kRankThreads = kScanSectors, kRankCtas = 6;
+constexpr int kRankThreads = 256, kRankCtas = 6;
+constexpr int kRankGroups = 3 * kRankThreads;             // groups of tiles: at most 683 of a bitmap store, see validate
+static_assert(kScanSectors == 8 * 32, "a tile has eight parts, one sector for each lane of a warp");
 
 __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const __grid_constant__ ScanArgs a) {
     await_predecessor();
     constexpr int kWarps = kRankThreads / 32;
-    __shared__ uint32_t s_before[kWarps], s_warp[kWarps];
-    __shared__ int s_over[2];                             // cells over the cap and their points: sum, then base
+    __shared__ uint32_t s_groups[2][kRankGroups], s_sum[2][kWarps];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const uint32_t listed = *a.st.listed;
+    const uint32_t listed = *a.st.listed, step = gridDim.x * kWarps;
 #pragma unroll
     for (int v = 0; v < 2; ++v)                           // vox_count has read the notes
         for (int i = blockIdx.x * kRankThreads + t; i < a.st.words[v]; i += gridDim.x * kRankThreads) a.st.marked[v][i] = 0u;
-    uint32_t entry = blockIdx.x < listed ? a.st.list[blockIdx.x] : 0u, next = 0u;
-    // Voxels of both scales, and this CTA's share of their accumulators cleared: a few tiles hold most of the
-    // voxels, so the clearing is not tied to the tiles.  Done here, just before they are added to, it also brings
-    // them into L2 (cleared after use by vox_finalize, vox_accum took 48 instead of 43 us on four nuScenes-shaped
-    // frames and vox_finalize 40 instead of 37).
+    uint32_t k = (uint32_t)warp * gridDim.x + blockIdx.x, next = 0u;
+    uint32_t entry = k < listed ? a.st.list[k] : 0u;
+    // Voxels before every group of tiles, and of both scales.
     uint32_t all[2] = {0u, 0u};
+    {
+        uint32_t n[2][3], inc[2], sum[2];
 #pragma unroll
-    for (int v = 0; v < 2; ++v)
-        for (int i = t; i * kTilesPerGroup < a.tiles[v]; i += kRankThreads) all[v] += a.st.group_voxels[v][i];
+        for (int v = 0; v < 2; ++v) {
 #pragma unroll
-    for (int v = 0; v < 2; ++v) {
-        all[v] = __reduce_add_sync(0xFFFFFFFFu, all[v]);
-        if (lane == 0) (v ? s_warp : s_before)[warp] = all[v];
+            for (int i = 0; i < 3; ++i) n[v][i] = (3 * t + i) * kTilesPerGroup < a.tiles[v] ? a.st.group_voxels[v][3 * t + i] : 0u;
+        }
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            sum[v] = n[v][0] + n[v][1] + n[v][2];
+            inc[v] = warp_incl_scan(sum[v]);
+            if (lane == 31) s_sum[v][warp] = inc[v];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            const uint32_t own = lane < kWarps ? s_sum[v][lane] : 0u;
+            all[v] = __reduce_add_sync(0xFFFFFFFFu, own);
+            uint32_t run = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? own : 0u) + inc[v] - sum[v];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) { s_groups[v][3 * t + i] = run; run += n[v][i]; }
+        }
+        __syncthreads();
     }
-    __syncthreads();
-#pragma unroll
-    for (int v = 0; v < 2; ++v) all[v] = __reduce_add_sync(0xFFFFFFFFu, lane < kWarps ? (v ? s_warp : s_before)[lane] : 0u);
     if (blockIdx.x == 0 && t < 2 && !a.s[t].design) {
         // More voxels than a call's points allow: the store was not all zero when the call began (two
         // calls on one handle at once).  The scale is then not ranked and reports no voxels, and the
@@ -275,71 +304,27 @@ __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const
         if (dirty) atomicOr(a.status, kStatusDirtyStore);
         else if ((int)n > a.capacity[t]) atomicOr(a.status, kStatusCapacity);
     }
-    {
-        const size_t n0 = (size_t)min(all[0], a.s[0].max_list) * a.s[0].acc_f4, n1 = (size_t)min(all[1], a.s[1].max_list) * a.s[1].acc_f4;
-        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (size_t i = (size_t)blockIdx.x * kRankThreads + t; i < n0; i += (size_t)gridDim.x * kRankThreads) a.s[0].acc[i] = z;
-        for (size_t i = (size_t)blockIdx.x * kRankThreads + t; i < n1; i += (size_t)gridDim.x * kRankThreads) a.s[1].acc[i] = z;
-    }
-    __syncthreads();
-    for (uint32_t k = blockIdx.x; k < listed; k += gridDim.x, entry = next) {
-        if (k + gridDim.x < listed) next = a.st.list[k + gridDim.x];
-        const int sc = (int)(entry >> 31), tile = (int)(entry & 0x7FFFFFFFu);
+    // The listed parts, a warp each; the warps of a CTA are far apart in the list.
+    for (; k < listed; k += step, entry = next) {
+        if (k + step < listed) next = a.st.list[k + step];
+        const int sc = (int)(entry >> 31), tile = (int)(entry >> 3 & 0x0FFFFFFFu), part = (int)(entry & 7u);
         const ScaleDev& g = a.s[sc];
         if (!voxels_possible(sc ? all[1] : all[0], g.max_list)) continue;
         const bool bitmap = g.mode == MODE_BITMAP;
-        const uint32_t sector = (uint32_t)tile * kScanSectors + t;
+        const uint32_t sector = (uint32_t)tile * kScanSectors + part * 32 + lane;
         uint4* const at = reinterpret_cast<uint4*>(g.store) + (size_t)sector * 2;
         uint4 p = at[0], q = at[1];
-        // Voxels before the tile: groups before its group, tiles of its group before it.
-        const int group = tile / kTilesPerGroup, in_group = tile % kTilesPerGroup;
-        uint32_t before = 0;
-        if (t < in_group) before = a.st.tile_voxels[sc][group * kTilesPerGroup + t];
-        for (int i = kRankThreads - 1 - t; i < group; i += kRankThreads) before += a.st.group_voxels[sc][i];
-        before = __reduce_add_sync(0xFFFFFFFFu, before);
+        // Voxels before the part: groups before its group, tiles of its group before its tile, parts of its tile before it.
+        const int in_group = tile % kTilesPerGroup, k0 = 4 * lane;
+        uint4 four = make_uint4(0u, 0u, 0u, 0u);
+        if (k0 < in_group) four = *reinterpret_cast<const uint4*>(a.st.tile_voxels[sc] + (tile - in_group) + k0);
+        uint32_t before = lane < part ? reinterpret_cast<const uint16_t*>(a.st.tile_parts[sc] + tile)[lane] : 0u;
+        before += (k0 < in_group ? four.x : 0u) + (k0 + 1 < in_group ? four.y : 0u) + (k0 + 2 < in_group ? four.z : 0u) +
+                  (k0 + 3 < in_group ? four.w : 0u);
+        before = __reduce_add_sync(0xFFFFFFFFu, before) + s_groups[sc][tile / kTilesPerGroup];
         const uint32_t c = sector_voxels(bitmap, p, q);
         const uint32_t inc = warp_incl_scan(c);
-        if (lane == 31) { s_before[warp] = before; s_warp[warp] = inc; }
-        if (t < 2) s_over[t] = 0;
-        __syncthreads();
-        const uint32_t base = __reduce_add_sync(0xFFFFFFFFu, lane < kWarps ? s_before[lane] : 0u);
-        const uint32_t own = lane < kWarps ? s_warp[lane] : 0u;
-        uint32_t m = base + __reduce_add_sync(0xFFFFFFFFu, lane < warp ? own : 0u) + inc - c;
-        // Cells over the cap take the next places among such cells, and their points the next slots of
-        // the index list, in any order: one ticket per tile.
-        uint32_t j = 0, off = 0;
-        bool list_over = false;
-        if (!bitmap && g.cap > 0) {
-            const uint32_t n[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
-            uint32_t cells = 0, points = 0;
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                if (n[i] > (uint32_t)g.cap) { cells += 1; points += clamp_points(n[i]); }
-            if (__any_sync(0xFFFFFFFFu, cells != 0)) {
-                points = clamp_points(points);
-                const uint32_t ic = warp_incl_scan(cells), ip = warp_incl_scan(points);
-                int wc = 0, wp = 0;                       // the warp's share starts here inside the tile's
-                if (lane == 31) { wc = atomicAdd(&s_over[0], (int)ic); wp = atomicAdd(&s_over[1], (int)clamp_points(ip)); }
-                j = (uint32_t)__shfl_sync(0xFFFFFFFFu, wc, 31) + ic - cells;
-                off = (uint32_t)__shfl_sync(0xFFFFFFFFu, wp, 31) + ip - points;
-            }
-            __syncthreads();
-            if (t == 0 && s_over[0] > 0) {
-                const uint32_t tc = (uint32_t)s_over[0], tp = (uint32_t)s_over[1];
-                unsigned long long first = 0;
-                bool fits = tp <= g.max_list;
-                if (fits) {
-                    first = atomicAdd(reinterpret_cast<unsigned long long*>(g.totals + 2), (unsigned long long)over_ticket(tc, tp));
-                    fits = over_fits(first, tc, tp, g.max_ovf, g.max_list);
-                }
-                if (!fits) refuse_lists(g, a.status);
-                s_over[0] = fits ? (int)(first >> 32) : -1; s_over[1] = (int)(uint32_t)first;
-            }
-            __syncthreads();
-            list_over = s_over[0] >= 0;
-            j += (uint32_t)s_over[0];
-            off += (uint32_t)s_over[1];
-        }
+        uint32_t m = before + inc - c;
         if (bitmap) {
             const uint32_t w[6] = {p.x, p.y, p.z, q.x, q.y, q.z};
             if (c != 0u) {
@@ -354,31 +339,68 @@ __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const
                 for (uint32_t bits = w[i]; bits; bits &= bits - 1u, ++m)
                     if (m < g.max_list) g.cell_list[m] = cell + (uint32_t)__ffs(bits) - 1u;
             }
-        } else {
-            if (c != 0u) {
-                const uint32_t cell = sector * 8u;
-                uint32_t n[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    if (n[i] == 0u) continue;
-                    const bool over = list_over && n[i] > (uint32_t)g.cap;
-                    if (m < (uint32_t)a.capacity[sc]) a.counts[sc][m] = over ? g.cap : (int)n[i];
-                    if (m < g.max_list) g.cell_list[m] = over ? (cell + i) | kOverCap : cell + i;
-                    if (over) {
-                        g.ovf_vox[j] = (int)m; g.ovf_off[j] = (int)off; g.ovf_cell[j] = cell + i;
-                        g.ovf_cursor[(size_t)j * kCursorStride] = 0;
-                        off += n[i];
-                        n[i] = kOverCap | j++;
-                    } else {
-                        n[i] = m;
-                    }
-                    ++m;
-                }
-                at[0] = make_uint4(n[0], n[1], n[2], n[3]);
-                at[1] = make_uint4(n[4], n[5], n[6], n[7]);
-            }
+            continue;
         }
-        __syncthreads();                                  // the shared counters are used again
+        // Cells over the cap take the next places among such cells, and their points the next slots of
+        // the index list, in any order: one ticket per part.
+        uint32_t n[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+        uint32_t j = 0, off = 0, cells = 0, points = 0;
+        bool list_over = false;
+        if (g.cap > 0) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (n[i] > (uint32_t)g.cap) { cells += 1; points += clamp_points(n[i]); }
+        }
+        if (__any_sync(0xFFFFFFFFu, cells != 0)) {
+            points = clamp_points(points);
+            const uint32_t ic = warp_incl_scan(cells), ip = warp_incl_scan(points);
+            unsigned long long first = 0;
+            bool fits = false;
+            if (lane == 31) {
+                fits = ip <= g.max_list;
+                if (fits) {
+                    first = atomicAdd(reinterpret_cast<unsigned long long*>(g.totals + 2), (unsigned long long)over_ticket(ic, ip));
+                    fits = over_fits(first, ic, ip, g.max_ovf, g.max_list);
+                }
+                if (!fits) refuse_lists(g, a.status);
+            }
+            list_over = __shfl_sync(0xFFFFFFFFu, fits ? 1 : 0, 31) != 0;
+            j = __shfl_sync(0xFFFFFFFFu, (uint32_t)(first >> 32), 31) + ic - cells;
+            off = __shfl_sync(0xFFFFFFFFu, (uint32_t)first, 31) + ip - points;
+        }
+        if (c != 0u) {
+            const uint32_t cell = sector * 8u;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                if (n[i] == 0u) continue;
+                const bool over = list_over && n[i] > (uint32_t)g.cap;
+                if (m < (uint32_t)a.capacity[sc]) a.counts[sc][m] = over ? g.cap : (int)n[i];
+                if (m < g.max_list) g.cell_list[m] = over ? (cell + i) | kOverCap : cell + i;
+                if (over) {
+                    g.ovf_vox[j] = (int)m; g.ovf_off[j] = (int)off; g.ovf_cell[j] = cell + i;
+                    g.ovf_cursor[(size_t)j * kCursorStride] = 0;
+                    off += n[i];
+                    n[i] = kOverCap | j++;
+                } else {
+                    n[i] = m;
+                }
+                ++m;
+            }
+            at[0] = make_uint4(n[0], n[1], n[2], n[3]);
+            at[1] = make_uint4(n[4], n[5], n[6], n[7]);
+        }
+    }
+    // This CTA's share of the accumulators of the voxels cleared: a few tiles hold most of the voxels, so the clearing is
+    // not tied to the tiles.  Done here, just before they are added to, it also brings
+    // them into L2 (cleared after use by vox_finalize, vox_accum took 48 instead of 43 us on four nuScenes-shaped
+    // frames and vox_finalize 40 instead of 37).
+    const uint32_t thread = blockIdx.x * kRankThreads + t, threads = gridDim.x * kRankThreads;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+        const ScaleDev& g = a.s[v];
+        const uint32_t voxels = min(all[v], g.max_list);
+        for (size_t i = thread; i < (size_t)voxels * g.acc_f4; i += threads) g.acc[i] = zero;
     }
     release_successor();
 }

@@ -85,6 +85,25 @@ def test_units_tiles_and_groups_of_the_stores(oracle, which, C):
     check_voxels(w, np.ascontiguousarray(pts), oracle, rules=which in ("edges", "last_cells"))
 
 
+@pytest.mark.parametrize("B", [1, 3])
+@pytest.mark.parametrize("share", [1.0, 0.02])
+def test_parts_of_the_tiles_of_a_table_store(oracle, B, share):
+    """Parts of 32 sectors (256 cells): cells over the cap on both sides of their edges, every part or a few holding voxels."""
+    rng = np.random.default_rng(11)
+    frames = []
+    for _ in range(B):
+        few = [a for e in range(0, TABLE.cells, 256) for a in range(e - 2, e + 3) if 0 <= a < TABLE.cells and rng.random() < share]
+        few += [0, TABLE.cells - 1]
+        frames.append(centres(rng.permutation(np.repeat(few, rng.integers(1, 6, len(few)))), TABLE, 4, rng))
+    N = max(map(len, frames))
+    pts = np.full((B, N, 4), -1.0, np.float32)                 # padding outside both grids
+    for b, f in enumerate(frames):
+        pts[b, :len(f)] = f
+    fine = Grid(min=(0.0, 0.0, 0.0), voxel=(1.0, 1.0, 1.0), dims=(4099, 4099, 1), max_points=2)      # a cap on a bitmap store
+    w = replace(gen.KITTI.with_shape(B, N), grids=(fine, TABLE))
+    check_voxels(w, pts, oracle)
+
+
 @pytest.mark.parametrize("dims", [(1408, 1600, 40), (61, 7, 3), (2_000_000, 2, 2)])
 def test_cells_of_points_on_cell_boundaries(oracle, dims):
     """Points a few ulps around multiples of the cell size, far away, and not finite: cells as by subtract, divide, floor."""
