@@ -102,6 +102,12 @@ int validate(const emc2_config_t& c) {
     return EMC2_OK;
 }
 
+// float4 per accumulator.  Four channels need one where the points of a voxel are counted elsewhere: in the words of a table
+// store, or for a bitmap scale without a cap in the caller's counts.  The other dedup designs count in the accumulators.
+int accumulator_f4(const ScaleDev& d, int point_floats) {
+    return point_floats == 4 && d.design == 0 && (d.mode == MODE_TABLE || d.cap == 0) ? 1 : 2;
+}
+
 struct SlabPlan {
     size_t off = 0;
     size_t take(size_t bytes) {
@@ -159,8 +165,7 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out) {
         d.mode = total_cells <= (uint64_t)kMaxTableCells ? MODE_TABLE : MODE_BITMAP;
         const uint64_t per_tile = d.mode == MODE_BITMAP ? kBitmapTileCells : kTableTileCells;
         d.tiles = (uint32_t)((total_cells + per_tile - 1) / per_tile + kCountTiles - 1) / kCountTiles * kCountTiles;
-        // A table store knows the cells' point counts without accumulating them: four channels need one float4.
-        d.acc_f4 = d.mode == MODE_TABLE && c.point_floats == 4 ? 1 : 2;
+        d.acc_f4 = accumulator_f4(d, c.point_floats);
         d.max_ovf = d.cap > 0 ? (uint32_t)(maxpts / ((size_t)d.cap + 1) + 1) : 0;
         d.max_list = (uint32_t)maxpts;
         o_store[s] = plan.take((size_t)d.tiles * kScanTileBytes);
@@ -631,8 +636,7 @@ int emc2_bridge_set_tuning(emc2_bridge_t* h, int32_t knob, int32_t value) {
             if (rc != EMC2_OK) return rc;
         }
         h->scale[s].design = value;
-        // The other designs keep no counts per cell: the accumulators do.
-        h->scale[s].acc_f4 = value == 0 && h->scale[s].mode == MODE_TABLE && h->cfg.point_floats == 4 ? 1 : 2;
+        h->scale[s].acc_f4 = accumulator_f4(h->scale[s], h->cfg.point_floats);
         h->scale[s].point_rank = value ? h->arm.point_rank[s] : nullptr;
     }
     h->tune[knob] = value;

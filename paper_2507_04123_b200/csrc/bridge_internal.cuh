@@ -118,7 +118,7 @@ struct ScaleDev {
     uint32_t* store;        // bitmap: 16-byte units {96 cell bits, rank}; table: one word per cell, its point
                             // count while marking, then its rank or kOverCap | index among the cells over the
                             // cap.  All zero between calls
-    int acc_f4;             // float4 per accumulator: 1 or 2
+    int acc_f4;             // float4 per accumulator: 1 or 2, see accumulator_f4
     float4* acc;            // [max voxels][acc_f4] per-voxel accumulators
     uint32_t* cell_list;    // [max voxels] cell id of each unique voxel (table stores: bit 31 = over the cap)
     int* ovf_off;           // per cell over the cap j: start of its points in ovf_list
