@@ -262,6 +262,7 @@ __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const
     await_predecessor();
     constexpr int kWarps = kRankThreads / 32;
     __shared__ uint32_t s_groups[2][kRankGroups], s_sum[2][kWarps];
+    __shared__ uint2 s_words[kWarps][6 * 32];             // words of a part that have a bit
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const uint32_t listed = *a.st.listed, step = gridDim.x * kWarps;
 #pragma unroll
@@ -336,12 +337,30 @@ __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const
                 at[0] = p;
                 at[1] = q;
             }
-            uint32_t cell = sector * (2u * kUnitCells);
+            // The words with voxels side by side in shared memory, {word, voxels of the part before it, place in the part}, then a
+            // lane per word.
+            uint32_t some = 0u;
 #pragma unroll
-            for (int i = 0; i < 6; ++i, cell += 32u) {
-                for (uint32_t bits = w[i]; bits; bits &= bits - 1u, ++m)
-                    if (m < g.max_list) g.cell_list[m] = cell + (uint32_t)__ffs(bits) - 1u;
+            for (int i = 0; i < 6; ++i) some += w[i] != 0u;
+            uint32_t to = warp_incl_scan(some), rel = inc - c;
+            const uint32_t words = __shfl_sync(0xFFFFFFFFu, to, 31);
+            to -= some;
+#pragma unroll
+            for (int i = 0; i < 6; ++i) {
+                if (w[i] == 0u) continue;
+                s_words[warp][to++] = make_uint2(w[i], rel << 8 | (6u * lane + i));
+                rel += __popc(w[i]);
             }
+            __syncwarp();
+            const uint32_t cell0 = (sector - lane) * (2u * kUnitCells);
+            for (uint32_t i = lane; i < words; i += 32u) {
+                const uint2 word = s_words[warp][i];
+                const uint32_t cell = cell0 + (word.y & 255u) * 32u;
+                uint32_t row = before + (word.y >> 8);
+                for (uint32_t bits = word.x; bits; bits &= bits - 1u, ++row)
+                    if (row < g.max_list) g.cell_list[row] = cell + (uint32_t)__ffs(bits) - 1u;
+            }
+            __syncwarp();                                 // the words are used again
             continue;
         }
         // Cells over the cap take the next places among such cells, and their points the next slots of
