@@ -295,17 +295,26 @@ inline ScanReset scan_reset(const emc2_bridge* h) {
     return r;
 }
 
+// Bytes of both stores of a frame.
+inline uint64_t store_bytes(const emc2_bridge* h) {
+    uint64_t bytes = 0;
+    for (int s = 0; s < 2; ++s) {
+        const ScaleDev& g = h->scale[s];
+        if (!g.design) bytes += g.mode == MODE_BITMAP ? g.cells / kUnitCells * 16ull : g.cells * 4ull;
+    }
+    return bytes;
+}
+
 // Whether the marking pass of this call notes the tiles it touches; a handle's other dedup designs have no stores.
 inline bool keeps_tile_marks(const emc2_bridge* h, int B, int N) {
-    uint64_t words = 0, bytes = 0;
+    uint64_t words = 0;
     for (int s = 0; s < 2; ++s) {
         const ScaleDev& g = h->scale[s];
         if (g.design) return false;
         const bool bitmap = g.mode == MODE_BITMAP;
         words += most_frame_words(g.cells, bitmap ? kBitmapTileCells : kTableTileCells);
-        bytes += bitmap ? g.cells / kUnitCells * 16ull : g.cells * 4ull;
     }
-    return keeps_notes(bytes, words, B, N);
+    return keeps_notes(store_bytes(h), words, B, N);
 }
 
 inline TileMarks tile_marks(const emc2_bridge* h, int B, int N) {

@@ -218,6 +218,7 @@ struct PrArgs {
     int N, tiles, K, H, W;
     float min_depth;
     RouteParams rp;
+    int B, frames_log;
     int frame0;           // kMark: frame index (in the whole batch) of this launch's first frame
     ScaleDev s0, s1;      // kMark: the voxel grids whose cells the points mark
     float4* bev;          // kMark: BEV image to zero (bev_n4 float4), or null
@@ -226,7 +227,7 @@ struct PrArgs {
     TileMarks marks;      // kNote
 };
 
-// grid = (tiles per frame, B); tiles never straddle frames.  kMark: the kernel also does the
+// grid = (tiles per frame << frames_log, groups of frames), see frames_side_by_side; tiles never straddle frames.  kMark: the kernel also does the
 // voxelizer's marking pass (every point marks its cell in both scales' stores, and the BEV image
 // is zeroed, spread over the grid), so that stage 1 starts from marked stores and reads the
 // points once less; the reductions are fire-and-forget and land while the projection computes.
@@ -238,14 +239,15 @@ __global__ void __launch_bounds__(kThreads, 8) project_route_kernel(const __grid
     __shared__ __align__(16) float suvd[kTile * 3];
     __shared__ int hist[EMC2_MAX_EXPERTS];
     __shared__ Camera sP[EMC2_MAX_CAMERAS];
-    const int b = blockIdx.y, tile = blockIdx.x, t = threadIdx.x, lane = t & 31;
-    load_cameras(a.proj, b, 1, a.K, sP);
+    const int t = threadIdx.x, lane = t & 31;
+    const int tile = (int)(blockIdx.x >> a.frames_log), b = (int)((blockIdx.y << a.frames_log) + (blockIdx.x & ((1u << a.frames_log) - 1u)));
+    if (b < a.B) load_cameras(a.proj, b, 1, a.K, sP);
     const int i0 = tile * kTile;
-    const int npts = min(kTile, a.N - i0);
+    const int npts = b < a.B ? min(kTile, a.N - i0) : 0;       // the last group can have fewer frames
     const size_t g0 = (size_t)b * a.N + i0;
     if (t < EMC2_MAX_EXPERTS) hist[t] = 0;
     FrameTiles* const tiles = frame_tiles<kNote>();
-    if (kNote) begin_tiles(*tiles, a.s0, a.s1, (uint32_t)(a.frame0 + b));
+    if (kNote && b < a.B) begin_tiles(*tiles, a.s0, a.s1, (uint32_t)(a.frame0 + b));
     __syncthreads();
     int e = -1;
     if (t < npts) {
@@ -284,8 +286,8 @@ __global__ void __launch_bounds__(kThreads, 8) project_route_kernel(const __grid
         if (lane == 0 && m) atomicAdd(&hist[k], __popc(m));
     }
     __syncthreads();
-    if (t < a.rp.E) a.tile_counts[((size_t)b * a.tiles + tile) * a.rp.E + t] = hist[t];
-    if (kNote) publish_tiles(*tiles, a.marks);
+    if (t < a.rp.E && b < a.B) a.tile_counts[((size_t)b * a.tiles + tile) * a.rp.E + t] = hist[t];
+    if (kNote && b < a.B) publish_tiles(*tiles, a.marks);
     if (kMark) {
         const size_t cta = (size_t)blockIdx.y * gridDim.x + blockIdx.x, nthreads = (size_t)gridDim.x * gridDim.y * kThreads;
         reset_scan(a.reset, cta * kThreads + t, nthreads);
@@ -799,7 +801,8 @@ int launch_project_route(emc2_bridge* h, int b0, int B, int N, const float* d_po
     const emc2_config_t& c = h->cfg;
     const int tiles = (N + kTile - 1) / kTile;
     if (B == 0 || tiles == 0) return EMC2_OK;
-    const dim3 grid(tiles, B);
+    const int frames_log = frames_side_by_side(store_bytes(h), B);
+    const dim3 grid(tiles << frames_log, (B + (1 << frames_log) - 1) >> frames_log);
     const size_t p0 = (size_t)b0 * N;                      // first point of the range
     PrArgs pa;
     pa.pts = d_points + p0 * c.point_floats; pa.proj = d_proj + (size_t)b0 * c.num_cameras * 12;
@@ -808,6 +811,7 @@ int launch_project_route(emc2_bridge* h, int b0, int B, int N, const float* d_po
     pa.N = N; pa.tiles = tiles; pa.K = c.num_cameras; pa.H = c.img_h; pa.W = c.img_w;
     pa.min_depth = c.min_depth;
     pa.rp = route_params(h);
+    pa.B = B; pa.frames_log = frames_log;
     pa.frame0 = b0;
     pa.s0 = h->scale[0]; pa.s1 = h->scale[1];
     pa.bev = nullptr; pa.bev_n4 = 0;

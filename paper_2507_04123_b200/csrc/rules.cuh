@@ -142,6 +142,19 @@ inline bool keeps_notes(uint64_t frame_bytes, uint64_t words, int B, int N) {
     return words <= kMarkWords && B * frame_bytes >= (uint64_t)24 << 20 && N <= 1 << 17;
 }
 
+// ---- which tile of which frame a CTA of a marking pass takes: groups of 1 << log frames, whose tiles take turns
+// Marks that land in one sector of a store are served one after another, and the sector of pillars next to the sensor gets about
+// a thousand of a nuScenes-shaped frame's 300,000 points: frame after frame, four of them took project_route 45 us.  With the
+// frames side by side those marks are spread over the whole kernel: 37 (vox_mark 37 -> 29).  Their stores should fit in L2
+// together, us without / with groups of 32, 64, 128 and 256 MB: four nuScenes-shaped frames 44.7 / 38.7, 37.2, 37.2, 37.3; eight
+// KITTI-shaped ones, whose first ring of points is farther away, 43.6 / 42.9, 42.6, 43.1, 42.7; 32 frames of 262,144
+// KITTI-shaped points (480 MB) 193 / 198, 198, 201, 205, all 32 side by side 222.
+inline int frames_side_by_side(uint64_t frame_bytes, int B) {
+    int log = 0;
+    while ((1 << log) < B && (frame_bytes << (log + 1)) <= (uint64_t)64 << 20) ++log;
+    return log;
+}
+
 // Four bytes that are 0 or 1 -> four bits, the lowest byte in the lowest bit.
 EMC2_RULE uint32_t bits_of_bytes(uint32_t bytes) { return bytes * 0x01020408u >> 24 & 15u; }
 

@@ -72,15 +72,17 @@ __device__ __forceinline__ bool counts_in_output(const ScaleDev& g) { return g.m
 __device__ __forceinline__ float cell_corner(float mn, float vs, int i) { return __fmaf_rn((float)i, vs, mn); }
 
 // ------------------------------------------------------------------ pass 1: mark cells
-// grid = (tiles per frame, B), at least; tiles never straddle frames.
+// grid = (tiles per frame << frames_log, groups of frames), at least, see frames_side_by_side; tiles never straddle frames.
 template <int C>
 __global__ void __launch_bounds__(kThreads)
-vox_mark_kernel(const float* __restrict__ pts, int N, const __grid_constant__ ScaleDev s0, const __grid_constant__ ScaleDev s1,
+vox_mark_kernel(const float* __restrict__ pts, int B, int N, int frames_log, const __grid_constant__ ScaleDev s0, const __grid_constant__ ScaleDev s1,
                 float4* bev, size_t bev_n4, ScanReset reset, TileMarks marks) {
     __shared__ FrameTiles tiles;
     const size_t thread = ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * kThreads + threadIdx.x;
     const size_t nthreads = (size_t)gridDim.x * gridDim.y * kThreads;
-    const int b = blockIdx.y, i = blockIdx.x * kThreads + threadIdx.x;
+    const int b = (int)((blockIdx.y << frames_log) + (blockIdx.x & ((1u << frames_log) - 1u)));
+    const int i = (int)((blockIdx.x >> frames_log) * kThreads + threadIdx.x);
+    if (b >= B) N = 0;                            // the last group can have fewer frames
     float x = 0.f, y = 0.f, z = 0.f;
     if (i < N) {
         const float* p = pts + ((size_t)b * N + i) * C;
@@ -91,7 +93,7 @@ vox_mark_kernel(const float* __restrict__ pts, int N, const __grid_constant__ Sc
             x = __ldg(p); y = __ldg(p + 1); z = __ldg(p + 2);
         }
     }
-    if (marks.marked[0]) {
+    if (marks.marked[0] && b < B) {
         begin_tiles(tiles, s0, s1, (uint32_t)b);
         __syncthreads();
     }
@@ -106,7 +108,7 @@ vox_mark_kernel(const float* __restrict__ pts, int N, const __grid_constant__ Sc
         const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
         for (size_t k = thread; k < bev_n4; k += nthreads) __stcs(bev + k, zero);
     }
-    if (marks.marked[0]) {
+    if (marks.marked[0] && b < B) {
         __syncthreads();
         publish_tiles(tiles, marks);
     }
@@ -830,10 +832,11 @@ int run_voxelize(emc2_bridge* h, int B, int N, const float* d_points, int32_t* c
     if (!marked) {
         // Also zeroes the BEV image; with no points it still runs for that.
         const int zeroing = bev_n && bev_vec ? (h->num_sms + B - 1) / B : 0;
-        const dim3 grid(max((N + kTile - 1) / kTile, zeroing), B);
+        const int frames_log = frames_side_by_side(store_bytes(h), B);
+        const dim3 grid(max((N + kTile - 1) / kTile, zeroing) << frames_log, (B + (1 << frames_log) - 1) >> frames_log);
         if (B > 0 && grid.x > 0) {
             LaunchScope ls(h, K_VOX_MARK, st);
-            vox_mark_kernel<C><<<grid, kThreads, 0, st>>>(d_points, N, sa.s[0], sa.s[1],
+            vox_mark_kernel<C><<<grid, kThreads, 0, st>>>(d_points, B, N, frames_log, sa.s[0], sa.s[1],
                                                           bev_vec ? reinterpret_cast<float4*>(d_bev) : nullptr,
                                                           bev_vec ? bev_n >> 2 : 0, scan_reset(h), tile_marks(h, B, N));
         }
