@@ -181,7 +181,7 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out) {
     const size_t o_tiles = plan.take((tiles[0] + tiles[1]) * sizeof(uint32_t));
     const size_t o_parts = plan.take((tiles[0] + tiles[1]) * sizeof(uint4));
     const size_t marked[2] = {(tiles[0] + 31) / 32, (tiles[1] + 31) / 32};
-    const size_t o_marked = plan.take((marked[0] + marked[1]) * sizeof(uint32_t));
+    const size_t o_marked = plan.take(kNoteCopies * ((marked[0] + marked[1] + 31) / 32 * 32) * sizeof(uint32_t));
     const size_t o_list = plan.take((tiles[0] + tiles[1]) * 8 * sizeof(uint32_t));
     h->scan_reset_words = (int)(groups[0] + groups[1] + 1);
     const size_t o_groups = plan.take((size_t)h->scan_reset_words * sizeof(uint32_t));
@@ -226,6 +226,7 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out) {
     h->scan.list = reinterpret_cast<uint32_t*>(base + o_list);
     h->scan.marked[0] = reinterpret_cast<uint32_t*>(base + o_marked);
     h->scan.marked[1] = h->scan.marked[0] + marked[0];
+    h->scan.note_stride = (uint32_t)((marked[0] + marked[1] + 31) / 32 * 32);
     h->scan.group_voxels[0] = reinterpret_cast<uint32_t*>(base + o_groups);
     h->scan.group_voxels[1] = h->scan.group_voxels[0] + groups[0];
     h->scan.listed = h->scan.group_voxels[1] + groups[1];

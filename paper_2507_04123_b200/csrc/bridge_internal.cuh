@@ -150,12 +150,20 @@ struct ScanState {
     uint32_t* listed;           // parts in `list`; zero when the scan begins
     uint32_t* list;             // [8 * tiles of both scales] parts that hold voxels, in any order: 8 * tile + part; bit 31: scale 1
     uint32_t* marked[2];        // a bit per tile of a store: a cell of it was marked; zero between calls
+    uint32_t note_stride;       // words from one copy of the notes to the next
     int words[2];               // words of `marked` to clear, 0 where the marking pass does not keep it
 };
+
+// The notes are kept in this many copies, and a CTA sends its own to one of them: reductions on one word are served one after another,
+// and every CTA has some for the few words of the ground plane.  us for 1, 4, 8 and 16 copies: eight KITTI-shaped frames
+// 42.4, 33.8, 33.4, 33.1 (project_route; 32.1 without notes), the call 202.4, 194.3, 193.6, 193.8; vox_mark 36.5, 28.0, 27.6,
+// 27.2.  Reading a word first, to send only what is new, adds to the same queue: 52.8 with one copy.
+constexpr uint32_t kNoteCopies = 8;
 
 // Where the marking pass notes the tiles that it touches (see keeps_tile_marks), or null.
 struct TileMarks {
     uint32_t* marked[2];
+    uint32_t stride;            // words from one copy to the next
 };
 
 // What of it is zeroed when a call begins, by whichever kernel marks the cells.
@@ -314,11 +322,11 @@ inline bool keeps_tile_marks(const emc2_bridge* h, int B, int N) {
         const bool bitmap = g.mode == MODE_BITMAP;
         words += most_frame_words(g.cells, bitmap ? kBitmapTileCells : kTableTileCells);
     }
-    return keeps_notes(store_bytes(h), words, B, N);
+    return keeps_notes(store_bytes(h), words, B, (N + (int)kNoteCopies - 1) / (int)kNoteCopies);
 }
 
 inline TileMarks tile_marks(const emc2_bridge* h, int B, int N) {
-    TileMarks m = {{nullptr, nullptr}};
+    TileMarks m = {{nullptr, nullptr}, h->scan.note_stride};
     if (keeps_tile_marks(h, B, N))
         for (int s = 0; s < 2; ++s) m.marked[s] = h->scan.marked[s];
     return m;
@@ -458,10 +466,8 @@ __device__ __forceinline__ void note_tiles(FrameTiles& f, const int tile[2]) {
     if (tile[1] >= 0) f.seen[32 * f.words[0] + tile[1] - 32 * f.word0[1]] = 1;
 }
 
-// One fire-and-forget reduction per word: a load first, to send only what is not noted yet, holds the CTA until its marks
-// have drained (eight KITTI-shaped frames: project_route 45 instead of 42 us, 31 without the notes).  A byte or a sector
-// per tile instead of a bit: 45 and 58.
-__device__ __forceinline__ void publish_tiles(const FrameTiles& f, const TileMarks& to) {
+// One fire-and-forget reduction per word, in copy `copy` % kNoteCopies of the notes.
+__device__ __forceinline__ void publish_tiles(const FrameTiles& f, const TileMarks& to, uint32_t copy) {
     const uint32_t t = threadIdx.x, n0 = f.words[0];
     if (t >= n0 + f.words[1]) return;
     const uint4* bytes = reinterpret_cast<const uint4*>(f.seen) + 2 * t;
@@ -469,7 +475,7 @@ __device__ __forceinline__ void publish_tiles(const FrameTiles& f, const TileMar
     const uint32_t mine = bits_of_bytes(p.x) | bits_of_bytes(p.y) << 4 | bits_of_bytes(p.z) << 8 | bits_of_bytes(p.w) << 12 |
                           bits_of_bytes(q.x) << 16 | bits_of_bytes(q.y) << 20 | bits_of_bytes(q.z) << 24 | bits_of_bytes(q.w) << 28;
     uint32_t* w = t < n0 ? to.marked[0] + f.word0[0] + t : to.marked[1] + f.word0[1] + (t - n0);
-    if (mine) atomicOr(w, mine);
+    if (mine) atomicOr(w + (copy % kNoteCopies) * to.stride, mine);
 }
 
 __device__ __forceinline__ void reset_scan(const ScanReset& r, size_t thread, size_t nthreads) {

@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(kThreads, 8) project_route_kernel(const __grid
     }
     __syncthreads();
     if (t < a.rp.E && b < a.B) a.tile_counts[((size_t)b * a.tiles + tile) * a.rp.E + t] = hist[t];
-    if (kNote && b < a.B) publish_tiles(*tiles, a.marks);
+    if (kNote && b < a.B) publish_tiles(*tiles, a.marks, (uint32_t)tile);
     if (kMark) {
         const size_t cta = (size_t)blockIdx.y * gridDim.x + blockIdx.x, nthreads = (size_t)gridDim.x * gridDim.y * kThreads;
         reset_scan(a.reset, cta * kThreads + t, nthreads);

@@ -127,16 +127,15 @@ EMC2_RULE uint32_t frame_words(uint32_t b, uint32_t cells, uint32_t per_tile) {
 }
 inline uint32_t most_frame_words(uint32_t cells, uint32_t per_tile) { return cells / per_tile / 32u + 2u; }
 
-// Whether the marking pass of a call keeps the notes: frames of N points whose stores take `frame_bytes` each (8 KB tiles
-// `words` words of notes).  The counting pass then reads the noted tiles instead of the whole stores, three quarters of
-// which are empty space.  One frame's stores are read as fast as the notes come back (voxels and rulebooks of 30,000 points
-// 56 and 57 us); frames of many points pay more for noting, whose reductions meet in the few sectors of the ground plane, than
-// the reading costs.  us per call without / with the notes, KITTI-shaped frames of 64 channels: 2 of 30,000 points 33.6 / 32.4,
-// 32 of 16,384 284 / 237, 8 of 60,000 139.5 / 130.8, of 100,000 191.1 / 187.2, of 131,072 228.6 / 226.2, of 160,000 261.2 /
-// 260.9; 32 of 131,072 853.9 / 853.5.  Six cameras and 80 channels: 2 of 2,000 47.1 / 42.3, 8 of 131,072 320.7 / 315.0, of
-// 160,000 373 / 366.7.  Voxel lists alone: 4 of 300,000 KITTI-shaped 102.3 / 112.1, nuScenes-shaped 141.6 / 140.0, 32 of
-// 131,072 458 / 463 and 600 / 585.  The 72 words hold the frames of both grid families (64 and 55 words); larger grids, which
-// would need more shared memory, have not been measured with notes.
+// Whether the marking pass of a call keeps the notes: frames of which N points note in the same copy (see kNoteCopies) and whose
+// stores take `frame_bytes` each (8 KB tiles, `words` words of notes).  The counting pass then reads the noted tiles instead of
+// the whole stores, three quarters of which are empty space.  One frame's stores are read as fast as the notes come back (voxels
+// and rulebooks of 30,000 points 56 and 57 us).  The more points note in one copy the longer the queues at its words: with a single
+// copy notes lost from about 2^17 points on (voxel lists of four KITTI-shaped frames of 300,000 points 102 us without, 112 with);
+// with eight, us per call without / with the notes: four nuScenes-shaped frames of 300,000 points 302 / 296.6, their voxels and
+// rulebooks 216.4 / 212.0, 32 KITTI-shaped frames of 262,144 points and six cameras 1,766 / 1,732, eight of 120,000 points 207.0 /
+// 193.6.  Frames of more than 2^20 points have not been measured.  The 72 words hold the frames of both grid families (64 and 55
+// words); larger grids, which would need more shared memory, have not been measured with notes.
 constexpr uint32_t kMarkWords = 72;
 inline bool keeps_notes(uint64_t frame_bytes, uint64_t words, int B, int N) {
     return words <= kMarkWords && B * frame_bytes >= (uint64_t)24 << 20 && N <= 1 << 17;

@@ -110,7 +110,7 @@ vox_mark_kernel(const float* __restrict__ pts, int B, int N, int frames_log, con
     }
     if (marks.marked[0] && b < B) {
         __syncthreads();
-        publish_tiles(tiles, marks);
+        publish_tiles(tiles, marks, blockIdx.x >> frames_log);
     }
     release_successor();
 }
@@ -224,8 +224,8 @@ __global__ void __launch_bounds__(kThreads) vox_count_kernel(const __grid_consta
 
 // The same where the marking pass noted the tiles it touched: only those are looked at (vox_rank clears the notes).  A
 // fixed grid of CTAs, each with at most kThreads groups of four tiles.  us by events, whole stores / noted tiles: eight
-// KITTI-shaped frames (127 MB of stores) 28.3 / 15.4, while the marking pass goes from 27.5 to 38.4 and project_route, where
-// it does the marking, from 32.5 to 42.3; four of 60,000 points 18.8 / 12.7 and 14.6 / 16.2.  See keeps_notes for whole calls.
+// KITTI-shaped frames (127 MB of stores) 28.7 / 16.9, while project_route, which does the marking, goes from 32.1 to 33.4; four
+// nuScenes-shaped ones 16.8 / 11.4 and 37.3 / 39.5.  See keeps_notes for whole calls.
 __global__ void __launch_bounds__(kThreads) vox_count_marked_kernel(const __grid_constant__ ScanArgs a) {
     await_predecessor();
     __shared__ uint32_t s_warp[kCountTiles][kThreads / 32], s_which[kThreads];
@@ -234,7 +234,9 @@ __global__ void __launch_bounds__(kThreads) vox_count_marked_kernel(const __grid
     uint32_t which = 0u;
     if (mine < words) {
         const int sc = mine < words1 ? 1 : 0, w = sc ? mine : mine - words1;
-        which = a.st.marked[sc][w / 8] >> (w % 8 * 4) & 15u;
+#pragma unroll
+        for (uint32_t r = 0; r < kNoteCopies; ++r) which |= a.st.marked[sc][w / 8 + r * a.st.note_stride];
+        which = which >> (w % 8 * 4) & 15u;
         if (!which) *reinterpret_cast<uint4*>(a.st.tile_voxels[sc] + w * kCountTiles) = make_uint4(0u, 0u, 0u, 0u);
     }
     s_which[t] = which;
@@ -269,7 +271,9 @@ __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const
     const uint32_t listed = *a.st.listed, step = gridDim.x * kWarps;
 #pragma unroll
     for (int v = 0; v < 2; ++v)                           // vox_count has read the notes
-        for (int i = blockIdx.x * kRankThreads + t; i < a.st.words[v]; i += gridDim.x * kRankThreads) a.st.marked[v][i] = 0u;
+        for (int i = blockIdx.x * kRankThreads + t; i < a.st.words[v]; i += gridDim.x * kRankThreads)
+#pragma unroll
+            for (uint32_t r = 0; r < kNoteCopies; ++r) a.st.marked[v][i + r * a.st.note_stride] = 0u;
     uint32_t k = (uint32_t)warp * gridDim.x + blockIdx.x, next = 0u;
     uint32_t entry = k < listed ? a.st.list[k] : 0u;
     // Voxels before every group of tiles, and of both scales.

@@ -236,6 +236,25 @@ def test_pooled_sampling_of_cut_windows(oracle, cf, hw, p):
     br.close()
 
 
+@pytest.mark.parametrize("base,B,N", [(gen.KITTI, 3, 700), (gen.KITTI, 5, 257), (gen.NUSCENES, 9, 300), (gen.KITTI, 2, 140000),
+                                      (gen.DENSE, 2, 3000)], ids=lambda v: getattr(v, "name", str(v)))
+def test_frames_that_take_turns_with_notes(oracle, base, B, N):
+    """Groups of frames that are not full, frames of one tile and a little, and more points per frame than one copy of the notes takes."""
+    w = replace(base.with_shape(B, N), feat_c=4)
+    refs = []
+    for i in range(2):
+        batch = gen.make_batch(w, frames=[B * i + k for k in range(B)])
+        refs.append((batch, oracle.bridge(w, batch)))
+    for step in ("run", "run_staged"):
+        br = bridge_for(w)
+        for batch, ref in (refs[0], refs[1], refs[0]):
+            d = to_dev(batch)
+            bufs = getattr(br, step)(d["points"], d["proj"], d["feat"])
+            br.status()
+            compare_bridge(w, ref, bufs)
+        br.close()
+
+
 @pytest.mark.parametrize("base,B,N,cf", [(gen.KITTI, 1, 131072, 256), (gen.KITTI, 1, 131073, 256), (gen.KITTI, 2, 66000, 260),
                                          (gen.NUSCENES, 2, 209715, 80), (gen.NUSCENES, 2, 209716, 80)],
                          ids=lambda v: getattr(v, "name", str(v)))

@@ -114,6 +114,19 @@ def test_calls_that_keep_notes(rules):
         assert not rules.notes(frame, words, 32, (1 << 17) + 1) and not rules.notes(frame, 73, 32, 1000)
 
 
+def test_frames_side_by_side(rules):
+    """Groups are as large as the frames need or 64 MB of stores allow, and their CTAs take every tile of every frame once."""
+    for frame in (0, 1, 13_488_272, 15_898_656, 32 << 20, (32 << 20) + 1, 64 << 20, 65 << 20, 700 << 20):
+        for B in (1, 2, 3, 4, 5, 7, 8, 9, 31, 32):
+            log = rules.frames_log(frame, B)
+            G = 1 << log
+            assert G == 1 or (G * frame <= 64 << 20 and G < 2 * B)
+            assert G >= B or 2 * G * frame > 64 << 20
+            groups = (B + G - 1) >> log
+            taken = [((y << log) + (x & (G - 1)), x >> log) for y in range(groups) for x in range(3 << log)]
+            assert sorted(t for t in taken if t[0] < B) == [(b, i) for b in range(B) for i in range(3)]
+
+
 def test_gathered_rows_that_stay_in_l2(rules):
     for points, feat_c, stays in ((120000, 256, 1), (131072, 256, 1), (131073, 256, 0), (419430, 80, 1), (419431, 80, 0), (1, 4, 1),
                                   (1 << 24, 1020, 0)):
