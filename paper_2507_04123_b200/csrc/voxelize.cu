@@ -259,14 +259,15 @@ __device__ __forceinline__ void refuse_lists(const ScaleDev& g, int* status) {
 }
 
 constexpr int kRankThreads = 256, kRankCtas = 6;
-constexpr int kRankGroups = 3 * kRankThreads;             // groups of tiles: at most 683 of a bitmap store, see validate
+static_assert(0xFFFFFF00u / kBitmapTileCells / kTilesPerGroup < 3 * kRankThreads, "a thread has up to three groups of tiles of a scale, see validate");
 static_assert(kScanSectors == 8 * 32, "a tile has eight parts, one sector for each lane of a warp");
 
 __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const __grid_constant__ ScanArgs a) {
     await_predecessor();
     constexpr int kWarps = kRankThreads / 32;
-    __shared__ uint32_t s_groups[2][kRankGroups], s_sum[2][kWarps];
-    __shared__ uint2 s_words[kWarps][6 * 32];             // words of a part that have a bit
+    extern __shared__ uint32_t s_groups[];                // [groups of both scales]
+    __shared__ uint32_t s_sum[2][kWarps], s_words[kWarps][6 * 32];    // words of a part that have a bit
+    const uint32_t groups0 = (uint32_t)(a.tiles[0] + kTilesPerGroup - 1) / kTilesPerGroup;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const uint32_t listed = *a.st.listed, step = gridDim.x * kWarps;
 #pragma unroll
@@ -298,7 +299,10 @@ __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const
             all[v] = __reduce_add_sync(0xFFFFFFFFu, own);
             uint32_t run = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? own : 0u) + inc[v] - sum[v];
 #pragma unroll
-            for (int i = 0; i < 3; ++i) { s_groups[v][3 * t + i] = run; run += n[v][i]; }
+            for (int i = 0; i < 3; ++i) {
+                if ((3 * t + i) * kTilesPerGroup < a.tiles[v]) s_groups[v * groups0 + 3 * t + i] = run;
+                run += n[v][i];
+            }
         }
         __syncthreads();
     }
@@ -331,7 +335,7 @@ __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const
         uint32_t before = lane < part ? reinterpret_cast<const uint16_t*>(a.st.tile_parts[sc] + tile)[lane] : 0u;
         before += (k0 < in_group ? four.x : 0u) + (k0 + 1 < in_group ? four.y : 0u) + (k0 + 2 < in_group ? four.z : 0u) +
                   (k0 + 3 < in_group ? four.w : 0u);
-        before = __reduce_add_sync(0xFFFFFFFFu, before) + s_groups[sc][tile / kTilesPerGroup];
+        before = __reduce_add_sync(0xFFFFFFFFu, before) + s_groups[sc * groups0 + tile / kTilesPerGroup];
         const uint32_t c = sector_voxels(bitmap, p, q);
         const uint32_t inc = warp_incl_scan(c);
         uint32_t m = before + inc - c;
@@ -343,7 +347,7 @@ __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const
                 at[0] = p;
                 at[1] = q;
             }
-            // The words with voxels side by side in shared memory, {word, voxels of the part before it, place in the part}, then a
+            // The words with voxels side by side in shared memory, {voxels of the part before it, number, lane that has it}, then a
             // lane per word.
             uint32_t some = 0u;
 #pragma unroll
@@ -354,16 +358,22 @@ __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const
 #pragma unroll
             for (int i = 0; i < 6; ++i) {
                 if (w[i] == 0u) continue;
-                s_words[warp][to++] = make_uint2(w[i], rel << 8 | (6u * lane + i));
+                s_words[warp][to++] = rel << 8 | i << 5 | lane;
                 rel += __popc(w[i]);
             }
             __syncwarp();
             const uint32_t cell0 = (sector - lane) * (2u * kUnitCells);
-            for (uint32_t i = lane; i < words; i += 32u) {
-                const uint2 word = s_words[warp][i];
-                const uint32_t cell = cell0 + (word.y & 255u) * 32u;
-                uint32_t row = before + (word.y >> 8);
-                for (uint32_t bits = word.x; bits; bits &= bits - 1u, ++row)
+            for (uint32_t i0 = 0u; i0 < words; i0 += 32u) {
+                const uint32_t word = i0 + lane < words ? s_words[warp][i0 + lane] : 7u << 5;
+                const uint32_t number = word >> 5 & 7u, from = word & 31u;
+                uint32_t bits = 0u;
+#pragma unroll
+                for (int i = 0; i < 6; ++i) {
+                    const uint32_t theirs = __shfl_sync(0xFFFFFFFFu, w[i], from);
+                    if (number == i) bits = theirs;
+                }
+                const uint32_t cell = cell0 + from * (2u * kUnitCells) + number * 32u;
+                for (uint32_t row = before + (word >> 8); bits; bits &= bits - 1u, ++row)
                     if (row < g.max_list) g.cell_list[row] = cell + (uint32_t)__ffs(bits) - 1u;
             }
             __syncwarp();                                 // the words are used again
@@ -862,7 +872,8 @@ int run_voxelize(emc2_bridge* h, int B, int N, const float* d_points, int32_t* c
                 launch_kernel(!marked || chained, vox_count_kernel, tiles / kCountTiles, kThreads, 0, st, sa);
         }
         LaunchScope ls(h, K_VOX_RANK, st);
-        launch_chained(vox_rank_kernel, min(tiles, kRankCtas * h->num_sms), kRankThreads, 0, st, sa);
+        const int groups = (sa.tiles[0] + kTilesPerGroup - 1) / kTilesPerGroup + (sa.tiles[1] + kTilesPerGroup - 1) / kTilesPerGroup;
+        launch_chained(vox_rank_kernel, min(tiles, kRankCtas * h->num_sms), kRankThreads, groups * sizeof(uint32_t), st, sa);
     }
     if (total > 0) {
         LaunchScope ls(h, K_VOX_ACCUM, st);
