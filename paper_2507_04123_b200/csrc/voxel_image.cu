@@ -6,7 +6,7 @@
 // Rows are 256/320 bytes: adding them up with reductions would cost twenty 16-byte requests per
 // point.  Instead the visible points are listed per voxel and each voxel reads its points' rows whole:
 //   vif_scan   exclusive prefix sums of the voxels' kept-point counts (the prefix-sum indexing of Sec. 3.6) -> start
-//              of every voxel's list.  The sums go over 4096 voxels; a CTA takes their part of the list array with one
+//              of every voxel's list.  The sums go over 1024 voxels; a CTA takes their part of the list array with one
 //              ticket, so that no pass over all the counts has to come first.
 //   vif_fill   every kept point that a camera sees takes a ticket in its voxel's list (one atomic with return).
 //   vif_mean   16 voxels x Cf/4 columns of threads per CTA: a voxel's threads walk its list and
@@ -50,8 +50,10 @@ __device__ __forceinline__ int voxels_in_use(const VifArgs& a) { return min(*a.n
 // A warp has kScanRows * 32 consecutive voxels, a CTA eight times as many and one ticket: tickets on one address are
 // served one after another (about 10 ns each).  As a cooperative launch that summed all counts before any start was known
 // this took 14.3 us for the lists of four nuScenes-shaped frames (mean of both scales, by events), now 10.7; the fill, which
-// looked the start up and listed invisible points as well, 26.9, now 22.7; both scales together 300.7 -> 282.1 us.
-constexpr int kScanRows = 16, kScanVoxels = kThreads * kScanRows;
+// looked the start up and listed invisible points as well, 26.9, now 22.7; both scales together 300.7 -> 282.1 us.  A CTA of 4,096,
+// 2,048, 1,024 or 512 voxels: both scales of four nuScenes-shaped frames 274.8, 269.7, 268.7, 270.2 us (more CTAs in flight, more
+// tickets), of two KITTI-shaped frames 50.2, 45.7, 44.6, 44.7.
+constexpr int kScanRows = 4, kScanVoxels = kThreads * kScanRows;
 
 __global__ void __launch_bounds__(kThreads) vif_scan_kernel(const __grid_constant__ VifArgs a) {
     __shared__ int wsum[kThreads / 32];
