@@ -163,7 +163,9 @@ constexpr uint32_t kNoteCopies = 8;
 // Where the marking pass notes the tiles that it touches (see keeps_tile_marks), or null.
 struct TileMarks {
     uint32_t* marked[2];
-    uint32_t stride;            // words from one copy to the next
+    uint32_t stride;                        // words from one copy to the next
+    uint16_t word0[2][EMC2_MAX_BATCH];      // first word of `marked` that has tiles of the frame, per scale (a store has at most
+    uint16_t words[2][EMC2_MAX_BATCH];      // 2,731 words), and how many
 };
 
 // What of it is zeroed when a call begins, by whichever kernel marks the cells.
@@ -326,11 +328,23 @@ inline bool keeps_tile_marks(const emc2_bridge* h, int B, int N) {
 }
 
 inline TileMarks tile_marks(const emc2_bridge* h, int B, int N) {
-    TileMarks m = {{nullptr, nullptr}, h->scan.note_stride};
-    if (keeps_tile_marks(h, B, N))
-        for (int s = 0; s < 2; ++s) m.marked[s] = h->scan.marked[s];
+    TileMarks m = {};
+    if (!keeps_tile_marks(h, B, N)) return m;
+    m.stride = h->scan.note_stride;
+    for (int s = 0; s < 2; ++s) {
+        const ScaleDev& g = h->scale[s];
+        const uint32_t per = g.mode == MODE_BITMAP ? kBitmapTileCells : kTableTileCells;
+        m.marked[s] = h->scan.marked[s];
+        for (int b = 0; b < B; ++b) {
+            m.word0[s][b] = (uint16_t)frame_first_word((uint32_t)b, g.cells, per);
+            m.words[s][b] = (uint16_t)frame_words((uint32_t)b, g.cells, per);
+        }
+    }
     return m;
 }
+
+// Whether the marking kernels zero a BEV image of n floats: whole float4, counted in 32 bits (a grid has far less than 2^30 threads).
+inline bool bev_by_kernel(size_t n) { return (n & 3) == 0 && n >> 2 < (size_t)3 << 30; }
 
 inline RouteParams route_params(const emc2_bridge* h) {
     RouteParams rp;
@@ -434,8 +448,6 @@ __device__ __forceinline__ void mark_point(const ScaleDev& s0, const ScaleDev& s
 
 // ---- the tiles of the stores that a CTA of a marking pass touches, all of one frame
 struct FrameTiles {
-    uint32_t word0[2];                      // first word of `marked` that has tiles of the frame, per scale
-    uint32_t words[2];                      // and how many
     __align__(16) uint8_t seen[kMarkWords * 32];        // a byte per tile, scale 1 behind scale 0
 };
 
@@ -451,39 +463,41 @@ __device__ __forceinline__ FrameTiles* frame_tiles() {
 }
 
 // The caller synchronises the CTA before the first note_tiles and before publish_tiles.
-__device__ __forceinline__ void begin_tiles(FrameTiles& f, const ScaleDev& s0, const ScaleDev& s1, uint32_t b) {
-    if (threadIdx.x < 2) {
-        const ScaleDev& g = threadIdx.x ? s1 : s0;
-        const uint32_t per = g.mode == MODE_BITMAP ? kBitmapTileCells : kTableTileCells;
-        f.word0[threadIdx.x] = frame_first_word(b, g.cells, per);
-        f.words[threadIdx.x] = frame_words(b, g.cells, per);
-    }
+__device__ __forceinline__ void begin_tiles(FrameTiles& f) {
     if (threadIdx.x < kMarkWords * 2) reinterpret_cast<uint4*>(f.seen)[threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-__device__ __forceinline__ void note_tiles(FrameTiles& f, const int tile[2]) {
-    if (tile[0] >= 0) f.seen[tile[0] - 32 * f.word0[0]] = 1;
-    if (tile[1] >= 0) f.seen[32 * f.words[0] + tile[1] - 32 * f.word0[1]] = 1;
+__device__ __forceinline__ void note_tiles(FrameTiles& f, const TileMarks& to, int b, const int tile[2]) {
+    if (tile[0] >= 0) f.seen[tile[0] - 32 * (int)to.word0[0][b]] = 1;
+    if (tile[1] >= 0) f.seen[tile[1] - 32 * ((int)to.word0[1][b] - (int)to.words[0][b])] = 1;
 }
 
-// One fire-and-forget reduction per word, in copy `copy` % kNoteCopies of the notes.
-__device__ __forceinline__ void publish_tiles(const FrameTiles& f, const TileMarks& to, uint32_t copy) {
-    const uint32_t t = threadIdx.x, n0 = f.words[0];
-    if (t >= n0 + f.words[1]) return;
+// One fire-and-forget reduction per word, in copy `copy` % kNoteCopies of the notes of frame b.
+__device__ __forceinline__ void publish_tiles(const FrameTiles& f, const TileMarks& to, int b, uint32_t copy) {
+    const uint32_t t = threadIdx.x, n0 = to.words[0][b];
+    if (t >= n0 + to.words[1][b]) return;
     const uint4* bytes = reinterpret_cast<const uint4*>(f.seen) + 2 * t;
     const uint4 p = bytes[0], q = bytes[1];
     const uint32_t mine = bits_of_bytes(p.x) | bits_of_bytes(p.y) << 4 | bits_of_bytes(p.z) << 8 | bits_of_bytes(p.w) << 12 |
                           bits_of_bytes(q.x) << 16 | bits_of_bytes(q.y) << 20 | bits_of_bytes(q.z) << 24 | bits_of_bytes(q.w) << 28;
-    uint32_t* w = t < n0 ? to.marked[0] + f.word0[0] + t : to.marked[1] + f.word0[1] + (t - n0);
+    uint32_t* w = t < n0 ? to.marked[0] + to.word0[0][b] + t : to.marked[1] + to.word0[1][b] + (t - n0);
     if (mine) atomicOr(w + (copy % kNoteCopies) * to.stride, mine);
 }
 
-__device__ __forceinline__ void reset_scan(const ScanReset& r, size_t thread, size_t nthreads) {
-    for (size_t i = thread; i < (size_t)r.n; i += nthreads) r.words[i] = 0u;
-    if (thread == 0 && r.totals[0]) {
+// By one CTA.
+__device__ __forceinline__ void reset_scan(const ScanReset& r) {
+    for (int i = threadIdx.x; i < r.n; i += blockDim.x) r.words[i] = 0u;
+    if (threadIdx.x == 0 && r.totals[0]) {
         *reinterpret_cast<int4*>(r.totals[0]) = make_int4(0, 0, 0, 0);
         *reinterpret_cast<int4*>(r.totals[1]) = make_int4(0, 0, 0, 0);
     }
+}
+
+// Spread over the whole grid.
+__device__ __forceinline__ void zero_bev(float4* bev, uint32_t n4) {
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    const uint32_t step = gridDim.x * gridDim.y * blockDim.x;
+    for (uint32_t i = (blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x; i < n4; i += step) __stcs(bev + i, zero);
 }
 
 __device__ __forceinline__ int warp_sum(int v) { return __reduce_add_sync(0xFFFFFFFFu, v); }

@@ -76,10 +76,8 @@ __device__ __forceinline__ float cell_corner(float mn, float vs, int i) { return
 template <int C>
 __global__ void __launch_bounds__(kThreads)
 vox_mark_kernel(const float* __restrict__ pts, int B, int N, int frames_log, const __grid_constant__ ScaleDev s0, const __grid_constant__ ScaleDev s1,
-                float4* bev, size_t bev_n4, ScanReset reset, TileMarks marks) {
+                float4* bev, uint32_t bev_n4, ScanReset reset, TileMarks marks) {
     __shared__ FrameTiles tiles;
-    const size_t thread = ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * kThreads + threadIdx.x;
-    const size_t nthreads = (size_t)gridDim.x * gridDim.y * kThreads;
     const int b = (int)((blockIdx.y << frames_log) + (blockIdx.x & ((1u << frames_log) - 1u)));
     const int i = (int)((blockIdx.x >> frames_log) * kThreads + threadIdx.x);
     if (b >= B) N = 0;                            // the last group can have fewer frames
@@ -94,23 +92,20 @@ vox_mark_kernel(const float* __restrict__ pts, int B, int N, int frames_log, con
         }
     }
     if (marks.marked[0] && b < B) {
-        begin_tiles(tiles, s0, s1, (uint32_t)b);
+        begin_tiles(tiles);
         __syncthreads();
     }
     if (i < N) {
         int tile[2];
         mark_point(s0, s1, x, y, z, b, tile);
-        if (marks.marked[0]) note_tiles(tiles, tile);
+        if (marks.marked[0]) note_tiles(tiles, marks, b, tile);
     }
-    reset_scan(reset, thread, nthreads);
+    if (blockIdx.x + blockIdx.y == 0) reset_scan(reset);
     // The BEV image is zeroed here, spread over the whole grid, so it costs no extra launch.
-    if (bev) {
-        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (size_t k = thread; k < bev_n4; k += nthreads) __stcs(bev + k, zero);
-    }
+    if (bev) zero_bev(bev, bev_n4);
     if (marks.marked[0] && b < B) {
         __syncthreads();
-        publish_tiles(tiles, marks, blockIdx.x >> frames_log);
+        publish_tiles(tiles, marks, b, blockIdx.x >> frames_log);
     }
     release_successor();
 }
@@ -841,7 +836,7 @@ int run_voxelize(emc2_bridge* h, int B, int N, const float* d_points, int32_t* c
     aa.status = h->d_status;
 
     const size_t bev_n = d_bev ? (size_t)B * C * h->scale[1].dims[1] * h->scale[1].dims[0] : 0;
-    const bool bev_vec = (bev_n & 3) == 0;
+    const bool bev_vec = bev_by_kernel(bev_n);
     if (!marked && bev_n && !bev_vec) cudaMemsetAsync(d_bev, 0, bev_n * sizeof(float), st);
     if (!marked) {
         // Also zeroes the BEV image; with no points it still runs for that.
@@ -852,7 +847,7 @@ int run_voxelize(emc2_bridge* h, int B, int N, const float* d_points, int32_t* c
             LaunchScope ls(h, K_VOX_MARK, st);
             vox_mark_kernel<C><<<grid, kThreads, 0, st>>>(d_points, B, N, frames_log, sa.s[0], sa.s[1],
                                                           bev_vec ? reinterpret_cast<float4*>(d_bev) : nullptr,
-                                                          bev_vec ? bev_n >> 2 : 0, scan_reset(h), tile_marks(h, B, N));
+                                                          bev_vec ? (uint32_t)(bev_n >> 2) : 0u, scan_reset(h), tile_marks(h, B, N));
         }
     }
     for (int s = 0; s < 2; ++s) {
