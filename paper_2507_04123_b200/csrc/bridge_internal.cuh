@@ -30,7 +30,7 @@ inline int row_threads(int cf4) {
 // cells streams 2: 75 instead of 50 MB for four frames of the nuScenes-shaped grid, and the scan is paid by
 // the grid's volume).  Small grids: one word per cell.
 constexpr uint32_t kUnitCells = 96;
-constexpr size_t kScanTileBytes = 8192;   // of the store, per CTA of the ranking pass
+constexpr size_t kScanTileBytes = 8192;   // of the store; the ranking pass takes eighths of them
 constexpr uint32_t kBitmapTileCells = (uint32_t)(kScanTileBytes / 16) * kUnitCells;
 constexpr uint32_t kTableTileCells = (uint32_t)(kScanTileBytes / 4);
 constexpr int kMaxTableCells = 1 << 24;  // a word per cell up to 16 Mi cells per batch (64 MB)
@@ -149,7 +149,7 @@ struct ScanState {
     uint32_t* group_voxels[2];  // [ceil(tiles / 128)] per group of tiles; zero when the scan begins
     uint32_t* listed;           // parts in `list`; zero when the scan begins
     uint32_t* list;             // [8 * tiles of both scales] parts that hold voxels, in any order: 8 * tile + part; bit 31: scale 1
-    uint32_t* marked[2];        // a bit per tile of a store: a cell of it was marked; zero between calls
+    uint32_t* marked[2];        // a bit per tile of a store: a cell of it was marked; kNoteCopies of them, zero between calls
     uint32_t note_stride;       // words from one copy of the notes to the next
     int words[2];               // words of `marked` to clear, 0 where the marking pass does not keep it
 };

@@ -9,8 +9,8 @@
 //
 //   vox_mark      every point marks its two cells with one fire-and-forget reduction each;
 //                 the same launch zeroes the BEV image.
-//   vox_count,    the rank scan, two launches: voxels per tile of the store (of the tiles that the marking pass
-//                 noted, where it notes them), then the exclusive prefix
+//   vox_count,    the rank scan, two launches: voxels per tile of the store and eighth of it (of the tiles that the marking
+//                 pass noted, where it notes them), then the exclusive prefix
 //   vox_rank      sums (the parallel prefix-sum index search of Sec. 3.6) are written into the rank
 //                 fields and the occupied cell ids listed in that order; the bookkeeping of cells over
 //                 the cap is laid out.
