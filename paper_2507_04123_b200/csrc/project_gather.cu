@@ -76,8 +76,8 @@ __device__ __forceinline__ void chains(const Camera& c, float x, float y, float 
 // after it.  `cam`: the frame's K cameras in shared memory.
 // A warp of the six-camera workload took 860 instructions with a test per camera in scalar arithmetic and divides for
 // the six cell indices, now 680.  That shows in project_route_kernel where instruction issue bounds it: 32 frames of
-// 262,144 points 222 -> 179 us, eight KITTI-shaped frames 33.9 -> 31.2.  On four nuScenes-shaped frames it does not
-// (43.9 and 44.3 us): there the kernel waits for the marks, whose sectors of the cell store are not in L2.
+// 262,144 points 222 -> 179 us, eight KITTI-shaped frames 33.9 -> 31.2.  On four nuScenes-shaped frames it did not
+// (43.9 and 44.3 us) as long as their marks were queueing at the hottest sectors of the stores (see frames_side_by_side).
 __device__ __forceinline__ Projected project_point(const Camera* cam, int K, float x, float y, float z,
                                                     int W, int H, float min_depth) {
     Projected r;
