@@ -160,6 +160,9 @@ EMC2_RULE uint32_t bits_of_bytes(uint32_t bytes) { return bytes * 0x01020408u >>
 // ---- voxels found by the rank scan: at most one per point of a call, or the store was not all zero when it began
 EMC2_RULE bool voxels_possible(uint32_t voxels, uint32_t max_list) { return voxels <= max_list; }
 
+// Rows of such a scale, and the voxels it reports: none where the store was not.
+EMC2_RULE uint32_t voxels_ranked(uint32_t voxels, uint32_t max_list) { return voxels_possible(voxels, max_list) ? voxels : 0u; }
+
 // The scan covers whole tiles, which can reach past the call's last frame; a cell found there was left over as well,
 // and the caller's BEV image has no such frame.
 EMC2_RULE bool frame_in_call(uint32_t frame, uint32_t frames) { return frame < frames; }

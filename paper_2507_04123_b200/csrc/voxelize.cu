@@ -308,8 +308,8 @@ __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const
         const ScaleDev& g = a.s[t];
         const uint32_t n = t ? all[1] : all[0];
         const bool dirty = !voxels_possible(n, g.max_list);
-        g.totals[0] = dirty ? 0 : (int)n;
-        a.num_voxels[t] = dirty ? 0 : (int)n;
+        g.totals[0] = (int)voxels_ranked(n, g.max_list);
+        a.num_voxels[t] = (int)voxels_ranked(n, g.max_list);
         if (dirty) atomicOr(a.status, kStatusDirtyStore);
         else if ((int)n > a.capacity[t]) atomicOr(a.status, kStatusCapacity);
     }
@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(kRankThreads, kRankCtas) vox_rank_kernel(const
 #pragma unroll
     for (int v = 0; v < 2; ++v) {
         const ScaleDev& g = a.s[v];
-        const uint32_t voxels = min(all[v], g.max_list);
+        const uint32_t voxels = voxels_ranked(all[v], g.max_list);
         for (size_t i = thread; i < (size_t)voxels * g.acc_f4; i += threads) g.acc[i] = zero;
         if (counts_in_output(g))
             for (uint32_t i = thread; i < min(voxels, (uint32_t)a.capacity[v]); i += threads) a.counts[v][i] = 0;
@@ -514,7 +514,9 @@ vox_accum_kernel(const float* __restrict__ pts, long long total, int N, const __
         const float dz = __fsub_rn(f[2], cell_corner(s.mn[2], s.vs[2], c[sc][2]));
         float4* row = s.acc + (size_t)at.m * s.acc_f4;
         atomicAdd(row, make_float4(dx, dy, dz, f[3]));
-        if (counts_in_output(s)) atomicAdd(a.counts[sc] + at.m, 1);
+        // A scale that was not ranked reports no voxels, whatever its store holds, and the caller's counts stay as they were.  The
+        // total is read here and not with the look-ups, where it cost eight KITTI-shaped frames 22.4 -> 23.2 us (here 22.5).
+        if (counts_in_output(s)) { if (at.m < s.totals[0]) atomicAdd(a.counts[sc] + at.m, 1); }
         else if (s.mode == MODE_BITMAP) atomicAdd(reinterpret_cast<float2*>(row + 1), make_float2(C > 4 ? f[C - 1] : 0.0f, 1.0f));
         else if (C > 4) atomicAdd(reinterpret_cast<float*>(row + 1), f[C - 1]);
     }

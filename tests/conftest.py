@@ -33,6 +33,7 @@ def rules(tmp_path_factory):
     u32, u64 = ctypes.c_uint32, ctypes.c_uint64
     so.clamp.restype, so.clamp.argtypes = u32, [u32]
     so.fits.restype, so.fits.argtypes = ctypes.c_int, [u64, u32, u32, u32, u32]
+    so.ranked.restype, so.ranked.argtypes = u32, [u32, u32]
     so.ticket.restype, so.ticket.argtypes = u64, [u32, u32]
     so.tile_frames.restype, so.tile_frames.argtypes = ctypes.c_int64, [ctypes.c_int64, ctypes.c_int64]
     for f in (so.first_word, so.words_of_frame):

@@ -23,6 +23,7 @@ int notes(uint64_t bytes, uint64_t words, int B, int N) { return keeps_notes(byt
 int frames_log(uint64_t bytes, int B) { return frames_side_by_side(bytes, B); }
 int rows_aside(uint64_t points, uint64_t feat_c, int both) { return rows_on_other_stream(points, feat_c, both != 0); }
 int rows_stay(uint64_t points, uint64_t feat_c) { return rows_stay_in_l2(points, feat_c); }
+uint32_t ranked(uint32_t voxels, uint32_t max_list) { return voxels_ranked(voxels, max_list); }
 uint64_t ticket(uint32_t cells, uint32_t points) { return over_ticket(cells, points); }
 
 // Cells of n points (x, y, z), -1 -1 -1 outside the grid; returns for how many of them no divide was needed.

@@ -67,6 +67,21 @@ def test_a_scale_with_more_voxels_than_points_is_not_ranked():
         assert guard < loop.index(write), write
 
 
+def test_a_scale_that_is_not_ranked_leaves_the_callers_counts_alone(rules):
+    """It has no rows: vox_rank clears no counts for it and vox_accum, which counts there for some scales, adds none."""
+    for most in (0, 1, 5, 1 << 24):
+        for n in {0, 1, most, most + 1, 1 << 25, 0xFFFFFFFF}:
+            assert rules.ranked(n, most) == (n if n <= most else 0)
+    text = open(os.path.join(CSRC, "voxelize.cu")).read()
+    rank = text[text.index("vox_rank_kernel("):text.index("pass 3: accumulate")]
+    clear = rank.index("a.counts[v][i] = 0")
+    assert "const uint32_t voxels = voxels_ranked(all[v], g.max_list);" in rank[:clear]
+    assert "i < min(voxels, (uint32_t)a.capacity[v])" in rank[clear - 120:clear]
+    assert "g.totals[0] = (int)voxels_ranked(n, g.max_list);" in rank
+    accum = text[text.index("vox_accum_kernel("):text.index("per-voxel cap on a bitmap scale")]
+    assert accum.count("a.counts[sc]") == 1 and "if (at.m < s.totals[0]) atomicAdd(a.counts[sc] + at.m, 1);" in accum
+
+
 def test_the_bev_image_is_written_for_frames_of_the_call_only():
     """A pillar scan's tiles cover cells of frames past the call's last one: every write into the image tests the frame."""
     text = open(os.path.join(CSRC, "voxelize.cu")).read()
