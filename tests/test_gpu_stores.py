@@ -104,6 +104,23 @@ def test_parts_of_the_tiles_of_a_table_store(oracle, B, share):
     check_voxels(w, pts, oracle)
 
 
+@pytest.mark.parametrize("most", [1, 4, 5])
+def test_parts_listed_by_sectors_and_by_words(oracle, most):
+    """Parts (6,144 cells) whose fullest sector (192 cells) holds as many voxels as one lane lists, or one more: in the first, the
+    last or any sector, in one word or at both ends of the sector, the other sectors empty or not."""
+    rng = np.random.default_rng(most)
+    at = []
+    for part in range(24):
+        p0 = 6144 * (part if part < 12 else 2700 + part)
+        full = (0, 31, int(rng.integers(32)))[part % 3]
+        at += [p0 + 192 * full + d for d in ([191 - k for k in range(most)] if part % 2 else [0, 95, 96, 191, 33][:most])]
+        if part % 4 > 1:
+            at += [p0 + 192 * s + int(rng.integers(192)) for s in range(32) if s != full]
+    assert max(at) < BITMAP.cells and np.bincount(np.unique(at) // 192).max() == most
+    pts = centres(rng.permutation(np.repeat(np.unique(at), 2)), BITMAP, 4, rng)[None]
+    check_voxels(replace(gen.KITTI.with_shape(1, pts.shape[1]), grids=(BITMAP, TABLE)), pts, oracle)
+
+
 @pytest.mark.parametrize("dims", [(1408, 1600, 40), (61, 7, 3), (2_000_000, 2, 2)])
 def test_cells_of_points_on_cell_boundaries(oracle, dims):
     """Points a few ulps around multiples of the cell size, far away, and not finite: cells as by subtract, divide, floor."""
