@@ -305,6 +305,9 @@ inline ScanReset scan_reset(const emc2_bridge* h) {
     return r;
 }
 
+// Grid of a marking pass: `tiles` CTAs per frame, (tiles * frames of a group, groups); `group` divides by the frames of a group.
+inline dim3 marking_grid(int tiles, int B, const FastDiv& group) { return dim3(tiles * group.d, (B + group.d - 1) / group.d); }
+
 // Bytes of both stores of a frame.
 inline uint64_t store_bytes(const emc2_bridge* h) {
     uint64_t bytes = 0;

@@ -218,7 +218,8 @@ struct PrArgs {
     int N, tiles, K, H, W;
     float min_depth;
     RouteParams rp;
-    int B, frames_log;
+    int B;
+    FastDiv group;        // frames of a group, see marking_grid
     int frame0;           // kMark: frame index (in the whole batch) of this launch's first frame
     ScaleDev s0, s1;      // kMark: the voxel grids whose cells the points mark
     float4* bev;          // kMark: BEV image to zero (bev_n4 float4), or null
@@ -227,7 +228,7 @@ struct PrArgs {
     TileMarks marks;      // kNote
 };
 
-// grid = (tiles per frame << frames_log, groups of frames), see frames_side_by_side; tiles never straddle frames.  kMark: the kernel also does the
+// See marking_grid; tiles never straddle frames.  kMark: the kernel also does the
 // voxelizer's marking pass (every point marks its cell in both scales' stores, and the BEV image
 // is zeroed, spread over the grid), so that stage 1 starts from marked stores and reads the
 // points once less; the reductions are fire-and-forget and land while the projection computes.
@@ -244,7 +245,9 @@ __global__ void __launch_bounds__(kThreads, 8) project_route_kernel(const __grid
     __shared__ int hist[EMC2_MAX_EXPERTS];
     __shared__ Camera sP[EMC2_MAX_CAMERAS];
     const int t = threadIdx.x, lane = t & 31;
-    const int tile = (int)(blockIdx.x >> a.frames_log), b = (int)((blockIdx.y << a.frames_log) + (blockIdx.x & ((1u << a.frames_log) - 1u)));
+    uint32_t tile_u, in_group;
+    a.group.divmod(blockIdx.x, tile_u, in_group);
+    const int tile = (int)tile_u, b = (int)(blockIdx.y * a.group.d + in_group);
     if (b < a.B) load_cameras(a.proj, b, 1, a.K, sP);
     const int i0 = tile * kTile;
     const int npts = b < a.B ? min(kTile, a.N - i0) : 0;       // the last group can have fewer frames
@@ -805,8 +808,8 @@ int launch_project_route(emc2_bridge* h, int b0, int B, int N, const float* d_po
     const emc2_config_t& c = h->cfg;
     const int tiles = (N + kTile - 1) / kTile;
     if (B == 0 || tiles == 0) return EMC2_OK;
-    const int frames_log = frames_side_by_side(store_bytes(h), B);
-    const dim3 grid(tiles << frames_log, (B + (1 << frames_log) - 1) >> frames_log);
+    const FastDiv group = make_fast_div((uint32_t)frames_per_group(store_bytes(h), B));
+    const dim3 grid = marking_grid(tiles, B, group);
     const size_t p0 = (size_t)b0 * N;                      // first point of the range
     PrArgs pa;
     pa.pts = d_points + p0 * c.point_floats; pa.proj = d_proj + (size_t)b0 * c.num_cameras * 12;
@@ -815,7 +818,7 @@ int launch_project_route(emc2_bridge* h, int b0, int B, int N, const float* d_po
     pa.N = N; pa.tiles = tiles; pa.K = c.num_cameras; pa.H = c.img_h; pa.W = c.img_w;
     pa.min_depth = c.min_depth;
     pa.rp = route_params(h);
-    pa.B = B; pa.frames_log = frames_log;
+    pa.B = B; pa.group = group;
     pa.frame0 = b0;
     pa.s0 = h->scale[0]; pa.s1 = h->scale[1];
     pa.bev = nullptr; pa.bev_n4 = 0;

@@ -141,17 +141,28 @@ inline bool keeps_notes(uint64_t frame_bytes, uint64_t words, int B, int N) {
     return words <= kMarkWords && B * frame_bytes >= (uint64_t)24 << 20 && N <= 1 << 17;
 }
 
-// ---- which tile of which frame a CTA of a marking pass takes: groups of 1 << log frames, whose tiles take turns
+// ---- which tile of which frame a CTA of a marking pass takes: groups of frames, whose tiles take turns
 // Marks that land in one sector of a store are served one after another, and the sector of pillars next to the sensor gets about
-// a thousand of a nuScenes-shaped frame's 300,000 points: frame after frame, four of them took project_route 45 us.  With the
-// frames side by side those marks are spread over the whole kernel: 37 (vox_mark 37 -> 29).  Their stores should fit in L2
-// together, us without / with groups of 32, 64, 128 and 256 MB: four nuScenes-shaped frames 44.7 / 38.7, 37.2, 37.2, 37.3; eight
-// KITTI-shaped ones, whose first ring of points is farther away, 43.6 / 42.9, 42.6, 43.1, 42.7; 32 frames of 262,144
-// KITTI-shaped points (480 MB) 193 / 198, 198, 201, 205, all 32 side by side 222.
+// a thousand of a nuScenes-shaped frame's 300,000 points.  With the frames side by side those marks are spread over the whole
+// kernel.  The stores of a group should fit in L2 together: four nuScenes-shaped frames with groups of 32, 64, 128 and 256 MB
+// took project_route 38.7, 37.2, 37.2 and 37.3 us, 32 KITTI-shaped ones of 262,144 points and six cameras 198, 198, 201 and 205,
+// all 32 side by side 222.  us, frame after frame / groups of at most 64 MB: project_route of four nuScenes-shaped frames 44.9 /
+// 37.5, their vox_mark 37.7 / 30.1, the call 301.1 / 293.3; of 32 KITTI-shaped frames of 262,144 points 167 / 161, the call 1,329 /
+// 1,322, through six cameras 203.9 / 205.5 and 1,746 / 1,744; of eight of 120,000, whose first ring of points is farther away, 33.1 /
+// 33.8, the call 189.6 / 189.8; voxel lists of 32 dense frames of 524,288 points 1,178 / 1,114.
+// The power of two that fits:
 inline int frames_side_by_side(uint64_t frame_bytes, int B) {
     int log = 0;
     while ((1 << log) < B && (frame_bytes << (log + 1)) <= (uint64_t)64 << 20) ++log;
     return log;
+}
+
+// Frames per group: as few groups as that allows, all of one size but for the last.  Groups of the power of two itself left CTAs
+// without a frame, which cost nine frames in groups of four, twelve places, up to 1.6 % (us): voxel lists of uniform frames of
+// 16,384 points 98.9, now 97.3, KITTI-shaped ones of 60,000 77.8, now 77.1, all stages of these 132.2, now 131.4.
+inline int frames_per_group(uint64_t frame_bytes, int B) {
+    const int most = 1 << frames_side_by_side(frame_bytes, B), groups = (B + most - 1) / most;
+    return groups > 0 ? (B + groups - 1) / groups : 1;
 }
 
 // Four bytes that are 0 or 1 -> four bits, the lowest byte in the lowest bit.

@@ -72,14 +72,16 @@ __device__ __forceinline__ bool counts_in_output(const ScaleDev& g) { return g.m
 __device__ __forceinline__ float cell_corner(float mn, float vs, int i) { return __fmaf_rn((float)i, vs, mn); }
 
 // ------------------------------------------------------------------ pass 1: mark cells
-// grid = (tiles per frame << frames_log, groups of frames), at least, see frames_side_by_side; tiles never straddle frames.
+// See marking_grid; tiles never straddle frames.
 template <int C>
 __global__ void __launch_bounds__(kThreads)
-vox_mark_kernel(const float* __restrict__ pts, int B, int N, int frames_log, const __grid_constant__ ScaleDev s0, const __grid_constant__ ScaleDev s1,
+vox_mark_kernel(const float* __restrict__ pts, int B, int N, const FastDiv group, const __grid_constant__ ScaleDev s0, const __grid_constant__ ScaleDev s1,
                 float4* bev, uint32_t bev_n4, ScanReset reset, TileMarks marks) {
     __shared__ FrameTiles tiles;
-    const int b = (int)((blockIdx.y << frames_log) + (blockIdx.x & ((1u << frames_log) - 1u)));
-    const int i = (int)((blockIdx.x >> frames_log) * kThreads + threadIdx.x);
+    uint32_t tile, in_group;
+    group.divmod(blockIdx.x, tile, in_group);
+    const int b = (int)(blockIdx.y * group.d + in_group);
+    const int i = (int)(tile * kThreads + threadIdx.x);
     if (b >= B) N = 0;                            // the last group can have fewer frames
     float x = 0.f, y = 0.f, z = 0.f;
     if (i < N) {
@@ -105,7 +107,7 @@ vox_mark_kernel(const float* __restrict__ pts, int B, int N, int frames_log, con
     if (bev) zero_bev(bev, bev_n4);
     if (marks.marked[0] && b < B) {
         __syncthreads();
-        publish_tiles(tiles, marks, b, blockIdx.x >> frames_log);
+        publish_tiles(tiles, marks, b, tile);
     }
     release_successor();
 }
@@ -859,11 +861,11 @@ int run_voxelize(emc2_bridge* h, int B, int N, const float* d_points, int32_t* c
     if (!marked) {
         // Also zeroes the BEV image; with no points it still runs for that.
         const int zeroing = bev_n && bev_vec ? (h->num_sms + B - 1) / B : 0;
-        const int frames_log = frames_side_by_side(store_bytes(h), B);
-        const dim3 grid(max((N + kTile - 1) / kTile, zeroing) << frames_log, (B + (1 << frames_log) - 1) >> frames_log);
+        const FastDiv group = make_fast_div((uint32_t)frames_per_group(store_bytes(h), B));
+        const dim3 grid = marking_grid(max((N + kTile - 1) / kTile, zeroing), B, group);
         if (B > 0 && grid.x > 0) {
             LaunchScope ls(h, K_VOX_MARK, st);
-            vox_mark_kernel<C><<<grid, kThreads, 0, st>>>(d_points, B, N, frames_log, sa.s[0], sa.s[1],
+            vox_mark_kernel<C><<<grid, kThreads, 0, st>>>(d_points, B, N, group, sa.s[0], sa.s[1],
                                                           bev_vec ? reinterpret_cast<float4*>(d_bev) : nullptr,
                                                           bev_vec ? (uint32_t)(bev_n >> 2) : 0u, scan_reset(h), tile_marks(h, B, N));
         }

@@ -42,6 +42,7 @@ def rules(tmp_path_factory):
     so.four_bits.restype, so.four_bits.argtypes = u32, [u32]
     so.notes.argtypes = [u64, u64, ctypes.c_int, ctypes.c_int]
     so.frames_log.argtypes = [u64, ctypes.c_int]
+    so.frames_in_group.argtypes = [u64, ctypes.c_int]
     so.rows_aside.argtypes = [u64, u64, ctypes.c_int]
     so.rows_stay.argtypes = [u64, u64]
     return so

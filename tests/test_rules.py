@@ -142,6 +142,18 @@ def test_frames_side_by_side(rules):
             assert sorted(t for t in taken if t[0] < B) == [(b, i) for b in range(B) for i in range(3)]
 
 
+def test_groups_of_frames_are_as_large_as_the_batch_needs(rules):
+    """No more groups than the power of two takes, fewer places without a frame than there are groups, every tile taken once."""
+    for frame in (0, 1, 13_488_272, 15_898_656, 32 << 20, (32 << 20) + 1, 700 << 20):
+        for B in range(0, 33):
+            most, G = 1 << rules.frames_log(frame, B), rules.frames_in_group(frame, B)
+            groups = -(-B // G)
+            assert 1 <= G <= most and groups == -(-B // most) and (B == 0 or 0 <= groups * G - B < groups)
+            taken = [(y * G + x % G, x // G) for y in range(groups) for x in range(3 * G)]
+            assert sorted(t for t in taken if t[0] < B) == [(b, i) for b in range(B) for i in range(3)]
+    assert rules.frames_in_group(15_898_656, 9) == 3 and rules.frames_in_group(15_898_656, 5) == 3
+
+
 def test_gathered_rows_that_stay_in_l2(rules):
     for points, feat_c, stays in ((120000, 256, 1), (131072, 256, 1), (131073, 256, 0), (419430, 80, 1), (419431, 80, 0), (1, 4, 1),
                                   (1 << 24, 1020, 0)):
