@@ -154,12 +154,6 @@ struct ScanState {
     int words[2];               // words of `marked` to clear, 0 where the marking pass does not keep it
 };
 
-// The notes are kept in this many copies, and a CTA sends its own to one of them: reductions on one word are served one after another,
-// and every CTA has some for the few words of the ground plane.  us for 1, 4, 8 and 16 copies: eight KITTI-shaped frames
-// 42.4, 33.8, 33.4, 33.1 (project_route; 32.1 without notes), the call 202.4, 194.3, 193.6, 193.8; vox_mark 36.5, 28.0, 27.6,
-// 27.2.  Reading a word first, to send only what is new, adds to the same queue: 52.8 with one copy.
-constexpr uint32_t kNoteCopies = 8;
-
 // Where the marking pass notes the tiles that it touches (see keeps_tile_marks), or null.
 struct TileMarks {
     uint32_t* marked[2];
@@ -327,7 +321,7 @@ inline bool keeps_tile_marks(const emc2_bridge* h, int B, int N) {
         const bool bitmap = g.mode == MODE_BITMAP;
         words += most_frame_words(g.cells, bitmap ? kBitmapTileCells : kTableTileCells);
     }
-    return keeps_notes(store_bytes(h), words, B, (N + (int)kNoteCopies - 1) / (int)kNoteCopies);
+    return keeps_frame_notes(store_bytes(h), words, B, N);
 }
 
 inline TileMarks tile_marks(const emc2_bridge* h, int B, int N) {

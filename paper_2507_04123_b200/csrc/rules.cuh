@@ -127,18 +127,33 @@ EMC2_RULE uint32_t frame_words(uint32_t b, uint32_t cells, uint32_t per_tile) {
 }
 inline uint32_t most_frame_words(uint32_t cells, uint32_t per_tile) { return cells / per_tile / 32u + 2u; }
 
-// Whether the marking pass of a call keeps the notes: frames of which N points note in the same copy (see kNoteCopies) and whose
-// stores take `frame_bytes` each (8 KB tiles, `words` words of notes).  The counting pass then reads the noted tiles instead of
-// the whole stores, three quarters of which are empty space.  One frame's stores are read as fast as the notes come back (voxels
-// and rulebooks of 30,000 points 56 and 57 us).  The more points note in one copy the longer the queues at its words: with a single
-// copy notes lost from about 2^17 points on (voxel lists of four KITTI-shaped frames of 300,000 points 102 us without, 112 with);
-// with eight, us per call without / with the notes: four nuScenes-shaped frames of 300,000 points 302 / 296.6, their voxels and
-// rulebooks 216.4 / 212.0, 32 KITTI-shaped frames of 262,144 points and six cameras 1,766 / 1,732, eight of 120,000 points 207.0 /
-// 193.6.  Frames of more than 2^20 points have not been measured.  The 72 words hold the frames of both grid families (64 and 55
-// words); larger grids, which would need more shared memory, have not been measured with notes.
+// Whether the marking pass of a call keeps the notes: frames of which N points note in the same copy and whose stores take
+// `frame_bytes` each (8 KB tiles, `words` words of notes).  The counting pass then reads the noted tiles instead of the whole
+// stores, three quarters of which are empty space.  One frame's stores are read as fast as the notes come back (voxels and
+// rulebooks of 30,000 points 56 and 57 us).  The more points note in one copy the longer the queues at its words: with a single
+// copy notes lost from about 2^17 points on.  The 72 words hold the frames of both grid families (64 and 55 words); larger grids,
+// which would need more shared memory, have not been measured with notes.
 constexpr uint32_t kMarkWords = 72;
 inline bool keeps_notes(uint64_t frame_bytes, uint64_t words, int B, int N) {
     return words <= kMarkWords && B * frame_bytes >= (uint64_t)24 << 20 && N <= 1 << 17;
+}
+
+// The notes are kept in this many copies, and a CTA sends its own to one of them: reductions on one word are served one after another,
+// and every CTA has some for the few words of the ground plane.  us for 1, 4, 8 and 16 copies: eight KITTI-shaped frames
+// 42.4, 33.8, 33.4, 33.1 (project_route; 32.1 without notes), the call 202.4, 194.3, 193.6, 193.8; vox_mark 36.5, 28.0, 27.6,
+// 27.2.  Reading a word first, to send only what is new, adds to the same queue: 52.8 with one copy.
+constexpr uint32_t kNoteCopies = 8;
+
+// The same for frames of N points, which are spread over the copies: up to 2^20 points.  us per call without / with the notes:
+//   voxel lists: four KITTI-shaped frames of 300,000 points 88.6 / 82.5, of 700,000 186 / 183, of 1,000,000 236 / 232; eight of
+//   850,000 in firing order 421 / 410; four nuScenes-shaped ones of 300,000 127 / 121.5, of 1,000,000 381 / 376.
+//   all stages, where the notes are taken by the projection: four KITTI-shaped frames of 300,000 points 207 / 200, of 524,288 334.6 /
+//   332, of 700,000 441 / 441, of 850,000 525 / 528, of 1,000,000 460 / 464 (32 channels); four nuScenes-shaped ones of 300,000 257 /
+//   251.5, of 700,000 551 / 551, of 850,000 665 / 670.
+// So they lose up to 1 % of the calls of all stages from about 700,000 points on and gain 1 to 2 % of the voxel lists there.  Larger
+// frames have not been measured.
+inline bool keeps_frame_notes(uint64_t frame_bytes, uint64_t words, int B, int N) {
+    return keeps_notes(frame_bytes, words, B, (N + (int)kNoteCopies - 1) / (int)kNoteCopies);
 }
 
 // ---- which tile of which frame a CTA of a marking pass takes: groups of frames, whose tiles take turns

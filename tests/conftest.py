@@ -40,6 +40,7 @@ def rules(tmp_path_factory):
         f.restype, f.argtypes = u32, [u32, u32, u32]
     so.most_words.restype, so.most_words.argtypes = u32, [u32, u32]
     so.four_bits.restype, so.four_bits.argtypes = u32, [u32]
+    so.frame_notes.argtypes = [u64, u64, ctypes.c_int, ctypes.c_int]
     so.notes.argtypes = [u64, u64, ctypes.c_int, ctypes.c_int]
     so.frames_log.argtypes = [u64, ctypes.c_int]
     so.frames_in_group.argtypes = [u64, ctypes.c_int]

@@ -20,6 +20,7 @@ uint32_t words_of_frame(uint32_t b, uint32_t cells, uint32_t per) { return frame
 uint32_t most_words(uint32_t cells, uint32_t per) { return most_frame_words(cells, per); }
 uint32_t four_bits(uint32_t bytes) { return bits_of_bytes(bytes); }
 int notes(uint64_t bytes, uint64_t words, int B, int N) { return keeps_notes(bytes, words, B, N); }
+int frame_notes(uint64_t bytes, uint64_t words, int B, int N) { return keeps_frame_notes(bytes, words, B, N); }
 int frames_log(uint64_t bytes, int B) { return frames_side_by_side(bytes, B); }
 int frames_in_group(uint64_t bytes, int B) { return frames_per_group(bytes, B); }
 int rows_aside(uint64_t points, uint64_t feat_c, int both) { return rows_on_other_stream(points, feat_c, both != 0); }

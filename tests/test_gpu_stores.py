@@ -256,7 +256,8 @@ def test_pooled_sampling_of_cut_windows(oracle, cf, hw, p):
 @pytest.mark.parametrize("base,B,N", [(gen.KITTI, 3, 700), (gen.KITTI, 5, 257), (gen.NUSCENES, 9, 300), (gen.KITTI, 2, 140000),
                                       (gen.DENSE, 2, 3000)], ids=lambda v: getattr(v, "name", str(v)))
 def test_frames_that_take_turns_with_notes(oracle, base, B, N):
-    """Groups of frames that are not full, frames of one tile and a little, and more points per frame than one copy of the notes takes."""
+    """Groups of frames that are not full, frames of one tile and a little, and more points per frame than one copy of the notes would
+    take by itself."""
     w = replace(base.with_shape(B, N), feat_c=4)
     refs = []
     for i in range(2):
@@ -270,6 +271,20 @@ def test_frames_that_take_turns_with_notes(oracle, base, B, N):
             br.status()
             compare_bridge(w, ref, bufs)
         br.close()
+
+
+@pytest.mark.parametrize("N", [1 << 20, (1 << 20) + 1])
+def test_frames_on_either_side_of_the_most_points_that_are_noted(oracle, N):
+    w = replace(gen.KITTI.with_shape(2, N), feat_c=4)
+    batch = gen.make_batch(w)
+    ref = oracle.bridge(w, batch)
+    d = to_dev(batch)
+    br = bridge_for(w)
+    for step in (br.run, br.run_staged, br.run):
+        bufs = step(d["points"], d["proj"], d["feat"])
+        br.status()
+        compare_bridge(w, ref, bufs)
+    br.close()
 
 
 @pytest.mark.parametrize("base,B,N,cf", [(gen.KITTI, 1, 131072, 256), (gen.KITTI, 1, 131073, 256), (gen.KITTI, 2, 66000, 260),

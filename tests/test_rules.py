@@ -129,6 +129,18 @@ def test_calls_that_keep_notes(rules):
         assert not rules.notes(frame, words, 32, (1 << 17) + 1) and not rules.notes(frame, 73, 32, 1000)
 
 
+def test_frames_that_keep_notes(rules):
+    """By points per frame, which the copies of the notes share: the limit that calls have."""
+    kitti, nuscenes = 15_018_656 + 880_000, 12_439_696 + 1_048_576
+    for frame, words in ((kitti, 64), (nuscenes, 55)):
+        assert rules.frame_notes(frame, words, 2, 1) and rules.frame_notes(frame, words, 2, 1 << 20)
+        assert not rules.frame_notes(frame, words, 2, (1 << 20) + 1) and not rules.frame_notes(frame, words, 1, 1000)
+        assert not rules.frame_notes(frame, 73, 2, 1000)
+    text = open(os.path.join(CSRC, "bridge_internal.cuh")).read()
+    body = text[text.index("inline bool keeps_tile_marks("):text.index("inline TileMarks tile_marks(")]
+    assert "return keeps_frame_notes(store_bytes(h), words, B, N);" in body
+
+
 def test_frames_side_by_side(rules):
     """Groups are as large as the frames need or 64 MB of stores allow, and their CTAs take every tile of every frame once."""
     for frame in (0, 1, 13_488_272, 15_898_656, 32 << 20, (32 << 20) + 1, 64 << 20, 65 << 20, 700 << 20):
