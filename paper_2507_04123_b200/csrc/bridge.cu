@@ -406,7 +406,7 @@ static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_poi
             rc2 = launch_project_route(h, 0, B, N, d_points, d_proj, d_uvd, d_vis_mask, d_cam, d_expert, false, nullptr, 0, marks, st);
         const int tiles = (N + kTile - 1) / kTile;
         if (rc2 == EMC2_OK) {
-            launch_route_scan(h, 0, half0, tiles, N, d_offsets, N > 0 && !rows_aside, row_st);
+            launch_route_scan(h, 0, half0, tiles, d_offsets, N > 0 && !rows_aside, row_st);
             if (early_copy) {
                 // Enqueued after the kernels: from memory that is not page-locked the host copies while they run.
                 e = cudaEventRecord(h->ev_scan, st);
@@ -426,7 +426,7 @@ static int run_bridge(emc2_bridge_t* h, int32_t B, int32_t N, const float* d_poi
             e = cudaStreamWaitEvent(st, h->ev_half, 0);
             if (e != cudaSuccess) rc2 = check_cuda(h, e);
             else {
-                launch_route_scan(h, half0, B - half0, tiles, N, d_offsets + (size_t)half0 * (h->cfg.num_experts + 1), false, st);
+                launch_route_scan(h, half0, B - half0, tiles, d_offsets + (size_t)half0 * (h->cfg.num_experts + 1), false, st);
                 if (early_copy) {                         // the copy of the offsets takes those of both halves
                     e = cudaEventRecord(h->ev_scan, st);
                     if (e != cudaSuccess) rc2 = check_cuda(h, e);

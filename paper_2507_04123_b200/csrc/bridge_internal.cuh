@@ -368,7 +368,7 @@ int launch_scene_route(emc2_bridge* h, int B, const int32_t* d_offsets, const ui
                        int32_t* d_scene_expert, cudaStream_t st);
 // Tile histograms (handle scratch) of frames [b0, b0 + B) -> d_offsets (of frame b0 on) and tile bases.
 // `chained` (here and below): the call's previous work on `st` is one kernel, see launch_chained.
-void launch_route_scan(emc2_bridge* h, int b0, int B, int tiles, int N, int32_t* d_offsets, bool chained, cudaStream_t st);
+void launch_route_scan(emc2_bridge* h, int b0, int B, int tiles, int32_t* d_offsets, bool chained, cudaStream_t st);
 // Stages 2 - 4 in one pass over the feature rows (the one-call path), in two parts: projection +
 // routing per point (which, with `d_bev_to_zero`/`mark`, also marks the voxel cells of both scales
 // and zeroes the BEV image, so that stage 1 reads the points once less), then, after launch_route_scan, the rows.

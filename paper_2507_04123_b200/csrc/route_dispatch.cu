@@ -242,7 +242,7 @@ int launch_scene_route(emc2_bridge* h, int B, const int32_t* d_offsets, const ui
     return check_cuda(h, cudaGetLastError());
 }
 
-void launch_route_scan(emc2_bridge* h, int b0, int B, int tiles, int N, int32_t* d_offsets, bool chained, cudaStream_t st) {
+void launch_route_scan(emc2_bridge* h, int b0, int B, int tiles, int32_t* d_offsets, bool chained, cudaStream_t st) {
     LaunchScope ls(h, K_ROUTE_SCAN, st);
     const size_t t0 = (size_t)b0 * tiles * h->cfg.num_experts;
     launch_kernel(chained, route_scan_kernel, dim3(h->cfg.num_experts, B), scan_threads(tiles), 0, st, h->d_tile_counts + t0,
