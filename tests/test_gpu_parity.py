@@ -481,6 +481,40 @@ def test_rulebook_at_full_size(b200, oracle):
     br.close()
 
 
+@pytest.mark.parametrize("cells", [2_097_152, 2_097_153, 4_410_000])
+def test_rulebook_of_lists_that_take_several_rounds(b200, cells):
+    """Lists of one, two and three rounds of the prefix sums over their tiles of 256 voxels (8,192 tiles each): a plane of cells with
+    holes, listed in order; the pairs are the neighbours that are listed, and nothing else."""
+    from dataclasses import replace
+    from emc2_gen.configs import Grid
+    gx, gy = 2100, -(-cells * 103 // (100 * 2100))
+    w = replace(gen.KITTI.with_shape(1, cells), feat_c=4,
+                grids=(Grid(min=(0.0, 0.0, 0.0), voxel=(1.0, 1.0, 1.0), dims=(gx, gy, 1)), gen.KITTI.grids[1]))
+    br = b200.Bridge(b200.config_from_workload(w))
+    g = torch.Generator(device="cuda").manual_seed(5)
+    ids = torch.randperm(gx * gy, generator=g, device="cuda")[:cells].sort().values
+    y, x = ids // gx, ids % gx
+    zero = torch.zeros_like(x)
+    coords = torch.stack([zero, zero, y, x], dim=1).int().contiguous()
+    vox = {"coords": [coords], "num_voxels": torch.tensor([cells, 0], dtype=torch.int32, device="cuda")}
+    at = torch.full((gy + 2, gx + 2), -1, dtype=torch.int32, device="cuda")
+    at[y + 1, x + 1] = torch.arange(cells, dtype=torch.int32, device="cuda")
+    out = br.rulebook(vox, 0, pair_capacity=9 * cells)
+    br.status()
+    off = np_(out["offsets"]).astype(np.int64)
+    for k in range(27):
+        dz, dy, dx = k // 9 - 1, (k // 3) % 3 - 1, k % 3 - 1
+        got = slice(off[k], off[k + 1])
+        if dz != 0:
+            assert off[k] == off[k + 1], k
+            continue
+        other = at[y + 1 + dy, x + 1 + dx]
+        rows = (other >= 0).nonzero()[:, 0]
+        assert off[k + 1] - off[k] == len(rows), k
+        assert torch.equal(out["rule_out"][got], rows.int()) and torch.equal(out["rule_in"][got], other[rows]), k
+    br.close()
+
+
 def test_rulebook_errors_only_the_device_sees(b200, oracle):
     w = gen.KITTI.with_shape(1, 20_000)
     batch = gen.make_batch(w)
@@ -544,6 +578,25 @@ def test_occlusion_and_routing_of_occluded_points(b200, oracle, cid, B, N, cell,
     assert np.array_equal(np_(rd["perm"]), perm)
     assert (ex != ref["expert"]).any()
     br.close()
+
+
+@pytest.mark.parametrize("E,B,N", [(1, 2, 300), (5, 2, 1031), (6, 1, 33333), (11, 5, 777), (16, 3, 4099), (16, 1, 1), (6, 1, 262401),
+                                   (16, 2, 300001)])
+def test_any_number_of_experts(b200, oracle, E, B, N):
+    """Every bucket of distance and both of visibility in use: experts beyond the five of one packed sum, the experts before each
+    one summed, and frames of more tiles than the route scan has threads (262,144 points)."""
+    from dataclasses import replace
+    w = replace(gen.KITTI.with_shape(B, N), feat_c=4, thresholds=(4.0, 6.0, 9.0, 13.0, 20.0, 30.0, 45.0), num_experts=E,
+                lut=(tuple(k % E for k in range(8)), tuple((8 + k) % E for k in range(8))))
+    batch = gen.make_batch(w)
+    for staged in (False, True):
+        ref, bufs = run_case(b200, oracle, w, batch=batch, repeat=2, staged=staged)
+    assert N < 300 or (np.diff(ref["offsets"], axis=1) > 0).sum() >= (12 if E == 16 else E)
+    out = {k: torch.zeros_like(v) for k, v in bufs["rd"].items()}
+    d = to_dev(batch)
+    b200.route_dispatch_static(b200.config_from_workload(w), d["points"], bufs["pg"]["vis_mask"], bufs["pg"]["gathered"], out)
+    for k, v in bufs["rd"].items():
+        assert torch.equal(out[k].view(torch.uint8), v.view(torch.uint8)), k
 
 
 def test_scene_route_matches_the_oracle(b200, oracle):
@@ -687,6 +740,41 @@ def test_capacity_overflow_is_reported_and_handle_recovers(b200, oracle):
     bufs = br.run(d["points"], d["proj"], d["feat"])              # scratch is clean again
     br.status()
     compare_bridge(w, ref, bufs)
+    br.close()
+
+
+@pytest.mark.parametrize("cap_fine", [0, 3])
+@pytest.mark.parametrize("which", ["kitti", "nuscenes"])
+def test_rows_past_the_voxels_or_the_capacity_stay_as_they_were(b200, oracle, which, cap_fine):
+    """Lists with room to spare, with room for exactly the voxels, cut in the middle and of no rows at all: the rows that fit are
+    right, means included, and nothing is written behind them (a scale can count its points in the caller's array)."""
+    from dataclasses import replace
+    base = gen.KITTI.with_shape(3, 5001) if which == "kitti" else gen.NUSCENES.with_shape(2, 5001)
+    w = replace(base, grids=(replace(base.grids[0], max_points=cap_fine), base.grids[1]))
+    pts = gen.make_batch(w)["points"]
+    pts[:, 1::2] = pts[:, ::2][:, :pts[:, 1::2].shape[1]]              # two points and more in a voxel
+    refs = [oracle.voxelize(pts, g.min, g.voxel, g.dims, g.max_points) for g in w.grids]
+    M = [r["num_voxels"] for r in refs]
+    br = b200.Bridge(b200.config_from_workload(w))
+    d = torch.from_numpy(pts).cuda()
+    size = w.B * w.N + 64
+    for cap in ([w.B * w.N] * 2, M, [m // 2 + 1 for m in M], [33, 0], [0, 7], [w.B * w.N] * 2):
+        out = {"coords": [torch.full((size, 4), -7, dtype=torch.int32, device="cuda") for _ in range(2)],
+               "counts": [torch.full((size,), -7, dtype=torch.int32, device="cuda") for _ in range(2)],
+               "mean": [torch.full((size, w.C), -7.0, device="cuda") for _ in range(2)], "bev": None,
+               "point_voxel": [torch.full((w.B, w.N), -7, dtype=torch.int32, device="cuda") for _ in range(2)],
+               "num_voxels": torch.full((2,), -7, dtype=torch.int32, device="cuda")}
+        br.voxelize(d, capacity=cap, out=out)
+        over = any(m > c for m, c in zip(M, cap))
+        assert br.status(raise_on_error=False) == (b200.bridge.EMC2_ERR_CAPACITY if over else b200.bridge.EMC2_OK)
+        assert np_(out["num_voxels"]).tolist() == M
+        for s in range(2):
+            n = min(M[s], cap[s])
+            assert np.array_equal(np_(out["coords"][s])[:n], refs[s]["coords"][:n])
+            assert np.array_equal(np_(out["counts"][s])[:n], refs[s]["counts"][:n])
+            assert close(np_(out["mean"][s])[:n], refs[s]["mean"][:n])[0]
+            for k in ("coords", "counts", "mean"):
+                assert bool((out[k][s][n:] == -7).all()), (k, s, cap)
     br.close()
 
 
