@@ -113,7 +113,9 @@ int emc2_bridge_create(const emc2_config_t* config, emc2_bridge_t** out);
  *   d_num_voxels     int32 [2]               number of unique voxels found per scale (true count
  *                                            even when it exceeds capacity[s])
  *   d_bev            float [B, C, Gy, Gx] of grid[1], or NULL: pillar means at (iy, ix), else 0
- * d_points is float [B, N, C].  Rows past num_voxels are left untouched.  All integer outputs
+ * d_points is float [B, N, C].  Rows past num_voxels are left untouched; those before it can hold intermediate
+ * values while the call runs (d_counts is counted up in place on some scales), and a capped scale that reports none
+ * because its lists were refused (EMC2_ERR_INTERNAL) can have rows written.  All integer outputs
  * (coordinates, counts, point rows, the number of voxels) are the same on every run; the means
  * and the BEV image are sums of fp32 reductions whose order is not fixed, so they are
  * reproducible to the comparison tolerance (1e-4 + 1e-5 |x|), not bit for bit.  The same holds

@@ -61,7 +61,8 @@ int validate(const emc2_config_t& c) {
     if (c.device < 0) return EMC2_ERR_BAD_CONFIG;
     if (c.max_batch < 1 || c.max_batch > EMC2_MAX_BATCH) return EMC2_ERR_BAD_CONFIG;
     if (c.max_points < 1) return EMC2_ERR_BAD_CONFIG;
-    // Per-voxel point counts are accumulated in fp32, which is exact up to 2^24.
+    // Where a voxel's points are counted in its accumulator, that is in fp32, which is exact up to 2^24; the lists of cells over
+    // the cap rely on the same limit (see kPointsClamp).
     if ((int64_t)c.max_batch * c.max_points > (int64_t)1 << 24) return EMC2_ERR_BAD_CONFIG;
     if (c.point_floats != 4 && c.point_floats != 5) return EMC2_ERR_BAD_CONFIG;
     for (int s = 0; s < 2; ++s) {

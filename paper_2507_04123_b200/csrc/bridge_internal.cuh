@@ -154,7 +154,7 @@ struct ScanState {
     int words[2];               // words of `marked` to clear, 0 where the marking pass does not keep it
 };
 
-// Where the marking pass notes the tiles that it touches (see keeps_tile_marks), or null.
+// Where the marking pass notes the tiles that it touches (see keeps_tile_marks and kNoteCopies), or null.
 struct TileMarks {
     uint32_t* marked[2];
     uint32_t stride;                        // words from one copy to the next

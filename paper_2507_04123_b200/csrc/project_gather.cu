@@ -232,13 +232,14 @@ struct PrArgs {
 // voxelizer's marking pass (every point marks its cell in both scales' stores, and the BEV image
 // is zeroed, spread over the grid), so that stage 1 starts from marked stores and reads the
 // points once less; the reductions are fire-and-forget and land while the projection computes.
-// kNote: and notes the tiles that they touch (see keeps_notes).  A variant of its own, so that calls without notes have
+// kNote: and notes the tiles that they touch (see keeps_frame_notes).  A variant of its own, so that calls without notes have
 // neither their shared memory nor their code: one frame of 30,000 points and 256 channels 47.2 -> 46.0 us, of 20,000 and 192
 // 39.2 -> 38.0.
 // Bound by instruction issue (0.82 per cycle and scheduler) where the marks' sectors are in L2: the experts are counted by one
 // reduction of packed fields per warp, the words of a frame's notes come from a table, one CTA resets the scan and a warp
-// stores its own pixels.  With ballots per expert, divides for the words and the pixels stored by the CTA four nuScenes-shaped
-// frames took 39.2 us, now 37.3, and 32 frames of 262,144 points 209, now 193; eight KITTI-shaped ones 33.4 either way.
+// stores its own pixels.  With ballots per expert, divides for the words and the pixels stored by the CTA (with notes, us)
+// four nuScenes-shaped frames took 39.4, now 38.0, 32 KITTI-shaped ones of 262,144 points 168.5, now 161, with six cameras 220, now
+// 210; eight of 120,000 points 33.3, now 33.1.
 template <int C, bool kMark, bool kNote = false>
 __global__ void __launch_bounds__(kThreads, 8) project_route_kernel(const __grid_constant__ PrArgs a) {
     __shared__ __align__(16) float suvd[kTile * 3];

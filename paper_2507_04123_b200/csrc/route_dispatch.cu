@@ -93,7 +93,12 @@ inline int scan_threads(int tiles) { return min(max((tiles + 31) / 32 * 32, 128)
 // The counts may still be in the making while this kernel is set up (see launch_chained), so they are not declared read-only.
 // Bound by one round trip to memory and the launch; as one CTA per frame, with the experts one after another, it took 8.5 us by events
 // for eight KITTI-shaped frames and 10.9 for four nuScenes-shaped ones, now 6.8 and 8.5; their calls 192.4 -> 190.7 and 296.1 ->
-// 294.1, one dense frame 69.1 -> 67.8, stage calls with occlusion 126.5 -> 124.7.
+// 294.1, one dense frame 69.1 -> 67.8, stage calls with occlusion 126.5 -> 124.7.  With 16 experts one frame of 120,000 points
+// took 16.8, now 8.7 (the call 43.4 -> 35.9), one of 16,000,000 1,998, now 618; the sum over the experts before grows with them, and
+// is read from L2.  The rows start 2 us earlier, in some small calls ahead of stage 1's rank scan instead of behind it: two frames of
+// 33,333 uniform points 40.9 -> 44.3, three nuScenes-shaped ones of 33,333 51.5 -> 54.2, one of 262,144 with 128 channels 101 -> 106,
+// but 30,000 points with 256 channels 43 -> 33, eight frames of 16,384 uniform points 105 -> 103, 32 KITTI-shaped ones of 4,000 122 ->
+// 118.  Nothing tried that holds the rows back (an ordinary launch, a fork behind vox_count) keeps the one without losing the other.
 __global__ void __launch_bounds__(kScanThreads)
 route_scan_kernel(const int* tile_counts, int* tile_base, int32_t* offsets, int tiles, int E) {
     await_predecessor();

@@ -15,8 +15,9 @@
 //                 fields and the occupied cell ids listed in that order; the bookkeeping of cells over
 //                 the cap is laid out.
 //   vox_accum     every point looks its rank up, writes point_voxel and adds itself to its
-//                 voxels' accumulators with two fp32 vector reductions (offsets from the cell
-//                 corner, the other channels, the count).
+//                 voxels' accumulators with one or two fp32 vector reductions (offsets from the cell
+//                 corner, the other channels).  Points are counted in the words of a table store while they are
+//                 marked; on a bitmap scale here, in the caller's array (four channels, no cap) or in the accumulator.
 //                 Points of cells over the cap go to per-cell lists instead.
 //   vox_finalize  a warp per 32 consecutive voxels: coordinates from the listed cell id, count,
 //                 mean and BEV cell, with contiguous row traffic, and the store back to zero; in the same launch
@@ -116,7 +117,7 @@ vox_mark_kernel(const float* __restrict__ pts, int B, int N, const FastDiv group
 struct ScanArgs {
     ScaleDev s[2];
     int capacity[2];
-    int32_t* counts[2];         // table stores: the kept points of every voxel go straight to the output
+    int32_t* counts[2];         // the caller's: written for a table store, cleared where vox_accum counts in them
     int32_t* num_voxels;
     int* status;
     int tiles[2];               // 8 KB tiles covering this call's B frames
@@ -126,16 +127,18 @@ struct ScanArgs {
 // Two launches.
 //   vox_count   voxels per 8 KB tile of the store and per eighth of it (a part: 32 sectors), their sum per 128 tiles, and a
 //               list of the parts that hold any (most of a fine grid is empty space).  One kernel streams the whole store, a CTA
-//               per four tiles; another, where the marking pass keeps notes (see keeps_notes), reads the noted tiles only.
+//               per four tiles; another, where the marking pass keeps notes (see keeps_frame_notes), reads the noted tiles only.
 //   vox_rank    a warp per listed part finds the voxels before it (groups of tiles before its group, tiles of the group
 //               and parts of the tile before it: a load each), ranks its units or cells and lists the
 //               occupied cells in rank order.
 // The counting is bound by the read of the store or of the noted tiles, vox_rank by the latency of
 // its three dependent round trips and by the parts on the ground plane that hold most voxels: a lane
 // has one sector of 32 bytes, and a warp lists the cells of its 32 sectors together.  Nothing in its loop waits for another
-// warp.  By events, us, a CTA per listed tile with three barriers each / a warp per part of the listed tiles / per listed part:
-// tiny frame 12.6 / 12.9 / 10.7, eight KITTI-shaped frames 34.1 / 32.7 / 28.3, four nuScenes-shaped 34.4 / 30.8 / 30.6, 32 frames
-// of 262,144 points 152 / 137 / 125; the next part's sectors requested ahead: 29.9, 30.3, 125.
+// warp.  By events, us, with a CTA per listed tile and three barriers each / now: tiny frame 12.8 / 11.5, eight KITTI-shaped
+// frames 33.7 / 26.1, four nuScenes-shaped 33.0 / 28.2, 32 KITTI-shaped frames of 262,144 points 146.8 / 99.7, of 524,288, which take
+// more tickets for cells over the cap, 210 / 143.  (As it was first, cells listed by sectors and accumulators of 32 bytes, the
+// second to fourth of these took 28.3, 30.6 and 125, with a warp for the empty parts of the listed tiles too 32.7, 30.8 and 137,
+// with the next part's sectors requested ahead 29.9, 30.3 and 125.)
 __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t x) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
@@ -220,9 +223,9 @@ __global__ void __launch_bounds__(kThreads) vox_count_kernel(const __grid_consta
 }
 
 // The same where the marking pass noted the tiles it touched: only those are looked at (vox_rank clears the notes).  A
-// fixed grid of CTAs, each with at most kThreads groups of four tiles.  us by events, whole stores / noted tiles: eight
-// KITTI-shaped frames (127 MB of stores) 28.7 / 16.9, while project_route, which does the marking, goes from 32.1 to 33.4; four
-// nuScenes-shaped ones 16.8 / 11.4 and 37.3 / 39.5.  See keeps_notes for whole calls.
+// fixed grid of CTAs, each with at most kThreads groups of four tiles.  us by events, without / with notes: eight KITTI-shaped
+// frames (127 MB of stores) 28.5 / 16.8, and project_route, which does the marking, 32.3 / 33.2; four nuScenes-shaped ones 16.9 / 11.5
+// and 35.4 / 37.4; 32 KITTI-shaped ones of 262,144 points 88.5 / 50.0 and 154 / 161.  See keeps_frame_notes for whole calls.
 __global__ void __launch_bounds__(kThreads) vox_count_marked_kernel(const __grid_constant__ ScanArgs a) {
     await_predecessor();
     __shared__ uint32_t s_warp[kCountTiles][kThreads / 32], s_which[kThreads];
